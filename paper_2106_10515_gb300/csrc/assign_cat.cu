@@ -236,11 +236,12 @@ __device__ __forceinline__ int heavy_bit(uint32_t x, const uint32_t *__restrict_
     return (lo < nheavy && hv_item[lo] == x) ? hv_bit[lo] : -1;
 }
 
+template <int W>
 __global__ void k_heavy_masks(int64_t k, const int64_t *__restrict__ coff, const uint32_t *__restrict__ citems,
                               const uint32_t *__restrict__ hv_item, const int16_t *__restrict__ hv_bit, int nheavy,
                               int HW, uint64_t *__restrict__ cmask, int32_t *__restrict__ clen) {
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < k; j += (int64_t)gridDim.x * blockDim.x) {
-        uint64_t m[JX_HW] = {};
+        uint64_t m[W] = {};
         for (int64_t p = coff[j]; p < coff[j + 1]; p++) {
             const int b = heavy_bit(citems[p], hv_item, hv_bit, nheavy);
             if (b >= 0) m[b >> 6] |= 1ull << (b & 63);
@@ -255,7 +256,7 @@ __global__ void k_heavy_masks(int64_t k, const int64_t *__restrict__ coff, const
 // counter array (cleared after use).  Every centre is then scored exactly:
 // J_j = inter / (|A| + |C_j| - inter), compared by cross-multiplication.
 // (The dense path: every centre is scanned per set.  It serves the sets
-// whose light candidates overflow the shared-memory table of k_jac_light;
+// with more items than k_jac_tiled takes;
 // rows lists them, na_fix >= 0 replaces |A| by a fixed size.)
 __global__ void __launch_bounds__(256) k_assign_jaccard(
     int64_t n, const int64_t *__restrict__ off, const uint32_t *__restrict__ items, int64_t k,
@@ -335,30 +336,51 @@ __global__ void __launch_bounds__(256) k_assign_jaccard(
     }
 }
 
-// Exact Jaccard argmax, tiled over the centres.  A block takes JX_S sets
-// (one warp each) and walks the centres in tiles of KT; per tile, every
-// item of a set reads the part of its posting list (centres containing the
-// item, ascending) that falls in the tile, found from precomputed per-tile
-// offsets, and adds one to the set's counter of each centre there (packed
-// 8- or 16-bit counters in shared memory: a counter counts the set's light
-// items in one centre, at most the variant's MAXI).  The counters are
-// then |A n C_j| for every centre of the tile: J_j = I / (|A| + |C_j| - I) is
-// compared exactly (64-bit cross products), larger fraction then smaller
-// index; with no positive J the label is 0.  Sets with more than MAXI
-// items are listed for the dense path.
-constexpr int JX_S = 8;
-constexpr int JX_THREADS = 32 * JX_S;
-// NARROW: sets of at most 128 items, 8-bit counters, tiles of 8192 centres
-// (74 KB of shared memory: three blocks per SM); otherwise up to 512 items,
-// 16-bit counters, tiles of 4096 centres (104 KB).
+// Exact Jaccard argmax, tiled over the centres; a warp per set, warps
+// independent of one another.  Per tile of `kt` centres every item of the set
+// reads the part of its posting list (centres containing the item, ascending)
+// that falls in the tile and adds one to the warp's counter of each centre
+// there (packed 8- or 16-bit counters in shared memory: a counter counts the
+// set's light items in one centre, at most MAXI), so the counters plus the
+// heavy items' bitmask give |A n C_j|.
+//
+// Visiting every (set, centre) pair is what a plain form pays for: scoring a
+// pair costs about 15 operations, a set meets 8,192 centres per tile, and
+// the few hundred most frequent items alone give 9 of 10 counter increments.
+// So there are two passes:
+//  k_jac_prune (every set): the JX_MW * 64 most frequent items stay out of
+//    the counters.  A centre beats or ties the best fraction bn / bd so far
+//    only if |A n C| >= bn (|A| + |C|) / (bn + bd), so its counter is at least
+//    that (with the tile's smallest |C|) less the set's number of frequent
+//    items: the warp tests the counters of a 16-byte load against this
+//    threshold with one add and mask per word and scores the few that pass
+//    exactly (64-bit cross products, larger fraction then smaller index; with
+//    no positive J the label is 0).  The centre of a tile's largest counter
+//    gives the first bound; a tile met while the threshold is not positive is
+//    taken again at the end, and if it still is not (a set unlike every
+//    centre), the set goes to the second pass.
+//  k_jac_count (those sets): only the 64 most frequent items stay out, and
+//    every centre is scored, lane per centre.
+// Sets with more than MAXI items are listed for the dense path.
+// 2,000,000 sets of 59 items against 47,686 centres (mean 58 items): the
+// counters get 3,200 increments per set instead of 28,600, and the two passes
+// take 44 + 37 ms; scoring every pair took 173 ms.  500,000 DOPH rows of 400
+// tokens against 425 centres: 4.5 + 5.0 ms, before 31 ms.
+constexpr int JX_WARPS = 8;
+constexpr int JX_THREADS = 32 * JX_WARPS;
+constexpr int JX_MW = 8;  // mask words of the frequent items k_jac_prune leaves out
+// NARROW: sets of at most 128 items, 8-bit counters, tiles of up to 8192
+// centres; otherwise up to 512 items, 16-bit counters, tiles of up to 4096
+// (8 KB of counters per warp either way; fewer when k is smaller).
 template <bool NARROW> struct Jx {
-    static constexpr int KT = NARROW ? 8192 : 4096;  // centres per tile
+    static constexpr int KT = NARROW ? 8192 : 4096;  // centres per tile, at most
     static constexpr int MAXI = NARROW ? 128 : 512;  // items per set on the tiled path
     static constexpr int LG = NARROW ? 2 : 1;        // log2 counters per word
     static constexpr int CBITS = 32 >> LG;
     static constexpr uint32_t CMASK = NARROW ? 0xFFu : 0xFFFFu;
-    static constexpr int CW = KT >> LG;              // counter words per set
-    static constexpr size_t SMEM = (size_t)JX_S * CW * 4 + (size_t)JX_S * MAXI * (4 + 4 + 2);
+    static constexpr uint32_t ONES = NARROW ? 0x01010101u : 0x00010001u;
+    static constexpr uint32_t TOP = NARROW ? 0x80u : 0x8000u;
+    static constexpr int STEP = 128 << LG;           // counters per warp-wide 16-byte load
 };
 
 // the largest set: max over i of off[i + 1] - off[i]
@@ -391,189 +413,328 @@ __global__ void k_tile_offsets(int64_t nr, const int64_t *__restrict__ post_off,
     }
 }
 
+// tile_min[t] = the smallest |C| among the centres of tile t (block per tile)
+__global__ void __launch_bounds__(256) k_tile_min_len(int64_t k, int kt, const int32_t *__restrict__ clen,
+                                                      int32_t *__restrict__ tile_min) {
+    __shared__ int s_min;
+    if (threadIdx.x == 0) s_min = INT32_MAX;
+    __syncthreads();
+    const int64_t c0 = (int64_t)blockIdx.x * kt, c1 = min(k, c0 + kt);
+    int m = INT32_MAX;
+    for (int64_t c = c0 + threadIdx.x; c < c1; c += 256) m = min(m, clen[c]);
+    atomicMin(&s_min, m);
+    __syncthreads();
+    if (threadIdx.x == 0) tile_min[blockIdx.x] = s_min;
+}
+
+// posting entries as centre indices within their tile
+__global__ void k_tile_local(int64_t m, const uint32_t *__restrict__ post_centre, int kt, uint16_t *__restrict__ out) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x)
+        out[e] = (uint16_t)(post_centre[e] % (uint32_t)kt);
+}
+
+// lut[item] for items up to the largest in any centre: -2 - rank for one of
+// the 64 JX_MW most frequent items, else its posting list (>= 0), -1 for an
+// item no centre holds
+__global__ void k_item_lut(int64_t nlight, const uint32_t *__restrict__ litem, int32_t *__restrict__ lut) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nlight; e += (int64_t)gridDim.x * blockDim.x)
+        lut[litem[e]] = (int32_t)e;
+}
+__global__ void k_freq_lut(int nfreq, const uint32_t *__restrict__ fq_item, const int16_t *__restrict__ fq_bit,
+                           int32_t *__restrict__ lut) {
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nfreq; q += gridDim.x * blockDim.x)
+        lut[fq_item[q]] = -2 - (int32_t)fq_bit[q];
+}
+// posting list of each frequent item by rank (ranks below 64 JX_HW have none)
+__global__ void k_freq_list(int nfreq, const int64_t *__restrict__ fq_run, const int16_t *__restrict__ fq_bit,
+                            const int64_t *__restrict__ lrun_pos, int32_t *__restrict__ fq_list) {
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nfreq; q += gridDim.x * blockDim.x)
+        fq_list[fq_bit[q]] = fq_bit[q] < 64 * JX_HW ? -1 : (int32_t)lrun_pos[fq_run[q]];
+}
+
+// how the kernels find an item: the table when the items are small numbers
+// (n_lut entries), else binary searches
+struct JxIndex {
+    const int32_t *lut;
+    int64_t n_lut;
+    const uint32_t *fq_item;  // frequent items ascending, their ranks
+    const int16_t *fq_bit;
+    int nfreq;
+    const uint32_t *post_item;  // items with posting lists, ascending
+    int64_t n_post_items;
+    __device__ __forceinline__ int32_t find(uint32_t it) const {
+        if (lut) return (int64_t)it < n_lut ? lut[it] : -1;
+        const int hb = heavy_bit(it, fq_item, fq_bit, nfreq);
+        if (hb >= 0) return -2 - hb;
+        int64_t lo = 0, hi = n_post_items;
+        while (lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (post_item[mid] < it) lo = mid + 1;
+            else hi = mid;
+        }
+        return lo < n_post_items && post_item[lo] == it ? (int32_t)lo : -1;
+    }
+};
+
+struct JxArgs {
+    int64_t n;  // sets
+    const int64_t *off;
+    const uint32_t *items;
+    int na_fix;
+    int64_t k;
+    int kt, ntiles;
+    const int32_t *clen, *tile_min, *tile_off;
+    const uint16_t *post_local;
+    JxIndex X;
+    int32_t *labels;
+};
+
+// Counts one tile: every item of the warp's set adds one to the counter of
+// each centre of its posting list there.  The lanes take 32 items at a time; a
+// prefix sum of their range lengths turns the ranges into one run of entries,
+// walked 32 at a time with every lane busy (a range is 16 entries on
+// average).  Returns the lane's largest (count << 16 | counter) it produced.
+template <class C>
+__device__ __forceinline__ uint32_t jx_count(uint32_t *cw, const int32_t *ridx, int ni, int t, const JxArgs &A) {
+    const int lane = threadIdx.x & 31, ld = A.ntiles + 1;
+    uint32_t lm = 0;
+    for (int q0 = 0; q0 < ni; q0 += 32) {
+        const int32_t r = q0 + lane < ni ? ridx[q0 + lane] : -1;
+        int ps = 0, len = 0;
+        if (r >= 0) {
+            ps = A.tile_off[(int64_t)r * ld + t];
+            len = A.tile_off[(int64_t)r * ld + t + 1] - ps;
+        }
+        int inc = len;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        const int tot = __shfl_sync(0xffffffffu, inc, 31);
+        const int ex = inc - len, base = ps - ex;
+#pragma unroll 2
+        for (int e0 = 0; e0 < tot; e0 += 32) {
+            const int e = e0 + lane;
+            int src = 0;  // the last range starting at or before entry e
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (__shfl_sync(0xffffffffu, ex, src + o) <= e) src += o;
+            const int at = __shfl_sync(0xffffffffu, base, src) + e;
+            if (e < tot) {
+                const uint32_t cc = A.post_local[at];
+                const int sh = (cc & ((1 << C::LG) - 1)) * C::CBITS;
+                const uint32_t old = atomicAdd(&cw[cc >> C::LG], 1u << sh);
+                lm = max(lm, (((old >> sh) & C::CMASK) << 16) + 65536u + cc);
+            }
+        }
+    }
+    return lm;
+}
+
+// the best centre of a set: larger fraction n / d, then smaller index
+struct JxBest {
+    uint32_t n = 0, d = 1;
+    int j = 0x7FFFFFFF;
+    // |A| + |C| < 2^16: both cross products fit 32 bits
+    __device__ __forceinline__ void push(uint32_t on, uint32_t od, int oj) {
+        const uint32_t l = on * d, r = n * od;
+        if (l > r || (l == r && oj < j)) {
+            n = on;
+            d = od;
+            j = oj;
+        }
+    }
+    __device__ __forceinline__ void warp_merge() {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            push(__shfl_xor_sync(0xffffffffu, n, o), __shfl_xor_sync(0xffffffffu, d, o),
+                 __shfl_xor_sync(0xffffffffu, j, o));
+    }
+    // the smallest |A n C| that still beats or ties it, |C| >= cmin
+    __device__ __forceinline__ uint32_t need(uint32_t na, uint32_t cmin) const {
+        return max((n * (na + cmin) + n + d - 1) / (n + d), 1u);
+    }
+};
+
 template <bool NARROW>
-__global__ void __launch_bounds__(JX_THREADS) k_jac_tiled(
-    int64_t n, const int64_t *__restrict__ off, const uint32_t *__restrict__ items, int na_fix, int64_t k,
-    const int32_t *__restrict__ clen, const uint64_t *__restrict__ cmask, const uint32_t *__restrict__ hv_item,
-    const int16_t *__restrict__ hv_bit, int nheavy, int HW, const uint32_t *__restrict__ post_item,
-    const int32_t *__restrict__ tile_off, int ntiles, int64_t n_post_items, const uint32_t *__restrict__ post_centre,
-    int32_t *__restrict__ labels, int32_t *__restrict__ ovf_rows, unsigned long long *__restrict__ n_ovf) {
+__global__ void __launch_bounds__(JX_THREADS, 3) k_jac_prune(JxArgs A, const uint64_t *__restrict__ fmask, int FW,
+                                                             int32_t *__restrict__ ovf_rows,
+                                                             unsigned long long *__restrict__ n_ovf,
+                                                             int4 *__restrict__ hard_rows,
+                                                             unsigned long long *__restrict__ n_hard) {
     using C = Jx<NARROW>;
-    __shared__ unsigned long long s_am[JX_S][JX_HW];  // the sets' heavy-item masks
-    extern __shared__ uint32_t jx_smem[];
-    uint32_t *cnt = jx_smem;                                          // [S][KT / 2]
-    int32_t *ridx = reinterpret_cast<int32_t *>(cnt + JX_S * C::CW);        // [S][MAXI]: posting list of each item
-    int32_t *rps = ridx + JX_S * C::MAXI;                                  // [S][MAXI]: its range in the tile
-    uint16_t *rlen = reinterpret_cast<uint16_t *>(rps + JX_S * C::MAXI);   // [S][MAXI]
-    __shared__ int s_ni[JX_S];
-    __shared__ int64_t s_na[JX_S];
-    __shared__ uint32_t r_n[JX_S][JX_S], r_d[JX_S][JX_S];
-    __shared__ int r_j[JX_S][JX_S];
+    extern __shared__ uint4 jx_smem[];
+    __shared__ unsigned long long s_am[JX_WARPS][JX_MW];  // the set's frequent items
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int e = threadIdx.x; e < JX_S * C::CW; e += blockDim.x) cnt[e] = 0;
-    const int64_t ngroups = (n + JX_S - 1) / JX_S;
-    for (int64_t g = blockIdx.x; g < ngroups; g += gridDim.x) {
-        // the warp's set: posting ranges of its items
-        const int64_t i = g * JX_S + w;
-        int ni = 0;
-        if (i < n) {
-            const int64_t s0 = off[i], e0 = off[i + 1];
-            ni = (int)min(e0 - s0, (int64_t)C::MAXI + 1);
-            if (ni > C::MAXI) {
-                if (lane == 0) ovf_rows[atomicAdd(n_ovf, 1ull)] = (int32_t)i;
-                ni = 0;
-            }
-            if (lane < JX_HW) s_am[w][lane] = 0ull;
-            __syncwarp();
-            for (int p = lane; p < ni; p += 32) {
-                const uint32_t it = items[s0 + p];
-                const int hb = heavy_bit(it, hv_item, hv_bit, nheavy);
-                if (hb >= 0) {
-                    atomicOr(&s_am[w][hb >> 6], 1ull << (hb & 63));
-                    ridx[w * C::MAXI + p] = -1;
-                    continue;
-                }
-                int64_t lo = 0, hi = n_post_items;
-                while (lo < hi) {
-                    const int64_t mid = (lo + hi) >> 1;
-                    if (post_item[mid] < it) lo = mid + 1;
-                    else hi = mid;
-                }
-                const bool f = lo < n_post_items && post_item[lo] == it;
-                ridx[w * C::MAXI + p] = f ? (int32_t)lo : -1;
-            }
-            if (lane == 0) {
-                s_ni[w] = ni;
-                s_na[w] = na_fix >= 0 ? na_fix : e0 - s0;
-            }
-        } else if (lane == 0) {
-            s_ni[w] = 0;
-            s_na[w] = 0;
-            for (int h = 0; h < JX_HW; h++) s_am[w][h] = 0ull;
+    const int nv = A.kt / C::STEP;  // 16-byte loads per lane and tile
+    uint4 *c4 = jx_smem + (size_t)w * nv * 32;
+    uint32_t *cw = reinterpret_cast<uint32_t *>(c4);
+    int32_t *ridx = reinterpret_cast<int32_t *>(jx_smem + (size_t)JX_WARPS * nv * 32) + w * C::MAXI;
+    unsigned long long *am = s_am[w];
+    for (int v = lane; v < nv * 32; v += 32) c4[v] = make_uint4(0u, 0u, 0u, 0u);
+    const int64_t nwarps = (int64_t)gridDim.x * JX_WARPS;
+    for (int64_t i = (int64_t)blockIdx.x * JX_WARPS + w; i < A.n; i += nwarps) {
+        const int64_t s0 = A.off[i], e0 = A.off[i + 1];
+        if (e0 - s0 > C::MAXI) {
+            if (lane == 0) ovf_rows[atomicAdd(n_ovf, 1ull)] = (int32_t)i;
+            continue;
         }
-        __syncthreads();
-        uint32_t bn[JX_S], bd[JX_S], na[JX_S];
-        uint64_t am[JX_S][JX_HW];
-        int bj[JX_S];
-#pragma unroll
-        for (int q = 0; q < JX_S; q++) {
-            bn[q] = 0;
-            bd[q] = 1;
-            bj[q] = 0x7FFFFFFF;
-            na[q] = (uint32_t)s_na[q];
-#pragma unroll
-            for (int h = 0; h < JX_HW; h++) am[q][h] = s_am[q][h];
+        const int ni = (int)(e0 - s0);
+        const uint32_t na = (uint32_t)(A.na_fix >= 0 ? A.na_fix : ni);
+        __syncwarp();
+        if (lane < JX_MW) am[lane] = 0ull;
+        __syncwarp();
+        // the items: frequent ones into the mask, the others' posting lists
+        int mine = 0;
+#pragma unroll 2
+        for (int p = lane; p < ni; p += 32) {
+            const int32_t r = A.X.find(A.items[s0 + p]);
+            ridx[p] = r;
+            if (r < -1) {
+                const int hb = -2 - r;
+                atomicOr(&am[hb >> 6], 1ull << (hb & 63));
+                mine++;
+            }
         }
-        for (int64_t c0 = 0; c0 < k; c0 += C::KT) {
-            const int64_t c1 = min(k, c0 + C::KT);
-            // counting: lanes walk consecutive entries of one posting list
-            const int niw = s_ni[w];
-            uint32_t *cw = cnt + w * C::CW;
-            const int t = (int)(c0 / C::KT);
-            // the items' ranges in this tile, lane per item (independent loads)
-            for (int q = lane; q < niw; q += 32) {
-                const int32_t r = ridx[w * C::MAXI + q];
-                int32_t ps = 0, pe = 0;
-                if (r >= 0) {
-                    ps = tile_off[(int64_t)r * (ntiles + 1) + t];
-                    pe = tile_off[(int64_t)r * (ntiles + 1) + t + 1];
-                }
-                rps[w * C::MAXI + q] = ps;
-                rlen[w * C::MAXI + q] = (uint16_t)(pe - ps);
+        const int hcnt = __reduce_add_sync(0xffffffffu, mine);  // frequent items of the set
+        __syncwarp();
+        JxBest best;  // the same on every lane
+        auto score = [&](int64_t c, uint32_t l, JxBest &b) {
+            uint32_t in = l;
+            for (int h = 0; h < FW; h++) in += __popcll(am[h] & fmask[c * FW + h]);
+            if (in) b.push(in, na + (uint32_t)A.clen[c] - in, (int)c);
+        };
+        // tiles met without a positive threshold, taken again at the end
+        uint64_t again = 0;
+        bool hard = false;
+        for (int tt = 0, t = 0; !hard; tt++) {
+            const bool second = tt >= A.ntiles;
+            if (!second) {
+                t = tt;
+            } else {
+                if (!again) break;
+                t = __ffsll((long long)again) - 1;
+                again &= again - 1;
             }
+            const int64_t c0 = (int64_t)t * A.kt;
+            const uint32_t cmin = (uint32_t)A.tile_min[t];
+            int need = (int)best.need(na, cmin) - hcnt;
+            if (second && need <= 0) {
+                hard = true;
+                break;
+            }
+            const uint32_t lm = __reduce_max_sync(0xffffffffu, jx_count<C>(cw, ridx, ni, t, A));
             __syncwarp();
-            // short ranges: a lane walks one item's entries
-            for (int q = lane; q < niw; q += 32) {
-                const int len = rlen[w * C::MAXI + q];
-                if (len == 0 || len >= 32) continue;
-                const int32_t ps = rps[w * C::MAXI + q];
-                for (int e = 0; e < len; e++) {
-                    const int cc = (int)((int64_t)post_centre[ps + e] - c0);
-                    atomicAdd(&cw[cc >> C::LG], 1u << ((cc & ((1 << C::LG) - 1)) * C::CBITS));
+            if (need <= 0) {
+                // the centre of the tile's largest counter as a first bound
+                if (lm >> 16) score(c0 + (lm & 0xFFFFu), lm >> 16, best);
+                need = (int)best.need(na, cmin) - hcnt;
+                if (need <= 0) {
+                    if (t < 64) again |= 1ull << t;
+                    else hard = true;
                 }
             }
-            // long ranges: the warp walks one item's entries, lane per entry
-            for (int q = 0; q < niw; q++) {
-                const int len = rlen[w * C::MAXI + q];
-                if (len < 32) continue;
-                const int32_t ps = rps[w * C::MAXI + q];
-#pragma unroll 4
-                for (int p = lane; p < len; p += 32) {
-                    const int cc = (int)((int64_t)post_centre[ps + p] - c0);
-                    atomicAdd(&cw[cc >> C::LG], 1u << ((cc & ((1 << C::LG) - 1)) * C::CBITS));
-                }
+            if (need <= 0 || need > (int)(lm >> 16)) {  // taken again, or above every counter
+                for (int v = 0; v < nv; v++) c4[v * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
+                __syncwarp();
+                continue;
             }
-            __syncwarp();
-            __syncthreads();
-            // scoring: thread per centre of the tile, all JX_S sets
-            for (int cc = threadIdx.x; cc < (int)(c1 - c0); cc += blockDim.x) {
-                const int64_t c = c0 + cc;
-                const int64_t cl = clen[c];
-                uint64_t cm[JX_HW];
+            for (int v = 0; v < nv; v++) {
+                const uint4 q = c4[v * 32 + lane];
+                c4[v * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
+                if (need > (int)C::TOP) continue;  // the bound rose above every counter
+                const uint32_t ww[4] = {q.x, q.y, q.z, q.w};
+                // a counter b <= TOP reaches `need` exactly when b + TOP - need sets its top bit
+                const uint32_t add = (C::TOP - (uint32_t)need) * C::ONES, top = C::TOP * C::ONES;
+                uint32_t hit[4];
 #pragma unroll
-                for (int h = 0; h < JX_HW; h++) cm[h] = h < HW ? cmask[c * HW + h] : 0ull;
+                for (int u = 0; u < 4; u++) hit[u] = (ww[u] + add) & top;
+                JxBest b = best;
+                if (hit[0] | hit[1] | hit[2] | hit[3]) {
 #pragma unroll
-                for (int q = 0; q < JX_S; q++) {
-                    uint32_t in = (cnt[q * C::CW + (cc >> C::LG)] >> ((cc & ((1 << C::LG) - 1)) * C::CBITS)) & C::CMASK;
-#pragma unroll
-                    for (int h = 0; h < JX_HW; h++) in += __popcll(am[q][h] & cm[h]);
-                    if (in) {
-                        // |A| + |C| < 2^16: both cross products fit 32 bits
-                        const uint32_t un = na[q] + (uint32_t)cl - in;
-                        const uint32_t l = in * bd[q], r = bn[q] * un;
-                        if (l > r || (l == r && (int)c < bj[q])) {
-                            bn[q] = in;
-                            bd[q] = un;
-                            bj[q] = (int)c;
+                    for (int u = 0; u < 4; u++)
+                        for (uint32_t m = hit[u]; m; m &= m - 1) {
+                            const int p = (__ffs((int)m) - 1) / C::CBITS;
+                            score(c0 + ((((v * 32 + lane) * 4 + u) << C::LG) + p), (ww[u] >> (p * C::CBITS)) & C::CMASK, b);
                         }
-                    }
+                }
+                if (__any_sync(0xffffffffu, b.j != best.j)) {
+                    b.warp_merge();
+                    best = b;
+                    need = (int)best.need(na, cmin) - hcnt;  // does not fall: stays positive
                 }
             }
-            __syncthreads();
-            for (int e = threadIdx.x; e < JX_S * C::CW; e += blockDim.x) cnt[e] = 0;
-            __syncthreads();
+            __syncwarp();
         }
-        // per set: reduce the threads' bests (warp, then across warps)
-#pragma unroll
-        for (int q = 0; q < JX_S; q++) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const uint32_t on = __shfl_xor_sync(0xffffffffu, bn[q], o);
-                const uint32_t od = __shfl_xor_sync(0xffffffffu, bd[q], o);
-                const int oj = __shfl_xor_sync(0xffffffffu, bj[q], o);
-                const uint32_t l = on * bd[q], r = bn[q] * od;
-                if (l > r || (l == r && oj < bj[q])) {
-                    bn[q] = on;
-                    bd[q] = od;
-                    bj[q] = oj;
-                }
-            }
-            if (lane == 0) {
-                r_n[q][w] = bn[q];
-                r_d[q][w] = bd[q];
-                r_j[q][w] = bj[q];
-            }
+        // no positive J: every fraction is 0 and the smallest index wins
+        if (lane == 0) {
+            if (hard) hard_rows[atomicAdd(n_hard, 1ull)] = make_int4((int)i, (int)best.n, (int)best.d, best.j);
+            else A.labels[i] = best.n > 0 ? best.j : 0;
         }
-        __syncthreads();
-        if (threadIdx.x < JX_S) {
-            const int q = threadIdx.x;
-            uint32_t n0 = 0, d0 = 1;
-            int j0 = 0x7FFFFFFF;
-            for (int v = 0; v < JX_S; v++) {
-                const uint32_t l = r_n[q][v] * d0, r = n0 * r_d[q][v];
-                if (l > r || (l == r && r_j[q][v] < j0)) {
-                    n0 = r_n[q][v];
-                    d0 = r_d[q][v];
-                    j0 = r_j[q][v];
-                }
-            }
-            const int64_t ii = g * JX_S + q;
-            // no positive J: every fraction is 0 and the smallest index wins
-            if (ii < n) labels[ii] = (n0 > 0 && j0 != 0x7FFFFFFF) ? j0 : 0;
-        }
-        __syncthreads();
     }
 }
+
+template <bool NARROW>
+__global__ void __launch_bounds__(JX_THREADS, 3) k_jac_count(JxArgs A, const uint64_t *__restrict__ cmask, int HW,
+                                                             const int32_t *__restrict__ fq_list,
+                                                             const int4 *__restrict__ rows,
+                                                             const unsigned long long *__restrict__ n_rows) {
+    using C = Jx<NARROW>;
+    extern __shared__ uint4 jx_smem[];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int nv = A.kt / C::STEP;
+    uint4 *c4 = jx_smem + (size_t)w * nv * 32;
+    uint32_t *cw = reinterpret_cast<uint32_t *>(c4);
+    int32_t *ridx = reinterpret_cast<int32_t *>(jx_smem + (size_t)JX_WARPS * nv * 32) + w * C::MAXI;
+    for (int v = lane; v < nv * 32; v += 32) c4[v] = make_uint4(0u, 0u, 0u, 0u);
+    const int64_t nwarps = (int64_t)gridDim.x * JX_WARPS, nr = (int64_t)*n_rows;
+    for (int64_t q = (int64_t)blockIdx.x * JX_WARPS + w; q < nr; q += nwarps) {
+        const int4 row = rows[q];  // the set and its best centre so far
+        const int64_t i = row.x;
+        const int64_t s0 = A.off[i];
+        const int ni = (int)(A.off[i + 1] - s0);  // <= MAXI: the first pass listed it
+        const uint32_t na = (uint32_t)(A.na_fix >= 0 ? A.na_fix : ni);
+        uint64_t am = 0;
+        __syncwarp();
+#pragma unroll 2
+        for (int p = lane; p < ni; p += 32) {
+            int32_t r = A.X.find(A.items[s0 + p]);
+            if (r < -1) {
+                const int hb = -2 - r;
+                if (hb < 64 * JX_HW) am |= 1ull << hb;
+                r = fq_list[hb];
+            }
+            ridx[p] = r;
+        }
+        __syncwarp();
+        am = ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(am >> 32)) << 32) |
+             __reduce_or_sync(0xffffffffu, (uint32_t)am);
+        JxBest best;
+        best.n = (uint32_t)row.y;
+        best.d = (uint32_t)row.z;
+        best.j = row.w;
+        for (int t = 0; t < A.ntiles; t++) {
+            const int64_t c0 = (int64_t)t * A.kt;
+            jx_count<C>(cw, ridx, ni, t, A);
+            __syncwarp();
+            const uint32_t need = best.need(na, (uint32_t)A.tile_min[t]);
+            const int nc = (int)min((int64_t)A.kt, A.k - c0);
+#pragma unroll 4
+            for (int cc = lane; cc < nc; cc += 32) {
+                uint32_t in = (cw[cc >> C::LG] >> ((cc & ((1 << C::LG) - 1)) * C::CBITS)) & C::CMASK;
+                if (HW) in += __popcll(am & cmask[c0 + cc]);
+                if (in >= need) best.push(in, na + (uint32_t)A.clen[c0 + cc] - in, (int)(c0 + cc));
+            }
+            best.warp_merge();
+            __syncwarp();
+            for (int v = lane; v < nv * 32; v += 32) c4[v] = make_uint4(0u, 0u, 0u, 0u);
+            __syncwarp();
+        }
+        if (lane == 0) A.labels[i] = best.n > 0 ? best.j : 0;
+    }
+}
+static_assert(JX_HW == 1, "k_jac_count holds one mask word per centre");
 
 }  // namespace
 
@@ -778,20 +939,25 @@ geek_status jaccard_core(geek_ctx *ctx, Scratch &scr, const int64_t *off, const 
     std::vector<int32_t> ord(ni);
     GK_CUDA(ctx, cudaStreamSynchronize(st));
     for (int64_t r = 0; r < ni; r++) ord[r] = (int32_t)r;
-    const int64_t hmax = std::min<int64_t>(64 * JX_HW, ni);
-    std::partial_sort(ord.begin(), ord.begin() + hmax, ord.end(), [&](int32_t a, int32_t b) {
+    const int64_t fmax = std::min<int64_t>(64 * JX_MW, ni), hmax = std::min<int64_t>(64 * JX_HW, ni);
+    std::partial_sort(ord.begin(), ord.begin() + fmax, ord.end(), [&](int32_t a, int32_t b) {
         const int64_t la = hrs[a + 1] - hrs[a], lb = hrs[b + 1] - hrs[b];
         return la != lb ? la > lb : a < b;
     });
-    int nheavy = 0;
-    while (nheavy < hmax && hrs[ord[nheavy] + 1] - hrs[ord[nheavy]] >= 2) nheavy++;
-    const int HW = (nheavy + 63) / 64;
+    int nfreq = 0;  // frequent items, by rank: the first 64 JX_HW of them are the heavy ones
+    while (nfreq < fmax && hrs[ord[nfreq] + 1] - hrs[ord[nfreq]] >= 2) nfreq++;
+    const int nheavy = (int)std::min<int64_t>(nfreq, hmax);
+    const int HW = (nheavy + 63) / 64, FW = (nfreq + 63) / 64;
+    std::vector<int32_t> fq_runs(ord.begin(), ord.begin() + nfreq);
+    std::sort(fq_runs.begin(), fq_runs.end());
+    std::vector<int16_t> f_bit(nfreq);
     std::vector<int64_t> h_is(ni, 0);
     std::vector<int32_t> hv_runs(ord.begin(), ord.begin() + nheavy);
     std::sort(hv_runs.begin(), hv_runs.end());  // runs ascend with the item value
     std::vector<int16_t> h_bit(nheavy);
     std::vector<int32_t> rank_of(ni, -1);
-    for (int b = 0; b < nheavy; b++) rank_of[ord[b]] = b;  // bit = rank by posting length
+    for (int b = 0; b < nfreq; b++) rank_of[ord[b]] = b;  // bit = rank by posting length
+    for (int q = 0; q < nfreq; q++) f_bit[q] = (int16_t)rank_of[fq_runs[q]];
     for (int q = 0; q < nheavy; q++) {
         h_is[hv_runs[q]] = 1;
         h_bit[q] = (int16_t)rank_of[hv_runs[q]];
@@ -809,7 +975,23 @@ geek_status jaccard_core(geek_ctx *ctx, Scratch &scr, const int64_t *off, const 
     GK_TRY(scr.alloc(&lent_pos, std::max<int64_t>(ni, 1)));
     GK_TRY(scr.alloc(&nlight, 1));
     GK_TRY(scr.alloc(&nlent, 1));
+    uint32_t *fq_item;
+    int16_t *fq_bit;
+    int64_t *fq_run_dev;
+    int32_t *fq_list;
+    GK_TRY(scr.alloc(&fq_item, std::max(1, nfreq)));
+    GK_TRY(scr.alloc(&fq_bit, std::max(1, nfreq)));
+    GK_TRY(scr.alloc(&fq_run_dev, std::max(1, nfreq)));
+    GK_TRY(scr.alloc(&fq_list, std::max(1, nfreq)));
     GK_CUDA(ctx, cudaMemcpyAsync(is_heavy, h_is.data(), 8 * ni, cudaMemcpyHostToDevice, st));
+    if (nfreq) {
+        std::vector<int64_t> fq_r64(fq_runs.begin(), fq_runs.end());
+        GK_CUDA(ctx, cudaMemcpyAsync(fq_run_dev, fq_r64.data(), 8 * nfreq, cudaMemcpyHostToDevice, st));
+        GK_CUDA(ctx, cudaMemcpyAsync(fq_bit, f_bit.data(), 2 * nfreq, cudaMemcpyHostToDevice, st));
+        GK_COUNT();
+        k_run_items<<<G(ctx, nfreq), 256, 0, st>>>(nfreq, fq_run_dev, rs, ikey, fq_item);
+        GK_LAUNCH(ctx);
+    }
     if (nheavy) {
         std::vector<int64_t> hv_r64(hv_runs.begin(), hv_runs.end());
         GK_CUDA(ctx, cudaMemcpyAsync(hv_run_dev, hv_r64.data(), 8 * nheavy, cudaMemcpyHostToDevice, st));
@@ -836,12 +1018,20 @@ geek_status jaccard_core(geek_ctx *ctx, Scratch &scr, const int64_t *off, const 
     k_light_emit<<<G(ctx, ni), 256, 0, st>>>(ni, rs, ikey, pairs, is_heavy, lrun_pos, lent_pos, d_litem, d_loff,
                                              d_lcentre, nlent, h_nlight);
     GK_LAUNCH(ctx);
-    uint64_t *cmask;
+    if (nfreq) {
+        GK_COUNT();
+        k_freq_list<<<G(ctx, nfreq), 256, 0, st>>>(nfreq, fq_run_dev, fq_bit, lrun_pos, fq_list);
+        GK_LAUNCH(ctx);
+    }
+    uint64_t *cmask, *fmask;
     int32_t *clen, *counts;
     GK_TRY(scr.alloc(&cmask, (size_t)k * std::max(HW, 1)));
     GK_TRY(scr.alloc(&clen, k));
     GK_COUNT();
-    k_heavy_masks<<<G(ctx, k), 256, 0, st>>>(k, coff, citems, hv_item, hv_bit, nheavy, HW, cmask, clen);
+    k_heavy_masks<JX_HW><<<G(ctx, k), 256, 0, st>>>(k, coff, citems, hv_item, hv_bit, nheavy, HW, cmask, clen);
+    GK_TRY(scr.alloc(&fmask, (size_t)k * std::max(FW, 1)));
+    GK_COUNT();
+    k_heavy_masks<JX_MW><<<G(ctx, k), 256, 0, st>>>(k, coff, citems, fq_item, fq_bit, nfreq, FW, fmask, clen);
     GK_LAUNCH(ctx);
     if (nci > 0x7FFFFFFFLL) return set_error(ctx, GEEK_ERR_UNSUPPORTED, "more than 2^31 centre items");
     // the tiled kernel compares fractions in 32 bits: |A| <= MAXI (else the
@@ -849,6 +1039,7 @@ geek_status jaccard_core(geek_ctx *ctx, Scratch &scr, const int64_t *off, const 
     // more than its MAXI items
     bool tiled_ok = na_fix < 32768;
     unsigned long long h_amax = 0, *d_amax;
+    uint64_t h_last = 0;  // the largest item of any centre
     GK_TRY(scr.alloc(&d_amax, 1));
     GK_CUDA(ctx, cudaMemsetAsync(d_amax, 0, sizeof(unsigned long long), st));
     if (na_fix < 0 && n > 0) {
@@ -860,6 +1051,9 @@ geek_status jaccard_core(geek_ctx *ctx, Scratch &scr, const int64_t *off, const 
         std::vector<int64_t> hco(k + 1);
         GK_CUDA(ctx, cudaMemcpyAsync(hco.data(), coff, 8 * (k + 1), cudaMemcpyDeviceToHost, st));
         GK_CUDA(ctx, cudaMemcpyAsync(&h_amax, d_amax, sizeof h_amax, cudaMemcpyDeviceToHost, st));
+        // the items ascend with the runs: the last entry holds the largest
+        if (nci > 0)
+            GK_CUDA(ctx, cudaMemcpyAsync(&h_last, ikey + nci - 1, sizeof h_last, cudaMemcpyDeviceToHost, st));
         GK_CUDA(ctx, cudaStreamSynchronize(st));
         for (int64_t j = 0; j < k && tiled_ok; j++) tiled_ok = hco[j + 1] - hco[j] < 32768;
     }
@@ -870,38 +1064,72 @@ geek_status jaccard_core(geek_ctx *ctx, Scratch &scr, const int64_t *off, const 
     GK_TRY(scr.alloc(&n_ovf, 1));
     GK_CUDA(ctx, cudaMemsetAsync(n_ovf, 0, sizeof(unsigned long long), st));
     {
-        static bool attr = false;
-        if (!attr) {
-            GK_CUDA(ctx, cudaFuncSetAttribute(k_jac_tiled<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)Jx<true>::SMEM));
-            GK_CUDA(ctx, cudaFuncSetAttribute(k_jac_tiled<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)Jx<false>::SMEM));
-            attr = true;
-        }
-        const int kt = narrow ? Jx<true>::KT : Jx<false>::KT;
+        // tiles of kt centres (the last one may be short), a multiple of the
+        // counters one warp-wide load covers
+        const int step = narrow ? Jx<true>::STEP : Jx<false>::STEP;
+        const int kt = (int)std::min<int64_t>(narrow ? Jx<true>::KT : Jx<false>::KT, ceil_div(k, step) * step);
         const int ntiles = (int)ceil_div(k, kt);
-        int32_t *toff;
+        const size_t smem = (size_t)JX_WARPS * (narrow ? kt + 4 * Jx<true>::MAXI : 2 * kt + 4 * Jx<false>::MAXI);
+        int32_t *toff, *tile_min;
+        uint16_t *d_lloc;
         GK_TRY(scr.alloc(&toff, (size_t)std::max<int64_t>(h_nlight, 1) * (ntiles + 1)));
+        GK_TRY(scr.alloc(&tile_min, ntiles));
+        GK_TRY(scr.alloc(&d_lloc, std::max<int64_t>(1, h_nlent)));
         GK_COUNT();
         k_tile_offsets<<<G(ctx, h_nlight * (ntiles + 1)), 256, 0, st>>>(h_nlight, d_loff, d_lcentre, ntiles, kt, toff);
+        GK_COUNT();
+        k_tile_local<<<G(ctx, h_nlent), 256, 0, st>>>(h_nlent, d_lcentre, kt, d_lloc);
+        GK_COUNT();
+        k_tile_min_len<<<ntiles, 256, 0, st>>>(k, kt, clen, tile_min);
+        // the largest centre item decides between the table and the searches:
+        // above 2^24 (a 64 MB table) the fill would outweigh the searches' 20
+        // dependent loads per item
+        JxIndex X{nullptr, 0, fq_item, fq_bit, nfreq, d_litem, h_nlight};
+        if (h_last < (1u << 24)) {
+            int32_t *lut;
+            X.n_lut = (int64_t)h_last + 1;
+            GK_TRY(scr.alloc(&lut, (size_t)X.n_lut));
+            GK_CUDA(ctx, cudaMemsetAsync(lut, 0xFF, sizeof(int32_t) * (size_t)X.n_lut, st));
+            GK_COUNT();
+            k_item_lut<<<G(ctx, h_nlight), 256, 0, st>>>(h_nlight, d_litem, lut);
+            if (nfreq) {
+                GK_COUNT();
+                k_freq_lut<<<G(ctx, nfreq), 256, 0, st>>>(nfreq, fq_item, fq_bit, lut);
+            }
+            X.lut = lut;
+        }
         EvTimer tk(ctx, "kernel.jaccard", st);
-        tk.work = (double)n * (double)k;  // (set, centre) pairs scored
+        tk.work = (double)n * (double)k;  // (set, centre) pairs decided
         if (!tiled_ok) {  // very large central sets: every set takes the dense path
             GK_COUNT();
             k_iota_rows<<<G(ctx, n), 256, 0, st>>>(n, ovf, n_ovf);
             GK_LAUNCH(ctx);
         } else {
-        GK_COUNT();
-        const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(n, JX_S), (int64_t)ctx->num_sms * 3);
-        if (narrow)
-            k_jac_tiled<true><<<grid, JX_THREADS, Jx<true>::SMEM, st>>>(n, off, items, na_fix, k, clen, cmask, hv_item,
-                                                                      hv_bit, nheavy, HW, d_litem, toff, ntiles,
-                                                                      h_nlight, d_lcentre, labels, ovf, n_ovf);
-        else
-            k_jac_tiled<false><<<grid, JX_THREADS, Jx<false>::SMEM, st>>>(n, off, items, na_fix, k, clen, cmask,
-                                                                        hv_item, hv_bit, nheavy, HW, d_litem, toff,
-                                                                        ntiles, h_nlight, d_lcentre, labels, ovf,
-                                                                        n_ovf);
+        int4 *hard;
+        unsigned long long *n_hard;
+        GK_TRY(scr.alloc(&hard, n));
+        GK_TRY(scr.alloc(&n_hard, 1));
+        GK_CUDA(ctx, cudaMemsetAsync(n_hard, 0, sizeof(unsigned long long), st));
+        const JxArgs A{n, off, items, na_fix, k, kt, ntiles, clen, tile_min, toff, d_lloc, X, labels};
+        auto run = [&](auto *prune, auto *count) -> geek_status {
+            int per_sm[2] = {1, 1};
+            const void *fn[2] = {(const void *)prune, (const void *)count};
+            for (int f = 0; f < 2; f++) {
+                GK_CUDA(ctx, cudaFuncSetAttribute(fn[f], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+                GK_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[f], fn[f], JX_THREADS, smem));
+            }
+            auto grid = [&](int f) {
+                return (unsigned)std::min<int64_t>(ceil_div(n, JX_WARPS), (int64_t)ctx->num_sms * std::max(per_sm[f], 1));
+            };
+            GK_COUNT();
+            prune<<<grid(0), JX_THREADS, smem, st>>>(A, fmask, FW, ovf, n_ovf, hard, n_hard);
+            GK_COUNT();
+            count<<<grid(1), JX_THREADS, smem, st>>>(A, cmask, HW, fq_list, hard, n_hard);
+            GK_LAUNCH(ctx);
+            return GEEK_OK;
+        };
+        if (narrow) GK_TRY(run(k_jac_prune<true>, k_jac_count<true>));
+        else GK_TRY(run(k_jac_prune<false>, k_jac_count<false>));
         GK_LAUNCH(ctx);
         }
     }
