@@ -915,11 +915,18 @@ __global__ void k_label_keys(int64_t n, const int32_t *__restrict__ labels, int6
     }
 }
 
-// sort key of centre j: descending member count, then ascending index
-__global__ void k_size_order(int64_t k, const unsigned long long *__restrict__ cnt, uint64_t *__restrict__ key) {
+// sort key of centre j: descending member count, then ascending index; nseg[j] =
+// segments of a large centre (else 0), *n_large += 1 for each
+constexpr int UL_M = 128;        // members per segment
+constexpr int UL_MIN = 16384;    // a centre of more members is cut into segments
+__global__ void k_size_order(int64_t k, const unsigned long long *__restrict__ cnt, uint64_t *__restrict__ key,
+                             int64_t *__restrict__ nseg, unsigned long long *__restrict__ n_large) {
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < k; j += (int64_t)gridDim.x * blockDim.x) {
         const uint64_t cj = cnt[j] > 0xFFFFFFFFull ? 0xFFFFFFFFull : cnt[j];
         key[j] = ((0xFFFFFFFFull - cj) << 32) | (uint64_t)j;
+        const bool large = cj > UL_MIN;
+        nseg[j] = large ? (int64_t)((cj + UL_M - 1) / UL_M) : 0;
+        if (large) atomicAdd(n_large, 1ull);
     }
 }
 
@@ -1109,6 +1116,7 @@ __global__ void __launch_bounds__(UC_T) k_update_centres(const float *__restrict
                                                          const int64_t *__restrict__ off,
                                                          const unsigned long long *__restrict__ cnt,
                                                          const int32_t *__restrict__ ids, const uint64_t *__restrict__ order,
+                                                         const unsigned long long *__restrict__ n_large,
                                                          unsigned long long *__restrict__ next, double *__restrict__ c,
                                                          int *__restrict__ err) {
     extern __shared__ float uc_ring[];  // [UC_P][UC_S][32 rows][32 floats]
@@ -1130,7 +1138,8 @@ __global__ void __launch_bounds__(UC_T) k_update_centres(const float *__restrict
         const uint32_t ring_s = su32(ring);
         const bool vec = (((uintptr_t)x & 15) == 0) && ((ldx & 3) == 0);
         const int64_t np = (int64_t)gridDim.x * UC_P;
-        int64_t it = (int64_t)pr * gridDim.x + blockIdx.x;  // first wave: slices of a centre on different SMs
+        const int64_t it0 = (int64_t)*n_large * nsl;        // the large centres come first in the order
+        int64_t it = it0 + (int64_t)pr * gridDim.x + blockIdx.x;  // first wave: slices of a centre on different SMs
         uint32_t sn = 0;                                    // stages issued by this pair
         bool ok = true;
         for (;;) {
@@ -1195,7 +1204,7 @@ __global__ void __launch_bounds__(UC_T) k_update_centres(const float *__restrict
             if (done || !ok) break;
             unsigned long long got = 0;
             if (lane == 0) got = atomicAdd(next, 1ull);
-            it = np + (int64_t)__shfl_sync(0xffffffffu, got, 0);
+            it = it0 + np + (int64_t)__shfl_sync(0xffffffffu, got, 0);
         }
         asm volatile("cp.async.wait_all;" ::: "memory");  // own copies landed before the block ends
     } else {
@@ -1227,6 +1236,237 @@ __global__ void __launch_bounds__(UC_T) k_update_centres(const float *__restrict
     }
 }
 
+// ---- large centres: the chain in parallel segments -------------------------
+// One warp walks a chain at about 42 ns per member, so a cluster of 950,000
+// members held the whole pass for 38 ms (10M x 128, k = 20,000 with Zipf
+// weights).  The chain s <- RN(s + x_i) can be cut into segments of UL_M
+// members that run in parallel, bit for bit:
+//  While s stays inside one binade, |s| in [2^e, 2^(e+1)), every FP64 value
+//  there is a multiple of q = 2^(e-52), and RN(s + x) = s + q round(x / q) with
+//  the ties of x / q broken by the parity of s / q.  So a whole segment moves
+//  S = s / q by an integer that depends on S only through its parity: two
+//  integers (for S even and odd) describe it, computed without knowing s, only
+//  its binade.  The binade comes from the segments' approximate sums.
+//  k_ul_sums    approximate sum of every (segment, coordinate), in a
+//               compensated FP32 sum
+//  k_ul_starts  their running sums: the approximate s at each segment's start
+//  k_ul_deltas  the segment's two integers in the unit of that s's binade, and
+//               the range of the partial sums on the way
+//  k_ul_chain   a warp per (centre, 32 coordinates) walks the segments with the
+//               exact s: where s has the assumed exponent and S plus the range
+//               stays in [2^52 + 1, 2^53 - 1] (then every exact s + x lies in
+//               the binade before its rounding), s moves by the integer;
+//               otherwise (the first segments, a segment that crosses a power
+//               of two, a member comparable to s or not finite) the segment
+//               runs through chain_chunk.
+// Both sides of the line: a centre of UL_MIN members takes 0.7 ms on one warp
+// pair, about what the whole pass over the segments takes at 10M x 128, and
+// its first segments run through chain_chunk either way.
+struct UlArgs {
+    const float *x;
+    int64_t ldx;
+    int d;
+    int64_t k;
+    const int64_t *off;
+    const unsigned long long *cnt;
+    const int32_t *ids;
+    const int64_t *seg_off;        // k: first segment of each centre
+    const int64_t *n_seg;          // all segments
+    const uint64_t *order;         // centres by descending count
+    const unsigned long long *n_large;
+    double *start;                 // [segment][d]: sums, then s at the start (approximate)
+    int64_t *d0, *d1, *mn, *mx;    // [segment][d]
+    int32_t *ex;                   // [segment][d]: biased exponent assumed, -1: none
+    double *c;                     // k x d
+};
+
+// item (segment, 32-coordinate slice) -> centre, member range, coordinate
+struct UlItem {
+    int64_t j, seg;
+    const int32_t *mid;
+    int rows, t;
+    bool act;
+};
+__device__ __forceinline__ UlItem ul_item(const UlArgs &A, int64_t it, int nsl) {
+    UlItem q;
+    q.seg = it / nsl;
+    q.t = (int)(it % nsl) * 32 + (threadIdx.x & 31);
+    q.act = q.t < A.d;
+    q.j = find_inst(A.seg_off, (int)A.k, q.seg);  // centres without segments share their successor's offset
+    const int64_t m0 = (q.seg - A.seg_off[q.j]) * UL_M;
+    q.rows = (int)min((int64_t)UL_M, (int64_t)A.cnt[q.j] - m0);
+    q.mid = A.ids + A.off[q.j] + m0;
+    return q;
+}
+
+// calls f(x) for the item's members in order, UL_F rows' loads in flight
+constexpr int UL_F = 16;
+template <class Fn>
+__device__ __forceinline__ void ul_rows(const UlArgs &A, const UlItem &q, Fn f) {
+    const int lane = threadIdx.x & 31;
+    const float *xs = A.x + (q.act ? q.t : 0);
+    for (int m0 = 0; m0 < q.rows; m0 += 32) {
+        const int32_t id = m0 + lane < q.rows ? q.mid[m0 + lane] : 0;
+        const int nr = min(32, q.rows - m0);
+#pragma unroll
+        for (int h = 0; h < 32; h += UL_F) {
+            float v[UL_F];
+#pragma unroll
+            for (int r = 0; r < UL_F; r++) {
+                const int32_t row = __shfl_sync(0xffffffffu, id, h + r);
+                v[r] = h + r < nr ? xs[(int64_t)row * A.ldx] : 0.f;
+            }
+#pragma unroll
+            for (int r = 0; r < UL_F; r++)
+                if (h + r < nr) f(v[r]);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(256) k_ul_sums(UlArgs A) {
+    const int nsl = (A.d + 31) >> 5;
+    const int64_t items = *A.n_seg * nsl, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t it = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < items; it += nw) {
+        const UlItem q = ul_item(A, it, nsl);
+        float sh = 0.f, sl = 0.f;
+        ul_rows(A, q, [&](float v) { csum_add(sh, sl, v); });
+        if (q.act) A.start[q.seg * A.d + q.t] = (double)sh + (double)sl;
+    }
+}
+
+// warp per (large centre, slice): sums -> the running sum before each segment
+__global__ void __launch_bounds__(128) k_ul_starts(UlArgs A) {
+    const int nsl = (A.d + 31) >> 5, lane = threadIdx.x & 31;
+    const int64_t items = (int64_t)*A.n_large * nsl, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t it = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < items; it += nw) {
+        const int64_t j = (int64_t)(A.order[it / nsl] & 0xFFFFFFFFull);
+        const int t = (int)(it % nsl) * 32 + lane;
+        if (t >= A.d) continue;
+        const int64_t ns = ((int64_t)A.cnt[j] + UL_M - 1) / UL_M;
+        double *p = A.start + A.seg_off[j] * A.d + t;
+        double run = 0.0;
+        for (int64_t s0 = 0; s0 < ns; s0 += 16) {
+            double v[16];
+#pragma unroll
+            for (int u = 0; u < 16; u++) v[u] = s0 + u < ns ? p[(s0 + u) * A.d] : 0.0;
+#pragma unroll
+            for (int u = 0; u < 16; u++) {
+                if (s0 + u < ns) p[(s0 + u) * A.d] = run;
+                run += v[u];
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(256) k_ul_deltas(UlArgs A) {
+    const int nsl = (A.d + 31) >> 5;
+    const int64_t items = *A.n_seg * nsl, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t it = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < items; it += nw) {
+        const UlItem q = ul_item(A, it, nsl);
+        const int64_t at = q.seg * A.d + q.t;
+        const double s = q.act ? A.start[at] : 0.0;
+        const int E = (int)(((uint64_t)__double_as_longlong(s) >> 52) & 0x7FF);
+        bool ok = E > 64 && E < 0x7FE - 64;
+        int64_t D0 = 0, D1 = 0, mn = 0, mx = 0;
+        ul_rows(A, q, [&](float v) {
+            // v / q = m 2^sh, m a 24-bit integer
+            const uint32_t b = __float_as_uint(v);
+            const int e = (int)((b >> 23) & 0xFFu);
+            const int32_t ma = (int32_t)((b & 0x7FFFFFu) | ((uint32_t)min(e, 1) << 23));
+            const int32_t m = (b >> 31) ? -ma : ma;
+            const int sh = max(e, 1) + 925 - E;
+            ok = ok && sh <= 28 && e != 0xFF;  // 128 values of at most 2^52 units each: no overflow
+            int64_t r0, r1;
+            if (sh >= 0) {
+                r0 = r1 = (int64_t)((uint64_t)(int64_t)m << min(sh, 28));
+            } else if (sh < -25) {
+                r0 = r1 = 0;  // below half a unit
+            } else {
+                const int32_t F = m >> -sh, rem = m & ((1 << -sh) - 1), half = 1 << (-sh - 1);
+                r0 = r1 = F + (rem > half);
+                if (rem == half) {  // a tie: to the even one of S + F, S + F + 1
+                    r0 = F + ((D0 + F) & 1);
+                    r1 = F + ((1 + D1 + F) & 1);
+                }
+            }
+            D0 += r0;
+            D1 += r1;
+            mn = min(mn, min(D0, D1));
+            mx = max(mx, max(D0, D1));
+        });
+        if (q.act) {
+            A.d0[at] = D0;
+            A.d1[at] = D1;
+            A.mn[at] = mn;
+            A.mx[at] = mx;
+            A.ex[at] = ok ? E : -1;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(32) k_ul_chain(UlArgs A) {
+    const int nsl = (A.d + 31) >> 5, lane = threadIdx.x;
+    const int64_t items = (int64_t)*A.n_large * nsl;
+    constexpr int64_t LO = (1ll << 52) + 1, HI = (1ll << 53) - 1;
+    for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
+        const int64_t j = (int64_t)(A.order[it / nsl] & 0xFFFFFFFFull);
+        const int t = (int)(it % nsl) * 32 + lane;
+        const bool act = t < A.d;
+        const int64_t cj = (int64_t)A.cnt[j], ns = (cj + UL_M - 1) / UL_M;
+        const int32_t *mid = A.ids + A.off[j];
+        const float *xs = A.x + (act ? t : 0);
+        const int64_t a0 = A.seg_off[j] * A.d + (act ? t : 0);
+        double s = 0.0;
+        for (int64_t g0 = 0; g0 < ns; g0 += 4) {
+            // four segments' integers requested together
+            int64_t D0[4], D1[4], mn[4], mx[4];
+            int ex[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const int64_t at = a0 + min(g0 + u, ns - 1) * A.d;
+                D0[u] = A.d0[at];
+                D1[u] = A.d1[at];
+                mn[u] = A.mn[at];
+                mx[u] = A.mx[at];
+                ex[u] = A.ex[at];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                if (g0 + u >= ns) break;
+                const uint64_t bits = (uint64_t)__double_as_longlong(s);
+                const int E = (int)((bits >> 52) & 0x7FF);
+                const int64_t a = (int64_t)((bits & ((1ull << 52) - 1)) | (1ull << 52));
+                const bool neg = bits >> 63;
+                const int64_t S = neg ? -a : a;
+                const bool ok = !act || (ex[u] == E && (neg ? S + mx[u] <= -LO && S + mn[u] >= -HI
+                                                            : S + mn[u] >= LO && S + mx[u] <= HI));
+                const int64_t T = S + ((S & 1) ? D1[u] : D0[u]);
+                const uint64_t b = (uint64_t)(T < 0 ? -T : T);
+                const double moved = __longlong_as_double(
+                    (long long)((bits & (1ull << 63)) | ((uint64_t)E << 52) | (b & ((1ull << 52) - 1))));
+                double walked = s;
+                if (!__all_sync(0xffffffffu, ok)) {
+                    const int64_t m0 = (g0 + u) * UL_M;
+                    for (int64_t p = m0; p < min(cj, m0 + UL_M); p += UC_B) {
+                        const int ma = (int)min((int64_t)UC_B, cj - p);
+                        const int32_t id = lane < ma ? mid[p + lane] : 0;
+                        float v[UC_B];
+#pragma unroll
+                        for (int r = 0; r < UC_B; r++) {
+                            const int32_t row = __shfl_sync(0xffffffffu, id, r);
+                            v[r] = r < ma ? xs[(int64_t)row * A.ldx] : 0.f;
+                        }
+                        walked = ma == UC_B ? chain_chunk<true>(walked, v, ma, act && !ok)
+                                            : chain_chunk<false>(walked, v, ma, act && !ok);
+                    }
+                }
+                s = ok ? moved : walked;
+            }
+        }
+        if (act) A.c[j * A.d + t] = __ddiv_rn(s, (double)cj);
+    }
+}
+
 geek_status refine_dense(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx, int64_t n, int d, double *centres,
                          int64_t k, int passes, int precision, int32_t *labels, geek_assign_stats *stats,
                          cudaStream_t st) {
@@ -1251,11 +1491,19 @@ geek_status refine_dense(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ld
         GK_TRY(radix_sort_segments(ctx, ps, 1, n, &key, nullptr, &ids, bit_length_u64((uint64_t)k), st));
         GK_TRY(exclusive_scan_i64(ctx, ps, (const int64_t *)cnt, off, k, nullptr, st));
         uint64_t *order;
+        int64_t *nseg, *seg_off, *seg_tot;
+        unsigned long long *n_large;
         GK_TRY(ps.alloc(&order, k));
+        GK_TRY(ps.alloc(&nseg, k));
+        GK_TRY(ps.alloc(&seg_off, k));
+        GK_TRY(ps.alloc(&seg_tot, 1));
+        GK_TRY(ps.alloc(&n_large, 1));
+        GK_CUDA(ctx, cudaMemsetAsync(n_large, 0, sizeof(unsigned long long), st));
         GK_COUNT();
-        k_size_order<<<grid_for(k, 256, ctx->num_sms), 256, 0, st>>>(k, cnt, order);
+        k_size_order<<<grid_for(k, 256, ctx->num_sms), 256, 0, st>>>(k, cnt, order, nseg, n_large);
         GK_LAUNCH(ctx);
         GK_TRY(radix_sort_segments(ctx, ps, 1, k, &order, nullptr, nullptr, 64, st));
+        GK_TRY(exclusive_scan_i64(ctx, ps, nseg, seg_off, k, seg_tot, st));
         tg.stop();
         unsigned long long *next;
         int *uc_err;
@@ -1269,10 +1517,33 @@ geek_status refine_dense(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ld
             uc_attr = true;
         }
         EvTimer tu(ctx, "kernel.update_centres", st);
+        if (n > UL_MIN) {  // else no centre is large
+            const size_t segs = (size_t)(n / UL_M + n / UL_MIN + 1);  // at most
+            UlArgs U{x, ldx, d, k, off, cnt, (const int32_t *)ids, seg_off, seg_tot, order, n_large};
+            GK_TRY(ps.alloc(&U.start, segs * d));
+            GK_TRY(ps.alloc(&U.d0, segs * d));
+            GK_TRY(ps.alloc(&U.d1, segs * d));
+            GK_TRY(ps.alloc(&U.mn, segs * d));
+            GK_TRY(ps.alloc(&U.mx, segs * d));
+            GK_TRY(ps.alloc(&U.ex, segs * d));
+            U.c = centres;
+            const int nsl = (d + 31) / 32;
+            const int gs = grid_for((int64_t)segs * nsl * 32, 256, ctx->num_sms);
+            const int64_t most = (n / UL_MIN) * nsl;  // (large centre, slice) items, at most
+            GK_COUNT();
+            k_ul_sums<<<gs, 256, 0, st>>>(U);
+            GK_COUNT();
+            k_ul_starts<<<grid_for(most * 32, 128, ctx->num_sms), 128, 0, st>>>(U);
+            GK_COUNT();
+            k_ul_deltas<<<gs, 256, 0, st>>>(U);
+            GK_COUNT();
+            k_ul_chain<<<(unsigned)std::min<int64_t>(most, (int64_t)ctx->num_sms * 16), 32, 0, st>>>(U);
+            GK_LAUNCH(ctx);
+        }
         GK_COUNT();
         k_update_centres<<<(unsigned)std::min<int64_t>((k * ((d + 31) / 32) + UC_P - 1) / UC_P, (int64_t)ctx->num_sms),
-                           UC_T, UC_SMEM, st>>>(x, ldx, d, k, off, cnt, (const int32_t *)ids, order, next, centres,
-                                                uc_err);
+                           UC_T, UC_SMEM, st>>>(x, ldx, d, k, off, cnt, (const int32_t *)ids, order, n_large, next,
+                                                centres, uc_err);
         GK_LAUNCH(ctx);
         tu.stop();
         int h_bad = 0, h_uc = 0;
