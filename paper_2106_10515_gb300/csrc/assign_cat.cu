@@ -92,8 +92,11 @@ constexpr int CAT_TILE = 64;
 constexpr int CAT_MAXA = 32;
 __global__ void __launch_bounds__(256) k_assign_cat(int64_t n, int A, int64_t k, const uint64_t *__restrict__ attrs,
                                                     const uint64_t *__restrict__ modes, int32_t *__restrict__ labels,
-                                                    int32_t *__restrict__ matches) {
+                                                    unsigned long long *__restrict__ hist) {
     __shared__ uint64_t ms[CAT_TILE * CAT_MAXA];
+    __shared__ unsigned s_hist[CAT_MAXA + 1];
+    if (threadIdx.x <= CAT_MAXA) s_hist[threadIdx.x] = 0;
+    __syncthreads();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     uint64_t x[CAT_MAXA];
     for (int a = 0; a < CAT_MAXA; a++) x[a] = (i < n && a < A) ? attrs[i * A + a] : 0;
@@ -116,8 +119,11 @@ __global__ void __launch_bounds__(256) k_assign_cat(int64_t n, int A, int64_t k,
     }
     if (i < n) {
         labels[i] = bj;
-        if (matches) matches[i] = bm;
+        if (hist && bm >= 0) atomicAdd(&s_hist[bm], 1u);
     }
+    __syncthreads();
+    if (hist && threadIdx.x <= A && s_hist[threadIdx.x])
+        atomicAdd(&hist[threadIdx.x], (unsigned long long)s_hist[threadIdx.x]);
 }
 
 // ---- set data --------------------------------------------------------------
@@ -811,10 +817,8 @@ geek_status assign_hetero(geek_ctx *ctx, Scratch &scr, const geek_buckets *b, co
     if (A > CAT_MAXA) return set_error(ctx, GEEK_ERR_UNSUPPORTED, "more than %d categorical attributes", CAT_MAXA);
     if (n == 0) return GEEK_OK;
     uint64_t *attrs, *modes;
-    int32_t *matches;
     GK_TRY(scr.alloc(&attrs, (size_t)n * A));
     GK_TRY(scr.alloc(&modes, (size_t)std::max<int64_t>(k, 1) * A));
-    GK_TRY(scr.alloc(&matches, n));
     int32_t *rep = nullptr;
     if (keep && k) GK_TRY(scr.alloc(&rep, (size_t)k * A));
     GK_COUNT();
@@ -849,19 +853,27 @@ geek_status assign_hetero(geek_ctx *ctx, Scratch &scr, const geek_buckets *b, co
             GK_CUDA(ctx, cudaStreamSynchronize(st));
         }
     }
-    GK_COUNT();
-    k_assign_cat<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(n, A, k, attrs, modes, labels, matches);
-    GK_LAUNCH(ctx);
+    unsigned long long *hist;  // rows by their number of matching attributes
+    GK_TRY(scr.alloc(&hist, A + 1));
+    GK_CUDA(ctx, cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * (A + 1), st));
+    if (match_bits_eligible(k, A)) {
+        GK_TRY(match_bits_assign(ctx, scr, n, A, attrs, k, modes, labels, stats ? hist : nullptr, st));
+    } else {
+        GK_COUNT();
+        k_assign_cat<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(n, A, k, attrs, modes, labels, stats ? hist : nullptr);
+        GK_LAUNCH(ctx);
+    }
     if (stats) {
-        // SSE in the categorical distance 1 - m / (2A - m), computed on the host
-        std::vector<int32_t> hm(n);
-        GK_CUDA(ctx, cudaMemcpyAsync(hm.data(), matches, 4 * n, cudaMemcpyDeviceToHost, st));
+        // the categorical distance 1 - m / (2A - m) takes A + 1 values: the
+        // SSE is their sum weighted by the rows that have each
+        unsigned long long hm[CAT_MAXA + 1];
+        GK_CUDA(ctx, cudaMemcpyAsync(hm, hist, sizeof(unsigned long long) * (A + 1), cudaMemcpyDeviceToHost, st));
         GK_CUDA(ctx, cudaStreamSynchronize(st));
         double sse = 0.0, rmax = 0.0;
-        for (int64_t i = 0; i < n; i++) {
-            if (hm[i] < 0) continue;
-            const double dd = 1.0 - (double)hm[i] / (double)(2 * A - hm[i]);
-            sse += dd;
+        for (int m = A; m >= 0; m--) {
+            if (!hm[m]) continue;
+            const double dd = 1.0 - (double)m / (double)(2 * A - m);
+            sse += (double)hm[m] * dd;
             rmax = std::max(rmax, dd);
         }
         stats->sse = sse;
@@ -1192,9 +1204,10 @@ __global__ void k_run_flags(int64_t m, const uint64_t *__restrict__ sorted, int6
 // reduced dimension.  Central vector = the mode of each dimension over the
 // seed's members (Sect. 3.3: the mode of sparse data after DOPH; ties to the
 // smallest token); distance 1 - Jaccard of the token sets, i.e. the label
-// maximises the number of dimensions equal to the centre's mode.  Tokens map
-// to 32-bit ids of the distinct mode tokens and the Jaccard engine decides,
-// with |A| = |C| = D'.
+// maximises the number of dimensions equal to the centre's mode
+// (match_bits.cu).  Where the mask table would be too large, tokens map to
+// 32-bit ids of the distinct mode tokens and the Jaccard engine decides, with
+// |A| = |C| = D'.
 geek_status assign_doph(geek_ctx *ctx, Scratch &scr, const geek_buckets *b, const silk_seeds *s, int32_t *labels,
                         geek_assign_stats *stats, geek_centres *keep, cudaStream_t st) {
     const int64_t n = b->n, k = s->k;
@@ -1219,6 +1232,7 @@ geek_status assign_doph(geek_ctx *ctx, Scratch &scr, const geek_buckets *b, cons
     k_modes<<<G(ctx, km), 256, 0, st>>>(k, D, s->off, s->ids, b->doph_tok, modes, nullptr);
     GK_LAUNCH(ctx);
     if (keep) GK_CUDA(ctx, cudaMemcpyAsync(keep->modes, modes, 8 * km, cudaMemcpyDeviceToDevice, st));
+    if (match_bits_eligible(k, D)) return match_bits_assign(ctx, scr, n, D, b->doph_tok, k, modes, labels, nullptr, st);
     // distinct mode tokens, ascending
     GK_CUDA(ctx, cudaMemcpyAsync(srt, modes, 8 * km, cudaMemcpyDeviceToDevice, st));
     GK_TRY(radix_sort_segments(ctx, scr, 1, km, &srt, nullptr, nullptr, 64, st));
