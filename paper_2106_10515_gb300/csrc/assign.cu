@@ -80,11 +80,7 @@ struct FArgs {
 };
 struct GatherUnits {
     const RInst *R;
-    const int32_t *grows;
-    const int *unit_inst;
-    const int64_t *unit_start;
-    const int *unit_cnt;
-    const int *n_units;
+    FlagUnits f;
 };
 
 __device__ __forceinline__ unsigned long long ffma2(unsigned long long a, unsigned long long b, unsigned long long c) {
@@ -106,13 +102,13 @@ __global__ void __launch_bounds__(256, 2) k_assign_fp32(FArgs A, GatherUnits U) 
     extern __shared__ __align__(16) float sm[];
     __shared__ int64_t s_rows[AS_TR];
     const int t = threadIdx.x, cg = t & 15, rg = t >> 4;
-    const int64_t nunits = GATHER ? (int64_t)*U.n_units : A.ntiles;
+    const int64_t nunits = GATHER ? (int64_t)*U.f.n_units : A.ntiles;
     for (int64_t u = blockIdx.x; u < nunits; u += gridDim.x) {
         int64_t row0 = u * AS_TR;
         int nrows = (int)min((int64_t)AS_TR, A.n - row0);
         int64_t rbase = 0;
         if (GATHER) {
-            const RInst &I = U.R[U.unit_inst[u]];
+            const RInst &I = U.R[U.f.unit_inst[u]];
             A.x = I.x;
             A.ldx = I.ldx;
             A.d = I.d;
@@ -122,9 +118,9 @@ __global__ void __launch_bounds__(256, 2) k_assign_fp32(FArgs A, GatherUnits U) 
             A.cmax = __uint_as_float(*I.cmax_bits);
             A.labels = I.labels;
             rbase = I.row_base;
-            nrows = U.unit_cnt[u];
+            nrows = U.f.unit_cnt[u];
             __syncthreads();  // s_rows of the previous unit fully used
-            if (t < nrows) s_rows[t] = (int64_t)U.grows[U.unit_start[u] + t] - rbase;
+            if (t < nrows) s_rows[t] = (int64_t)U.f.grows[U.f.unit_start[u] + t] - rbase;
             __syncthreads();
         }
         const int d = A.d;
@@ -328,15 +324,15 @@ __global__ void __launch_bounds__(256) k_assign_decide64(GatherUnits U, const fl
     __shared__ int s_qn;
     constexpr unsigned long long DINF = 0x7FF0000000000000ull;  // above every finite D
     const int t = threadIdx.x, cg = t & 15, rg = t >> 4;
-    const int64_t nunits = (int64_t)*U.n_units;
+    const int64_t nunits = (int64_t)*U.f.n_units;
     for (int64_t u = blockIdx.x; u < nunits; u += gridDim.x) {
-        const RInst &I = U.R[U.unit_inst[u]];
+        const RInst &I = U.R[U.f.unit_inst[u]];
         const int d = I.d;
         const int64_t k = I.k;
         const int64_t rbase = I.row_base;
-        const int nrows = U.unit_cnt[u];
+        const int nrows = U.f.unit_cnt[u];
         __syncthreads();  // s_rows and xs of the previous unit fully used
-        if (t < nrows) s_rows[t] = (int64_t)U.grows[U.unit_start[u] + t] - rbase;
+        if (t < nrows) s_rows[t] = (int64_t)U.f.grows[U.f.unit_start[u] + t] - rbase;
         if (t < AS_TR) {
             sbD[t] = DINF;
             prevD[t] = DINF;
@@ -468,11 +464,11 @@ __global__ void k_flag_count(const int32_t *__restrict__ flags, const unsigned l
         atomicAdd(&cnt[find_inst(row_off, count, flags[q])], 1);
 }
 
-// one block: segment offsets and 128-row units per instance; cursor[i] =
-// segment start for the scatter
+// one block: the rows (seg_off) and 128-row units (unit_off) before each
+// instance, count + 1 entries; cursor[i] = segment start for the scatter
 __global__ void __launch_bounds__(1024) k_flag_units(const int *__restrict__ cnt, int count, int64_t *__restrict__ cursor,
-                                                     int *__restrict__ unit_inst, int64_t *__restrict__ unit_start,
-                                                     int *__restrict__ unit_cnt, int *__restrict__ n_units) {
+                                                     int64_t *__restrict__ seg_off, int64_t *__restrict__ unit_off,
+                                                     int *__restrict__ n_units) {
     __shared__ int64_t seg_carry, unit_carry;
     __shared__ int64_t s_seg[1024], s_unit[1024];
     if (threadIdx.x == 0) seg_carry = unit_carry = 0;
@@ -484,7 +480,7 @@ __global__ void __launch_bounds__(1024) k_flag_units(const int *__restrict__ cnt
         s_seg[threadIdx.x] = c;
         s_unit[threadIdx.x] = nu;
         __syncthreads();
-        for (int o = 1; o < 1024; o <<= 1) {  // inclusive scans
+        for (int o = 1; o < 1024 && o < count; o <<= 1) {  // inclusive scans
             const int64_t a = threadIdx.x >= o ? s_seg[threadIdx.x - o] : 0;
             const int64_t b = threadIdx.x >= o ? s_unit[threadIdx.x - o] : 0;
             __syncthreads();
@@ -492,23 +488,36 @@ __global__ void __launch_bounds__(1024) k_flag_units(const int *__restrict__ cnt
             s_unit[threadIdx.x] += b;
             __syncthreads();
         }
-        const int64_t so = seg_carry + s_seg[threadIdx.x] - c, uo = unit_carry + s_unit[threadIdx.x] - nu;
         if (i < count) {
-            cursor[i] = so;
-            for (int64_t q = 0; q < nu; q++) {
-                unit_inst[uo + q] = i;
-                unit_start[uo + q] = so + q * AS_TR;
-                unit_cnt[uo + q] = (int)min((int64_t)AS_TR, c - q * AS_TR);
-            }
+            cursor[i] = seg_off[i] = seg_carry + s_seg[threadIdx.x] - c;
+            unit_off[i] = unit_carry + s_unit[threadIdx.x] - nu;
         }
         __syncthreads();
-        if (threadIdx.x == 1023) {
-            seg_carry += s_seg[1023];
-            unit_carry += s_unit[1023];
+        if (threadIdx.x == 0) {
+            const int last = min(1024, count - base) - 1;
+            seg_carry += s_seg[last];
+            unit_carry += s_unit[last];
         }
         __syncthreads();
     }
-    if (threadIdx.x == 0) *n_units = (int)unit_carry;
+    if (threadIdx.x == 0) {
+        seg_off[count] = seg_carry;
+        unit_off[count] = unit_carry;
+        *n_units = (int)unit_carry;
+    }
+}
+
+// unit u: its instance, first row (in grows) and row count
+__global__ void k_fill_units(int count, const int64_t *__restrict__ seg_off, const int64_t *__restrict__ unit_off,
+                             int *__restrict__ unit_inst, int64_t *__restrict__ unit_start, int *__restrict__ unit_cnt) {
+    const int64_t nu = unit_off[count];
+    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < nu; u += (int64_t)gridDim.x * blockDim.x) {
+        const int i = find_inst(unit_off, count, u);
+        const int64_t s = seg_off[i] + (u - unit_off[i]) * AS_TR;
+        unit_inst[u] = i;
+        unit_start[u] = s;
+        unit_cnt[u] = (int)min((int64_t)AS_TR, seg_off[i + 1] - s);
+    }
 }
 
 __global__ void k_flag_scatter(const int32_t *__restrict__ flags, const unsigned long long *__restrict__ n_flag,
@@ -1684,15 +1693,20 @@ geek_status assign_dense_centres(geek_ctx *ctx, Scratch &scr, const float *x, in
     float cmax;
     memcpy(&cmax, &h_bits, sizeof cmax);
     int32_t *flag_rows;
-    float *flag_m = nullptr;  // the FP32 pass's smallest value per flagged row
+    float *flag_m;  // the fast pass's smallest value per flagged row
     unsigned long long *n_flag;
     GK_TRY(scr.alloc(&flag_rows, n));
-    if (precision == GEEK_PREC_FP32) GK_TRY(scr.alloc(&flag_m, n));
+    GK_TRY(scr.alloc(&flag_m, n));
     GK_TRY(scr.alloc(&n_flag, 1));
     GK_CUDA(ctx, cudaMemsetAsync(n_flag, 0, sizeof(unsigned long long), st));
+    TcPlan plan;
+    struct Free {
+        TcPlan *p;
+        ~Free() { tc_plan_free(p); }
+    } plan_free{&plan};
     if (precision == GEEK_PREC_BF16 || precision == GEEK_PREC_BF16X3) {
         GK_TRY(assign_tc_bf16(ctx, scr, x, ldx, n, d, centres, k, precision == GEEK_PREC_BF16X3, labels, flag_rows,
-                              n_flag, st));
+                              flag_m, n_flag, &plan, st));
     } else {
         const size_t smem = fp32_smem(d);
         GK_CUDA(ctx, cudaFuncSetAttribute(k_assign_fp32<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1719,7 +1733,9 @@ geek_status assign_dense_centres(geek_ctx *ctx, Scratch &scr, const float *x, in
             GK_LAUNCH(ctx);
             h_fp64 = h_flag;
         } else {
-            GK_TRY(decide_flags(ctx, ri, roff, 1, d, flag_rows, n_flag, db, st));
+            GK_TRY(tc_emit_alloc(ctx, &scr, &plan, (int64_t)h_flag, st));
+            GK_TRY(decide_flags(ctx, plan, ri, roff, 1, d, flag_rows, flag_m, n_flag, (int64_t)h_flag, db, st));
+            GK_TRY(tc_plan_check(ctx, plan, st));  // the candidates' pass, too, ran to its end
         }
     }
     if (stats) {
@@ -1821,6 +1837,10 @@ geek_status decide_bufs_alloc(geek_ctx *ctx, Scratch *scr, int count, int64_t n_
     GK_TRY(al(&B.unit_start, nu));
     GK_TRY(al(&B.unit_cnt, nu));
     GK_TRY(al(&B.n_units, 1));
+    GK_TRY(al(&B.seg_off, count + 1));
+    GK_TRY(al(&B.unit_off, count + 1));
+    GK_TRY(al(&B.left, std::max<int64_t>(n_total, 1)));
+    GK_TRY(al(&B.n_left, 1));
     GK_TRY(al(&B.grows, std::max<int64_t>(n_total, 1)));
     GK_TRY(al(&B.flags2, std::max<int64_t>(n_total, 1)));
     GK_TRY(al(&B.flags2_m, std::max<int64_t>(n_total, 1)));
@@ -1834,23 +1854,44 @@ void decide_bufs_free(DecideBufs &B) {
     B.owned.clear();
 }
 
-// Decides the flagged rows of a fast pass exactly: rows grouped by
-// instance, a tiled FP32 pass (narrow FP32 window) over each group, then the
-// FP64 reference for the rows still uncertain.  No host synchronisation.
-geek_status decide_flags(geek_ctx *ctx, const RInst *R, const int64_t *row_off, int count, int dmax,
-                         const int32_t *flags, const unsigned long long *n_flag, const DecideBufs &B,
-                         cudaStream_t st) {
-    EvTimer tk(ctx, "kernel.assign_recheck", st);
+// the listed rows grouped by instance in units of 128 (B.grows, B.unit_*)
+static geek_status group_flags(geek_ctx *ctx, const int64_t *row_off, int count, const int32_t *flags,
+                               const unsigned long long *n_flag, const DecideBufs &B, cudaStream_t st) {
     const int g = ctx->num_sms * 4;
     GK_CUDA(ctx, cudaMemsetAsync(B.cnt, 0, sizeof(int) * count, st));
-    GK_CUDA(ctx, cudaMemsetAsync(B.n_flag2, 0, sizeof(unsigned long long), st));
     GK_COUNT();
     k_flag_count<<<g, 256, 0, st>>>(flags, n_flag, row_off, count, B.cnt);
     GK_COUNT();
-    k_flag_units<<<1, 1024, 0, st>>>(B.cnt, count, B.cursor, B.unit_inst, B.unit_start, B.unit_cnt, B.n_units);
+    k_flag_units<<<1, 1024, 0, st>>>(B.cnt, count, B.cursor, B.seg_off, B.unit_off, B.n_units);
+    GK_COUNT();
+    k_fill_units<<<g, 256, 0, st>>>(count, B.seg_off, B.unit_off, B.unit_inst, B.unit_start, B.unit_cnt);
     GK_COUNT();
     k_flag_scatter<<<g, 256, 0, st>>>(flags, n_flag, row_off, count, B.cursor, B.grows);
     GK_LAUNCH(ctx);
+    return GEEK_OK;
+}
+
+// Decides the flagged rows of a tensor-core pass exactly (flags: global rows;
+// flag_m: their smallest fast values).  Nearly all of them among their
+// candidates, by direct FP32 distances (tc_decide_candidates); the rest (near
+// duplicates of one centre, values that are not finite) by a tiled FP32 scan of
+// every centre (narrow FP32 window), then the FP64 reference for the rows still
+// uncertain.  max_rows: at most so many flagged rows.  No host synchronisation.
+// Alg. 1 pipeline at 10M x 128, k = 1,751, split-BF16: 4.7M flagged rows of 35
+// candidates each take 26 ms; the two scans over every centre took 162.
+geek_status decide_flags(geek_ctx *ctx, const TcPlan &P, const RInst *R, const int64_t *row_off, int count, int dmax,
+                         const int32_t *flags, const float *flag_m, const unsigned long long *n_flag,
+                         int64_t max_rows, const DecideBufs &B, cudaStream_t st) {
+    EvTimer tk(ctx, "kernel.assign_recheck", st);
+    const int g = ctx->num_sms * 4;
+    const FlagUnits F{B.grows, B.unit_inst, B.unit_start, B.unit_cnt, B.n_units};
+    GK_CUDA(ctx, cudaMemsetAsync(B.n_flag2, 0, sizeof(unsigned long long), st));
+    GK_CUDA(ctx, cudaMemsetAsync(B.n_left, 0, sizeof(unsigned long long), st));
+    GK_TRY(group_flags(ctx, row_off, count, flags, n_flag, B, st));
+    GK_COUNT();
+    k_scatter_m<<<g, 256, 0, st>>>(flags, flag_m, n_flag, B.mrow);
+    GK_TRY(tc_decide_candidates(ctx, P, R, F, B.mrow, max_rows, B.left, B.n_left, st));
+    GK_TRY(group_flags(ctx, row_off, count, B.left, B.n_left, B, st));
     const size_t smem = (size_t)dmax * AS_TR * sizeof(float) + (size_t)AS_KC * AS_TC * sizeof(float);
     GK_CUDA(ctx, cudaFuncSetAttribute(k_assign_fp32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)fp32_smem(AS_MAXD)));
@@ -1858,7 +1899,7 @@ geek_status decide_flags(geek_ctx *ctx, const RInst *R, const int64_t *row_off, 
     A.flag_rows = B.flags2;
     A.flag_m = B.flags2_m;
     A.n_flag = B.n_flag2;
-    GatherUnits U{R, B.grows, B.unit_inst, B.unit_start, B.unit_cnt, B.n_units};
+    const GatherUnits U{R, F};
     EvTimer t32(ctx, "kernel.assign_refine32", st);
     GK_COUNT();
     k_assign_fp32<true><<<ctx->num_sms * 2, 256, fp32_smem(dmax), st>>>(A, U);
@@ -1866,22 +1907,11 @@ geek_status decide_flags(geek_ctx *ctx, const RInst *R, const int64_t *row_off, 
     t32.stop();
     // the rows still uncertain, grouped by instance again, go to the tiled
     // FP64 decision with their smallest FP32 value
-    static bool attr64 = false;
-    if (!attr64) {
-        const size_t mx =
-            (size_t)AS_MAXD * AS_TR * sizeof(float) + (size_t)AS_KC * AS_TC * sizeof(float) + DQ_BYTES;
-        GK_CUDA(ctx, cudaFuncSetAttribute(k_assign_decide64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx));
-        attr64 = true;
-    }
-    GK_CUDA(ctx, cudaMemsetAsync(B.cnt, 0, sizeof(int) * count, st));
+    const size_t mx = (size_t)AS_MAXD * AS_TR * sizeof(float) + (size_t)AS_KC * AS_TC * sizeof(float) + DQ_BYTES;
+    GK_CUDA(ctx, cudaFuncSetAttribute(k_assign_decide64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx));
     GK_COUNT();
     k_scatter_m<<<g, 256, 0, st>>>(B.flags2, B.flags2_m, B.n_flag2, B.mrow);
-    GK_COUNT();
-    k_flag_count<<<g, 256, 0, st>>>(B.flags2, B.n_flag2, row_off, count, B.cnt);
-    GK_COUNT();
-    k_flag_units<<<1, 1024, 0, st>>>(B.cnt, count, B.cursor, B.unit_inst, B.unit_start, B.unit_cnt, B.n_units);
-    GK_COUNT();
-    k_flag_scatter<<<g, 256, 0, st>>>(B.flags2, B.n_flag2, row_off, count, B.cursor, B.grows);
+    GK_TRY(group_flags(ctx, row_off, count, B.flags2, B.n_flag2, B, st));
     EvTimer t64(ctx, "kernel.assign_decide64", st);
     GK_COUNT();
     k_assign_decide64<<<ctx->num_sms * 2, 256, smem + DQ_BYTES, st>>>(U, B.mrow);

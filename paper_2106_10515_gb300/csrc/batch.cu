@@ -151,6 +151,7 @@ struct geek_batch {
     double *part_sum = nullptr, *sse_d = nullptr, *rmax_d = nullptr;
     float *part_max = nullptr;
     int32_t *flag_rows = nullptr;
+    float *flag_m = nullptr;
     unsigned long long *n_flag = nullptr;
     DecideBufs dec;                  // grouping and FP32 / FP64 decision of flagged rows
     cudaGraphExec_t g_assign = nullptr;
@@ -215,6 +216,7 @@ struct geek_batch {
         dfree(seeds.off);
         dfree(seeds.ids);
         dfree(flag_rows);
+        dfree(flag_m);
         dfree(n_flag);
         if (cs) cudaStreamDestroy(cs);
     }
@@ -282,6 +284,7 @@ geek_status batch_create(geek_ctx *ctx, const geek_instance *inst, int count, co
     GK_TRY(dalloc(ctx, &b->members, (size_t)N * L));
     GK_TRY(dalloc(ctx, &b->obj_bucket, (size_t)N * L));
     GK_TRY(dalloc(ctx, &b->flag_rows, (size_t)std::max<int64_t>(N, 1)));
+    GK_TRY(dalloc(ctx, &b->flag_m, (size_t)std::max<int64_t>(N, 1)));
     GK_TRY(dalloc(ctx, &b->n_flag, 1));
     b->k.assign(count, 0);
     b->seed_base.assign(count + 1, 0);
@@ -533,6 +536,7 @@ geek_status build_assign(geek_batch *b, int32_t *labels, cudaStream_t st) {
     b->tc.allow_split = b->p.precision == GEEK_PREC_AUTO;
     GK_TRY(tc_plan_build(ctx, nullptr, tp, &b->tc, st));
     GK_TRY(decide_bufs_alloc(ctx, nullptr, count, b->N, b->dec));
+    GK_TRY(tc_emit_alloc(ctx, nullptr, &b->tc, b->N, st));
     GK_CUDA(ctx, cudaStreamSynchronize(st));
     b->a_k = b->k;
     b->a_labels = labels;
@@ -556,8 +560,9 @@ geek_status enqueue_assign(geek_batch *b, int32_t *labels, cudaStream_t s) {
     GK_CUDA(ctx, cudaMemsetAsync(b->n_flag, 0, sizeof(unsigned long long), s));
     GK_TRY(fill_labels(ctx, labels, b->N, -1, s));
     GK_TRY(enqueue_centres(b, s));
-    GK_TRY(tc_plan_launch(ctx, b->tc, b->flag_rows, b->n_flag, s));
-    GK_TRY(decide_flags(ctx, b->rinst, b->hb.row_off, b->count, b->dmax, b->flag_rows, b->n_flag, b->dec, s));
+    GK_TRY(tc_plan_launch(ctx, b->tc, b->flag_rows, b->flag_m, b->n_flag, s));
+    GK_TRY(decide_flags(ctx, b->tc, b->rinst, b->hb.row_off, b->count, b->dmax, b->flag_rows, b->flag_m, b->n_flag, b->N,
+                        b->dec, s));
     GK_TRY(centre_split(ctx, b->c64, b->kd_tot, b->chi, b->clo, s));
     GK_TRY(stats_batch(ctx, b->sinst, b->st_units, b->n_st_units, b->st_uoff, b->count, b->part_sum, b->part_max,
                        b->sse_d, b->rmax_d, s));
@@ -603,11 +608,12 @@ geek_status autotune(geek_batch *b, cudaStream_t st) {
         for (auto c = classes.begin(); c != classes.end() && rc == GEEK_OK; ++c) {
             // at most ~8 units per SM of this class's instances
             std::vector<int> which;
-            int64_t units = 0;
+            int64_t units = 0, rows = 0;
             for (int i : c->second) {
                 if (units > (int64_t)ctx->num_sms * 8) break;
                 which.push_back(i);
                 units += ceil_div(b->inst[i].n, 128);
+                rows += b->inst[i].n;
             }
             const int dcls = b->inst[c->second[0]].d;
             for (int q = 0; q < nc && rc == GEEK_OK; q++) {
@@ -619,10 +625,10 @@ geek_status autotune(geek_batch *b, cudaStream_t st) {
                 for (int rep = 0; rep < 2 && rc == GEEK_OK; rep++) {
                     cudaMemsetAsync(b->n_flag, 0, sizeof(unsigned long long), st);
                     cudaEventRecord(e0, st);
-                    rc = tc_plan_launch_subset(ctx, &b->tc, which, b->flag_rows, b->n_flag, st);
+                    rc = tc_plan_launch_subset(ctx, &b->tc, which, b->flag_rows, b->flag_m, b->n_flag, st);
                     if (rc == GEEK_OK)
-                        rc = decide_flags(ctx, b->rinst, b->hb.row_off, b->count, b->dmax, b->flag_rows, b->n_flag,
-                                          b->dec, st);
+                        rc = decide_flags(ctx, b->tc, b->rinst, b->hb.row_off, b->count, b->dmax, b->flag_rows,
+                                          b->flag_m, b->n_flag, rows, b->dec, st);
                     cudaEventRecord(e1, st);
                     if (cudaEventSynchronize(e1) != cudaSuccess && rc == GEEK_OK)
                         rc = set_error(ctx, GEEK_ERR_CUDA, "autotune run failed: %s", cudaGetErrorString(cudaGetLastError()));

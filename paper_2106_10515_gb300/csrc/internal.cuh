@@ -1,5 +1,8 @@
 // Host-side entry points shared between translation units.
 #pragma once
+#include <cuda.h>
+#include <cuda_bf16.h>
+
 #include <vector>
 
 #include "common.cuh"
@@ -213,29 +216,50 @@ struct TcPlan {
     float *xnorm = nullptr;
     unsigned *cmax_bits = nullptr;
     int *err = nullptr;
+    // the exact decision's waves (tc_emit_alloc): gathered rows of kg columns,
+    // their limits and candidate masks of kw words
+    __nv_bfloat16 *xg = nullptr;
+    float *emit_lim = nullptr;
+    uint32_t *emit_masks = nullptr;
+    CUtensorMap *tmG = nullptr;
+    int kg = 0, kw = 0;
+    int64_t emit_units = 0;
     std::vector<void *> owned;
 };
+// Flagged rows grouped by instance in units of up to 128: unit u holds the
+// global rows grows[unit_start[u] .. + unit_cnt[u]] of instance unit_inst[u].
+struct FlagUnits {
+    const int32_t *grows;
+    const int *unit_inst;
+    const int64_t *unit_start;
+    const int *unit_cnt;
+    const int *n_units;
+};
+struct RInst;
+geek_status tc_emit_alloc(geek_ctx *ctx, Scratch *scr, TcPlan *P, int64_t max_rows, cudaStream_t st);
+geek_status tc_decide_candidates(geek_ctx *ctx, const TcPlan &P, const RInst *R, const FlagUnits &F, const float *mrow,
+                                 int64_t max_rows, int32_t *left, unsigned long long *n_left, cudaStream_t st);
 // scr == nullptr: buffers are cudaMalloc'd and owned by the plan
 geek_status tc_plan_build(geek_ctx *ctx, Scratch *scr, const std::vector<TcPlanInst> &desc, TcPlan *P,
                           cudaStream_t st);
 // conversions of X and the centres (BF16, norms, max |c|^2)
 geek_status tc_plan_convert(geek_ctx *ctx, const TcPlan &P, cudaStream_t st);
 // the persistent tcgen05 pass (after tc_plan_convert); n_flag zeroed by the caller
-geek_status tc_plan_launch(geek_ctx *ctx, const TcPlan &P, int32_t *flag_rows, unsigned long long *n_flag,
-                           cudaStream_t st);
-geek_status tc_plan_enqueue(geek_ctx *ctx, const TcPlan &P, int32_t *flag_rows, unsigned long long *n_flag,
-                            cudaStream_t st);
+geek_status tc_plan_launch(geek_ctx *ctx, const TcPlan &P, int32_t *flag_rows, float *flag_m,
+                           unsigned long long *n_flag, cudaStream_t st);
+geek_status tc_plan_enqueue(geek_ctx *ctx, const TcPlan &P, int32_t *flag_rows, float *flag_m,
+                            unsigned long long *n_flag, cudaStream_t st);
 geek_status tc_plan_upload(geek_ctx *ctx, TcPlan *P, cudaStream_t st);
 geek_status tc_plan_set_modes(geek_ctx *ctx, TcPlan *P, const std::vector<int> &N, const std::vector<int> &split,
                               cudaStream_t st);
 geek_status tc_plan_launch_subset(geek_ctx *ctx, TcPlan *P, const std::vector<int> &which, int32_t *flag_rows,
-                                  unsigned long long *n_flag, cudaStream_t st);
+                                  float *flag_m, unsigned long long *n_flag, cudaStream_t st);
 geek_status tc_plan_check(geek_ctx *ctx, const TcPlan &P, cudaStream_t st);
 void tc_plan_free(TcPlan *P);
 int tc_tile_candidates(const int **tiles);
 geek_status assign_tc_bf16(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx, int64_t n, int d,
                            const double *centres, int64_t k, int split, int32_t *labels, int32_t *flag_rows,
-                           unsigned long long *n_flag, cudaStream_t st);
+                           float *flag_m, unsigned long long *n_flag, TcPlan *P, cudaStream_t st);
 
 // assign.cu
 // Centre preparation of one instance (device copies): FP32 copy and |c|^2
@@ -295,6 +319,9 @@ struct DecideBufs {
     int64_t *unit_start = nullptr;
     int *unit_cnt = nullptr;
     int *n_units = nullptr;
+    int64_t *seg_off = nullptr, *unit_off = nullptr;  // count + 1: rows, units before an instance
+    int32_t *left = nullptr;       // rows undecided among their candidates
+    unsigned long long *n_left = nullptr;
     int32_t *grows = nullptr;      // flagged rows grouped by instance
     int32_t *flags2 = nullptr;     // rows left to the FP64 reference
     float *flags2_m = nullptr;     // their smallest FP32 value (NaN: none)
@@ -304,9 +331,9 @@ struct DecideBufs {
 };
 geek_status decide_bufs_alloc(geek_ctx *ctx, Scratch *scr, int count, int64_t n_total, DecideBufs &B);
 void decide_bufs_free(DecideBufs &B);
-geek_status decide_flags(geek_ctx *ctx, const RInst *R, const int64_t *row_off, int count, int dmax,
-                         const int32_t *flags, const unsigned long long *n_flag, const DecideBufs &B,
-                         cudaStream_t st);
+geek_status decide_flags(geek_ctx *ctx, const TcPlan &P, const RInst *R, const int64_t *row_off, int count, int dmax,
+                         const int32_t *flags, const float *flag_m, const unsigned long long *n_flag,
+                         int64_t max_rows, const DecideBufs &B, cudaStream_t st);
 geek_status assign_dense_centres(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx,
                                  int64_t n, int d, const double *centres, int64_t k, int precision,
                                  int32_t *labels, geek_assign_stats *stats, cudaStream_t st);

@@ -40,6 +40,7 @@ struct TcInst {
     int64_t n, k;
     int64_t row_base;            // global row of local row 0 (flag list entries)
     int ntiles_c, Kp, d, N;      // centre tiles of N columns, padded d, d, tile N
+    int split;                   // stored as [hi | lo] pairs
 };
 
 // Per-instance conversion arguments (device copies).
@@ -80,14 +81,28 @@ constexpr int TC_B_STAGE_X3 = TC_B_STAGE / 2;
 static_assert(TC_A_STAGE_X3 + TC_B_STAGE_X3 == TC_A_STAGE + TC_B_STAGE, "both modes share one layout size");
 constexpr uint32_t TC_TMEM_COLS = 512;
 
+// EMIT: a wave of gathered flagged rows instead of an instance's own.  Slot s of
+// the wave is row s of the gathered buffer; unit u (128 slots) belongs to
+// instance unit_inst[u0 + u].
+struct TcEmit {
+    const CUtensorMap *tmG;      // gathered rows, box {64, 128}
+    const float *lim;            // per slot: a centre up to this value is a candidate
+    uint32_t *masks;             // per slot kw words: bit j = centre j is a candidate
+    int kw;
+    const int *unit_inst;
+    const int *n_units;          // of all waves
+    int64_t u0;                  // first unit of this wave
+};
 struct TcArgs {
     const TcInst *inst;
     const int2 *units;           // (instance, row tile); null: instance 0, unit = row tile
     int64_t nunits;
-    int32_t *flag_rows;          // global rows whose argmin needs the FP64 decision
+    int32_t *flag_rows;          // global rows whose argmin needs the exact decision
+    float *flag_m;               // their smallest values (NaN: none finite), beside flag_rows
     unsigned long long *n_flag;
     int *err;
     int lg_ns;                   // log2 of the centre-tile ring's stages (1..3)
+    TcEmit e;
 };
 
 // three-input minimum
@@ -179,6 +194,35 @@ __device__ __forceinline__ void epi_tile(uint32_t tbase, int64_t jb, float &b1, 
     }
 }
 
+// The candidates of one warp's rows among NCH 32-column chunks: bit i of
+// out[ch] = column jb + 32 ch + i is at most lim.
+template <int NCH>
+__device__ __forceinline__ void emit_tile(uint32_t tbase, float lim, uint32_t *__restrict__ out) {
+    uint32_t ra[32], rb[32];
+    tmem_ld32_async(tbase, ra);
+    tmem_wait_ld();
+#pragma unroll
+    for (int ch = 0; ch < NCH; ch++) {
+        if (ch + 1 < NCH) {
+            if (ch & 1) tmem_ld32_async(tbase + (ch + 1) * 32, ra);
+            else tmem_ld32_async(tbase + (ch + 1) * 32, rb);
+        }
+        const uint32_t *r = (ch & 1) ? rb : ra;
+        float tm = FLT_MAX;
+#pragma unroll
+        for (int i = 0; i < 30; i += 3)
+            tm = fminf(tm, min3f(__uint_as_float(r[i]), __uint_as_float(r[i + 1]), __uint_as_float(r[i + 2])));
+        tm = min3f(tm, __uint_as_float(r[30]), __uint_as_float(r[31]));
+        uint32_t m = 0;
+        if (tm <= lim) {
+#pragma unroll
+            for (int i = 0; i < 32; i++) m |= (__uint_as_float(r[i]) <= lim ? 1u : 0u) << i;
+        }
+        out[ch] = m;
+        if (ch + 1 < NCH) tmem_wait_ld();
+    }
+}
+
 // Index (first position) of the minimum in the saved chunk and the exact
 // runner-up over all columns.
 __device__ __forceinline__ void epi_resolve(float b1, float b2o, const float (&sv)[32], int64_t sj, float &b2,
@@ -203,7 +247,10 @@ __device__ __forceinline__ void epi_resolve(float b1, float b2o, const float (&s
 // SPLIT = true: x = x_h + x_l and c = c_h + c_l in BF16 pairs, S = x_h . c_h +
 // x_l . c_h + x_h . c_l: three MMAs per k-step into the same accumulator
 // (window_bf16x3, ~100x narrower).
-template <bool SPLIT>
+// EMIT: the rows are gathered flagged rows and the epilogue writes, instead of
+// the argmin, the mask of every row's candidates (units of the other mode's
+// instances are left to the launch of that mode).
+template <bool SPLIT, bool EMIT>
 __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc(const __grid_constant__ TcArgs A) {
     constexpr int A_ST = SPLIT ? TC_A_STAGE_X3 : TC_A_STAGE;
     constexpr int B_ST = SPLIT ? TC_B_STAGE_X3 : TC_B_STAGE;
@@ -255,6 +302,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc(const __grid_consta
     __syncthreads();
     fence_after();
     const uint32_t tmem = *tmem_slot;
+    const int64_t nunits = EMIT ? max((int64_t)0, min(A.nunits, (int64_t)*A.e.n_units - A.e.u0)) : A.nunits;
+    auto unit = [&](int64_t u) {
+        if (EMIT) return make_int2(A.e.unit_inst[A.e.u0 + u], (int)u);
+        return A.units ? A.units[u] : make_int2(0, (int)u);
+    };
 
     // Every role walks the same unit sequence (unit u = blockIdx.x + j *
     // gridDim.x); an instance's Kp, N and centre-tile count fix the per-unit
@@ -266,9 +318,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc(const __grid_consta
             uint32_t issued_b[8] = {0, 0, 0, 0, 0, 0, 0, 0};
             bool ok = true;
             int64_t it = 0;
-            for (int64_t u = blockIdx.x; u < A.nunits && ok; u += gridDim.x, it++) {
-                const int2 un = A.units ? A.units[u] : make_int2(0, (int)u);
+            for (int64_t u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
+                const int2 un = unit(u);
                 const TcInst &I = A.inst[un.x];
+                if (EMIT && (I.split != 0) != SPLIT) continue;
                 const int nkb = KW * I.Kp / TC_KB, N = I.N;  // stored k-blocks
                 const uint32_t a_bytes = (uint32_t)TC_M * KW * I.Kp * 2, b_bytes = (uint32_t)N * KW * I.Kp * 2;
                 const int ab = (int)(it & 1);
@@ -276,8 +329,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc(const __grid_consta
                 if (!(ok = mbar_wait(&empty_a[ab], (ua & 1) ^ 1, A.err))) break;
                 mbar_expect_tx(&full_a[ab], a_bytes);
                 for (int kb = 0; kb < nkb; kb++)
-                    tma_load_2d(su32(sA0 + ab * A_ST + kb * TC_M * 128), &I.tmA, kb * TC_KB, un.y * TC_M,
-                                &full_a[ab]);
+                    tma_load_2d(su32(sA0 + ab * A_ST + kb * TC_M * 128), EMIT ? A.e.tmG : &I.tmA, kb * TC_KB,
+                                un.y * TC_M, &full_a[ab]);
                 for (int c = 0; c < I.ntiles_c; c++, ct++) {
                     const int s = (int)(ct & (uint64_t)(NS - 1));
                     const uint32_t uu = (uint32_t)(ct >> A.lg_ns);
@@ -288,6 +341,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc(const __grid_consta
                     tma_load_2d(su32(sX0 + s * XSTR), &I.tmX, 0, c * N, &full_b[s]);
                     issued_b[s] = uu + 1;
                 }
+                it++;
             }
             // drain: every centre-tile copy this thread issued has landed
             for (int s = 0; s < NS; s++)
@@ -300,9 +354,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc(const __grid_consta
             uint64_t ct = 0;
             bool ok = true;
             int64_t it = 0;
-            for (int64_t u = blockIdx.x; u < A.nunits && ok; u += gridDim.x, it++) {
-                const int2 un = A.units ? A.units[u] : make_int2(0, (int)u);
+            for (int64_t u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
+                const int2 un = unit(u);
                 const TcInst &I = A.inst[un.x];
+                if (EMIT && (I.split != 0) != SPLIT) continue;
                 const int nkb = I.Kp / TC_KB, N = I.N;  // logical k-blocks
                 const uint32_t idesc = idesc_bf16(TC_M, N);
                 const int ab = (int)(it & 1);
@@ -336,6 +391,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc(const __grid_consta
                     mma_commit(&full_acc[s]);
                 }
                 mma_commit(&empty_a[ab]);
+                it++;
             }
             // drain: all MMAs this thread issued have completed
             mma_commit(done_bar);
@@ -350,13 +406,38 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc(const __grid_consta
         const int rloc = 32 * q + lane;
         uint64_t ct = 0;
         bool ok = true;
-        for (int64_t u = blockIdx.x; u < A.nunits; u += gridDim.x) {
-            const int2 un = A.units ? A.units[u] : make_int2(0, (int)u);
+        for (int64_t u = blockIdx.x; u < nunits; u += gridDim.x) {
+            const int2 un = unit(u);
             const TcInst &I = A.inst[un.x];
+            if (EMIT && (I.split != 0) != SPLIT) continue;
             const int N = I.N;
             const int gcols = N / TC_EPI_GROUPS;  // columns of this warp's group
             const int nch = gcols / 32;           // 32-column chunks (1, 2 or 4)
             const int64_t row = (int64_t)un.y * TC_M + rloc;
+            if (EMIT) {
+                const float lim = A.e.lim[row];
+                uint32_t *out = A.e.masks + row * A.e.kw;
+                for (int c = 0; c < I.ntiles_c; c++, ct++) {
+                    const int s = (int)(ct & 1);
+                    const uint32_t uu = (uint32_t)(ct >> 1);
+                    int w_ok = 0;
+                    if (lane == 0 && ok) w_ok = mbar_wait(&full_acc[s], uu & 1, A.err);
+                    w_ok = __shfl_sync(0xffffffffu, w_ok, 0);
+                    ok = ok && w_ok;
+                    if (ok) {
+                        fence_after();
+                        const uint32_t tbase = tmem + (uint32_t)(s * TC_N + h * gcols) + ((uint32_t)(32 * q) << 16);
+                        uint32_t *o = out + (c * N + h * gcols) / 32;
+                        if (nch == 4) emit_tile<4>(tbase, lim, o);
+                        else if (nch == 2) emit_tile<2>(tbase, lim, o);
+                        else emit_tile<1>(tbase, lim, o);
+                        fence_before();
+                    }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&empty_acc[s]);
+                }
+                continue;
+            }
             const float xn = row < I.n ? I.xnorm[row] : 0.f;
             const float cmax = sqrtf(__uint_as_float(*I.cmax_bits)) * (1.f + 1e-5f);
             const float W = 2.f * (SPLIT ? window_bf16x3(xn, cmax, I.d) : window_bf16(xn, cmax, I.d));
@@ -418,6 +499,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc(const __grid_consta
                 if (!sure) {
                     const unsigned long long qq = atomicAdd(A.n_flag, 1ull);
                     A.flag_rows[qq] = (int32_t)(I.row_base + row);
+                    A.flag_m[qq] = valid ? b1 : __int_as_float(0x7fc00000);
                 }
             }
             asm volatile("bar.sync 1, %0;" ::"r"(32 * TC_EPI_WARPS) : "memory");
@@ -588,6 +670,7 @@ geek_status make_inst(geek_ctx *ctx, const TcPlan &P, int i, int N, TcInst *out)
     T.Kp = Kp;
     T.d = I.d;
     T.N = N;
+    T.split = I.split;
     *out = T;
     return GEEK_OK;
 }
@@ -690,8 +773,9 @@ geek_status tc_plan_build(geek_ctx *ctx, Scratch *scr, const std::vector<TcPlanI
     GK_CUDA(ctx, cudaMemcpyAsync(P->kpad_off_dev, im.kpad_off.data(), sizeof(int64_t) * (count + 1),
                                  cudaMemcpyHostToDevice, st));
     GK_TRY(tc_plan_upload(ctx, P, st));
-    GK_CUDA(ctx, cudaFuncSetAttribute(k_assign_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem()));
-    GK_CUDA(ctx, cudaFuncSetAttribute(k_assign_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem()));
+    for (const void *fn : {(const void *)k_assign_tc<false, false>, (const void *)k_assign_tc<true, false>,
+                           (const void *)k_assign_tc<false, true>, (const void *)k_assign_tc<true, true>})
+        GK_CUDA(ctx, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem()));
     return GEEK_OK;
 }
 
@@ -770,11 +854,12 @@ int ring_lg(const TcPlan &P, const std::vector<int> *which, int split) {
 }
 
 geek_status launch_units(geek_ctx *ctx, const TcInst *inst, const int2 *units, int64_t n0, int64_t n1,
-                         int32_t *flag_rows, unsigned long long *n_flag, int *err, double work, int lg0, int lg1,
-                         cudaStream_t st) {
-    TcArgs A;
+                         int32_t *flag_rows, float *flag_m, unsigned long long *n_flag, int *err, double work, int lg0,
+                         int lg1, cudaStream_t st) {
+    TcArgs A{};
     A.inst = inst;
     A.flag_rows = flag_rows;
+    A.flag_m = flag_m;
     A.n_flag = n_flag;
     A.err = err;
     EvTimer tk(ctx, "kernel.assign_tc", st);
@@ -784,14 +869,14 @@ geek_status launch_units(geek_ctx *ctx, const TcInst *inst, const int2 *units, i
         A.nunits = n0;
         A.lg_ns = lg0;
         GK_COUNT();
-        k_assign_tc<false><<<(int)std::min<int64_t>(n0, ctx->num_sms), TC_THREADS, tc_smem(), st>>>(A);
+        k_assign_tc<false, false><<<(int)std::min<int64_t>(n0, ctx->num_sms), TC_THREADS, tc_smem(), st>>>(A);
     }
     if (n1 > 0) {
         A.units = units + n0;
         A.nunits = n1;
         A.lg_ns = lg1;
         GK_COUNT();
-        k_assign_tc<true><<<(int)std::min<int64_t>(n1, ctx->num_sms), TC_THREADS, tc_smem(), st>>>(A);
+        k_assign_tc<true, false><<<(int)std::min<int64_t>(n1, ctx->num_sms), TC_THREADS, tc_smem(), st>>>(A);
     }
     GK_LAUNCH(ctx);
     return GEEK_OK;
@@ -802,18 +887,18 @@ geek_status launch_units(geek_ctx *ctx, const TcInst *inst, const int2 *units, i
 // The persistent tcgen05 passes (BF16 units, then split-BF16 units) after
 // tc_plan_convert; flagged rows are appended to flag_rows / n_flag (zeroed
 // by the caller).
-geek_status tc_plan_launch(geek_ctx *ctx, const TcPlan &P, int32_t *flag_rows, unsigned long long *n_flag,
-                           cudaStream_t st) {
+geek_status tc_plan_launch(geek_ctx *ctx, const TcPlan &P, int32_t *flag_rows, float *flag_m,
+                           unsigned long long *n_flag, cudaStream_t st) {
     double work = 0.0;
     for (const TcPlanInst &I : P.desc) work += 2.0 * (double)I.n * (double)I.k * (double)I.d;
-    return launch_units(ctx, P.inst, P.units, P.nunits, P.nunits_x3, flag_rows, n_flag, P.err, work,
+    return launch_units(ctx, P.inst, P.units, P.nunits, P.nunits_x3, flag_rows, flag_m, n_flag, P.err, work,
                         ring_lg(P, nullptr, 0), ring_lg(P, nullptr, 1), st);
 }
 
-geek_status tc_plan_enqueue(geek_ctx *ctx, const TcPlan &P, int32_t *flag_rows, unsigned long long *n_flag,
-                            cudaStream_t st) {
+geek_status tc_plan_enqueue(geek_ctx *ctx, const TcPlan &P, int32_t *flag_rows, float *flag_m,
+                            unsigned long long *n_flag, cudaStream_t st) {
     GK_TRY(tc_plan_convert(ctx, P, st));
-    return tc_plan_launch(ctx, P, flag_rows, n_flag, st);
+    return tc_plan_launch(ctx, P, flag_rows, flag_m, n_flag, st);
 }
 
 // Sets every instance's tile width and mode (descriptors re-encoded, units
@@ -835,7 +920,7 @@ geek_status tc_plan_set_modes(geek_ctx *ctx, TcPlan *P, const std::vector<int> &
 // tc_plan_convert after tc_plan_set_modes).  Uses the plan's scratch
 // descriptor table; writes labels and flags of those rows.  No host sync.
 geek_status tc_plan_launch_subset(geek_ctx *ctx, TcPlan *P, const std::vector<int> &which, int32_t *flag_rows,
-                                  unsigned long long *n_flag, cudaStream_t st) {
+                                  float *flag_m, unsigned long long *n_flag, cudaStream_t st) {
     auto &im = *P->impl;
     std::vector<int2> u0, u1;
     make_units(*P, which, 0, u0);
@@ -856,8 +941,8 @@ geek_status tc_plan_launch_subset(geek_ctx *ctx, TcPlan *P, const std::vector<in
     GK_CUDA(ctx, cudaMemcpyAsync(P->tune_units, u0.data(), sizeof(int2) * u0.size(), cudaMemcpyHostToDevice, st));
     GK_CUDA(ctx, cudaStreamSynchronize(st));  // u0 is pageable and about to go out of scope
     (void)im;
-    return launch_units(ctx, P->inst, P->tune_units, n0, n1, flag_rows, n_flag, P->err, 0.0, ring_lg(*P, &which, 0),
-                        ring_lg(*P, &which, 1), st);
+    return launch_units(ctx, P->inst, P->tune_units, n0, n1, flag_rows, flag_m, n_flag, P->err, 0.0,
+                        ring_lg(*P, &which, 0), ring_lg(*P, &which, 1), st);
 }
 
 geek_status tc_plan_check(geek_ctx *ctx, const TcPlan &P, cudaStream_t st) {
@@ -879,24 +964,247 @@ void tc_plan_free(TcPlan *P) {
 }
 
 // BF16 (split = 0) or split-BF16 (split = 1) tcgen05 pass of one data set:
-// labels for every object, flagged rows appended to flag_rows / n_flag for
-// the FP64 decision.  d <= 128.
+// labels for every object, flagged rows appended to flag_rows / flag_m / n_flag
+// for the exact decision, which may use the plan P (buffers in scr).  d <= 128.
 geek_status assign_tc_bf16(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx, int64_t n, int d,
                            const double *centres, int64_t k, int split, int32_t *labels, int32_t *flag_rows,
-                           unsigned long long *n_flag, cudaStream_t st) {
+                           float *flag_m, unsigned long long *n_flag, TcPlan *P, cudaStream_t st) {
     if (d > 128) return set_error(ctx, GEEK_ERR_UNSUPPORTED, "BF16 tensor-core assignment supports d <= 128");
-    TcPlan P;
     std::vector<TcPlanInst> one(1);
     // BF16: N = 256 (two stages; 128-wide tiles read A from shared memory
     // twice as often per flop and measured ~60% slower at d = 128).  Split:
     // the widest tile whose hi|lo stage fits
     const int N = split ? (d <= 64 ? 128 : 64) : TC_N;
     one[0] = TcPlanInst{x, ldx, n, d, centres, k, labels, 0, N, split};
-    struct Free {
-        TcPlan *p;
-        ~Free() { tc_plan_free(p); }
-    } fr{&P};
-    GK_TRY(tc_plan_build(ctx, &scr, one, &P, st));
-    GK_TRY(tc_plan_enqueue(ctx, P, flag_rows, n_flag, st));
-    return tc_plan_check(ctx, P, st);
+    GK_TRY(tc_plan_build(ctx, &scr, one, P, st));
+    GK_TRY(tc_plan_enqueue(ctx, *P, flag_rows, flag_m, n_flag, st));
+    return tc_plan_check(ctx, *P, st);
+}
+
+// ---- candidates of the flagged rows ------------------------------------------
+namespace {
+
+// Slot s of the wave starting at unit u0: the flagged row's stored BF16 row
+// (warp per slot, 16 bytes per lane) and its limit m + 2W: every centre that
+// can be the exact argmin has a fast value of at most that (m: the smallest
+// fast value the first pass saw, W the rigorous half-window of the mode).  A
+// slot without a row, or whose limit is not finite, gets -inf: no candidate.
+__global__ void __launch_bounds__(256) k_gather_flagged(const TcInst *__restrict__ inst, const TcXPrep *__restrict__ X,
+                                                        const int64_t *__restrict__ row_off, FlagUnits F,
+                                                        const float *__restrict__ mrow, int64_t u0, int64_t umax,
+                                                        __nv_bfloat16 *__restrict__ xg, int kg,
+                                                        float *__restrict__ lim) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t nslots = TC_M * max((int64_t)0, min(umax, (int64_t)*F.n_units - u0));
+    for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < nslots; s += nw) {
+        const int64_t u = u0 + s / TC_M;
+        const int r = (int)(s % TC_M), ii = F.unit_inst[u];
+        float l = -INFINITY;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (r < F.unit_cnt[u]) {
+            const int64_t g = F.grows[F.unit_start[u] + r], i = g - row_off[ii];
+            const TcXPrep &P = X[ii];
+            const TcInst &I = inst[ii];
+            const int W = P.split ? 2 * P.Kp : P.Kp;
+            if (8 * lane < W) v = *reinterpret_cast<const uint4 *>(P.xb + i * W + 8 * lane);
+            const float cmax = sqrtf(__uint_as_float(*I.cmax_bits)) * (1.f + 1e-5f);
+            const float w2 = 2.f * (P.split ? window_bf16x3(I.xnorm[i], cmax, P.d) : window_bf16(I.xnorm[i], cmax, P.d));
+            const float m = mrow[g], q = fmaf(w2, 1.f + 1e-6f, m) + fabsf(m) * 1.2e-7f;
+            if (fabsf(q) < FLT_MAX) l = q;
+        }
+        if (8 * lane < kg) *reinterpret_cast<uint4 *>(xg + s * kg + 8 * lane) = v;
+        if (lane == 0) lim[s] = l;
+    }
+}
+
+// The exact argmin among a flagged row's candidates, a warp per slot.  The
+// direct distance D = sum (x - c)^2 in FP32 has none of the cancellation of
+// |c|^2 - 2 x.c: with u = 2^-24, C = max |c| and D' its FP32 value (centres
+// rounded to FP32, differences, FMA chain over lanes and a shuffle tree),
+//   |D' - D| <= ((d + 6) u D' + 2.001 u C sqrt(D') + 4.1 u^2 C^2)(1 + 10^-4)
+// (|x - c32| is off by u|x - c32| + u|c| per coordinate, Cauchy-Schwarz over the
+// coordinates, gamma_(d+4) for the sum), and the FP64 reference's own error
+// is below d 2^-52 D; err() rounds all of it up by 5 %.  Where the smallest
+// D' is apart from the second by both errors the label is decided; else (and
+// without a candidate) the row goes on to `left`, for the FP32 scan and the
+// FP64 reference.  A warp's eight-lane groups take a candidate each, lane l of a
+// group the coordinates 4 l .. 4 l + 3 of each 32: a group's loads of a centre
+// are whole 128-byte lines.
+__global__ void __launch_bounds__(256) k_decide_candidates(const RInst *__restrict__ R, FlagUnits F, int64_t u0,
+                                                           int64_t umax, const uint32_t *__restrict__ masks, int kw,
+                                                           int32_t *__restrict__ left,
+                                                           unsigned long long *__restrict__ n_left) {
+    __shared__ uint16_t s_list[8][1024];
+    const int lane = threadIdx.x & 31, grp = lane >> 3, sub = lane & 7;
+    uint16_t *list = s_list[threadIdx.x >> 5];
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t nslots = TC_M * max((int64_t)0, min(umax, (int64_t)*F.n_units - u0));
+    for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < nslots; s += nw) {
+        const int64_t u = u0 + s / TC_M;
+        const int r = (int)(s % TC_M);
+        if (r >= F.unit_cnt[u]) continue;
+        const RInst &I = R[F.unit_inst[u]];
+        const int64_t g = F.grows[F.unit_start[u] + r], row = g - I.row_base;
+        const int d = I.d;
+        const bool vec = ((d & 3) == 0) && ((I.ldx & 3) == 0) && ((((uintptr_t)I.x) | ((uintptr_t)I.c32)) & 15) == 0;
+        auto load4 = [&](const float *p, int t) {  // coordinates t .. t + 3, zeros past d
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (vec) {
+                if (t < d) v = *reinterpret_cast<const float4 *>(p + t);
+            } else {
+                if (t < d) v.x = p[t];
+                if (t + 1 < d) v.y = p[t + 1];
+                if (t + 2 < d) v.z = p[t + 2];
+                if (t + 3 < d) v.w = p[t + 3];
+            }
+            return v;
+        };
+        float4 xv[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) xv[q] = load4(I.x + row * I.ldx, 32 * q + 4 * sub);
+        const uint32_t *mk = masks + s * kw;
+        const int nwords = (int)((I.k + 31) >> 5);
+        float b1 = FLT_MAX, b2 = FLT_MAX;  // this group's smallest and second D'
+        int bj = 0x7FFFFFFF, total = 0;
+        bool bad = false;
+        for (int w0 = 0; w0 < nwords; w0 += 32) {
+            uint32_t m = w0 + lane < nwords ? mk[w0 + lane] : 0u;
+            if (w0 + lane == nwords - 1 && (I.k & 31)) m &= (1u << (I.k & 31)) - 1u;  // no index past the centres
+            int inc = __popc(m);
+            const int mine = inc;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += y;
+            }
+            const int cnt = __shfl_sync(0xffffffffu, inc, 31);
+            if (cnt == 0) continue;
+            __syncwarp();
+            for (int at = inc - mine; m; m &= m - 1, at++) list[at] = (uint16_t)(32 * lane + __ffs((int)m) - 1);
+            __syncwarp();
+            total += cnt;
+            for (int q0 = 0; q0 < cnt; q0 += 8) {  // two candidates per group in flight
+                float D[2];
+                int j[2];
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    const int q = q0 + 4 * h + grp;
+                    j[h] = q < cnt ? 32 * w0 + (int)list[q] : -1;
+                    const float *c = I.c32 + (int64_t)max(j[h], 0) * d;
+                    D[h] = 0.f;
+#pragma unroll
+                    for (int e = 0; e < 4; e++) {
+                        if (32 * e >= d) break;
+                        const float4 cv = load4(c, 32 * e + 4 * sub);
+                        const float e0 = xv[e].x - cv.x, e1 = xv[e].y - cv.y;
+                        const float e2 = xv[e].z - cv.z, e3 = xv[e].w - cv.w;
+                        D[h] = fmaf(e3, e3, fmaf(e2, e2, fmaf(e1, e1, fmaf(e0, e0, D[h]))));
+                    }
+                }
+#pragma unroll
+                for (int o = 1; o < 8; o <<= 1) {
+                    D[0] += __shfl_xor_sync(0xffffffffu, D[0], o);
+                    D[1] += __shfl_xor_sync(0xffffffffu, D[1], o);
+                }
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    if (j[h] < 0) continue;
+                    bad = bad || !(D[h] < FLT_MAX);
+                    if (D[h] < b1) {
+                        b2 = b1;
+                        b1 = D[h];
+                        bj = j[h];
+                    } else {
+                        b2 = fminf(b2, D[h]);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int o = 8; o < 32; o <<= 1) {  // the four groups
+            const float o1 = __shfl_xor_sync(0xffffffffu, b1, o), o2 = __shfl_xor_sync(0xffffffffu, b2, o);
+            const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
+            b2 = fminf(fminf(b2, o2), fmaxf(b1, o1));
+            if (o1 < b1) bj = oj;
+            b1 = fminf(b1, o1);
+        }
+        bad = __any_sync(0xffffffffu, bad);
+        if (lane == 0) {
+            const float C = __uint_as_float(*I.cmax_bits), uu = 5.9604645e-8f;
+            auto err = [&](float D) {
+                return 1.05f * ((float)(d + 6) * uu * D + 2.001f * uu * C * sqrtf(D) + 4.1f * uu * uu * C * C) + 1e-37f;
+            };
+            const bool sure = !bad && (total == 1 || (total > 1 && (b2 - b1) * (1.f - 1e-6f) > err(b1) + err(b2)));
+            if (sure) I.labels[row] = bj;
+            else left[atomicAdd(n_left, 1ull)] = (int32_t)g;
+        }
+    }
+}
+
+}  // namespace
+
+// The plan's part of the exact decision: per wave of flagged units (grouped by
+// decide_flags: F, every row's smallest value in mrow), gather the rows, find
+// their candidates with a second tcgen05 pass over them, and decide among the
+// candidates; what stays undecided is appended to left / n_left.  max_rows
+// bounds the flagged rows; no allocation and no host synchronisation (the
+// buffers are the plan's, tc_emit_alloc).
+geek_status tc_decide_candidates(geek_ctx *ctx, const TcPlan &P, const RInst *R, const FlagUnits &F, const float *mrow,
+                                 int64_t max_rows, int32_t *left, unsigned long long *n_left, cudaStream_t st) {
+    int64_t units = ceil_div(std::min(max_rows, P.N_total), TC_M) + P.count;
+    bool mode[2] = {false, false};
+    for (const TcPlanInst &I : P.desc)
+        if (I.n > 0 && I.k > 0) mode[I.split ? 1 : 0] = true;
+    EvTimer tk(ctx, "kernel.assign_candidates", st);
+    for (int64_t u0 = 0; u0 < units; u0 += P.emit_units) {
+        GK_COUNT();
+        k_gather_flagged<<<ctx->num_sms * 8, 256, 0, st>>>(P.inst, P.xprep, P.row_off, F, mrow, u0, P.emit_units,
+                                                           P.xg, P.kg, P.emit_lim);
+        TcArgs A{};
+        A.inst = P.inst;
+        A.nunits = P.emit_units;
+        A.err = P.err;
+        A.e = TcEmit{P.tmG, P.emit_lim, P.emit_masks, P.kw, F.unit_inst, F.n_units, u0};
+        for (int sp = 0; sp < 2; sp++) {
+            if (!mode[sp]) continue;
+            A.lg_ns = ring_lg(P, nullptr, sp);
+            GK_COUNT();
+            const int grid = (int)std::min<int64_t>(P.emit_units, ctx->num_sms);
+            if (sp) k_assign_tc<true, true><<<grid, TC_THREADS, tc_smem(), st>>>(A);
+            else k_assign_tc<false, true><<<grid, TC_THREADS, tc_smem(), st>>>(A);
+        }
+        GK_COUNT();
+        k_decide_candidates<<<ctx->num_sms * 8, 256, 0, st>>>(R, F, u0, P.emit_units, P.emit_masks, P.kw, left, n_left);
+        GK_LAUNCH(ctx);
+    }
+    return GEEK_OK;
+}
+
+// Buffers of tc_decide_candidates for at most max_rows flagged rows: a wave
+// holds as many units as fit EMIT_BYTES (gathered rows and masks), at least one
+// per SM.
+geek_status tc_emit_alloc(geek_ctx *ctx, Scratch *scr, TcPlan *P, int64_t max_rows, cudaStream_t st) {
+    constexpr int64_t EMIT_BYTES = 1ll << 30;
+    int kg = 64;
+    int64_t kw = 8;
+    for (const TcPlanInst &I : P->desc) {
+        const int Kp = I.d <= 64 ? 64 : 128;
+        kg = std::max(kg, (I.split || P->allow_split) ? 2 * Kp : Kp);
+        kw = std::max(kw, ceil_div(I.k, TC_N) * (TC_N / 32));
+    }
+    const int64_t unit_bytes = TC_M * (2 * (int64_t)kg + 4 * kw + 4);
+    const int64_t all = ceil_div(std::min(max_rows, P->N_total), TC_M) + P->count;
+    const int64_t units = std::min(all, std::max<int64_t>(EMIT_BYTES / unit_bytes, ctx->num_sms));
+    P->kg = kg;
+    P->kw = (int)kw;
+    P->emit_units = units;
+    GK_TRY(plan_alloc(ctx, scr, P->owned, &P->xg, (size_t)(units * TC_M * kg)));
+    GK_TRY(plan_alloc(ctx, scr, P->owned, &P->emit_lim, (size_t)(units * TC_M)));
+    GK_TRY(plan_alloc(ctx, scr, P->owned, &P->emit_masks, (size_t)(units * TC_M * kw)));
+    GK_TRY(plan_alloc(ctx, scr, P->owned, &P->tmG, 1));
+    CUtensorMap tm;
+    GK_TRY(encode_bf16_2d(ctx, &tm, P->xg, kg, (uint64_t)(units * TC_M), TC_KB, TC_M));
+    GK_CUDA(ctx, cudaMemcpyAsync(P->tmG, &tm, sizeof tm, cudaMemcpyHostToDevice, st));
+    return GEEK_OK;
 }
