@@ -8,6 +8,7 @@
 // order, each operation rounded to nearest, no fused multiply-add; ties go
 // to the smallest centre index.
 #include <cfloat>
+#include <cstddef>
 #include <type_traits>
 
 #include "internal.cuh"
@@ -71,7 +72,7 @@ struct FArgs {
     int d;
     const float *c32, *cn;
     int64_t k;
-    float cmax;
+    const unsigned *cmax_bits;
     int32_t *labels;
     int32_t *flag_rows;
     float *flag_m;  // may be null: the row's smallest fast value, beside flag_rows
@@ -115,7 +116,7 @@ __global__ void __launch_bounds__(256, 2) k_assign_fp32(FArgs A, GatherUnits U) 
             A.c32 = I.c32;
             A.cn = I.cn;
             A.k = I.k;
-            A.cmax = __uint_as_float(*I.cmax_bits);
+            A.cmax_bits = I.cmax_bits;
             A.labels = I.labels;
             rbase = I.row_base;
             nrows = U.f.unit_cnt[u];
@@ -232,6 +233,7 @@ __global__ void __launch_bounds__(256, 2) k_assign_fp32(FArgs A, GatherUnits U) 
                 B[r] = best_merge(B[r], o_);
             }
         }
+        const float cmax = __uint_as_float(*A.cmax_bits);
         // |x|^2 of the row group's rows, the coordinates over its 16 lanes
         float xs2[AS_RPT];
 #pragma unroll
@@ -251,7 +253,7 @@ __global__ void __launch_bounds__(256, 2) k_assign_fp32(FArgs A, GatherUnits U) 
                 if (rr >= nrows) continue;
                 const int64_t row = GATHER ? s_rows[rr] : row0 + rr;
                 const float xn = sqrtf(xs2[r]) * (1.f + 1.0e-3f);
-                const float W = 2.f * window_fp32(xn, A.cmax, d);
+                const float W = 2.f * window_fp32(xn, cmax, d);
                 // no finite value (non-finite input): undecided here, FP64 decides
                 const bool valid = B[r].i1 != 0x7FFFFFFF;
                 A.labels[row] = valid ? B[r].i1 : -1;
@@ -636,25 +638,46 @@ __global__ void __launch_bounds__(256) k_assign_recheck(const RInst *__restrict_
     }
 }
 
-// centre preparation: FP32 copy, |c|^2 (FP64 then rounded), max |c|;
-// thread per global centre e of instance find_inst(k_off, e)
-__global__ void k_centre_prep(const CInst *__restrict__ C, const int64_t *__restrict__ k_off, int count,
-                              int64_t ktot) {
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < ktot;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const CInst &I = C[find_inst(k_off, count, e)];
-        const int64_t j = e - I.k_base;
-        const int d = I.d;
-        double s = 0.0;
-        for (int t = 0; t < d; t++) {
-            const double v = I.c64[j * d + t];
-            I.c32[j * d + t] = (float)v;
-            s += v * v;
-        }
+// centre preparation: FP32 copy, |c|^2 (FP64 then rounded), max |c|; a warp per
+// centre, lanes over coordinates (a thread per centre took 26 us for 2,000
+// centres of 96 coordinates: a serial chain of FP64 adds and scattered loads)
+__device__ __forceinline__ void centre_prep(const CInst &I, int64_t j) {
+    const int lane = threadIdx.x & 31, d = I.d;
+    double s = 0.0;
+    for (int t = lane; t < d; t += 32) {
+        const double v = I.c64[j * d + t];
+        I.c32[j * d + t] = (float)v;
+        s += v * v;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) {
         I.cn[j] = (float)s;
         const float nrm = (float)sqrt(s) * (1.f + 1e-6f);
         atomicMax(I.cmax_bits, __float_as_uint(nrm));  // non-negative floats order as uints
     }
+}
+
+// global centre e of instance find_inst(k_off, e)
+__global__ void k_centre_prep(const CInst *__restrict__ C, const int64_t *__restrict__ k_off, int count,
+                              int64_t ktot) {
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < ktot; e += nw) {
+        const CInst &I = C[find_inst(k_off, count, e)];
+        centre_prep(I, e - I.k_base);
+    }
+}
+
+// one data set: its centres, and the one-instance tables of the kernels that
+// read them from memory (one launch instead of four small copies)
+struct OneTables {
+    RInst r;
+    int64_t row_off[2];
+};
+__global__ void k_centre_prep_one(CInst I, int64_t k, OneTables T, OneTables *__restrict__ out) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *out = T;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; j < k; j += nw) centre_prep(I, j);
 }
 
 // double-float split of the FP64 centres: c = hi + lo with hi = (float)c
@@ -796,17 +819,31 @@ __global__ void __launch_bounds__(256) k_assign_stats(const float *__restrict__ 
     }
 }
 
-__global__ void k_stats_final(const double *__restrict__ ps, const float *__restrict__ pm, int nb,
-                              double *__restrict__ out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        float m = 0.f;
-        for (int i = 0; i < nb; i++) {
-            s += ps[i];
-            m = fmaxf(m, pm[i]);
+// one block: the block partials in a fixed order (thread t takes partials t, t +
+// 256, ..., then a tree); a single thread took 0.25 ms for 4,864 of them
+__global__ void __launch_bounds__(256) k_stats_final(const double *__restrict__ ps, const float *__restrict__ pm, int nb,
+                                                     double *__restrict__ out) {
+    __shared__ double ss[256];
+    __shared__ float sx[256];
+    const int t = threadIdx.x;
+    double s = 0.0;
+    float m = 0.f;
+    for (int i = t; i < nb; i += 256) {
+        s += ps[i];
+        m = fmaxf(m, pm[i]);
+    }
+    ss[t] = s;
+    sx[t] = m;
+    for (int o = 128; o > 0; o >>= 1) {
+        __syncthreads();
+        if (t < o) {
+            ss[t] += ss[t + o];
+            sx[t] = fmaxf(sx[t], sx[t + o]);
         }
-        out[0] = s;
-        out[1] = sqrt((double)m);
+    }
+    if (t == 0) {
+        out[0] = ss[0];
+        out[1] = sqrt((double)sx[0]);
     }
 }
 
@@ -1661,44 +1698,32 @@ geek_status assign_dense_centres(geek_ctx *ctx, Scratch &scr, const float *x, in
     if (d > AS_MAXD) return set_error(ctx, GEEK_ERR_UNSUPPORTED, "dense assignment supports d <= %d", AS_MAXD);
     if (precision != GEEK_PREC_FP32 && precision != GEEK_PREC_BF16 && precision != GEEK_PREC_BF16X3)
         return set_error(ctx, GEEK_ERR_INVALID, "bad precision");
+    // the call's small words and tables share one allocation and one fill
+    struct Words {
+        unsigned long long n_flag;
+        double stats[2];
+        unsigned cmax_bits;
+        OneTables one;
+    } *w;
     float *c32, *cn;
-    unsigned *cmax_bits;
-    GK_TRY(scr.alloc(&c32, (size_t)k * d));
-    GK_TRY(scr.alloc(&cn, k));
-    GK_TRY(scr.alloc(&cmax_bits, 1));
-    GK_CUDA(ctx, cudaMemsetAsync(cmax_bits, 0, sizeof(unsigned), st));
-    // one-instance tables for the instance-driven kernels
-    CInst *ci;
-    RInst *ri;
-    int64_t *koff, *roff;
-    GK_TRY(scr.alloc(&ci, 1));
-    GK_TRY(scr.alloc(&ri, 1));
-    GK_TRY(scr.alloc(&koff, 2));
-    GK_TRY(scr.alloc(&roff, 2));
+    GK_TRY(scr.alloc(&w, 1));
+    GK_TRY(scr.alloc(&c32, (size_t)k * (d + 1)));
+    cn = c32 + (size_t)k * d;
+    GK_CUDA(ctx, cudaMemsetAsync(w, 0, sizeof(Words), st));
+    unsigned long long *n_flag = &w->n_flag;
+    const RInst *ri = &w->one.r;
+    const int64_t *roff = w->one.row_off;
     {
-        const CInst hc{centres, c32, cn, cmax_bits, d, 0};
-        const RInst hr{x, ldx, d, c32, cn, centres, k, cmax_bits, labels, 0};
-        const int64_t hk[2] = {0, k}, hn[2] = {0, n};
-        GK_CUDA(ctx, cudaMemcpyAsync(ci, &hc, sizeof hc, cudaMemcpyHostToDevice, st));
-        GK_CUDA(ctx, cudaMemcpyAsync(ri, &hr, sizeof hr, cudaMemcpyHostToDevice, st));
-        GK_CUDA(ctx, cudaMemcpyAsync(koff, hk, sizeof hk, cudaMemcpyHostToDevice, st));
-        GK_CUDA(ctx, cudaMemcpyAsync(roff, hn, sizeof hn, cudaMemcpyHostToDevice, st));
+        const CInst hc{centres, c32, cn, &w->cmax_bits, d, 0};
+        const OneTables one{RInst{x, ldx, d, c32, cn, centres, k, &w->cmax_bits, labels, 0}, {0, n}};
+        GK_COUNT();
+        k_centre_prep_one<<<grid_for(k * 32, 128, ctx->num_sms), 128, 0, st>>>(hc, k, one, &w->one);
+        GK_LAUNCH(ctx);
     }
-    GK_COUNT();
-    k_centre_prep<<<grid_for(k, 128, ctx->num_sms), 128, 0, st>>>(ci, koff, 1, k);
-    GK_LAUNCH(ctx);
-    unsigned h_bits = 0;
-    GK_CUDA(ctx, cudaMemcpyAsync(&h_bits, cmax_bits, sizeof h_bits, cudaMemcpyDeviceToHost, st));
-    GK_CUDA(ctx, cudaStreamSynchronize(st));
-    float cmax;
-    memcpy(&cmax, &h_bits, sizeof cmax);
     int32_t *flag_rows;
     float *flag_m;  // the fast pass's smallest value per flagged row
-    unsigned long long *n_flag;
     GK_TRY(scr.alloc(&flag_rows, n));
     GK_TRY(scr.alloc(&flag_m, n));
-    GK_TRY(scr.alloc(&n_flag, 1));
-    GK_CUDA(ctx, cudaMemsetAsync(n_flag, 0, sizeof(unsigned long long), st));
     TcPlan plan;
     struct Free {
         TcPlan *p;
@@ -1713,38 +1738,38 @@ geek_status assign_dense_centres(geek_ctx *ctx, Scratch &scr, const float *x, in
                                           (int)fp32_smem(AS_MAXD)));
         EvTimer tk(ctx, "kernel.assign_fp32", st);
         tk.work = 2.0 * (double)n * (double)k * (double)d;
-        FArgs A{x, ldx, n, d, c32, cn, k, cmax, labels, flag_rows, flag_m, n_flag, ceil_div(n, AS_TR)};
+        FArgs A{x, ldx, n, d, c32, cn, k, &w->cmax_bits, labels, flag_rows, flag_m, n_flag, ceil_div(n, AS_TR)};
         GK_COUNT();
         k_assign_fp32<false><<<(unsigned)A.ntiles, 256, smem, st>>>(A, GatherUnits{});
         GK_LAUNCH(ctx);
     }
     unsigned long long h_flag = 0, h_fp64 = 0;
-    GK_CUDA(ctx, cudaMemcpyAsync(&h_flag, n_flag, sizeof h_flag, cudaMemcpyDeviceToHost, st));
-    GK_CUDA(ctx, cudaStreamSynchronize(st));
     DecideBufs db;
-    if (h_flag) {
-        GK_TRY(decide_bufs_alloc(ctx, &scr, 1, n, db));
-        if (precision == GEEK_PREC_FP32) {
-            // the FP32 pass already applied the FP32 window: straight to FP64
-            const int blocks = (int)std::min<unsigned long long>(ceil_div((int64_t)h_flag, 8), (unsigned long long)ctx->num_sms * 8);
-            EvTimer tk(ctx, "kernel.assign_recheck", st);
-            GK_COUNT();
-            k_assign_recheck<<<blocks, 256, 0, st>>>(ri, roff, 1, flag_rows, flag_m, n_flag);
-            GK_LAUNCH(ctx);
-            h_fp64 = h_flag;
-        } else {
+    if (precision == GEEK_PREC_FP32) {
+        // the FP32 pass already applied the FP32 window: straight to FP64.  The
+        // kernel reads the row count itself, so that the host need not wait
+        // for it (with none it ends at once)
+        EvTimer tk(ctx, "kernel.assign_recheck", st);
+        GK_COUNT();
+        k_assign_recheck<<<(unsigned)std::min<int64_t>(ceil_div(n, 8), (int64_t)ctx->num_sms * 8), 256, 0, st>>>(
+            ri, roff, 1, flag_rows, flag_m, n_flag);
+        GK_LAUNCH(ctx);
+    } else {
+        GK_CUDA(ctx, cudaMemcpyAsync(&h_flag, n_flag, sizeof h_flag, cudaMemcpyDeviceToHost, st));
+        GK_TRY(tc_plan_check(ctx, plan, st));  // synchronises
+        if (h_flag) {
+            GK_TRY(decide_bufs_alloc(ctx, &scr, 1, n, db));
             GK_TRY(tc_emit_alloc(ctx, &scr, &plan, (int64_t)h_flag, st));
             GK_TRY(decide_flags(ctx, plan, ri, roff, 1, d, flag_rows, flag_m, n_flag, (int64_t)h_flag, db, st));
-            GK_TRY(tc_plan_check(ctx, plan, st));  // the candidates' pass, too, ran to its end
+            if (!stats) GK_TRY(tc_plan_check(ctx, plan, st));  // the candidates' pass, too, ran to its end
         }
     }
     if (stats) {
         const int nb = grid_for(n, 256, ctx->num_sms);
-        double *ps, *out;
+        double *ps;
         float *pm;
         GK_TRY(scr.alloc(&ps, nb));
         GK_TRY(scr.alloc(&pm, nb));
-        GK_TRY(scr.alloc(&out, 2));
         float *chi, *clo;
         GK_TRY(scr.alloc(&chi, (size_t)k * d));
         GK_TRY(scr.alloc(&clo, (size_t)k * d));
@@ -1753,15 +1778,19 @@ geek_status assign_dense_centres(geek_ctx *ctx, Scratch &scr, const float *x, in
         GK_COUNT();
         k_assign_stats<<<nb, 256, 0, st>>>(x, ldx, n, d, chi, clo, k, labels, ps, pm);
         GK_COUNT();
-        k_stats_final<<<1, 32, 0, st>>>(ps, pm, nb, out);
+        k_stats_final<<<1, 256, 0, st>>>(ps, pm, nb, w->stats);
         GK_LAUNCH(ctx);
-        double h[2];
-        GK_CUDA(ctx, cudaMemcpyAsync(h, out, sizeof h, cudaMemcpyDeviceToHost, st));
-        if (h_flag && precision != GEEK_PREC_FP32)
+        Words h;
+        GK_CUDA(ctx, cudaMemcpyAsync(&h, w, offsetof(Words, cmax_bits), cudaMemcpyDeviceToHost, st));
+        if (h_flag) {
             GK_CUDA(ctx, cudaMemcpyAsync(&h_fp64, db.n_flag2, sizeof h_fp64, cudaMemcpyDeviceToHost, st));
-        GK_CUDA(ctx, cudaStreamSynchronize(st));
-        stats->sse = h[0];
-        stats->radius_max = h[1];
+            GK_TRY(tc_plan_check(ctx, plan, st));  // synchronises; the candidates' pass, too, ran to its end
+        } else {
+            GK_CUDA(ctx, cudaStreamSynchronize(st));
+        }
+        if (precision == GEEK_PREC_FP32) h_flag = h_fp64 = h.n_flag;
+        stats->sse = h.stats[0];
+        stats->radius_max = h.stats[1];
         stats->k = k;
         stats->n_recheck_rows = (int64_t)h_flag;
         stats->n_fp64_rows = (int64_t)h_fp64;
@@ -1783,7 +1812,7 @@ geek_status centre_prep_batch(geek_ctx *ctx, const CInst *C, const int64_t *k_of
                               cudaStream_t st) {
     if (ktot == 0) return GEEK_OK;
     GK_COUNT();
-    k_centre_prep<<<grid_for(ktot, 128, ctx->num_sms), 128, 0, st>>>(C, k_off, count, ktot);
+    k_centre_prep<<<grid_for(ktot * 32, 128, ctx->num_sms), 128, 0, st>>>(C, k_off, count, ktot);
     GK_LAUNCH(ctx);
     return GEEK_OK;
 }

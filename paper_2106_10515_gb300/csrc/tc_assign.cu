@@ -577,45 +577,57 @@ __global__ void k_x_to_bf16(const TcXPrep *__restrict__ X, const int64_t *__rest
 }
 
 // centres -> BF16 [kpad][Kp], |c|^2 (+inf for padding) and the max of |c|^2
-// over real centres; thread per global padded centre e of instance
-// find_inst(kpad_off, e)
+// over real centres; a warp per global padded centre e of instance
+// find_inst(kpad_off, e), lanes over column pairs (a thread per centre, each
+// store two bytes of another row, took 66 us for 2,048 split centres)
 __global__ void k_c_to_bf16(const TcCPrep *__restrict__ C, const int64_t *__restrict__ kpad_off, int count,
                             int64_t total) {
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-         e += (int64_t)gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < total; e += nw) {
         const int ii = find_inst(kpad_off, count, e);
         const TcCPrep &P = C[ii];
         const int64_t j = e - kpad_off[ii];
         const int W = P.split ? 2 * P.Kp : P.Kp;
         double s = 0.0;
-        for (int t = 0; t < P.Kp; t++) {
+        for (int t = 2 * lane; t < P.Kp; t += 64) {
             // -2 c: scaling by a power of two is exact in BF16
-            const double v = (j < P.k && t < P.d) ? P.c[j * P.d + t] : 0.0;
-            const __nv_bfloat16 h = __double2bfloat16(-2.0 * v);
-            P.cb[j * W + t] = h;
-            if (P.split) P.cb[j * W + P.Kp + t] = __double2bfloat16(-2.0 * v - (double)__bfloat162float(h));  // exact
-            s += v * v;
+            __nv_bfloat162 h2, l2;
+#pragma unroll
+            for (int q = 0; q < 2; q++) {
+                const double v = (j < P.k && t + q < P.d) ? P.c[j * P.d + t + q] : 0.0;
+                const __nv_bfloat16 h = __double2bfloat16(-2.0 * v);
+                const __nv_bfloat16 l = __double2bfloat16(-2.0 * v - (double)__bfloat162float(h));  // exact
+                if (q) h2.y = h, l2.y = l;
+                else h2.x = h, l2.x = l;
+                s += v * v;
+            }
+            *reinterpret_cast<__nv_bfloat162 *>(P.cb + j * W + t) = h2;
+            if (P.split) *reinterpret_cast<__nv_bfloat162 *>(P.cb + j * W + P.Kp + t) = l2;
         }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         // |c|^2 = hi + mid + lo in BF16 (within 2^-24 |c|^2); padding: +inf,
         // which never wins
-        __nv_bfloat16 *xr = P.cbx + j * 16;
-        if (j < P.k) {
-            const __nv_bfloat16 h = __double2bfloat16(s);
-            const double r1 = s - (double)__bfloat162float(h);
-            const __nv_bfloat16 m = __double2bfloat16(r1);
-            const double r2 = r1 - (double)__bfloat162float(m);
-            xr[0] = h;
-            xr[1] = m;
-            xr[2] = __double2bfloat16(r2);
-        } else {
-            xr[0] = __ushort_as_bfloat16((unsigned short)0x7F80);
-            xr[1] = __ushort_as_bfloat16((unsigned short)0);
-            xr[2] = __ushort_as_bfloat16((unsigned short)0);
+        if (lane < 16) {
+            __nv_bfloat16 v = __ushort_as_bfloat16((unsigned short)0);
+            if (j < P.k) {
+                const __nv_bfloat16 h = __double2bfloat16(s);
+                const double r1 = s - (double)__bfloat162float(h);
+                const __nv_bfloat16 m = __double2bfloat16(r1);
+                if (lane == 0) v = h;
+                else if (lane == 1) v = m;
+                else if (lane == 2) v = __double2bfloat16(r1 - (double)__bfloat162float(m));
+            } else if (lane == 0) {
+                v = __ushort_as_bfloat16((unsigned short)0x7F80);
+            }
+            P.cbx[j * 16 + lane] = v;
         }
-        for (int t = 3; t < 16; t++) xr[t] = __ushort_as_bfloat16((unsigned short)0);
-        const float f = (float)s;
-        P.cn[j] = j < P.k ? f : __int_as_float(0x7f800000);
-        if (j < P.k) atomicMax(P.cmax_bits, __float_as_uint(f));  // non-negative floats order as uints
+        if (lane == 0) {
+            const float f = (float)s;
+            P.cn[j] = j < P.k ? f : __int_as_float(0x7f800000);
+            if (j < P.k) atomicMax(P.cmax_bits, __float_as_uint(f));  // non-negative floats order as uints
+        }
     }
 }
 
@@ -819,7 +831,7 @@ geek_status tc_plan_convert(geek_ctx *ctx, const TcPlan &P, cudaStream_t st) {
     }
     if (P.kpad_total > 0) {
         GK_COUNT();
-        k_c_to_bf16<<<grid_for(P.kpad_total, 128, ctx->num_sms), 128, 0, st>>>(P.cprep, P.kpad_off_dev, count,
+        k_c_to_bf16<<<grid_for(P.kpad_total * 32, 128, ctx->num_sms), 128, 0, st>>>(P.cprep, P.kpad_off_dev, count,
                                                                                P.kpad_total);
     }
     GK_LAUNCH(ctx);
@@ -965,7 +977,8 @@ void tc_plan_free(TcPlan *P) {
 
 // BF16 (split = 0) or split-BF16 (split = 1) tcgen05 pass of one data set:
 // labels for every object, flagged rows appended to flag_rows / flag_m / n_flag
-// for the exact decision, which may use the plan P (buffers in scr).  d <= 128.
+// for the exact decision, which may use the plan P (buffers in scr); the caller
+// ends it with tc_plan_check.  d <= 128.
 geek_status assign_tc_bf16(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx, int64_t n, int d,
                            const double *centres, int64_t k, int split, int32_t *labels, int32_t *flag_rows,
                            float *flag_m, unsigned long long *n_flag, TcPlan *P, cudaStream_t st) {
@@ -977,8 +990,7 @@ geek_status assign_tc_bf16(geek_ctx *ctx, Scratch &scr, const float *x, int64_t 
     const int N = split ? (d <= 64 ? 128 : 64) : TC_N;
     one[0] = TcPlanInst{x, ldx, n, d, centres, k, labels, 0, N, split};
     GK_TRY(tc_plan_build(ctx, &scr, one, P, st));
-    GK_TRY(tc_plan_enqueue(ctx, *P, flag_rows, flag_m, n_flag, st));
-    return tc_plan_check(ctx, *P, st);
+    return tc_plan_enqueue(ctx, *P, flag_rows, flag_m, n_flag, st);
 }
 
 // ---- candidates of the flagged rows ------------------------------------------
