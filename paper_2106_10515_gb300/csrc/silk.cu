@@ -43,6 +43,8 @@ __device__ __forceinline__ uint64_t seen_pos(uint64_t hf, int t, uint64_t seen_m
 // [row_off[i], row_off[i + 1]); a set lies inside one instance, whose
 // coefficients (A/B + i * coef_stride) hash its local ids, and tag[g] = i.
 // (set_inst, when given, holds every set's instance: no search per set)
+// (sets of more than SIG_BIG members are left to k_set_sig_big)
+constexpr int64_t SIG_BIG = 32;
 __global__ void k_set_sig(int64_t nsets, const int64_t *__restrict__ soff,
                           const uint32_t *__restrict__ sids, int Ks, const uint64_t *__restrict__ A,
                           const uint64_t *__restrict__ B, const int64_t *__restrict__ row_off, int count,
@@ -60,6 +62,7 @@ __global__ void k_set_sig(int64_t nsets, const int64_t *__restrict__ soff,
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < nsets;
          g += (int64_t)gridDim.x * blockDim.x) {
         const int64_t s0 = soff[g], s1 = soff[g + 1];
+        if (s1 - s0 > SIG_BIG) continue;
         int inst = 0;
         uint32_t base = 0;
         if (count > 1 && s1 > s0) {
@@ -154,7 +157,7 @@ __global__ void __launch_bounds__(256, 3)
             wpos[u] = 0;
             bit[u] = 0;
             cand[u] = -1;
-            if (g >= nsets) continue;
+            if (g >= nsets || s1[u] - s0[u] > SIG_BIG) continue;
             uint32_t base = 0;
             if (count > 1 && s1[u] > s0[u]) {
                 if ((int)inst[u] != have) {
@@ -216,78 +219,129 @@ __global__ void __launch_bounds__(256, 3)
         for (int u = 0; u < SM_U; u++) {
             const int64_t g = gb + u * blockDim.x + threadIdx.x;
             if ((old[u] & bit[u]) || gi[u] >= 0) atomicOr(&seen2[wpos[u]], bit[u]);
-            if (ms && g < nsets) ms[t * nm + (g - g0)] = gi[u];
+            if (ms && g < nsets && s1[u] - s0[u] <= SIG_BIG) ms[t * nm + (g - g0)] = gi[u];
         }
     }
 }
 
-// The same signatures for sets of many members: a thread takes one set for
-// all S tables (its first SS_REG member ids stay in registers, the per-set
-// lookups are paid once), where k_set_sig spends a thread per (set, table).
-// With a few members per set the thread per (set, table) keeps more loads in
-// flight and is the faster form; with hundreds this one is.
-constexpr int SS_REG = 8;
-constexpr int64_t SS_WIDE = 32;  // members per set (mean) from which k_set_sig_sets is used
-__global__ void k_set_sig_sets(int64_t nsets, int S, const int64_t *__restrict__ soff,
-                          const uint32_t *__restrict__ sids, int Ks, const uint64_t *__restrict__ A,
-                          const uint64_t *__restrict__ B, const int64_t *__restrict__ row_off, int count,
-                          const uint32_t *__restrict__ set_inst, int64_t coef_stride, uint64_t *__restrict__ klo,
-                          uint64_t *__restrict__ khi, uint32_t *__restrict__ vals, uint32_t *__restrict__ tag,
-                          uint32_t *__restrict__ seen1 = nullptr, uint32_t *__restrict__ seen2 = nullptr,
-                          uint64_t seen_mask = 0, int64_t g0 = 0) {
+// sets g0 .. nsets-1 of more than SIG_BIG members, in any order
+__global__ void k_big_sets(int64_t nsets, int64_t g0, const int64_t *__restrict__ soff, uint32_t *__restrict__ list,
+                           unsigned *__restrict__ n_list) {
     for (int64_t g = g0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < nsets;
-         g += (int64_t)gridDim.x * blockDim.x) {
+         g += (int64_t)gridDim.x * blockDim.x)
+        if (soff[g + 1] - soff[g] > SIG_BIG) list[atomicAdd(n_list, 1u)] = (uint32_t)g;
+}
+
+// The same signatures, marks and claims for the listed sets, all S tables.  A
+// warp takes a set and SB_F consecutive functions (8, or 12 for KS = 3: SB_F /
+// KS tables), its lanes the members: the loads of the member list are
+// coalesced, a member read once serves SB_F hashes (three integer operations
+// each, what bounds the kernel), and one reduction per function ends it.  A
+// thread per set walked such a list alone, each lane in another 128-byte line:
+// Alg. 1's 200,000 buckets of 2,000 objects under 40 functions took 18.5 ms,
+// now 5.0 ms.
+template <int KS>
+__global__ void __launch_bounds__(256)
+    k_set_sig_big(const uint32_t *__restrict__ list, const unsigned *__restrict__ n_list, int64_t nsets, int S,
+                  const int64_t *__restrict__ soff, const uint32_t *__restrict__ sids, const uint64_t *__restrict__ A,
+                  const uint64_t *__restrict__ B, const int64_t *__restrict__ row_off, int count,
+                  const uint32_t *__restrict__ set_inst, int64_t coef_stride, uint64_t *__restrict__ klo,
+                  uint64_t *__restrict__ khi, uint32_t *__restrict__ vals, uint32_t *__restrict__ tag,
+                  uint32_t *__restrict__ seen1, uint32_t *__restrict__ seen2, uint64_t seen_mask, int64_t g0,
+                  const uint8_t *__restrict__ kst, int kst_stride, const int32_t *__restrict__ single_of,
+                  int32_t *__restrict__ ms) {
+    constexpr int SB_F = KS == 3 ? 12 : 8, TG = SB_F / KS;  // functions, tables per item
+    const int lane = threadIdx.x & 31;
+    const int groups = (S + TG - 1) / TG, nf = S * KS;
+    const int64_t items = (int64_t)*n_list * groups, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t it = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < items; it += nw) {
+        const int64_t g = list[it / groups];
+        const int f0 = (int)(it % groups) * SB_F;
         const int64_t s0 = soff[g], s1 = soff[g + 1];
         int inst = 0;
         uint32_t base = 0;
-        if (count > 1 && s1 > s0) {
+        const uint64_t *Ai = A, *Bi = B;
+        if (count > 1) {
             inst = set_inst ? (int)set_inst[g] : find_inst(row_off, count, (int64_t)sids[s0]);
             base = (uint32_t)row_off[inst];
+            Ai += (int64_t)inst * coef_stride;
+            Bi += (int64_t)inst * coef_stride;
         }
-        const uint64_t *Ai = A + (count > 1 ? (int64_t)inst * coef_stride : 0);
-        const uint64_t *Bi = B + (count > 1 ? (int64_t)inst * coef_stride : 0);
-        const int64_t len = s1 - s0;
-        uint32_t mc[SS_REG];
+        uint64_t a[SB_F], b[SB_F];
+        uint32_t m[SB_F];
 #pragma unroll
-        for (int i = 0; i < SS_REG; i++) mc[i] = i < len ? sids[s0 + i] - base : 0u;
-        for (int t = 0; t < S; t++) {
-            uint64_t a[4], b[4];
-            uint32_t m[4] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu};
+        for (int f = 0; f < SB_F; f++) {
+            a[f] = f0 + f < nf ? Ai[f0 + f] : 0;
+            b[f] = f0 + f < nf ? Bi[f0 + f] : 0;
+            m[f] = 0xFFFFFFFFu;
+        }
+        int64_t p = s0 + lane;
+        for (; p + 96 < s1; p += 128) {  // four members in flight
+            uint32_t id[4];
 #pragma unroll
-            for (int k = 0; k < 4; k++)
-                if (k < Ks) {
-                    a[k] = __ldg(Ai + t * Ks + k);
-                    b[k] = __ldg(Bi + t * Ks + k);
-                }
+            for (int q = 0; q < 4; q++) id[q] = sids[p + 32 * q] - base;
 #pragma unroll
-            for (int i = 0; i < SS_REG; i++)
-                if (i < len) {
+            for (int f = 0; f < SB_F; f++)
 #pragma unroll
-                    for (int k = 0; k < 4; k++)
-                        if (k < Ks) m[k] = min(m[k], mh_hash32(a[k], b[k], mc[i]));
-                }
-            for (int64_t p = s0 + SS_REG; p < s1; p++) {
-                const uint32_t id = sids[p] - base;
+                for (int q = 0; q < 4; q++) m[f] = min(m[f], mh_hash32(a[f], b[f], id[q]));
+        }
+        for (; p < s1; p += 32) {
+            const uint32_t id = sids[p] - base;
 #pragma unroll
-                for (int k = 0; k < 4; k++)
-                    if (k < Ks) m[k] = min(m[k], mh_hash32(a[k], b[k], id));
-            }
+            for (int f = 0; f < SB_F; f++) m[f] = min(m[f], mh_hash32(a[f], b[f], id));
+        }
+#pragma unroll
+        for (int f = 0; f < SB_F; f++) m[f] = __reduce_min_sync(0xffffffffu, m[f]);
+#pragma unroll
+        for (int q = 0; q < TG; q++) {
+            const int t = f0 / KS + q;
+            if (t >= S) break;
             uint64_t hi = 0, lo = 0;
 #pragma unroll
-            for (int k = 0; k < 4; k++)
-                if (k < Ks) {
-                    hi = (hi << 32) | (lo >> 32);
-                    lo = (lo << 32) | m[k];
-                }
+            for (int k = 0; k < KS; k++) {
+                hi = (hi << 32) | (lo >> 32);
+                lo = (lo << 32) | m[q * KS + k];
+            }
             const int64_t so = (int64_t)t * nsets;
-            klo[so + g] = lo;
-            if (khi) khi[so + g] = hi;
-            if (vals) vals[so + g] = (uint32_t)g;
-            if (tag) tag[so + g] = (uint32_t)inst;
-            if (seen1) {
-                const uint64_t pos = seen_pos(sig_hash(lo, hi, (uint32_t)inst), t, seen_mask);
-                const uint32_t bit = 1u << (pos & 31);
-                if (atomicOr(&seen1[pos >> 5], bit) & bit) atomicOr(&seen2[pos >> 5], bit);
+            // the one-object bucket with this signature (see k_set_sig_marks)
+            int32_t gi = -1;
+            if (ms) {
+                const int ks = (int)kst[(int64_t)inst * kst_stride + t];
+                uint32_t arg = 0, mk = 0;
+                uint64_t ak = 0, bk = 0;
+#pragma unroll
+                for (int k = 0; k < KS; k++)
+                    if (k == ks) {
+                        ak = a[q * KS + k];
+                        bk = b[q * KS + k];
+                        mk = m[q * KS + k];
+                    }
+                bool found = false;
+                if (ks < KS)
+                    for (int64_t p0 = s0; p0 < s1 && !found; p0 += 32) {
+                        const uint32_t id = p0 + lane < s1 ? sids[p0 + lane] - base : 0u;
+                        const uint32_t hit = __ballot_sync(0xffffffffu, p0 + lane < s1 && mh_hash32(ak, bk, id) == mk);
+                        if (hit) {
+                            arg = __shfl_sync(0xffffffffu, id, __ffs((int)hit) - 1);
+                            found = true;
+                        }
+                    }
+                bool all = found;
+#pragma unroll
+                for (int k = 0; k < KS; k++) all = all && mh_hash32(a[q * KS + k], b[q * KS + k], arg) == m[q * KS + k];
+                if (all) gi = single_of[(int64_t)arg + base];
+            }
+            if (lane == 0) {
+                klo[so + g] = lo;
+                if (khi) khi[so + g] = hi;
+                if (vals) vals[so + g] = (uint32_t)g;
+                if (tag) tag[so + g] = (uint32_t)inst;
+                if (seen1) {
+                    const uint64_t pos = seen_pos(sig_hash(lo, hi, (uint32_t)inst), t, seen_mask);
+                    const uint32_t bit = 1u << (pos & 31);
+                    if ((atomicOr(&seen1[pos >> 5], bit) & bit) || gi >= 0) atomicOr(&seen2[pos >> 5], bit);
+                }
+                if (ms) ms[t * (nsets - g0) + (g - g0)] = gi;
             }
         }
     }
@@ -1003,6 +1057,38 @@ geek_status d2h_i64(geek_ctx *ctx, const int64_t *dev, int64_t *host, cudaStream
     return GEEK_OK;
 }
 
+// k_set_sig_big over the sets g0 .. nsets-1 of more than SIG_BIG of nids members
+geek_status sign_big_sets(geek_ctx *ctx, Scratch &scr, int S, int64_t nsets, int64_t g0, const int64_t *soff,
+                          const uint32_t *sids, int64_t nids, int Ks, const uint64_t *A, const uint64_t *B,
+                          const SilkBatch *bt, const uint32_t *set_inst, int64_t coef_stride, uint64_t *klo,
+                          uint64_t *khi, uint32_t *vals, uint32_t *tag, uint32_t *seen1, uint32_t *seen2,
+                          uint64_t seen_mask, const uint8_t *kst, int kst_stride, const int32_t *single_of, int32_t *ms,
+                          cudaStream_t st) {
+    if (nids <= SIG_BIG || nsets <= g0) return GEEK_OK;
+    const bool tagged = bt && bt->count > 1;
+    uint32_t *list;
+    unsigned *n_list;
+    GK_TRY(scr.alloc(&list, nids / (SIG_BIG + 1) + 1));
+    GK_TRY(scr.alloc(&n_list, 1));
+    GK_CUDA(ctx, cudaMemsetAsync(n_list, 0, sizeof(unsigned), st));
+    GK_COUNT();
+    k_big_sets<<<G(ctx, nsets - g0), 256, 0, st>>>(nsets, g0, soff, list, n_list);
+    GK_COUNT();
+    const int64_t *row_off = tagged ? bt->row_off : nullptr;
+    const int count = tagged ? bt->count : 1;
+    auto run = [&](auto *k) {
+        k<<<ctx->num_sms * 8, 256, 0, st>>>(list, n_list, nsets, S, soff, sids, A, B, row_off, count, set_inst, coef_stride,
+                                            klo, khi, vals, tag, seen1, seen2, seen_mask, g0, kst, kst_stride, single_of,
+                                            ms);
+    };
+    if (Ks == 1) run(k_set_sig_big<1>);
+    else if (Ks == 2) run(k_set_sig_big<2>);
+    else if (Ks == 3) run(k_set_sig_big<3>);
+    else run(k_set_sig_big<4>);
+    GK_LAUNCH(ctx);
+    return GEEK_OK;
+}
+
 // Group nsets sets into bins by their Ks-function MinHash signature.
 // Returns perm (set index per sorted position), rank (bin per position),
 // rs (bin starts, nbins + 1) and nbins.
@@ -1030,12 +1116,10 @@ geek_status make_bins(geek_ctx *ctx, Scratch &scr, int S, int64_t nsets, const i
     GK_TRY(scr.alloc(perm, tot));
     const int gx = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(nsets, 256), (int64_t)ctx->num_sms * 8));
     GK_COUNT();
-    if (nids >= SS_WIDE * nsets)
-        k_set_sig_sets<<<gx, 256, 0, st>>>(nsets, S, soff, sids, Ks, A, B, tagged ? bt->row_off : nullptr,
+    k_set_sig<<<dim3(gx, S), 256, 0, st>>>(nsets, soff, sids, Ks, A, B, tagged ? bt->row_off : nullptr,
                                            tagged ? bt->count : 1, nullptr, coef_stride, klo, khi, *perm, tag);
-    else
-        k_set_sig<<<dim3(gx, S), 256, 0, st>>>(nsets, soff, sids, Ks, A, B, tagged ? bt->row_off : nullptr,
-                                               tagged ? bt->count : 1, nullptr, coef_stride, klo, khi, *perm, tag);
+    GK_TRY(sign_big_sets(ctx, scr, S, nsets, 0, soff, sids, nids, Ks, A, B, bt, nullptr, coef_stride, klo, khi, *perm, tag,
+                         nullptr, nullptr, 0, nullptr, 0, nullptr, nullptr, st));
     GK_COUNT();
     k_first_component<<<G(ctx, tot), 256, 0, st>>>(tot, klo, khi, tag, Ks, k0);
     GK_LAUNCH(ctx);
@@ -1106,10 +1190,8 @@ geek_status group_bins(geek_ctx *ctx, Scratch &scr, int S, int64_t nsets, const 
     const bool tagged = bt && bt->count > 1;
     // sets g0 .. nsets-1 go through the seen maps and the grouping tables;
     // one-object sets 0 .. ns1-1, on the claim path, are claimed by the sets
-    // that share their signature (sets of many members take k_set_sig_sets
-    // and no claims)
-    const bool wide = nids >= SS_WIDE * nsets;
-    const bool claims = ns1 > 0 && !wide && kst && single_of;
+    // that share their signature
+    const bool claims = ns1 > 0 && kst && single_of;
     const int64_t g0 = claims ? ns1 : 0, nm = nsets - g0;
     int64_t C = 64;
     while (C < 2 * nm) C <<= 1;
@@ -1147,7 +1229,6 @@ geek_status group_bins(geek_ctx *ctx, Scratch &scr, int S, int64_t nsets, const 
     GK_TRY(scr.alloc(&seen, (size_t)(M / 32) * 2));
     GK_CUDA(ctx, cudaMemsetAsync(seen, 0, sizeof(uint32_t) * (size_t)(M / 32) * 2, st));
     uint32_t *seen1 = seen, *seen2 = seen + M / 32;
-    const int gm = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(nm, 256), (int64_t)ctx->num_sms * 8));
     const int gi = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(nm, 256 * 4), (int64_t)ctx->num_sms * 8));
     static_assert(SM_U == 4 && GI_U == 4, "grid of the four-sets-per-thread kernels");
     int32_t *ms = nullptr;
@@ -1160,15 +1241,13 @@ geek_status group_bins(geek_ctx *ctx, Scratch &scr, int S, int64_t nsets, const 
     }
     if (nm > 0) {
         GK_COUNT();
-        if (wide)
-            k_set_sig_sets<<<gm, 256, 0, st>>>(nsets, S, soff, sids, Ks, A, B, tagged ? bt->row_off : nullptr,
-                                               tagged ? bt->count : 1, tagged ? bt->set_inst : nullptr, coef_stride,
-                                               klo, khi, nullptr, tag, seen1, seen2, (uint64_t)(Mt - 1), g0);
-        else
-            k_set_sig_marks<<<dim3(gi, S), 256, 0, st>>>(
-                nsets, soff, sids, Ks, A, B, tagged ? bt->row_off : nullptr, tagged ? bt->count : 1,
-                tagged ? bt->set_inst : nullptr, coef_stride, klo, khi, tag, seen1, seen2, (uint64_t)(Mt - 1), g0,
-                kst, kst_stride, single_of, ms);
+        k_set_sig_marks<<<dim3(gi, S), 256, 0, st>>>(
+            nsets, soff, sids, Ks, A, B, tagged ? bt->row_off : nullptr, tagged ? bt->count : 1,
+            tagged ? bt->set_inst : nullptr, coef_stride, klo, khi, tag, seen1, seen2, (uint64_t)(Mt - 1), g0, kst,
+            kst_stride, single_of, ms);
+        GK_TRY(sign_big_sets(ctx, scr, S, nsets, g0, soff, sids, nids, Ks, A, B, bt, tagged ? bt->set_inst : nullptr,
+                             coef_stride, klo, khi, nullptr, tag, seen1, seen2, (uint64_t)(Mt - 1), kst, kst_stride,
+                             single_of, ms, st));
         GK_COUNT();
         k_group_insert<<<dim3(gi, S), 256, 0, st>>>(nsets, C, klo, khi, tag, roff, rcap, slot, mkey, mval, counts,
                                                     seen2, (uint64_t)(Mt - 1), vw, soff, delta, *singles, counts + 1,
