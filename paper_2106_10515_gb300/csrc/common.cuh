@@ -227,11 +227,13 @@ geek_status sort_err_eval(geek_ctx *ctx, const int *h, cudaStream_t st);
 // Stable LSD radix sort of S segments of m elements each (m < 2^30).  Keys are up to
 // 128 bits: key_lo holds bits 0..63, key_hi (may be null when nbits <= 64)
 // bits 64..127.  vals (may be null) moves with the keys.  Only bits
-// [0, nbits) are examined.  On return the sorted data is in the buffers
+// [bit0, nbits) are examined (bit0 a multiple of 8): a 32-bit key above a
+// 32-bit value in one word moves 8 bytes per element and pass where a key and
+// vals move 12.  On return the sorted data is in the buffers
 // pointed to by *key_lo / *key_hi / *vals (which may have been swapped with
 // internal buffers allocated from `scr`).
 geek_status radix_sort_segments(geek_ctx *ctx, Scratch &scr, int S, int64_t m, uint64_t **key_lo,
-                                uint64_t **key_hi, uint32_t **vals, int nbits, cudaStream_t st);
+                                uint64_t **key_hi, uint32_t **vals, int nbits, cudaStream_t st, int bit0 = 0);
 
 // Buckets of S key-sorted segments of m elements (ids: object id at each
 // sorted position): obj_bucket[seg][id] = rank of the id's key among the

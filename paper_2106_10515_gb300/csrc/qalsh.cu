@@ -3,16 +3,22 @@
 // sizes floor((j + 1) n / t) - floor(j n / t).
 //
 // The projections are computed with compensated FP32 arithmetic (Dot2, see
-// k_qalsh_dot2) and each table is sorted by the double hi + lo.  With E a
-// bound on |(hi + lo) - s| that holds for every object (s the pinned FP64
-// dot product), the exact value tau at cut position p lies within E of the
-// sorted value there (order statistics move by at most the largest
-// perturbation).  So every object whose value is more than 2E below (above)
-// the value at p is exactly before (after) the cut, and only the objects in
-// the window [v_(p) - 2E, v_(p) + 2E] of the sorted order can change sides:
-// their FP64 values are computed and each window (windows that overlap are
-// merged) is re-sorted by (s, id).  Outside the windows the sorted position
-// already gives the exact part.
+// k_qalsh_dot2): w = hi + lo lies within E of s, the pinned FP64 dot product,
+// for every object.  Only the cuts have to be exact, not the order between
+// them, so each table is sorted by r = w rounded to FP32, as one 64-bit word
+// (order-preserving bits of r, object id): four 8-byte passes, where sorting
+// the doubles with their ids took eight 12-byte ones.  Rounding is monotone,
+// so the sorted r are the rounded sorted w, and the w at cut position p is
+// within half an ulp of r_(p); the exact value at p is within E of that (order
+// statistics move by at most the largest perturbation).  So every object whose
+// r is more than 2E and an ulp below (above) r_(p) is exactly before (after) the
+// cut, and only the objects in that window of the sorted order can change
+// sides: their FP64 values are computed and each window (windows that overlap
+// are merged) is re-sorted by (s, id).  Outside the windows the sorted position
+// already gives the exact part.  The members of a part in id order are a second
+// sort of (part, id) words by the part's bits alone.
+// 10M x 128, m = 40, t = 5,000: the sorts take 15 ms, before 28 ms (and 3.7 ms that
+// built the double keys).
 #include <algorithm>
 
 #include "internal.cuh"
@@ -25,12 +31,22 @@ __device__ __forceinline__ uint64_t f64_key(double v) {
     return (u >> 63) ? ~u : (u | (1ull << 63));
 }
 
-// first index in the ascending keys k[0..n) with k >= v (upper: k > v)
-__device__ __forceinline__ int64_t lower_key(const uint64_t *k, int64_t n, uint64_t v, bool upper) {
+__device__ __forceinline__ uint32_t f32_key(float v) {
+    const uint32_t u = __float_as_uint(v);
+    return (u >> 31) ? ~u : (u | (1u << 31));
+}
+__device__ __forceinline__ float key_f32(uint32_t k) {
+    return __uint_as_float((k >> 31) ? (k & ~(1u << 31)) : ~k);
+}
+
+// first index in the words k[0..n), ascending by their upper halves, with an
+// upper half >= v (upper: > v)
+__device__ __forceinline__ int64_t lower_key(const uint64_t *k, int64_t n, uint32_t v, bool upper) {
     int64_t lo = 0, hi = n;
     while (lo < hi) {
         const int64_t mid = (lo + hi) >> 1;
-        if (upper ? k[mid] <= v : k[mid] < v) lo = mid + 1;
+        const uint32_t q = (uint32_t)(k[mid] >> 32);
+        if (upper ? q <= v : q < v) lo = mid + 1;
         else hi = mid;
     }
     return lo;
@@ -62,7 +78,8 @@ struct QDArgs {
     int64_t ldx, n;
     int d, F, FPAD, FG, RG;
     const float *a;
-    float *hi, *lo;      // n x F
+    float *hi;           // n x F
+    uint64_t *words;     // F x n: (key of the rounded value, object id)
     unsigned *xmax_bits; // max row-norm bound (float bits)
 };
 
@@ -172,7 +189,9 @@ __global__ void __launch_bounds__(QD_T, 2) k_qalsh_dot2(QDArgs A) {
                 const int f = fg * QD_FPT + c;
                 if (f < A.F) {
                     A.hi[row * A.F + f] = sh[r][c];
-                    A.lo[row * A.F + f] = sc[r][c];
+                    // + 0: -0 and 0 are equal values, tied by id
+                    const float w = __fadd_rn(__double2float_rn((double)sh[r][c] + (double)sc[r][c]), 0.f);
+                    A.words[(int64_t)f * A.n + row] = ((uint64_t)f32_key(w) << 32) | (uint64_t)row;
                 }
             }
         }
@@ -182,40 +201,26 @@ __global__ void __launch_bounds__(QD_T, 2) k_qalsh_dot2(QDArgs A) {
     if ((t & 31) == 0 && xm > 0.f) atomicMax(A.xmax_bits, __float_as_uint(xm));
 }
 
-// keys[f][i] = key of the double hi + lo of (i, f); ids[f][i] = i
-__global__ void k_qalsh_keys2(int64_t n, int m, const float *__restrict__ hi, const float *__restrict__ lo,
-                              uint64_t *__restrict__ keys, uint32_t *__restrict__ ids) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        for (int f = 0; f < m; f++) {
-            const double v = __dadd_rn((double)hi[i * m + f], (double)lo[i * m + f]);
-            keys[(int64_t)f * n + i] = f64_key(__dadd_rn(v, 0.0));
-            ids[(int64_t)f * n + i] = (uint32_t)i;
-        }
-    }
-}
-
-__device__ __forceinline__ double key_f64(uint64_t k) {
-    return __longlong_as_double((long long)((k >> 63) ? (k & ~(1ull << 63)) : ~k));
-}
-
-// window of cut j (1 .. t-1) of table f in the compensated order: positions
-// whose value is within 2.01 E of the value at floor(j n / t)
-__global__ void k_qalsh_windows2(int64_t n, int m, int t, const uint64_t *__restrict__ keys,
-                                 const float *__restrict__ anorm, const unsigned *__restrict__ xmax_bits, double cf,
-                                 int64_t *__restrict__ q0, int64_t *__restrict__ q1) {
+// window of cut j (1 .. t-1) of table f: positions whose value r is within 2E
+// and an ulp of the value at floor(j n / t) (2.01 E and 2^-22 |r| cover the
+// roundings of this test, 1e-44 the subnormal ones)
+__global__ void k_qalsh_windows(int64_t n, int m, int t, const uint64_t *__restrict__ words,
+                                const float *__restrict__ anorm, const unsigned *__restrict__ xmax_bits, double cf,
+                                int64_t *__restrict__ q0, int64_t *__restrict__ q1) {
     const int64_t tot = (int64_t)m * (t - 1);
     const double xm = (double)__uint_as_float(*xmax_bits);
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
         const int f = (int)(e / (t - 1));
         const int64_t j = e % (t - 1) + 1;
-        const uint64_t *kf = keys + (int64_t)f * n;
-        const double v = key_f64(kf[j * n / t]);
-        const double E = cf * (double)anorm[f] * xm;
-        double lo = nextafter(__dsub_rn(v, 2.01 * E), -INFINITY), hi = nextafter(__dadd_rn(v, 2.01 * E), INFINITY);
-        if (lo == 0.0) lo = -0.0;
-        if (hi == 0.0) hi = 0.0;
-        q0[e] = lower_key(kf, n, f64_key(lo), false);
-        q1[e] = lower_key(kf, n, f64_key(hi), true);
+        const uint64_t *wf = words + (int64_t)f * n;
+        const double v = (double)key_f32((uint32_t)(wf[j * n / t] >> 32));
+        const double dv = 2.01 * (cf * (double)anorm[f] * xm) + fabs(v) * 2.384185791015625e-07 + 4e-45;
+        float lo = __double2float_rd(v - dv), hi = __double2float_ru(v + dv);
+        if (fabs(v) == INFINITY) lo = hi = (float)v;  // values beyond FP32: every one of them
+        if (lo == 0.f) lo = -0.f;
+        if (hi == 0.f) hi = 0.f;
+        q0[e] = lower_key(wf, n, f32_key(lo), false);
+        q1[e] = lower_key(wf, n, f32_key(hi), true);
     }
 }
 
@@ -224,7 +229,7 @@ __global__ void k_qalsh_windows2(int64_t n, int m, int t, const uint64_t *__rest
 // of the object there, keyed (window, FP64 value, id) for one sort of all
 // windows.  Per entry, not per window: merged windows can span whole tables.
 __global__ void k_qalsh_gather(int64_t W, int64_t nwin, const int *__restrict__ wf, const int64_t *__restrict__ wq0,
-                               const int64_t *__restrict__ woff, const uint32_t *__restrict__ ids, int64_t n,
+                               const int64_t *__restrict__ woff, const uint64_t *__restrict__ words, int64_t n,
                                const float *__restrict__ x, int64_t ldx, int d, const float *__restrict__ a,
                                uint64_t *__restrict__ klo, uint64_t *__restrict__ khi) {
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < W; e += (int64_t)gridDim.x * blockDim.x) {
@@ -236,7 +241,7 @@ __global__ void k_qalsh_gather(int64_t W, int64_t nwin, const int *__restrict__ 
         }
         const int64_t w = lo;
         const int f = wf[w];
-        const uint32_t id = ids[(int64_t)f * n + wq0[w] + (e - woff[w])];
+        const uint32_t id = (uint32_t)words[(int64_t)f * n + wq0[w] + (e - woff[w])];
         const float *xr = x + (int64_t)id * ldx;
         const float *af = a + (int64_t)f * d;
         double s = 0.0;
@@ -250,30 +255,32 @@ __global__ void k_qalsh_gather(int64_t W, int64_t nwin, const int *__restrict__ 
 // sorted list entry e back into its window: position wq0 + (e - woff)
 __global__ void k_qalsh_put(int64_t W, const uint64_t *__restrict__ klo, const uint64_t *__restrict__ khi,
                             const int *__restrict__ wf, const int64_t *__restrict__ wq0,
-                            const int64_t *__restrict__ woff, uint32_t *__restrict__ ids, int64_t n) {
+                            const int64_t *__restrict__ woff, uint64_t *__restrict__ words, int64_t n) {
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < W; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t w = (int64_t)(khi[e] >> 32);
-        ids[(int64_t)wf[w] * n + wq0[w] + (e - woff[w])] = (uint32_t)klo[e];
+        words[(int64_t)wf[w] * n + wq0[w] + (e - woff[w])] = (uint32_t)klo[e];  // only the id is read from here on
     }
 }
 
 // part of sorted position p: the largest j with floor(j n / t) <= p
-__global__ void k_qalsh_parts(int64_t n, int m, int t, const uint32_t *__restrict__ ids,
+__global__ void k_qalsh_parts(int64_t n, int m, int t, const uint64_t *__restrict__ words,
                               int32_t *__restrict__ obj_bucket) {
     const int f = blockIdx.y;
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
         const int64_t j = ((p + 1) * t + n - 1) / n - 1;
-        obj_bucket[(int64_t)f * n + ids[(int64_t)f * n + p]] = (int32_t)j;
+        obj_bucket[(int64_t)f * n + (uint32_t)words[(int64_t)f * n + p]] = (int32_t)j;
     }
 }
 
-// members: objects in id order keyed by their part, stably sorted
-__global__ void k_qalsh_member_keys(int64_t tot, int64_t n, const int32_t *__restrict__ obj_bucket,
-                                    uint64_t *__restrict__ key, uint32_t *__restrict__ ids) {
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
-        key[e] = (uint64_t)(uint32_t)obj_bucket[e];
-        ids[e] = (uint32_t)(e % n);
-    }
+// members: (part, id) words in id order, stably sorted by the part
+__global__ void k_qalsh_member_words(int64_t tot, int64_t n, const int32_t *__restrict__ obj_bucket,
+                                     uint64_t *__restrict__ words) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x)
+        words[e] = ((uint64_t)(uint32_t)obj_bucket[e] << 32) | (uint64_t)(e % n);
+}
+__global__ void k_qalsh_members(int64_t tot, const uint64_t *__restrict__ words, uint32_t *__restrict__ members) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x)
+        members[e] = (uint32_t)words[e];
 }
 
 __global__ void k_qalsh_boff(int64_t n, int m, int t, int64_t *__restrict__ boff) {
@@ -289,7 +296,7 @@ geek_status hash_qalsh(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx,
     if (m < 1 || m > 512) return set_error(ctx, GEEK_ERR_UNSUPPORTED, "QALSH: 1 <= m <= 512 tables");
     if (n > 0 && (t < 1 || t > n)) return set_error(ctx, GEEK_ERR_INVALID, "QALSH: need 1 <= t <= n");
     if (n > 0x7FFFFFFFLL) return set_error(ctx, GEEK_ERR_UNSUPPORTED, "QALSH: more than 2^31 objects");
-    float *anorm, *lo;
+    float *anorm;
     unsigned *xmax;
     GK_TRY(scr.alloc(&anorm, m));
     GK_TRY(scr.alloc(&xmax, 1));
@@ -306,7 +313,8 @@ geek_status hash_qalsh(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx,
         return GEEK_OK;
     }
     const int64_t tot = n * m;
-    GK_TRY(scr.alloc(&lo, tot));
+    uint64_t *words;
+    GK_TRY(scr.alloc(&words, tot));
     {
         QDArgs Q{};
         Q.x = x; Q.ldx = ldx; Q.n = n; Q.d = d; Q.F = m; Q.a = a;
@@ -314,7 +322,7 @@ geek_status hash_qalsh(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx,
         Q.FPAD = Q.FG * QD_FPT;
         Q.RG = std::max(1, std::min(64, QD_T / Q.FG));
         Q.hi = (float *)b->codes;  // the handle's codes: FP32 bit patterns of hi
-        Q.lo = lo;
+        Q.words = words;
         Q.xmax_bits = xmax;
         const int TR = Q.RG * QD_RPT;
         const int threads = (int)ceil_div(Q.FG * Q.RG, 32) * 32;
@@ -327,15 +335,9 @@ geek_status hash_qalsh(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx,
         k_qalsh_dot2<<<(unsigned)ceil_div(n, TR), threads, smem, st>>>(Q);
         GK_LAUNCH(ctx);
     }
-    uint64_t *keys;
-    GK_TRY(scr.alloc(&keys, tot));
-    uint32_t *ids = b->members;  // the sorted order first, the members at the end
-    GK_COUNT();
-    k_qalsh_keys2<<<grid_for(n, 256, ctx->num_sms), 256, 0, st>>>(n, m, (const float *)b->codes, lo, keys, ids);
-    GK_LAUNCH(ctx);
     {
         EvTimer tk(ctx, "hash.sort", st);
-        GK_TRY(radix_sort_segments(ctx, scr, m, n, &keys, nullptr, &ids, 64, st));
+        GK_TRY(radix_sort_segments(ctx, scr, m, n, &words, nullptr, nullptr, 64, st, 32));
     }
     if (t > 1) {
         const int64_t nc = (int64_t)m * (t - 1);
@@ -346,7 +348,7 @@ geek_status hash_qalsh(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx,
         // double sum hi + lo and the FP64 reference: (d + 2) 2^-52
         const double cf = 2.2 * (2.0 * d) * (d + 1.0) * 3.552713678800501e-15 + (d + 2.0) * 2.220446049250313e-16;
         GK_COUNT();
-        k_qalsh_windows2<<<grid_for(nc, 256, ctx->num_sms), 256, 0, st>>>(n, m, t, keys, anorm, xmax, cf, q0, q1);
+        k_qalsh_windows<<<grid_for(nc, 256, ctx->num_sms), 256, 0, st>>>(n, m, t, words, anorm, xmax, cf, q0, q1);
         GK_LAUNCH(ctx);
         std::vector<int64_t> h0(nc), h1(nc);
         GK_CUDA(ctx, cudaMemcpyAsync(h0.data(), q0, sizeof(int64_t) * nc, cudaMemcpyDeviceToHost, st));
@@ -398,13 +400,13 @@ geek_status hash_qalsh(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx,
             GK_TRY(scr.alloc(&klo, W));
             GK_TRY(scr.alloc(&khi, W));
             GK_COUNT();
-            k_qalsh_gather<<<grid_for(W, 256, ctx->num_sms), 256, 0, st>>>(W, nwin, d_wf, d_w0, d_wo, ids, n, x,
+            k_qalsh_gather<<<grid_for(W, 256, ctx->num_sms), 256, 0, st>>>(W, nwin, d_wf, d_w0, d_wo, words, n, x,
                                                                             ldx, d, a, klo, khi);
             GK_LAUNCH(ctx);
             GK_TRY(radix_sort_segments(ctx, scr, 1, W, &klo, &khi, nullptr, 96 + bit_length_u64((uint64_t)nwin),
                                        st));
             GK_COUNT();
-            k_qalsh_put<<<grid_for(W, 256, ctx->num_sms), 256, 0, st>>>(W, klo, khi, d_wf, d_w0, d_wo, ids, n);
+            k_qalsh_put<<<grid_for(W, 256, ctx->num_sms), 256, 0, st>>>(W, klo, khi, d_wf, d_w0, d_wo, words, n);
             GK_LAUNCH(ctx);
             // the pageable window tables above are read by the copies: keep
             // them until the stream got past them
@@ -412,16 +414,17 @@ geek_status hash_qalsh(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx,
         }
     }
     GK_COUNT();
-    k_qalsh_parts<<<dim3((unsigned)std::min<int64_t>(ceil_div(n, 256), 4096), m), 256, 0, st>>>(n, m, t, ids,
+    k_qalsh_parts<<<dim3((unsigned)std::min<int64_t>(ceil_div(n, 256), 4096), m), 256, 0, st>>>(n, m, t, words,
                                                                                               b->obj_bucket);
     GK_LAUNCH(ctx);
-    uint64_t *bkey;
-    GK_TRY(scr.alloc(&bkey, tot));
     GK_COUNT();
-    k_qalsh_member_keys<<<grid_for(tot, 256, ctx->num_sms), 256, 0, st>>>(tot, n, b->obj_bucket, bkey, ids);
+    k_qalsh_member_words<<<grid_for(tot, 256, ctx->num_sms), 256, 0, st>>>(tot, n, b->obj_bucket, words);
     GK_LAUNCH(ctx);
-    GK_TRY(radix_sort_segments(ctx, scr, m, n, &bkey, nullptr, &ids, std::max(1, bit_length_u64((uint64_t)(t - 1))),
-                               st));
+    GK_TRY(radix_sort_segments(ctx, scr, m, n, &words, nullptr, nullptr,
+                               32 + std::max(1, bit_length_u64((uint64_t)(t - 1))), st, 32));
+    GK_COUNT();
+    k_qalsh_members<<<grid_for(tot, 256, ctx->num_sms), 256, 0, st>>>(tot, words, b->members);
+    GK_LAUNCH(ctx);
     GK_COUNT();
     k_qalsh_boff<<<grid_for(b->NB + 1, 256, ctx->num_sms), 256, 0, st>>>(n, m, t, b->boff);
     GK_LAUNCH(ctx);

@@ -91,7 +91,7 @@ __device__ __forceinline__ unsigned long long sort_gtimer() {
 // Shared histograms per warp pair keep same-address atomics rare when a
 // high digit takes few values.
 __global__ void __launch_bounds__(256) k_rs_hist_all(const uint64_t *__restrict__ lo, const uint64_t *__restrict__ hi,
-                                                     int64_t m, int npass, uint32_t *__restrict__ counts) {
+                                                     int64_t m, int bit0, int npass, uint32_t *__restrict__ counts) {
     extern __shared__ uint32_t hs[];  // [4][npass][256]
     const int seg = blockIdx.y, t = threadIdx.x, sub = (t >> 6);
     for (int i = t; i < 4 * npass * 256; i += 256) hs[i] = 0;
@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(256) k_rs_hist_all(const uint64_t *__restrict_
         const uint64_t kl = l[p];
         const uint64_t kh = h ? h[p] : 0;
         for (int q = 0; q < npass; q++) {
-            const int sh = q * 8;
+            const int sh = bit0 + q * 8;
             const uint32_t d = (uint32_t)(((sh >= 64 ? kh : kl) >> (sh & 63)) & 0xFFu);
             atomicAdd(&my[q * 256 + d], 1u);
         }
@@ -533,8 +533,8 @@ void launch_iota_u32(uint32_t *v, int64_t n, int64_t period, cudaStream_t st) {
 }
 
 geek_status radix_sort_segments(geek_ctx *ctx, Scratch &scr, int S, int64_t m, uint64_t **key_lo,
-                                uint64_t **key_hi, uint32_t **vals, int nbits, cudaStream_t st) {
-    if (S <= 0 || m <= 1 || nbits <= 0) return GEEK_OK;
+                                uint64_t **key_hi, uint32_t **vals, int nbits, cudaStream_t st, int bit0) {
+    if (S <= 0 || m <= 1 || nbits <= bit0) return GEEK_OK;
     if (S > 65535) return set_error(ctx, GEEK_ERR_UNSUPPORTED, "radix sort: %d segments", S);
     if (m > (int64_t)LB_MASK) return set_error(ctx, GEEK_ERR_UNSUPPORTED, "radix sort: segment too long");
     if ((int64_t)S * ceil_div(m, RS_TILE) > 0xFFFFFFFFLL)
@@ -563,7 +563,7 @@ geek_status radix_sort_segments(geek_ctx *ctx, Scratch &scr, int S, int64_t m, u
         GK_CUDA(ctx, cudaFuncSetAttribute(k_rs_hist_all, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * 16 * 256 * 4));
         attr_done = true;
     }
-    const int npass = (nbits + 7) / 8;
+    const int npass = (nbits - bit0 + 7) / 8;
     // all digit offsets from one read of the keys
     uint32_t *dbase_all, *look, *ticket;
     GK_TRY(scr.alloc(&dbase_all, (size_t)S * npass * 256));
@@ -574,8 +574,8 @@ geek_status radix_sort_segments(geek_ctx *ctx, Scratch &scr, int S, int64_t m, u
     {
         const int hb = (int)std::min<int64_t>(HIST_BLOCKS_PER_SEG, ceil_div(m, 256 * 16));
         GK_COUNT();
-        k_rs_hist_all<<<dim3(std::max(hb, 1), S), 256, (size_t)4 * npass * 256 * 4, st>>>(alo, hi ? ahi : nullptr, m, npass,
-                                                                                        dbase_all);
+        k_rs_hist_all<<<dim3(std::max(hb, 1), S), 256, (size_t)4 * npass * 256 * 4, st>>>(alo, hi ? ahi : nullptr, m, bit0,
+                                                                                        npass, dbase_all);
         GK_LAUNCH(ctx);
         GK_COUNT();
         k_rs_base_all<<<S * npass, 256, 0, st>>>(dbase_all);
@@ -583,7 +583,7 @@ geek_status radix_sort_segments(geek_ctx *ctx, Scratch &scr, int S, int64_t m, u
     }
     const int64_t nblocks = (int64_t)S * tiles;
     for (int q = 0; q < npass; q++, passes++) {
-        const int sh = q * 8, dsel = sh >= 64, sv = sh & 63;
+        const int sh = bit0 + q * 8, dsel = sh >= 64, sv = sh & 63;
         GK_CUDA(ctx, cudaMemsetAsync(look, 0, sizeof(uint32_t) * ((size_t)S * tiles * 256 + 32), st));
         EvTimer tk(ctx, "kernel.rs_scatter", st);
         tk.work = 2.0 * (double)total * ((hi ? 16 : 8) + (hv ? 4 : 0));
