@@ -192,7 +192,7 @@ struct TcPlanInst {
     int32_t *labels;
     int64_t row_base;
     int N;
-    int split;  // 1: split-BF16 (three products, narrow window); needs N * Kp <= 8192
+    int split;  // 1: split-BF16 (three products, narrow window); in a batch N * Kp <= 8192
 };
 struct TcInst;
 struct TcXPrep;

@@ -74,11 +74,16 @@ constexpr int TC_THREADS = 32 * (2 + TC_EPI_WARPS);
 constexpr int TC_KP_MAX = 128;                      // d <= 128
 constexpr int TC_A_STAGE = TC_M * TC_KP_MAX * 2;    // bytes of one X tile stage
 constexpr int TC_B_STAGE = TC_N * TC_KP_MAX * 2;    // bytes of one centre tile stage
-// split-BF16 mode: tiles hold [hi | lo] (2 Kp columns); the same 192 KB is
-// cut into larger X stages and smaller centre stages (N * Kp <= 8192)
-constexpr int TC_A_STAGE_X3 = 2 * TC_A_STAGE;
-constexpr int TC_B_STAGE_X3 = TC_B_STAGE / 2;
-static_assert(TC_A_STAGE_X3 + TC_B_STAGE_X3 == TC_A_STAGE + TC_B_STAGE, "both modes share one layout size");
+// split-BF16 mode: an X stage holds one k-block's [hi | lo] pair.  Two stages are
+// the two k-blocks of a row tile of 128 columns, or two row tiles of 64; the
+// centre ring's stages hold a whole [hi | lo] tile or, where that exceeds half
+// the ring (N = 256, Kp = 128), one 64-column block of it, so that 256-wide
+// tiles fit: 64-wide tiles, the widest whole ones at Kp = 128, read the X block
+// from shared memory once per 64 columns (300,007 x 100, k = 1,999: 646 us,
+// 256-wide 381 us).  Instances of a batch have few centre tiles per row tile, so
+// the next row tile's X must be on its way early: with tiles of N Kp <= 8192
+// the X ring takes four stages and the centre ring what is left, 64 KB (the
+// 256-instance batch: 11.9 ms, with two X stages 16.7 ms).
 constexpr uint32_t TC_TMEM_COLS = 512;
 
 // EMIT: a wave of gathered flagged rows instead of an instance's own.  Slot s of
@@ -102,6 +107,8 @@ struct TcArgs {
     unsigned long long *n_flag;
     int *err;
     int lg_ns;                   // log2 of the centre-tile ring's stages (1..3)
+    int lg_nx;                   // log2 of the |c|^2 ring's stages: lg_ns, or 1 with tiles in parts
+    int lg_na;                   // log2 of the X ring's stages (1 or, split, 2), 32 KB each
     TcEmit e;
 };
 
@@ -252,20 +259,25 @@ __device__ __forceinline__ void epi_resolve(float b1, float b2o, const float (&s
 // instances are left to the launch of that mode).
 template <bool SPLIT, bool EMIT>
 __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc(const __grid_constant__ TcArgs A) {
-    constexpr int A_ST = SPLIT ? TC_A_STAGE_X3 : TC_A_STAGE;
-    constexpr int B_ST = SPLIT ? TC_B_STAGE_X3 : TC_B_STAGE;
+    constexpr int A_ST = TC_A_STAGE;
     constexpr int KW = SPLIT ? 2 : 1;  // stored column blocks per k-block
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t *sA0 = base, *sB0 = base + 2 * A_ST;
+    const int NA = 1 << A.lg_na;
+    uint8_t *sA0 = base, *sB0 = base + NA * TC_A_STAGE;
     uint64_t *bars = (uint64_t *)(base + 2 * TC_A_STAGE + 2 * TC_B_STAGE);
-    uint64_t *full_a = bars, *empty_a = bars + 2, *full_acc = bars + 4, *empty_acc = bars + 6;
-    uint64_t *done_bar = bars + 8, *full_b = bars + 9, *empty_b = bars + 17;  // B ring: up to 8 stages
-    uint32_t *tmem_slot = (uint32_t *)(bars + 25);
+    uint64_t *full_a = bars, *empty_a = bars + 4, *full_acc = bars + 8, *empty_acc = bars + 10;  // X ring: up to 4
+    uint64_t *done_bar = bars + 12, *full_b = bars + 13, *empty_b = bars + 21;  // centre ring: up to 8
+    uint32_t *tmem_slot = (uint32_t *)(bars + 29);
     // the centre-tile ring: the same bytes cut into NS stages (narrower tiles,
     // more stages in flight)
     const int NS = 1 << A.lg_ns;
-    const int BSTR = 2 * B_ST / NS, XSTR = 2 * TC_N * 32 / NS;
+    const int BSTR = (2 * TC_B_STAGE - (NA - 2) * TC_A_STAGE) / NS, XSTR = (2 * TC_N * 32) >> A.lg_nx;
+    // stored 64-column blocks per stage: the whole tile, or one (a part)
+    auto blocks_of = [&](const TcInst &I) {
+        const int all = KW * I.Kp / TC_KB;
+        return SPLIT && all * I.N * 128 > BSTR ? 1 : all;
+    };
     float *mrg = (float *)(bars + 32);  // [groups-1][128][3] results of column groups 1..
     // |c|^2 columns: an all-ones X block (128 x 16) and per stage the centres'
     // (hi, mid, lo, 0...) rows (N x 16), 32-byte swizzled; one extra K = 16
@@ -275,9 +287,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc(const __grid_consta
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        for (int i = 0; i < 2; i++) {
+        for (int i = 0; i < 4; i++) {
             mbar_init(&full_a[i], 1);
             mbar_init(&empty_a[i], 1);
+        }
+        for (int i = 0; i < 2; i++) {
             mbar_init(&full_acc[i], 1);
             mbar_init(&empty_acc[i], TC_EPI_WARPS);
         }
@@ -314,36 +328,48 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc(const __grid_consta
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
         if (lane == 0) {
-            uint64_t ct = 0;
-            uint32_t issued_b[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+            uint64_t ct = 0, pt = 0, ac = 0;  // centre tiles, ring stages and X stages so far
+            uint32_t issued_b[8] = {0, 0, 0, 0, 0, 0, 0, 0}, issued_a[4] = {0, 0, 0, 0};
             bool ok = true;
-            int64_t it = 0;
             for (int64_t u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
                 const int2 un = unit(u);
                 const TcInst &I = A.inst[un.x];
                 if (EMIT && (I.split != 0) != SPLIT) continue;
-                const int nkb = KW * I.Kp / TC_KB, N = I.N;  // stored k-blocks
-                const uint32_t a_bytes = (uint32_t)TC_M * KW * I.Kp * 2, b_bytes = (uint32_t)N * KW * I.Kp * 2;
-                const int ab = (int)(it & 1);
-                const uint32_t ua = (uint32_t)(it >> 1);
-                if (!(ok = mbar_wait(&empty_a[ab], (ua & 1) ^ 1, A.err))) break;
-                mbar_expect_tx(&full_a[ab], a_bytes);
-                for (int kb = 0; kb < nkb; kb++)
-                    tma_load_2d(su32(sA0 + ab * A_ST + kb * TC_M * 128), EMIT ? A.e.tmG : &I.tmA, kb * TC_KB,
-                                un.y * TC_M, &full_a[ab]);
-                for (int c = 0; c < I.ntiles_c; c++, ct++) {
-                    const int s = (int)(ct & (uint64_t)(NS - 1));
-                    const uint32_t uu = (uint32_t)(ct >> A.lg_ns);
-                    if (!(ok = mbar_wait(&empty_b[s], (uu & 1) ^ 1, A.err))) break;
-                    mbar_expect_tx(&full_b[s], b_bytes + (uint32_t)N * 32);
-                    for (int kb = 0; kb < nkb; kb++)
-                        tma_load_2d(su32(sB0 + s * BSTR + kb * N * 128), &I.tmB, kb * TC_KB, c * N, &full_b[s]);
-                    tma_load_2d(su32(sX0 + s * XSTR), &I.tmX, 0, c * N, &full_b[s]);
-                    issued_b[s] = uu + 1;
+                const int nkb = I.Kp / TC_KB, N = I.N;  // logical k-blocks
+                const int all = KW * nkb, bps = blocks_of(I);
+                // X: one stage with every k-block, or (split) a stage per
+                // k-block with its hi and lo columns
+                for (int c = 0; c < (SPLIT ? nkb : 1); c++, ac++) {
+                    const int ab = (int)(ac & (uint64_t)(NA - 1));
+                    const uint32_t ua = (uint32_t)(ac >> A.lg_na);
+                    if (!(ok = mbar_wait(&empty_a[ab], (ua & 1) ^ 1, A.err))) break;
+                    const int nb = SPLIT ? 2 : nkb;
+                    mbar_expect_tx(&full_a[ab], (uint32_t)(nb * TC_M * 128));
+                    for (int b = 0; b < nb; b++)
+                        tma_load_2d(su32(sA0 + ab * A_ST + b * TC_M * 128), EMIT ? A.e.tmG : &I.tmA,
+                                    SPLIT ? c * TC_KB + b * I.Kp : b * TC_KB, un.y * TC_M, &full_a[ab]);
+                    issued_a[ab] = ua + 1;
                 }
-                it++;
+                for (int c = 0; c < I.ntiles_c && ok; c++, ct++)
+                    for (int b0 = 0; b0 < all; b0 += bps, pt++) {
+                        const int s = (int)(pt & (uint64_t)(NS - 1));
+                        const uint32_t uu = (uint32_t)(pt >> A.lg_ns);
+                        if (!(ok = mbar_wait(&empty_b[s], (uu & 1) ^ 1, A.err))) break;
+                        mbar_expect_tx(&full_b[s], (uint32_t)(bps * N * 128) + (b0 == 0 ? (uint32_t)N * 32 : 0u));
+                        // split: blocks in the order hi 0, lo 0, hi 1, lo 1
+                        for (int b = 0; b < bps; b++) {
+                            const int q = b0 + b;
+                            tma_load_2d(su32(sB0 + s * BSTR + b * N * 128), &I.tmB,
+                                        SPLIT ? (q >> 1) * TC_KB + (q & 1) * I.Kp : q * TC_KB, c * N, &full_b[s]);
+                        }
+                        if (b0 == 0)
+                            tma_load_2d(su32(sX0 + (int)(ct & ((1u << A.lg_nx) - 1)) * XSTR), &I.tmX, 0, c * N, &full_b[s]);
+                        issued_b[s] = uu + 1;
+                    }
             }
-            // drain: every centre-tile copy this thread issued has landed
+            // drain: every copy this thread issued has landed
+            for (int s = 0; s < NA; s++)
+                if (issued_a[s]) mbar_wait(&full_a[s], (issued_a[s] - 1) & 1, A.err, true);
             for (int s = 0; s < NS; s++)
                 if (issued_b[s]) mbar_wait(&full_b[s], (issued_b[s] - 1) & 1, A.err, true);
         }
@@ -351,47 +377,85 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc(const __grid_consta
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
         if (lane == 0) {
-            uint64_t ct = 0;
+            uint64_t ct = 0, pt = 0, ac = 0;
             bool ok = true;
-            int64_t it = 0;
             for (int64_t u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
                 const int2 un = unit(u);
                 const TcInst &I = A.inst[un.x];
                 if (EMIT && (I.split != 0) != SPLIT) continue;
                 const int nkb = I.Kp / TC_KB, N = I.N;  // logical k-blocks
+                const int all = KW * nkb, bps = blocks_of(I);
                 const uint32_t idesc = idesc_bf16(TC_M, N);
-                const int ab = (int)(it & 1);
-                const uint32_t ua = (uint32_t)(it >> 1);
-                if (!(ok = mbar_wait(&full_a[ab], ua & 1, A.err))) break;
-                const uint32_t a_base = su32(sA0 + ab * A_ST);
-                for (int c = 0; c < I.ntiles_c; c++, ct++) {
-                    const int sb = (int)(ct & (uint64_t)(NS - 1));  // centre-tile stage
-                    const uint32_t ub = (uint32_t)(ct >> A.lg_ns);
-                    const int s = (int)(ct & 1);                     // accumulator buffer
+                for (int c = 0; c < I.ntiles_c && ok; c++, ct++) {
+                    const int s = (int)(ct & 1);  // accumulator buffer
                     const uint32_t uu = (uint32_t)(ct >> 1);
-                    if (!(ok = mbar_wait(&full_b[sb], ub & 1, A.err))) break;
-                    if (!(ok = mbar_wait(&empty_acc[s], (uu & 1) ^ 1, A.err))) break;
-                    fence_after();
-                    const uint32_t b_base = su32(sB0 + sb * BSTR);
                     const uint32_t dtm = tmem + (uint32_t)(s * TC_N);
-                    for (int kb = 0; kb < nkb; kb++)
+                    if (bps == all) {
+                        // the whole tile in one stage: few instructions per
+                        // MMA (a 64-wide one takes 32 cycles)
+                        const int sb = (int)(pt & (uint64_t)(NS - 1));
+                        if (!(ok = mbar_wait(&full_b[sb], (uint32_t)(pt >> A.lg_ns) & 1, A.err))) break;
+                        if (!(ok = mbar_wait(&empty_acc[s], (uu & 1) ^ 1, A.err))) break;
+                        if (c == 0)
+                            for (int q = 0; q < (SPLIT ? nkb : 1) && ok; q++)
+                                ok = mbar_wait(&full_a[(ac + q) & (uint64_t)(NA - 1)], (uint32_t)((ac + q) >> A.lg_na) & 1,
+                                               A.err);
+                        if (!ok) break;
+                        fence_after();
+                        uint64_t db = sdesc(su32(sB0 + sb * BSTR));
+                        const uint32_t bl = (uint32_t)(N * 128) >> 4;  // the next block, in descriptor units
+                        for (int kb = 0; kb < nkb; kb++, db += KW * bl) {
+                            const uint64_t at = SPLIT ? ac + kb : ac;
+                            const uint64_t da =
+                                sdesc(su32(sA0 + (int)(at & (uint64_t)(NA - 1)) * A_ST) + (SPLIT ? 0 : kb * TC_M * 128));
 #pragma unroll
-                        for (int ks = 0; ks < TC_KB / 16; ks++) {
-                            const uint32_t ao = kb * TC_M * 128 + ks * 32, bo = kb * N * 128 + ks * 32;
-                            mma_bf16(dtm, sdesc(a_base + ao), sdesc(b_base + bo), idesc, (kb | ks) != 0);
-                            if (SPLIT) {
-                                // x_l . c_h and x_h . c_l: the lo halves sit nkb k-blocks on
-                                mma_bf16(dtm, sdesc(a_base + ao + nkb * TC_M * 128), sdesc(b_base + bo), idesc, 1);
-                                mma_bf16(dtm, sdesc(a_base + ao), sdesc(b_base + bo + nkb * N * 128), idesc, 1);
+                            for (int ks = 0; ks < TC_KB / 16; ks++) {
+                                mma_bf16(dtm, da + 2 * ks, db + 2 * ks, idesc, (kb | ks) != 0);
+                                if (SPLIT) {  // x_l . c_h and x_h . c_l
+                                    mma_bf16(dtm, da + (TC_M * 128 >> 4) + 2 * ks, db + 2 * ks, idesc, 1);
+                                    mma_bf16(dtm, da + 2 * ks, db + bl + 2 * ks, idesc, 1);
+                                }
                             }
                         }
-                    // + |c|^2: ones (128 x 16) times the centres' (hi, mid, lo, 0...)
-                    mma_bf16(dtm, sdesc32(su32(sOnes)), sdesc32(su32(sX0 + sb * XSTR)), idesc, 1);
-                    mma_commit(&empty_b[sb]);
+                        // + |c|^2: ones (128 x 16) times the centres' (hi, mid, lo, 0...)
+                        mma_bf16(dtm, sdesc32(su32(sOnes)),
+                                 sdesc32(su32(sX0 + (int)(ct & ((1u << A.lg_nx) - 1)) * XSTR)), idesc, 1);
+                        mma_commit(&empty_b[sb]);
+                        if (SPLIT && c + 1 == I.ntiles_c)
+                            for (int q = 0; q < nkb; q++) mma_commit(&empty_a[(ac + q) & (uint64_t)(NA - 1)]);
+                        pt++;
+                    } else {
+                        // split, the tile in parts: hi 0, lo 0, hi 1, lo 1
+                        for (int q = 0; q < all; q++, pt++) {
+                            const int sb = (int)(pt & (uint64_t)(NS - 1)), kb = q >> 1;
+                            const int ab = (int)((ac + kb) & (uint64_t)(NA - 1));  // X stage
+                            if (!(ok = mbar_wait(&full_b[sb], (uint32_t)(pt >> A.lg_ns) & 1, A.err))) break;
+                            if (q == 0 && !(ok = mbar_wait(&empty_acc[s], (uu & 1) ^ 1, A.err))) break;
+                            if (c == 0 && (q & 1) == 0 &&
+                                !(ok = mbar_wait(&full_a[ab], (uint32_t)((ac + kb) >> A.lg_na) & 1, A.err)))
+                                break;
+                            fence_after();
+                            const uint64_t da = sdesc(su32(sA0 + ab * A_ST)), db = sdesc(su32(sB0 + sb * BSTR));
+#pragma unroll
+                            for (int ks = 0; ks < TC_KB / 16; ks++) {
+                                mma_bf16(dtm, da + 2 * ks, db + 2 * ks, idesc, (q | ks) != 0);
+                                // a hi block meets x_l too: x_h.c_h + x_l.c_h, then x_h.c_l
+                                if ((q & 1) == 0) mma_bf16(dtm, da + (TC_M * 128 >> 4) + 2 * ks, db + 2 * ks, idesc, 1);
+                            }
+                            if (q == 0)
+                                mma_bf16(dtm, sdesc32(su32(sOnes)),
+                                         sdesc32(su32(sX0 + (int)(ct & ((1u << A.lg_nx) - 1)) * XSTR)), idesc, 1);
+                            // X stage: last read of its k-block in the last centre tile
+                            if ((q & 1) && c + 1 == I.ntiles_c) mma_commit(&empty_a[ab]);
+                            mma_commit(&empty_b[sb]);
+                        }
+                    }
+                    if (!ok) break;
                     mma_commit(&full_acc[s]);
                 }
-                mma_commit(&empty_a[ab]);
-                it++;
+                if (!ok) break;
+                if (!SPLIT) mma_commit(&empty_a[ac & (uint64_t)(NA - 1)]);
+                ac += SPLIT ? nkb : 1;
             }
             // drain: all MMAs this thread issued have completed
             mma_commit(done_bar);
@@ -667,8 +731,8 @@ geek_status make_inst(geek_ctx *ctx, const TcPlan &P, int i, int N, TcInst *out)
     const TcXPrep &xp = P.impl->xp[i];
     const TcCPrep &cp = P.impl->cp[i];
     const int Kst = I.split ? 2 * Kp : Kp;  // stored columns
-    if (I.split && N * Kp > 8192)
-        return set_error(ctx, GEEK_ERR_INVALID, "split-BF16 tiles need N * Kp <= 8192 (N %d, Kp %d)", N, Kp);
+    if (I.split && N * Kp > 8192 && P.count != 1)
+        return set_error(ctx, GEEK_ERR_INVALID, "split-BF16 tiles of a batch need N * Kp <= 8192 (N %d, Kp %d)", N, Kp);
     if (I.n > 0) GK_TRY(encode_bf16_2d(ctx, &T.tmA, xp.xb, Kst, I.n, TC_KB, TC_M));
     if (I.k > 0) GK_TRY(encode_bf16_2d(ctx, &T.tmB, cp.cb, Kst, cp.kpad, TC_KB, N));
     if (I.k > 0) GK_TRY(encode_bf16_2d(ctx, &T.tmX, cp.cbx, 16, cp.kpad, 16, N, CU_TENSOR_MAP_SWIZZLE_32B));
@@ -840,12 +904,17 @@ geek_status tc_plan_convert(geek_ctx *ctx, const TcPlan &P, cudaStream_t st) {
 
 namespace {
 
-// log2 of the centre-tile ring's stages for the instances of one mode in a
-// launch: the widest stage among them fixes the stage size; the ring's bytes
-// are cut into as many stages as fit (2 .. 8). Two regions are cut: the
-// centre tiles (N x Kp BF16, twice that when split) and the |c|^2 rows
-// (N x 32 bytes out of 2 * TC_N * 32), so both bound the stage count.
-int ring_lg(const TcPlan &P, const std::vector<int> *which, int split) {
+// The rings for the instances of one mode in a launch: log2 of the centre
+// ring's stages (2 .. 8) and of the |c|^2 ring's.  The widest tile among them
+// fixes the stage size, and the ring's bytes are cut into as many stages as fit;
+// both regions bound the count (the |c|^2 rows, N x 32 bytes a tile, have 2 TC_N
+// * 32).  A tile wider than half the ring (one split instance, N = 256, Kp =
+// 128) goes through in 64-column parts, four stages, and its |c|^2 rows take
+// turns in two: a part's stage comes free only after every part before it.
+struct Rings {
+    int ns, nx, na;
+};
+Rings ring_lg(const TcPlan &P, const std::vector<int> *which, int split) {
     int64_t mx = 0, nmax = 0;
     auto consider = [&](int i) {
         const TcPlanInst &I = P.desc[i];
@@ -858,16 +927,19 @@ int ring_lg(const TcPlan &P, const std::vector<int> *which, int split) {
         for (int i : *which) consider(i);
     else
         for (int i = 0; i < P.count; i++) consider(i);
-    const int64_t ring = 2 * (int64_t)(split ? TC_B_STAGE_X3 : TC_B_STAGE);
+    // split tiles of N Kp <= 8192: four X stages, the centre ring half as large
+    const int lg_na = split && mx <= TC_B_STAGE / 2 ? 2 : 1;
+    const int64_t ring = 2 * (int64_t)TC_B_STAGE - ((1 << lg_na) - 2) * (int64_t)TC_A_STAGE;
+    if (mx > ring / 2) return Rings{2, 1, lg_na};
     int lg = 1;
     const int64_t xring = 2 * (int64_t)TC_N * 32;
     while (lg < 3 && mx > 0 && (ring >> (lg + 1)) >= mx && (xring >> (lg + 1)) >= nmax * 32) lg++;
-    return lg;
+    return Rings{lg, lg, lg_na};
 }
 
 geek_status launch_units(geek_ctx *ctx, const TcInst *inst, const int2 *units, int64_t n0, int64_t n1,
-                         int32_t *flag_rows, float *flag_m, unsigned long long *n_flag, int *err, double work, int lg0,
-                         int lg1, cudaStream_t st) {
+                         int32_t *flag_rows, float *flag_m, unsigned long long *n_flag, int *err, double work,
+                         Rings r0, Rings r1, cudaStream_t st) {
     TcArgs A{};
     A.inst = inst;
     A.flag_rows = flag_rows;
@@ -879,14 +951,18 @@ geek_status launch_units(geek_ctx *ctx, const TcInst *inst, const int2 *units, i
     if (n0 > 0) {
         A.units = units;
         A.nunits = n0;
-        A.lg_ns = lg0;
+        A.lg_ns = r0.ns;
+        A.lg_nx = r0.nx;
+        A.lg_na = r0.na;
         GK_COUNT();
         k_assign_tc<false, false><<<(int)std::min<int64_t>(n0, ctx->num_sms), TC_THREADS, tc_smem(), st>>>(A);
     }
     if (n1 > 0) {
         A.units = units + n0;
         A.nunits = n1;
-        A.lg_ns = lg1;
+        A.lg_ns = r1.ns;
+        A.lg_nx = r1.nx;
+        A.lg_na = r1.na;
         GK_COUNT();
         k_assign_tc<true, false><<<(int)std::min<int64_t>(n1, ctx->num_sms), TC_THREADS, tc_smem(), st>>>(A);
     }
@@ -984,11 +1060,9 @@ geek_status assign_tc_bf16(geek_ctx *ctx, Scratch &scr, const float *x, int64_t 
                            float *flag_m, unsigned long long *n_flag, TcPlan *P, cudaStream_t st) {
     if (d > 128) return set_error(ctx, GEEK_ERR_UNSUPPORTED, "BF16 tensor-core assignment supports d <= 128");
     std::vector<TcPlanInst> one(1);
-    // BF16: N = 256 (two stages; 128-wide tiles read A from shared memory
-    // twice as often per flop and measured ~60% slower at d = 128).  Split:
-    // the widest tile whose hi|lo stage fits
-    const int N = split ? (d <= 64 ? 128 : 64) : TC_N;
-    one[0] = TcPlanInst{x, ldx, n, d, centres, k, labels, 0, N, split};
+    // the widest tiles: 128-wide ones read the X tile from shared memory twice
+    // as often per flop and measured ~60% slower (BF16, d = 128)
+    one[0] = TcPlanInst{x, ldx, n, d, centres, k, labels, 0, TC_N, split};
     GK_TRY(tc_plan_build(ctx, &scr, one, P, st));
     return tc_plan_enqueue(ctx, *P, flag_rows, flag_m, n_flag, st);
 }
@@ -1180,7 +1254,10 @@ geek_status tc_decide_candidates(geek_ctx *ctx, const TcPlan &P, const RInst *R,
         A.e = TcEmit{P.tmG, P.emit_lim, P.emit_masks, P.kw, F.unit_inst, F.n_units, u0};
         for (int sp = 0; sp < 2; sp++) {
             if (!mode[sp]) continue;
-            A.lg_ns = ring_lg(P, nullptr, sp);
+            const Rings r = ring_lg(P, nullptr, sp);
+            A.lg_ns = r.ns;
+            A.lg_nx = r.nx;
+            A.lg_na = r.na;
             GK_COUNT();
             const int grid = (int)std::min<int64_t>(P.emit_units, ctx->num_sms);
             if (sp) k_assign_tc<true, true><<<grid, TC_THREADS, tc_smem(), st>>>(A);
