@@ -84,10 +84,9 @@ struct GatherUnits {
     FlagUnits f;
 };
 
-__device__ __forceinline__ unsigned long long ffma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-    unsigned long long r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
+// c += a b, two FP32 values each
+__device__ __forceinline__ void ffma2(unsigned long long &c, unsigned long long a, unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
 }
 
 constexpr int AS_ST = 3;                    // stages of the centre ring
@@ -127,12 +126,12 @@ __global__ void __launch_bounds__(256, 2) k_assign_fp32(FArgs A, GatherUnits U) 
         const int d = A.d;
         const int64_t k = A.k;
         const int nch = (d + AS_KC - 1) / AS_KC;   // 32-coordinate chunks
-        const int dp = nch * AS_KC;
+        const int dp = nch * AS_KC, dp16 = 16 * dp;
         float *xs = sm;                            // [AS_TR][dp], pieces swizzled
         float *cs = sm + (size_t)AS_TR * dp;       // [AS_ST][AS_TC][AS_KC], pieces swizzled
         const bool xvec = ((A.ldx & 3) == 0) && ((d & 3) == 0) && (((uintptr_t)A.x & 15) == 0);
         const bool cvec = ((d & 3) == 0) && (((uintptr_t)A.c32 & 15) == 0);
-        const int64_t nst = ((k + AS_TC - 1) / AS_TC) * nch;  // chunks of all centre tiles
+        const int ntile = (int)((k + AS_TC - 1) / AS_TC);
         // 16-byte piece p of row r at position p ^ (r & 7) within each group of
         // eight pieces; zeros outside the data
         auto put = [&](float *dst, const float *src, int nv, bool vec) {
@@ -146,18 +145,22 @@ __global__ void __launch_bounds__(256, 2) k_assign_fp32(FArgs A, GatherUnits U) 
                 for (int q = 0; q < 4; q++) dst[q] = q < nv ? src[q] : 0.f;
             }
         };
-        auto stage = [&](int64_t s) {  // chunk s into its ring slot
-            if (s < nst) {
-                const int64_t j0 = s / nch * AS_TC;
-                const int k0 = (int)(s % nch) * AS_KC;
-                float *buf = cs + (int)(s % AS_ST) * AS_CST;
+        // the next chunk (tile f_t, chunk f_c) into ring slot f_s; counters instead
+        // of divisions of a chunk number, which cost as much as the products
+        int f_t = 0, f_c = 0, f_s = 0;
+        auto stage = [&]() {
+            if (f_t < ntile) {
+                const int k0 = f_c * AS_KC;
+                float *buf = cs + f_s * AS_CST;
 #pragma unroll
                 for (int u = 0; u < AS_CST / 4 / 256; u++) {
                     const int e = t + 256 * u, c = e >> 3, p = e & 7;
-                    const int64_t j = j0 + c;
+                    const int64_t j = (int64_t)f_t * AS_TC + c;
                     put(buf + c * AS_KC + 4 * (p ^ (c & 7)), A.c32 + j * d + k0 + 4 * p,
                         j < k ? min(4, d - k0 - 4 * p) : 0, cvec);
                 }
+                if (++f_c == nch) f_c = 0, f_t++;
+                if (++f_s == AS_ST) f_s = 0;
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
@@ -167,40 +170,39 @@ __global__ void __launch_bounds__(256, 2) k_assign_fp32(FArgs A, GatherUnits U) 
             const int64_t row = r < nrows ? (GATHER ? s_rows[r] : row0 + r) : 0;
             put(xs + r * dp + 4 * (p ^ (r & 7)), A.x + row * A.ldx + 4 * p, r < nrows ? min(4, d - 4 * p) : 0, xvec);
         }
-        stage(0);
-        stage(1);
+        stage();
+        stage();
         Best B[AS_RPT];
 #pragma unroll
         for (int r = 0; r < AS_RPT; r++) B[r] = Best{FLT_MAX, FLT_MAX, 0x7FFFFFFF};
         unsigned long long acc[AS_RPT][AS_CPT];
-        int ch = 0;
-        int64_t j0 = 0;
-        for (int64_t s = 0; s < nst; s++) {
+        int ch = 0, slot = 0;
+        for (int tile = 0; tile < ntile;) {
             asm volatile("cp.async.wait_group 1;" ::: "memory");
-            __syncthreads();  // chunk s has landed; everyone is done with chunk s - 1's slot
-            stage(s + 2);
+            __syncthreads();  // this chunk has landed; everyone is done with the last one's slot
+            stage();
             if (ch == 0) {
 #pragma unroll
                 for (int r = 0; r < AS_RPT; r++)
 #pragma unroll
                     for (int c = 0; c < AS_CPT; c++) acc[r][c] = 0ull;
             }
-            const float *buf = cs + (int)(s % AS_ST) * AS_CST, *xb = xs + ch * AS_KC;
+            const float *buf = cs + slot * AS_CST + cg * AS_KC, *xb = xs + rg * dp + ch * AS_KC;
+            if (++slot == AS_ST) slot = 0;
             const int np = min(AS_KC, d - ch * AS_KC + 3) >> 2;  // pieces holding data
 #pragma unroll 1
             for (int p = 0; p < np; p++) {
                 ulonglong2 cv[AS_CPT];
 #pragma unroll
                 for (int c = 0; c < AS_CPT; c++)  // (cg + 16 c) & 7 == cg & 7
-                    cv[c] = *reinterpret_cast<const ulonglong2 *>(buf + (cg + 16 * c) * AS_KC + 4 * (p ^ (cg & 7)));
+                    cv[c] = *reinterpret_cast<const ulonglong2 *>(buf + 16 * c * AS_KC + 4 * (p ^ (cg & 7)));
 #pragma unroll
                 for (int r = 0; r < AS_RPT; r++) {
-                    const ulonglong2 xv =
-                        *reinterpret_cast<const ulonglong2 *>(xb + (rg + 16 * r) * dp + 4 * (p ^ (rg & 7)));
+                    const ulonglong2 xv = *reinterpret_cast<const ulonglong2 *>(xb + r * dp16 + 4 * (p ^ (rg & 7)));
 #pragma unroll
                     for (int c = 0; c < AS_CPT; c++) {
-                        acc[r][c] = ffma2(xv.x, cv[c].x, acc[r][c]);
-                        acc[r][c] = ffma2(xv.y, cv[c].y, acc[r][c]);
+                        ffma2(acc[r][c], xv.x, cv[c].x);
+                        ffma2(acc[r][c], xv.y, cv[c].y);
                     }
                 }
             }
@@ -208,16 +210,16 @@ __global__ void __launch_bounds__(256, 2) k_assign_fp32(FArgs A, GatherUnits U) 
                 ch = 0;
 #pragma unroll
                 for (int c = 0; c < AS_CPT; c++) {
-                    const int64_t j = j0 + cg + 16 * c;
+                    const int j = tile * AS_TC + cg + 16 * c;
                     if (j >= k) continue;
                     const float cnj = A.cn[j];
 #pragma unroll
                     for (int r = 0; r < AS_RPT; r++) {
                         const float dot = __uint_as_float((uint32_t)acc[r][c]) + __uint_as_float((uint32_t)(acc[r][c] >> 32));
-                        best_push(B[r], fmaf(-2.f, dot, cnj), (int)j);
+                        best_push(B[r], fmaf(-2.f, dot, cnj), j);
                     }
                 }
-                j0 += AS_TC;
+                tile++;
             }
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -1399,10 +1401,24 @@ struct UlArgs {
     const uint64_t *order;         // centres by descending count
     const unsigned long long *n_large;
     double *start;                 // [segment][d]: sums, then s at the start (approximate)
-    int64_t *d0, *d1, *mn, *mx;    // [segment][d]
-    int32_t *ex;                   // [segment][d]: biased exponent assumed, -1: none
+    int64_t *rec;                  // [3][segments][d], see ul_pack
+    int64_t segs;                  // segments the arrays hold
     double *c;                     // k x d
 };
+
+// A segment's three words for one coordinate: (D0, D1 - D0 + 1), (mn, low
+// exponent bits), (mx, high exponent bits; 7: not usable).  D1 - D0 is -1, 0
+// or 1 (rounding is monotone, so neighbours stay ordered, and they merge when
+// both round to the same even value), and the three integers are below 2^54
+// whenever the segment is usable.
+__device__ __forceinline__ void ul_pack(int64_t *w, int64_t stride, int64_t D0, int64_t D1, int64_t mn, int64_t mx, int E,
+                                        bool ok) {
+    constexpr int64_t LIM = 1ll << 54;
+    ok = ok && mn > -LIM && mx < LIM;
+    w[0] = ok ? D0 * 4 + (D1 - D0 + 1) : 0;
+    w[stride] = ok ? mn * 256 + (E & 0xFF) : 0;
+    w[2 * stride] = ok ? mx * 256 + (E >> 8) : 7;
+}
 
 // item (segment, 32-coordinate slice) -> centre, member range, coordinate
 struct UlItem {
@@ -1458,27 +1474,38 @@ __global__ void __launch_bounds__(256) k_ul_sums(UlArgs A) {
     }
 }
 
-// warp per (large centre, slice): sums -> the running sum before each segment
-__global__ void __launch_bounds__(128) k_ul_starts(UlArgs A) {
-    const int nsl = (A.d + 31) >> 5, lane = threadIdx.x & 31;
-    const int64_t items = (int64_t)*A.n_large * nsl, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t it = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < items; it += nw) {
+// block per (large centre, slice): sums -> the running sum before each segment;
+// each of the 8 warps takes an eighth of the segments, after the others' totals
+__global__ void __launch_bounds__(256) k_ul_starts(UlArgs A) {
+    __shared__ double s_tot[8][32];
+    const int nsl = (A.d + 31) >> 5, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t items = (int64_t)*A.n_large * nsl;
+    for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
         const int64_t j = (int64_t)(A.order[it / nsl] & 0xFFFFFFFFull);
         const int t = (int)(it % nsl) * 32 + lane;
-        if (t >= A.d) continue;
         const int64_t ns = ((int64_t)A.cnt[j] + UL_M - 1) / UL_M;
+        const int64_t b0 = ns * w / 8, b1 = t < A.d ? ns * (w + 1) / 8 : b0;
         double *p = A.start + A.seg_off[j] * A.d + t;
         double run = 0.0;
-        for (int64_t s0 = 0; s0 < ns; s0 += 16) {
-            double v[16];
+        for (int pass = 0; pass < 2; pass++) {
+            for (int64_t s0 = b0; s0 < b1; s0 += 16) {
+                double v[16];
 #pragma unroll
-            for (int u = 0; u < 16; u++) v[u] = s0 + u < ns ? p[(s0 + u) * A.d] : 0.0;
+                for (int u = 0; u < 16; u++) v[u] = s0 + u < b1 ? p[(s0 + u) * A.d] : 0.0;
 #pragma unroll
-            for (int u = 0; u < 16; u++) {
-                if (s0 + u < ns) p[(s0 + u) * A.d] = run;
-                run += v[u];
+                for (int u = 0; u < 16; u++) {
+                    if (pass && s0 + u < b1) p[(s0 + u) * A.d] = run;
+                    run += v[u];
+                }
+            }
+            if (pass == 0) {
+                s_tot[w][lane] = run;
+                __syncthreads();
+                run = 0.0;
+                for (int q = 0; q < w; q++) run += s_tot[q][lane];
             }
         }
+        __syncthreads();
     }
 }
 
@@ -1518,13 +1545,7 @@ __global__ void __launch_bounds__(256) k_ul_deltas(UlArgs A) {
             mn = min(mn, min(D0, D1));
             mx = max(mx, max(D0, D1));
         });
-        if (q.act) {
-            A.d0[at] = D0;
-            A.d1[at] = D1;
-            A.mn[at] = mn;
-            A.mx[at] = mx;
-            A.ex[at] = ok ? E : -1;
-        }
+        if (q.act) ul_pack(A.rec + at, A.segs * A.d, D0, D1, mn, mx, E, ok);
     }
 }
 
@@ -1541,45 +1562,61 @@ __global__ void __launch_bounds__(32) k_ul_chain(UlArgs A) {
         const float *xs = A.x + (act ? t : 0);
         const int64_t a0 = A.seg_off[j] * A.d + (act ? t : 0);
         double s = 0.0;
-        for (int64_t g0 = 0; g0 < ns; g0 += 4) {
-            // four segments' integers requested together
-            int64_t D0[4], D1[4], mn[4], mx[4];
-            int ex[4];
+        // UL_U segments' words at a time, the next ones on the way meanwhile
+        constexpr int UL_U = 4;
+        const int64_t stride = A.segs * A.d;
+        int64_t nw[UL_U][3];
+        auto fetch = [&](int64_t g0) {
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
-                const int64_t at = a0 + min(g0 + u, ns - 1) * A.d;
-                D0[u] = A.d0[at];
-                D1[u] = A.d1[at];
-                mn[u] = A.mn[at];
-                mx[u] = A.mx[at];
-                ex[u] = A.ex[at];
+            for (int u = 0; u < UL_U; u++) {
+                const int64_t *w = A.rec + a0 + min(g0 + u, ns - 1) * A.d;
+                nw[u][0] = w[0];
+                nw[u][1] = w[stride];
+                nw[u][2] = w[2 * stride];
             }
+        };
+        fetch(0);
+        for (int64_t g0 = 0; g0 < ns; g0 += UL_U) {
+            int64_t cw[UL_U][3];
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
+            for (int u = 0; u < UL_U; u++)
+#pragma unroll
+                for (int q = 0; q < 3; q++) cw[u][q] = nw[u][q];
+            fetch(g0 + UL_U);
+#pragma unroll
+            for (int u = 0; u < UL_U; u++) {
                 if (g0 + u >= ns) break;
+                const int64_t D0 = cw[u][0] >> 2, D1 = D0 + (cw[u][0] & 3) - 1, mn = cw[u][1] >> 8, mx = cw[u][2] >> 8;
+                const int ex = (int)(cw[u][1] & 0xFF) | (int)(cw[u][2] & 0xFF) << 8;  // 0x700 and more: not usable
                 const uint64_t bits = (uint64_t)__double_as_longlong(s);
                 const int E = (int)((bits >> 52) & 0x7FF);
                 const int64_t a = (int64_t)((bits & ((1ull << 52) - 1)) | (1ull << 52));
                 const bool neg = bits >> 63;
                 const int64_t S = neg ? -a : a;
-                const bool ok = !act || (ex[u] == E && (neg ? S + mx[u] <= -LO && S + mn[u] >= -HI
-                                                            : S + mn[u] >= LO && S + mx[u] <= HI));
-                const int64_t T = S + ((S & 1) ? D1[u] : D0[u]);
+                const bool ok = !act || (ex == E && (neg ? S + mx <= -LO && S + mn >= -HI : S + mn >= LO && S + mx <= HI));
+                const int64_t T = S + ((S & 1) ? D1 : D0);
                 const uint64_t b = (uint64_t)(T < 0 ? -T : T);
                 const double moved = __longlong_as_double(
                     (long long)((bits & (1ull << 63)) | ((uint64_t)E << 52) | (b & ((1ull << 52) - 1))));
                 double walked = s;
                 if (!__all_sync(0xffffffffu, ok)) {
                     const int64_t m0 = (g0 + u) * UL_M;
-                    for (int64_t p = m0; p < min(cj, m0 + UL_M); p += UC_B) {
-                        const int ma = (int)min((int64_t)UC_B, cj - p);
-                        const int32_t id = lane < ma ? mid[p + lane] : 0;
-                        float v[UC_B];
+                    float w[UC_B];  // the next chunk's rows, requested before this one's sums
+                    auto rows = [&](int64_t p) {
+                        const int32_t id = p + lane < cj ? mid[p + lane] : 0;
 #pragma unroll
                         for (int r = 0; r < UC_B; r++) {
                             const int32_t row = __shfl_sync(0xffffffffu, id, r);
-                            v[r] = r < ma ? xs[(int64_t)row * A.ldx] : 0.f;
+                            w[r] = p + r < cj ? xs[(int64_t)row * A.ldx] : 0.f;
                         }
+                    };
+                    rows(m0);
+                    for (int64_t p = m0; p < min(cj, m0 + UL_M); p += UC_B) {
+                        const int ma = (int)min((int64_t)UC_B, cj - p);
+                        float v[UC_B];
+#pragma unroll
+                        for (int r = 0; r < UC_B; r++) v[r] = w[r];
+                        if (p + UC_B < min(cj, m0 + UL_M)) rows(p + UC_B);
                         walked = ma == UC_B ? chain_chunk<true>(walked, v, ma, act && !ok)
                                             : chain_chunk<false>(walked, v, ma, act && !ok);
                     }
@@ -1645,11 +1682,8 @@ geek_status refine_dense(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ld
             const size_t segs = (size_t)(n / UL_M + n / UL_MIN + 1);  // at most
             UlArgs U{x, ldx, d, k, off, cnt, (const int32_t *)ids, seg_off, seg_tot, order, n_large};
             GK_TRY(ps.alloc(&U.start, segs * d));
-            GK_TRY(ps.alloc(&U.d0, segs * d));
-            GK_TRY(ps.alloc(&U.d1, segs * d));
-            GK_TRY(ps.alloc(&U.mn, segs * d));
-            GK_TRY(ps.alloc(&U.mx, segs * d));
-            GK_TRY(ps.alloc(&U.ex, segs * d));
+            GK_TRY(ps.alloc(&U.rec, 3 * segs * d));
+            U.segs = (int64_t)segs;
             U.c = centres;
             const int nsl = (d + 31) / 32;
             const int gs = grid_for((int64_t)segs * nsl * 32, 256, ctx->num_sms);
@@ -1657,7 +1691,7 @@ geek_status refine_dense(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ld
             GK_COUNT();
             k_ul_sums<<<gs, 256, 0, st>>>(U);
             GK_COUNT();
-            k_ul_starts<<<grid_for(most * 32, 128, ctx->num_sms), 128, 0, st>>>(U);
+            k_ul_starts<<<(unsigned)std::min<int64_t>(most, (int64_t)ctx->num_sms * 8), 256, 0, st>>>(U);
             GK_COUNT();
             k_ul_deltas<<<gs, 256, 0, st>>>(U);
             GK_COUNT();
