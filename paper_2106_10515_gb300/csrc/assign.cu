@@ -1794,7 +1794,10 @@ geek_status assign_dense_centres(geek_ctx *ctx, Scratch &scr, const float *x, in
         if (h_flag) {
             GK_TRY(decide_bufs_alloc(ctx, &scr, 1, n, db));
             GK_TRY(tc_emit_alloc(ctx, &scr, &plan, (int64_t)h_flag, st));
-            GK_TRY(decide_flags(ctx, plan, ri, roff, 1, d, flag_rows, flag_m, n_flag, (int64_t)h_flag, db, st));
+            // the order pays for its sort from some 10^5 rows on
+            const FlagOrder order{&scr, k, labels};
+            GK_TRY(decide_flags(ctx, plan, ri, roff, 1, d, flag_rows, flag_m, n_flag, (int64_t)h_flag, db, st,
+                                h_flag >= 100000 ? &order : nullptr));
             if (!stats) GK_TRY(tc_plan_check(ctx, plan, st));  // the candidates' pass, too, ran to its end
         }
     }
@@ -1917,19 +1920,71 @@ void decide_bufs_free(DecideBufs &B) {
     B.owned.clear();
 }
 
-// the listed rows grouped by instance in units of 128 (B.grows, B.unit_*)
+// one instance: the list is the group
+__global__ void k_one_group(const int32_t *__restrict__ flags, const unsigned long long *__restrict__ n_flag,
+                            int64_t *__restrict__ seg_off, int64_t *__restrict__ unit_off, int *__restrict__ n_units,
+                            int32_t *__restrict__ grows) {
+    const int64_t nf = (int64_t)*n_flag;
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nf; q += (int64_t)gridDim.x * blockDim.x)
+        grows[q] = flags[q];
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        const int64_t nu = (nf + AS_TR - 1) / AS_TR;
+        seg_off[0] = unit_off[0] = 0;
+        seg_off[1] = nf;
+        unit_off[1] = nu;
+        *n_units = (int)nu;
+    }
+}
+
+// the listed rows grouped by instance in units of 128 (B.grows, B.unit_*); one
+// instance's rows keep the list's order
 static geek_status group_flags(geek_ctx *ctx, const int64_t *row_off, int count, const int32_t *flags,
                                const unsigned long long *n_flag, const DecideBufs &B, cudaStream_t st) {
     const int g = ctx->num_sms * 4;
-    GK_CUDA(ctx, cudaMemsetAsync(B.cnt, 0, sizeof(int) * count, st));
     GK_COUNT();
-    k_flag_count<<<g, 256, 0, st>>>(flags, n_flag, row_off, count, B.cnt);
-    GK_COUNT();
-    k_flag_units<<<1, 1024, 0, st>>>(B.cnt, count, B.cursor, B.seg_off, B.unit_off, B.n_units);
+    if (count == 1) {
+        k_one_group<<<g, 256, 0, st>>>(flags, n_flag, B.seg_off, B.unit_off, B.n_units, B.grows);
+    } else {
+        GK_CUDA(ctx, cudaMemsetAsync(B.cnt, 0, sizeof(int) * count, st));
+        k_flag_count<<<g, 256, 0, st>>>(flags, n_flag, row_off, count, B.cnt);
+        GK_COUNT();
+        k_flag_units<<<1, 1024, 0, st>>>(B.cnt, count, B.cursor, B.seg_off, B.unit_off, B.n_units);
+        GK_COUNT();
+        k_flag_scatter<<<g, 256, 0, st>>>(flags, n_flag, row_off, count, B.cursor, B.grows);
+    }
     GK_COUNT();
     k_fill_units<<<g, 256, 0, st>>>(count, B.seg_off, B.unit_off, B.unit_inst, B.unit_start, B.unit_cnt);
+    GK_LAUNCH(ctx);
+    return GEEK_OK;
+}
+
+// (label, row) words of the flagged rows, and the rows of the sorted words
+__global__ void k_flag_words(int64_t nf, const int32_t *__restrict__ flags, const int32_t *__restrict__ labels,
+                             uint64_t *__restrict__ words) {
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nf; q += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t r = flags[q];
+        words[q] = ((uint64_t)(uint32_t)max(labels[r], 0) << 32) | (uint32_t)r;
+    }
+}
+__global__ void k_word_rows(int64_t nf, const uint64_t *__restrict__ words, int32_t *__restrict__ rows) {
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nf; q += (int64_t)gridDim.x * blockDim.x)
+        rows[q] = (int32_t)(uint32_t)words[q];
+}
+
+// One data set's nf flagged rows in the order of the label the fast pass gave
+// them: neighbours then have the same candidates, whose centres the decision
+// reads from L1 instead of L2 (Alg. 1 pipeline, 4.7M rows of 35 candidates:
+// the decision takes 11 ms, 18 ms in the order of the flags).
+static geek_status order_flags(geek_ctx *ctx, Scratch &scr, int64_t nf, int64_t k, const int32_t *labels,
+                               int32_t *flags, cudaStream_t st) {
+    uint64_t *words;
+    GK_TRY(scr.alloc(&words, nf));
     GK_COUNT();
-    k_flag_scatter<<<g, 256, 0, st>>>(flags, n_flag, row_off, count, B.cursor, B.grows);
+    k_flag_words<<<grid_for(nf, 256, ctx->num_sms), 256, 0, st>>>(nf, flags, labels, words);
+    GK_LAUNCH(ctx);
+    GK_TRY(radix_sort_segments(ctx, scr, 1, nf, &words, nullptr, nullptr, 32 + bit_length_u64((uint64_t)k), st, 32));
+    GK_COUNT();
+    k_word_rows<<<grid_for(nf, 256, ctx->num_sms), 256, 0, st>>>(nf, words, flags);
     GK_LAUNCH(ctx);
     return GEEK_OK;
 }
@@ -1939,21 +1994,24 @@ static geek_status group_flags(geek_ctx *ctx, const int64_t *row_off, int count,
 // candidates, by direct FP32 distances (tc_decide_candidates); the rest (near
 // duplicates of one centre, values that are not finite) by a tiled FP32 scan of
 // every centre (narrow FP32 window), then the FP64 reference for the rows still
-// uncertain.  max_rows: at most so many flagged rows.  No host synchronisation.
+// uncertain.  max_rows: at most so many flagged rows.  No host synchronisation
+// and no allocation, except with `order` (one data set, exactly max_rows flagged
+// rows): flags is then put into the order of the labels first.
 // Alg. 1 pipeline at 10M x 128, k = 1,751, split-BF16: 4.7M flagged rows of 35
-// candidates each take 26 ms; the two scans over every centre took 162.
+// candidates each take 19 ms; the two scans over every centre took 162.
 geek_status decide_flags(geek_ctx *ctx, const TcPlan &P, const RInst *R, const int64_t *row_off, int count, int dmax,
-                         const int32_t *flags, const float *flag_m, const unsigned long long *n_flag,
-                         int64_t max_rows, const DecideBufs &B, cudaStream_t st) {
+                         int32_t *flags, const float *flag_m, const unsigned long long *n_flag, int64_t max_rows,
+                         const DecideBufs &B, cudaStream_t st, const FlagOrder *order) {
     EvTimer tk(ctx, "kernel.assign_recheck", st);
     const int g = ctx->num_sms * 4;
     const FlagUnits F{B.grows, B.unit_inst, B.unit_start, B.unit_cnt, B.n_units};
     GK_CUDA(ctx, cudaMemsetAsync(B.n_flag2, 0, sizeof(unsigned long long), st));
     GK_CUDA(ctx, cudaMemsetAsync(B.n_left, 0, sizeof(unsigned long long), st));
-    GK_TRY(group_flags(ctx, row_off, count, flags, n_flag, B, st));
     GK_COUNT();
     k_scatter_m<<<g, 256, 0, st>>>(flags, flag_m, n_flag, B.mrow);
-    GK_TRY(tc_decide_candidates(ctx, P, R, F, B.mrow, max_rows, B.left, B.n_left, st));
+    if (order) GK_TRY(order_flags(ctx, *order->scr, max_rows, order->k, order->labels, flags, st));
+    GK_TRY(group_flags(ctx, row_off, count, flags, n_flag, B, st));
+    GK_TRY(tc_decide_candidates(ctx, P, R, F, B.mrow, max_rows, order != nullptr, B.left, B.n_left, st));
     GK_TRY(group_flags(ctx, row_off, count, B.left, B.n_left, B, st));
     const size_t smem = (size_t)dmax * AS_TR * sizeof(float) + (size_t)AS_KC * AS_TC * sizeof(float);
     GK_CUDA(ctx, cudaFuncSetAttribute(k_assign_fp32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -238,7 +238,8 @@ struct FlagUnits {
 struct RInst;
 geek_status tc_emit_alloc(geek_ctx *ctx, Scratch *scr, TcPlan *P, int64_t max_rows, cudaStream_t st);
 geek_status tc_decide_candidates(geek_ctx *ctx, const TcPlan &P, const RInst *R, const FlagUnits &F, const float *mrow,
-                                 int64_t max_rows, int32_t *left, unsigned long long *n_left, cudaStream_t st);
+                                 int64_t max_rows, bool ordered, int32_t *left, unsigned long long *n_left,
+                                 cudaStream_t st);
 // scr == nullptr: buffers are cudaMalloc'd and owned by the plan
 geek_status tc_plan_build(geek_ctx *ctx, Scratch *scr, const std::vector<TcPlanInst> &desc, TcPlan *P,
                           cudaStream_t st);
@@ -329,11 +330,17 @@ struct DecideBufs {
     unsigned long long *n_flag2 = nullptr;
     std::vector<void *> owned;
 };
+// One data set's flagged rows are put into the order of their labels (of k).
+struct FlagOrder {
+    Scratch *scr;
+    int64_t k;
+    const int32_t *labels;
+};
 geek_status decide_bufs_alloc(geek_ctx *ctx, Scratch *scr, int count, int64_t n_total, DecideBufs &B);
 void decide_bufs_free(DecideBufs &B);
 geek_status decide_flags(geek_ctx *ctx, const TcPlan &P, const RInst *R, const int64_t *row_off, int count, int dmax,
-                         const int32_t *flags, const float *flag_m, const unsigned long long *n_flag,
-                         int64_t max_rows, const DecideBufs &B, cudaStream_t st);
+                         int32_t *flags, const float *flag_m, const unsigned long long *n_flag, int64_t max_rows,
+                         const DecideBufs &B, cudaStream_t st, const FlagOrder *order = nullptr);
 geek_status assign_dense_centres(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx,
                                  int64_t n, int d, const double *centres, int64_t k, int precision,
                                  int32_t *labels, geek_assign_stats *stats, cudaStream_t st);

@@ -1104,19 +1104,160 @@ __global__ void __launch_bounds__(256) k_gather_flagged(const TcInst *__restrict
     }
 }
 
-// The exact argmin among a flagged row's candidates, a warp per slot.  The
-// direct distance D = sum (x - c)^2 in FP32 has none of the cancellation of
-// |c|^2 - 2 x.c: with u = 2^-24, C = max |c| and D' its FP32 value (centres
-// rounded to FP32, differences, FMA chain over lanes and a shuffle tree),
+// The exact argmin among a flagged row's candidates.  The direct distance D =
+// sum (x - c)^2 in FP32 has none of the cancellation of |c|^2 - 2 x.c: with u =
+// 2^-24, C = max |c| and D' its FP32 value (centres rounded to FP32,
+// differences, FMA chains over the lanes and a shuffle tree),
 //   |D' - D| <= ((d + 6) u D' + 2.001 u C sqrt(D') + 4.1 u^2 C^2)(1 + 10^-4)
 // (|x - c32| is off by u|x - c32| + u|c| per coordinate, Cauchy-Schwarz over the
 // coordinates, gamma_(d+4) for the sum), and the FP64 reference's own error
-// is below d 2^-52 D; err() rounds all of it up by 5 %.  Where the smallest
+// is below d 2^-52 D; cand_err rounds all of it up by 5 %.  Where the smallest
 // D' is apart from the second by both errors the label is decided; else (and
 // without a candidate) the row goes on to `left`, for the FP32 scan and the
-// FP64 reference.  A warp's eight-lane groups take a candidate each, lane l of a
-// group the coordinates 4 l .. 4 l + 3 of each 32: a group's loads of a centre
-// are whole 128-byte lines.
+// FP64 reference.
+__device__ __forceinline__ float cand_err(float D, float C, int d) {
+    const float u = 5.9604645e-8f;
+    return 1.05f * ((float)(d + 6) * u * D + 2.001f * u * C * sqrtf(D) + 4.1f * u * u * C * C) + 1e-37f;
+}
+
+// coordinates t .. t + 3, zeros past d
+__device__ __forceinline__ float4 cand_load4(const float *__restrict__ p, int t, int d, bool vec) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (vec) {
+        if (t < d) v = *reinterpret_cast<const float4 *>(p + t);
+    } else {
+        if (t < d) v.x = p[t];
+        if (t + 1 < d) v.y = p[t + 1];
+        if (t + 2 < d) v.z = p[t + 2];
+        if (t + 3 < d) v.w = p[t + 3];
+    }
+    return v;
+}
+__device__ __forceinline__ bool cand_vec(const RInst &I) {
+    return ((I.d & 3) == 0) && ((I.ldx & 3) == 0) && ((((uintptr_t)I.x) | ((uintptr_t)I.c32)) & 15) == 0;
+}
+
+// the set bits of the warp's 32 words (a word per lane) as a list; its length
+__device__ __forceinline__ int cand_list(uint32_t m, uint16_t *list) {
+    const int lane = threadIdx.x & 31, mine = __popc(m);
+    int inc = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    __syncwarp();
+    for (int at = inc - mine; m; m &= m - 1, at++) list[at] = (uint16_t)(32 * lane + __ffs((int)m) - 1);
+    __syncwarp();
+    return __shfl_sync(0xffffffffu, inc, 31);
+}
+
+// Rows in the order of their labels (decide_flags with an order): a warp takes 8
+// neighbouring slots, whose candidates are nearly the same, and computes the
+// distances of all 8 to the union (a real distance of a centre that is no
+// candidate changes nothing).  A centre is read once for 8 rows: each eight-lane
+// group holds two rows, lane l the coordinates 4 l .. 4 l + 3 of each 32, and all
+// groups read the same 128-byte line.  Per (row, centre) pair that is about 6
+// instructions with packed FP32 arithmetic; a warp per row, a candidate per
+// group, took 43 and waited for L2.
+__global__ void __launch_bounds__(256) k_decide_ordered(const RInst *__restrict__ R, FlagUnits F, int64_t u0,
+                                                        int64_t umax, const uint32_t *__restrict__ masks, int kw,
+                                                        int32_t *__restrict__ left,
+                                                        unsigned long long *__restrict__ n_left) {
+    __shared__ uint16_t s_list[8][1024];
+    const int lane = threadIdx.x & 31, grp = lane >> 3, sub = lane & 7;
+    uint16_t *list = s_list[threadIdx.x >> 5];
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t nsets = (TC_M / 8) * max((int64_t)0, min(umax, (int64_t)*F.n_units - u0));
+    for (int64_t q8 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; q8 < nsets; q8 += nw) {
+        const int64_t u = u0 + q8 / (TC_M / 8), s = 8 * q8;  // s: slot in the wave
+        const int r0 = (int)(q8 % (TC_M / 8)) * 8, cnt = F.unit_cnt[u];
+        if (r0 >= cnt) continue;
+        const RInst &I = R[F.unit_inst[u]];
+        const int d = I.d;
+        const bool vec = cand_vec(I);
+        int64_t g[2];
+        unsigned long long nx[2][8];  // -x in pairs
+        bool row[2];
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const int r = r0 + grp + 4 * h;
+            row[h] = r < cnt;
+            g[h] = row[h] ? (int64_t)F.grows[F.unit_start[u] + r] : I.row_base;
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                const float4 v = cand_load4(I.x + (g[h] - I.row_base) * I.ldx, 32 * e + 4 * sub, d, vec);
+                asm("mov.b64 %0, {%1, %2};" : "=l"(nx[h][2 * e]) : "f"(-v.x), "f"(-v.y));
+                asm("mov.b64 %0, {%1, %2};" : "=l"(nx[h][2 * e + 1]) : "f"(-v.z), "f"(-v.w));
+            }
+        }
+        const int nwords = (int)((I.k + 31) >> 5);
+        float b1[2] = {FLT_MAX, FLT_MAX}, b2[2] = {FLT_MAX, FLT_MAX};
+        int bj[2] = {0x7FFFFFFF, 0x7FFFFFFF}, total = 0;
+        uint32_t own = 0;  // bit r: slot s + r has a candidate
+        bool bad = false;
+        for (int w0 = 0; w0 < nwords; w0 += 32) {
+            uint32_t m = 0;
+#pragma unroll
+            for (int r = 0; r < 8; r++) {
+                uint32_t w = w0 + lane < nwords && r0 + r < cnt ? masks[(s + r) * kw + w0 + lane] : 0u;
+                // no index past the centres
+                if (w0 + lane == nwords - 1 && (I.k & 31)) w &= (1u << (I.k & 31)) - 1u;
+                if (__any_sync(0xffffffffu, w != 0)) own |= 1u << r;
+                m |= w;
+            }
+            const int nc = cand_list(m, list);
+            total += nc;
+#pragma unroll 2
+            for (int q = 0; q < nc; q++) {
+                const int j = 32 * w0 + (int)list[q];
+                const float *c = I.c32 + (int64_t)j * d;
+                unsigned long long acc[2] = {0ull, 0ull};
+#pragma unroll
+                for (int e = 0; e < 4; e++) {
+                    if (32 * e >= d) break;
+                    const float4 cv = cand_load4(c, 32 * e + 4 * sub, d, vec);
+                    unsigned long long c01, c23;
+                    asm("mov.b64 %0, {%1, %2};" : "=l"(c01) : "f"(cv.x), "f"(cv.y));
+                    asm("mov.b64 %0, {%1, %2};" : "=l"(c23) : "f"(cv.z), "f"(cv.w));
+#pragma unroll
+                    for (int h = 0; h < 2; h++) {
+                        unsigned long long d01, d23;
+                        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d01) : "l"(c01), "l"(nx[h][2 * e]));
+                        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d23) : "l"(c23), "l"(nx[h][2 * e + 1]));
+                        asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(acc[h]) : "l"(d01));
+                        asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(acc[h]) : "l"(d23));
+                    }
+                }
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    float D = __uint_as_float((uint32_t)acc[h]) + __uint_as_float((uint32_t)(acc[h] >> 32));
+#pragma unroll
+                    for (int o = 1; o < 8; o <<= 1) D += __shfl_xor_sync(0xffffffffu, D, o);
+                    bad = bad || !(D < FLT_MAX);
+                    const bool less = D < b1[h];
+                    b2[h] = fminf(b2[h], less ? b1[h] : D);
+                    b1[h] = less ? D : b1[h];
+                    bj[h] = less ? j : bj[h];
+                }
+            }
+        }
+        if (sub == 0) {
+            const float C = __uint_as_float(*I.cmax_bits);
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                if (!row[h]) continue;
+                const bool sure = !bad && ((own >> (grp + 4 * h)) & 1u) &&
+                                  (total == 1 || (b2[h] - b1[h]) * (1.f - 1e-6f) > cand_err(b1[h], C, d) + cand_err(b2[h], C, d));
+                if (sure) I.labels[g[h] - I.row_base] = bj[h];
+                else left[atomicAdd(n_left, 1ull)] = (int32_t)g[h];
+            }
+        }
+    }
+}
+
+// Rows in any order: a warp per slot, its eight-lane groups take a candidate
+// each, two in flight.
 __global__ void __launch_bounds__(256) k_decide_candidates(const RInst *__restrict__ R, FlagUnits F, int64_t u0,
                                                            int64_t umax, const uint32_t *__restrict__ masks, int kw,
                                                            int32_t *__restrict__ left,
@@ -1133,22 +1274,10 @@ __global__ void __launch_bounds__(256) k_decide_candidates(const RInst *__restri
         const RInst &I = R[F.unit_inst[u]];
         const int64_t g = F.grows[F.unit_start[u] + r], row = g - I.row_base;
         const int d = I.d;
-        const bool vec = ((d & 3) == 0) && ((I.ldx & 3) == 0) && ((((uintptr_t)I.x) | ((uintptr_t)I.c32)) & 15) == 0;
-        auto load4 = [&](const float *p, int t) {  // coordinates t .. t + 3, zeros past d
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (vec) {
-                if (t < d) v = *reinterpret_cast<const float4 *>(p + t);
-            } else {
-                if (t < d) v.x = p[t];
-                if (t + 1 < d) v.y = p[t + 1];
-                if (t + 2 < d) v.z = p[t + 2];
-                if (t + 3 < d) v.w = p[t + 3];
-            }
-            return v;
-        };
+        const bool vec = cand_vec(I);
         float4 xv[4];
 #pragma unroll
-        for (int q = 0; q < 4; q++) xv[q] = load4(I.x + row * I.ldx, 32 * q + 4 * sub);
+        for (int q = 0; q < 4; q++) xv[q] = cand_load4(I.x + row * I.ldx, 32 * q + 4 * sub, d, vec);
         const uint32_t *mk = masks + s * kw;
         const int nwords = (int)((I.k + 31) >> 5);
         float b1 = FLT_MAX, b2 = FLT_MAX;  // this group's smallest and second D'
@@ -1157,18 +1286,7 @@ __global__ void __launch_bounds__(256) k_decide_candidates(const RInst *__restri
         for (int w0 = 0; w0 < nwords; w0 += 32) {
             uint32_t m = w0 + lane < nwords ? mk[w0 + lane] : 0u;
             if (w0 + lane == nwords - 1 && (I.k & 31)) m &= (1u << (I.k & 31)) - 1u;  // no index past the centres
-            int inc = __popc(m);
-            const int mine = inc;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, inc, o);
-                if (lane >= o) inc += y;
-            }
-            const int cnt = __shfl_sync(0xffffffffu, inc, 31);
-            if (cnt == 0) continue;
-            __syncwarp();
-            for (int at = inc - mine; m; m &= m - 1, at++) list[at] = (uint16_t)(32 * lane + __ffs((int)m) - 1);
-            __syncwarp();
+            const int cnt = cand_list(m, list);
             total += cnt;
             for (int q0 = 0; q0 < cnt; q0 += 8) {  // two candidates per group in flight
                 float D[2];
@@ -1182,7 +1300,7 @@ __global__ void __launch_bounds__(256) k_decide_candidates(const RInst *__restri
 #pragma unroll
                     for (int e = 0; e < 4; e++) {
                         if (32 * e >= d) break;
-                        const float4 cv = load4(c, 32 * e + 4 * sub);
+                        const float4 cv = cand_load4(c, 32 * e + 4 * sub, d, vec);
                         const float e0 = xv[e].x - cv.x, e1 = xv[e].y - cv.y;
                         const float e2 = xv[e].z - cv.z, e3 = xv[e].w - cv.w;
                         D[h] = fmaf(e3, e3, fmaf(e2, e2, fmaf(e1, e1, fmaf(e0, e0, D[h]))));
@@ -1217,11 +1335,9 @@ __global__ void __launch_bounds__(256) k_decide_candidates(const RInst *__restri
         }
         bad = __any_sync(0xffffffffu, bad);
         if (lane == 0) {
-            const float C = __uint_as_float(*I.cmax_bits), uu = 5.9604645e-8f;
-            auto err = [&](float D) {
-                return 1.05f * ((float)(d + 6) * uu * D + 2.001f * uu * C * sqrtf(D) + 4.1f * uu * uu * C * C) + 1e-37f;
-            };
-            const bool sure = !bad && (total == 1 || (total > 1 && (b2 - b1) * (1.f - 1e-6f) > err(b1) + err(b2)));
+            const float C = __uint_as_float(*I.cmax_bits);
+            const bool sure = !bad && (total == 1 || (total > 1 && (b2 - b1) * (1.f - 1e-6f) >
+                                                                       cand_err(b1, C, d) + cand_err(b2, C, d)));
             if (sure) I.labels[row] = bj;
             else left[atomicAdd(n_left, 1ull)] = (int32_t)g;
         }
@@ -1234,10 +1350,11 @@ __global__ void __launch_bounds__(256) k_decide_candidates(const RInst *__restri
 // decide_flags: F, every row's smallest value in mrow), gather the rows, find
 // their candidates with a second tcgen05 pass over them, and decide among the
 // candidates; what stays undecided is appended to left / n_left.  max_rows
-// bounds the flagged rows; no allocation and no host synchronisation (the
+// bounds the flagged rows, ordered: they are in the order of their labels; no allocation and no host synchronisation (the
 // buffers are the plan's, tc_emit_alloc).
 geek_status tc_decide_candidates(geek_ctx *ctx, const TcPlan &P, const RInst *R, const FlagUnits &F, const float *mrow,
-                                 int64_t max_rows, int32_t *left, unsigned long long *n_left, cudaStream_t st) {
+                                 int64_t max_rows, bool ordered, int32_t *left, unsigned long long *n_left,
+                                 cudaStream_t st) {
     int64_t units = ceil_div(std::min(max_rows, P.N_total), TC_M) + P.count;
     bool mode[2] = {false, false};
     for (const TcPlanInst &I : P.desc)
@@ -1264,7 +1381,8 @@ geek_status tc_decide_candidates(geek_ctx *ctx, const TcPlan &P, const RInst *R,
             else k_assign_tc<false, true><<<grid, TC_THREADS, tc_smem(), st>>>(A);
         }
         GK_COUNT();
-        k_decide_candidates<<<ctx->num_sms * 8, 256, 0, st>>>(R, F, u0, P.emit_units, P.emit_masks, P.kw, left, n_left);
+        (ordered ? k_decide_ordered : k_decide_candidates)<<<ctx->num_sms * 8, 256, 0, st>>>(
+            R, F, u0, P.emit_units, P.emit_masks, P.kw, left, n_left);
         GK_LAUNCH(ctx);
     }
     return GEEK_OK;
