@@ -277,6 +277,97 @@ __global__ void __launch_bounds__(RS_THREADS, 4)
     }
 }
 
+// Segments of at most RB_MAX elements: one block sorts a segment in shared
+// memory, all passes in one launch (each pass of the tiled form is a launch of
+// its own plus the digit totals: 19 launches for 64 bits).  Ranking as in
+// k_rs_onesweep, the tile read back after each pass.
+constexpr int RB_THREADS = 512, RB_ITEMS = 10, RB_MAX = RB_THREADS * RB_ITEMS, RB_WARPS = RB_THREADS / 32;
+template <bool HI, bool VALS>
+__global__ void __launch_bounds__(RB_THREADS) k_rs_block(uint64_t *__restrict__ lo, uint64_t *__restrict__ hi,
+                                                         uint32_t *__restrict__ v, int m, int bit0, int npass) {
+    __shared__ uint32_t whist[RB_WARPS][256];
+    __shared__ uint32_t tstart[256];
+    __shared__ uint32_t wsum[32];
+    extern __shared__ uint64_t stage[];
+    uint64_t *st_lo = stage, *st_hi = stage + m;
+    uint32_t *st_v = reinterpret_cast<uint32_t *>(stage + (HI ? 2 : 1) * (size_t)m);
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int64_t so = (int64_t)blockIdx.x * m;
+    const uint32_t lt = (1u << lane) - 1;
+    uint64_t klo[RB_ITEMS], khi[RB_ITEMS];
+    uint32_t vv[RB_ITEMS], dr[RB_ITEMS];
+    const int p0 = warp * (RB_ITEMS * 32) + lane;
+#pragma unroll
+    for (int i = 0; i < RB_ITEMS; i++) {
+        const int p = p0 + i * 32;
+        klo[i] = p < m ? lo[so + p] : 0;
+        khi[i] = HI && p < m ? hi[so + p] : 0;
+        vv[i] = VALS && p < m ? v[so + p] : 0;
+    }
+    for (int q = 0; q < npass; q++) {
+        const int sh = bit0 + 8 * q;
+        for (int e = t; e < RB_WARPS * 256; e += RB_THREADS) whist[e >> 8][e & 255] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < RB_ITEMS; i++) {
+            const uint32_t d = p0 + i * 32 < m ? (uint32_t)(((sh >= 64 ? khi[i] : klo[i]) >> (sh & 63)) & 0xFFu) : 256u;
+            const uint32_t peers = __match_any_sync(0xffffffffu, d);
+            const int leader = __ffs(peers) - 1;
+            uint32_t old = 0;
+            if (lane == leader && d < 256) {
+                old = whist[warp][d];
+                whist[warp][d] = old + __popc(peers);
+            }
+            old = __shfl_sync(0xffffffffu, old, leader);
+            dr[i] = d | ((old + __popc(peers & lt)) << 9);
+        }
+        __syncthreads();
+        uint32_t run = 0;
+        if (t < 256) {
+#pragma unroll
+            for (int w = 0; w < RB_WARPS; w++) {
+                const uint32_t c = whist[w][t];
+                whist[w][t] = run;
+                run += c;
+            }
+        }
+        uint32_t tot;
+        const uint32_t ex = block_excl_scan<RB_THREADS>(run, &tot, wsum);
+        if (t < 256) tstart[t] = ex;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < RB_ITEMS; i++) {
+            const uint32_t d = dr[i] & 511u;
+            if (d < 256) {
+                const uint32_t lp = tstart[d] + whist[warp][d] + (dr[i] >> 9);
+                st_lo[lp] = klo[i];
+                if (HI) st_hi[lp] = khi[i];
+                if (VALS) st_v[lp] = vv[i];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < RB_ITEMS; i++) {
+            const int p = p0 + i * 32;
+            if (p < m) {
+                klo[i] = st_lo[p];
+                if (HI) khi[i] = st_hi[p];
+                if (VALS) vv[i] = st_v[p];
+            }
+        }
+        // the next pass writes the stage only after its first barriers
+    }
+#pragma unroll
+    for (int i = 0; i < RB_ITEMS; i++) {
+        const int p = p0 + i * 32;
+        if (p < m) {
+            lo[so + p] = klo[i];
+            if (HI) hi[so + p] = khi[i];
+            if (VALS) v[so + p] = vv[i];
+        }
+    }
+}
+
 // ---- run detection ---------------------------------------------------------
 // a run starts where the key (lo, hi) or the optional tag changes
 __device__ __forceinline__ bool run_start_at(const uint64_t *lo, const uint64_t *hi, const uint32_t *tag, int64_t p) {
@@ -477,6 +568,46 @@ __global__ void __launch_bounds__(RS_THREADS) k_i64_tile_apply(const int64_t *__
     for (int e = threadIdx.x; e < cnt; e += RS_THREADS) out[t0 + e] = tv[e];
 }
 
+// the same for up to SCAN_ONE values by one block (one launch instead of three):
+// thread t the values 16 t .. 16 t + 15
+constexpr int SCAN_ONE = 16384;
+__global__ void __launch_bounds__(1024) k_i64_scan_one(const int64_t *__restrict__ in, int64_t *__restrict__ out, int n,
+                                                       int64_t *__restrict__ total) {
+    __shared__ int64_t s_warp[32];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    int64_t v[16], s = 0;
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+        v[i] = 16 * t + i < n ? in[16 * t + i] : 0;
+        s += v[i];
+    }
+    int64_t x = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) s_warp[w] = x;
+    __syncthreads();
+    if (w == 0) {
+        int64_t z = s_warp[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t y = __shfl_up_sync(0xffffffffu, z, o);
+            if (lane >= o) z += y;
+        }
+        s_warp[lane] = z;
+    }
+    __syncthreads();
+    int64_t ex = x - s + (w ? s_warp[w - 1] : 0);
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+        if (16 * t + i < n) out[16 * t + i] = ex;
+        ex += v[i];
+    }
+    if (t == 0 && total) *total = s_warp[31];
+}
+
 __global__ void k_iota_u32(uint32_t *v, int64_t n, int64_t period) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
@@ -542,6 +673,23 @@ geek_status radix_sort_segments(geek_ctx *ctx, Scratch &scr, int S, int64_t m, u
     const bool hi = nbits > 64;
     if (hi && !(key_hi && *key_hi)) return set_error(ctx, GEEK_ERR_INVALID, "radix sort: missing hi word");
     const bool hv = vals && *vals;
+    const int npass = (nbits - bit0 + 7) / 8;
+    if (m <= RB_MAX) {
+        const size_t smem = (size_t)m * ((hi ? 16 : 8) + (hv ? 4 : 0));
+        EvTimer tk(ctx, "kernel.rs_scatter", st);
+        tk.work = 2.0 * (double)S * m * ((hi ? 16 : 8) + (hv ? 4 : 0)) * npass;
+        GK_COUNT();
+        auto run = [&](auto *k) -> geek_status {
+            GK_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, RB_MAX * 20));
+            k<<<S, RB_THREADS, smem, st>>>(*key_lo, hi ? *key_hi : nullptr, hv ? *vals : nullptr, (int)m, bit0, npass);
+            GK_LAUNCH(ctx);
+            return GEEK_OK;
+        };
+        if (hi && hv) return run(k_rs_block<true, true>);
+        if (hi) return run(k_rs_block<true, false>);
+        if (hv) return run(k_rs_block<false, true>);
+        return run(k_rs_block<false, false>);
+    }
     const int tiles = (int)ceil_div(m, RS_TILE);
     const int64_t total = (int64_t)S * m;
     uint64_t *lo2 = nullptr, *hi2 = nullptr;
@@ -563,14 +711,17 @@ geek_status radix_sort_segments(geek_ctx *ctx, Scratch &scr, int S, int64_t m, u
         GK_CUDA(ctx, cudaFuncSetAttribute(k_rs_hist_all, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * 16 * 256 * 4));
         attr_done = true;
     }
-    const int npass = (nbits - bit0 + 7) / 8;
     // all digit offsets from one read of the keys
-    uint32_t *dbase_all, *look, *ticket;
-    GK_TRY(scr.alloc(&dbase_all, (size_t)S * npass * 256));
-    GK_TRY(scr.alloc(&look, (size_t)S * tiles * 256 + 32));
-    ticket = look + (size_t)S * tiles * 256;
+    // digit totals, then per pass the look-back words and the ticket: small
+    // sorts clear all passes' words with the totals (one fill instead of npass
+    // + 1), larger ones reuse one pass's words, cleared before each
+    uint32_t *dbase_all, *look;
+    const size_t nd = (size_t)S * npass * 256, nl = (size_t)S * tiles * 256 + 32;
+    const bool one_fill = nl * npass <= ((size_t)4 << 20);  // 16 MB
+    GK_TRY(scr.alloc(&dbase_all, nd + (one_fill ? npass : 1) * nl));
+    look = dbase_all + nd;
     GK_TRY(sort_err_word(ctx));
-    GK_CUDA(ctx, cudaMemsetAsync(dbase_all, 0, sizeof(uint32_t) * S * npass * 256, st));
+    GK_CUDA(ctx, cudaMemsetAsync(dbase_all, 0, sizeof(uint32_t) * (nd + (one_fill ? npass * nl : 0)), st));
     {
         const int hb = (int)std::min<int64_t>(HIST_BLOCKS_PER_SEG, ceil_div(m, 256 * 16));
         GK_COUNT();
@@ -584,13 +735,14 @@ geek_status radix_sort_segments(geek_ctx *ctx, Scratch &scr, int S, int64_t m, u
     const int64_t nblocks = (int64_t)S * tiles;
     for (int q = 0; q < npass; q++, passes++) {
         const int sh = bit0 + q * 8, dsel = sh >= 64, sv = sh & 63;
-        GK_CUDA(ctx, cudaMemsetAsync(look, 0, sizeof(uint32_t) * ((size_t)S * tiles * 256 + 32), st));
+        if (!one_fill) GK_CUDA(ctx, cudaMemsetAsync(look, 0, sizeof(uint32_t) * nl, st));
+        uint32_t *const lk = look + (one_fill ? q * nl : 0), *const ticket = lk + (nl - 32);
         EvTimer tk(ctx, "kernel.rs_scatter", st);
         tk.work = 2.0 * (double)total * ((hi ? 16 : 8) + (hv ? 4 : 0));
         GK_COUNT();
 #define RS_OS(H, V)                                                                                              \
     k_rs_onesweep<H, V><<<(unsigned)nblocks, RS_THREADS, stage, st>>>(alo, ahi, av, blo, bhi, bv, m, tiles, dsel, sv, \
-                                                                      dbase_all + (size_t)q * 256, npass * 256, look, \
+                                                                      dbase_all + (size_t)q * 256, npass * 256, lk, \
                                                                       ticket, ctx->sort_err, ctx->lb_wait_ns, ctx->stall_tile)
         if (hi && hv) RS_OS(true, true);
         else if (hi) RS_OS(true, false);
@@ -701,6 +853,12 @@ geek_status exclusive_scan_i64(geek_ctx *ctx, Scratch &scr, const int64_t *in, i
                                int64_t n, int64_t *total_dev, cudaStream_t st) {
     if (n <= 0) {
         if (total_dev) GK_CUDA(ctx, cudaMemsetAsync(total_dev, 0, sizeof(int64_t), st));
+        return GEEK_OK;
+    }
+    if (n <= SCAN_ONE) {
+        GK_COUNT();
+        k_i64_scan_one<<<1, 1024, 0, st>>>(in, out, (int)n, total_dev);
+        GK_LAUNCH(ctx);
         return GEEK_OK;
     }
     const int64_t tiles = ceil_div(n, RS_TILE);
