@@ -231,9 +231,12 @@ geek_status sort_err_eval(geek_ctx *ctx, const int *h, cudaStream_t st);
 // 32-bit value in one word moves 8 bytes per element and pass where a key and
 // vals move 12.  On return the sorted data is in the buffers
 // pointed to by *key_lo / *key_hi / *vals (which may have been swapped with
-// internal buffers allocated from `scr`).
+// internal buffers allocated from `scr`).  iota (with vals, nbits > bit0): the
+// values are the elements' positions in their segments; the first pass makes
+// them and *vals needs no contents.
 geek_status radix_sort_segments(geek_ctx *ctx, Scratch &scr, int S, int64_t m, uint64_t **key_lo,
-                                uint64_t **key_hi, uint32_t **vals, int nbits, cudaStream_t st, int bit0 = 0);
+                                uint64_t **key_hi, uint32_t **vals, int nbits, cudaStream_t st, int bit0 = 0,
+                                bool iota = false);
 
 // Buckets of S key-sorted segments of m elements (ids: object id at each
 // sorted position): obj_bucket[seg][id] = rank of the id's key among the

@@ -537,11 +537,15 @@ __device__ __forceinline__ void shl_or(uint64_t &hi, uint64_t &lo, int b, uint64
 
 // key of table l for object i: fields codes[l*K1+k] - min (bits[f] wide),
 // then K2 MinHash values (32 bits each), the first field most significant.
-// One thread per object walks all L tables, so each code row is read once;
-// a block first copies its objects' code rows to shared memory with
-// coalesced loads (row stride F1 | 1 words: conflict-free row reads), when
-// they fit (PK_STAGE_MAX codes per row).
-constexpr int PK_THREADS = 256, PK_STAGE_MAX = 128;
+// A block copies the field rows of PK_ROWS objects to shared memory with
+// coalesced loads (row stride F | 1 words: conflict-free row reads), when they
+// fit (PK_STAGE_MAX fields per row), so each is read once; thread t then forms
+// the keys of row t % PK_ROWS for every (PK_THREADS / PK_ROWS)th table.  It is
+// one read and one write of memory: with 64 rows (25 KB at 96 fields, 8 blocks
+// per SM, where 256 rows let 2 resident blocks load or compute in turn) and
+// without the upper key word when no key needs it, 10M x 96 codes in 16 tables
+// take 0.99 ms (1.94 ms before).
+constexpr int PK_THREADS = 256, PK_ROWS = 64, PK_STAGE_MAX = 128;
 
 // copies `rows` consecutive code rows (F1 codes each, from row r0) to shared
 // rows of stride F1 | 1; the (row, column) of element e advance by fixed
@@ -589,6 +593,7 @@ __device__ __forceinline__ void pk_stage_rows(int32_t *cs, const int32_t *__rest
         }
     }
 }
+template <bool HI>
 __global__ void __launch_bounds__(PK_THREADS) k_pack_keys(int64_t n, int L, const int32_t *__restrict__ codes,
                                                           int F1, int K1, const int *__restrict__ fmin,
                                                           const int *__restrict__ bits,
@@ -596,8 +601,9 @@ __global__ void __launch_bounds__(PK_THREADS) k_pack_keys(int64_t n, int L, cons
                                                           uint64_t *__restrict__ klo, uint64_t *__restrict__ khi) {
     extern __shared__ int32_t cs[];
     __shared__ int s_min[PK_STAGE_MAX], s_bits[PK_STAGE_MAX];
-    const bool staged = F1 > 0 && F1 <= PK_STAGE_MAX;
-    const int rs = F1 | 1;
+    const int FS = F1 > 0 ? F1 : F2;  // the staged rows: the codes, or the MinHash values where there are no codes
+    const bool staged = FS > 0 && FS <= PK_STAGE_MAX;
+    const int rs = FS | 1;
     if (staged) {
         for (int f = threadIdx.x; f < F1; f += PK_THREADS) {
             s_min[f] = fmin[f];
@@ -606,26 +612,32 @@ __global__ void __launch_bounds__(PK_THREADS) k_pack_keys(int64_t n, int L, cons
     }
     const int *fm = staged ? s_min : fmin;
     const int *bt = staged ? s_bits : bits;
-    for (int64_t i0 = (int64_t)blockIdx.x * PK_THREADS; i0 < n; i0 += (int64_t)gridDim.x * PK_THREADS) {
-        const int64_t i = i0 + threadIdx.x;
+    const int row = threadIdx.x % PK_ROWS, l0 = threadIdx.x / PK_ROWS;
+    for (int64_t i0 = (int64_t)blockIdx.x * PK_ROWS; i0 < n; i0 += (int64_t)gridDim.x * PK_ROWS) {
+        const int64_t i = i0 + row;
         if (staged) {
             __syncthreads();
-            pk_stage_rows(cs, codes, i0, (int)min((int64_t)PK_THREADS, n - i0), F1);
+            pk_stage_rows(cs, F1 > 0 ? codes : (const int32_t *)mh, i0, (int)min((int64_t)PK_ROWS, n - i0), FS);
             __syncthreads();
         }
         if (i >= n) continue;
-        const int32_t *cr = staged ? cs + threadIdx.x * rs : codes + i * F1;
-        const uint32_t *mr = mh ? mh + i * F2 : nullptr;
-        for (int l = 0; l < L; l++) {
+        const int32_t *sr = cs + row * rs;
+        const int32_t *cr = staged ? sr : codes + i * F1;
+        const uint32_t *mr = staged && F1 == 0 ? (const uint32_t *)sr : mh ? mh + i * F2 : nullptr;
+        for (int l = l0; l < L; l += PK_THREADS / PK_ROWS) {
             uint64_t hi = 0, lo = 0;
             for (int k = 0; k < K1; k++) {
                 const int f = l * K1 + k;
                 const uint32_t v = (uint32_t)((int64_t)cr[f] - (int64_t)fm[f]);
-                shl_or(hi, lo, bt[f], v);
+                if (HI) shl_or(hi, lo, bt[f], v);
+                else lo = (lo << bt[f]) | v;
             }
-            for (int k = 0; k < K2; k++) shl_or(hi, lo, 32, mr[l * K2 + k]);
+            for (int k = 0; k < K2; k++) {
+                if (HI) shl_or(hi, lo, 32, mr[l * K2 + k]);
+                else lo = (lo << 32) | mr[l * K2 + k];
+            }
             klo[(int64_t)l * n + i] = lo;
-            if (khi) khi[(int64_t)l * n + i] = hi;
+            if (HI) khi[(int64_t)l * n + i] = hi;
         }
     }
 }
@@ -635,6 +647,7 @@ __global__ void __launch_bounds__(PK_THREADS) k_pack_keys(int64_t n, int L, cons
 // the instance's own packed K-tuple, so that one sort per table groups every
 // instance separately and keeps each instance's lexicographic order.
 // (code rows staged through shared memory as in k_pack_keys)
+template <bool HI>
 __global__ void __launch_bounds__(PK_THREADS) k_pack_keys_batch(int64_t N, int L, const int32_t *__restrict__ codes,
                                                                 int F1, int K1, const int64_t *__restrict__ row_off,
                                                                 int count, const int *__restrict__ fmin,
@@ -644,35 +657,38 @@ __global__ void __launch_bounds__(PK_THREADS) k_pack_keys_batch(int64_t N, int L
     extern __shared__ int32_t cs[];
     const bool staged = F1 <= PK_STAGE_MAX;
     const int rs = F1 | 1;
-    for (int64_t r0 = (int64_t)blockIdx.x * PK_THREADS; r0 < N; r0 += (int64_t)gridDim.x * PK_THREADS) {
-        const int64_t r = r0 + threadIdx.x;
+    const int row = threadIdx.x % PK_ROWS, l0 = threadIdx.x / PK_ROWS;
+    for (int64_t r0 = (int64_t)blockIdx.x * PK_ROWS; r0 < N; r0 += (int64_t)gridDim.x * PK_ROWS) {
+        const int64_t r = r0 + row;
         if (staged) {
             __syncthreads();
-            pk_stage_rows(cs, codes, r0, (int)min((int64_t)PK_THREADS, N - r0), F1);
+            pk_stage_rows(cs, codes, r0, (int)min((int64_t)PK_ROWS, N - r0), F1);
             __syncthreads();
         }
         if (r >= N) continue;
         const int i = find_inst(row_off, count, r);
-        const int32_t *cr = staged ? cs + threadIdx.x * rs : codes + r * F1;
+        const int32_t *cr = staged ? cs + row * rs : codes + r * F1;
         const int *fm = fmin + (int64_t)i * F1;
         const int *bt = bits + (int64_t)i * F1;
-        for (int l = 0; l < L; l++) {
+        for (int l = l0; l < L; l += PK_THREADS / PK_ROWS) {
             uint64_t hi = 0, lo = 0;
             for (int k = 0; k < K1; k++) {
                 const int f = l * K1 + k;
-                shl_or(hi, lo, bt[f], (uint32_t)((int64_t)cr[f] - (int64_t)fm[f]));
+                const uint32_t v = (uint32_t)((int64_t)cr[f] - (int64_t)fm[f]);
+                if (HI) shl_or(hi, lo, bt[f], v);
+                else lo = (lo << bt[f]) | v;
             }
             const uint64_t iv = (uint64_t)i;
             if (B >= 64) {
-                hi |= iv << (B - 64);
+                if (HI) hi |= iv << (B - 64);
             } else if (B > 0) {
                 lo |= iv << B;
-                hi |= iv >> (64 - B);
+                if (HI) hi |= iv >> (64 - B);
             } else {
                 lo = iv;
             }
             klo[(int64_t)l * N + r] = lo;
-            if (khi) khi[(int64_t)l * N + r] = hi;
+            if (HI) khi[(int64_t)l * N + r] = hi;
         }
     }
 }
@@ -903,11 +919,10 @@ geek_status pack_keys_batch(geek_ctx *ctx, int64_t N, int L, const int32_t *code
     if (N == 0) return GEEK_OK;
     GK_COUNT();
     const int F1 = K * L;
-    const size_t smem = F1 <= PK_STAGE_MAX ? (size_t)PK_THREADS * (F1 | 1) * sizeof(int32_t) : 0;
-    GK_CUDA(ctx, cudaFuncSetAttribute(k_pack_keys_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(PK_THREADS * (PK_STAGE_MAX | 1) * sizeof(int32_t))));
-    k_pack_keys_batch<<<grid_for(N, PK_THREADS, ctx->num_sms), PK_THREADS, smem, st>>>(N, L, codes, F1, K, row_off,
-                                                                                       count, fmin, bits, B, klo, khi);
+    const size_t smem = F1 <= PK_STAGE_MAX ? (size_t)PK_ROWS * (F1 | 1) * sizeof(int32_t) : 0;
+    (khi ? k_pack_keys_batch<true> : k_pack_keys_batch<false>)<<<grid_for(ceil_div(N, PK_ROWS), 1, ctx->num_sms),
+                                                                 PK_THREADS, smem, st>>>(
+        N, L, codes, F1, K, row_off, count, fmin, bits, B, klo, khi);
     GK_LAUNCH(ctx);
     return GEEK_OK;
 }
@@ -979,11 +994,10 @@ geek_status pack_keys(geek_ctx *ctx, int64_t n, int L, const int32_t *codes, int
                       uint64_t *klo, uint64_t *khi, cudaStream_t st) {
     if (n == 0) return GEEK_OK;
     GK_COUNT();
-    const size_t smem = (F1 > 0 && F1 <= PK_STAGE_MAX) ? (size_t)PK_THREADS * (F1 | 1) * sizeof(int32_t) : 0;
-    GK_CUDA(ctx, cudaFuncSetAttribute(k_pack_keys, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(PK_THREADS * (PK_STAGE_MAX | 1) * sizeof(int32_t))));
-    k_pack_keys<<<grid_for(n, PK_THREADS, ctx->num_sms), PK_THREADS, smem, st>>>(n, L, codes, F1, K1, fmin, bits, mh,
-                                                                                 F2, K2, klo, khi);
+    const int FS = F1 > 0 ? F1 : F2;
+    const size_t smem = FS <= PK_STAGE_MAX ? (size_t)PK_ROWS * (FS | 1) * sizeof(int32_t) : 0;
+    (khi ? k_pack_keys<true> : k_pack_keys<false>)<<<grid_for(ceil_div(n, PK_ROWS), 1, ctx->num_sms), PK_THREADS, smem,
+                                                     st>>>(n, L, codes, F1, K1, fmin, bits, mh, F2, K2, klo, khi);
     GK_LAUNCH(ctx);
     return GEEK_OK;
 }
@@ -992,11 +1006,9 @@ geek_status group_tables(geek_ctx *ctx, Scratch &scr, int64_t n, int L, uint64_t
                          uint64_t *khi, int nbits, uint32_t *ids, int32_t *obj_bucket,
                          int64_t **boff_out, std::vector<int64_t> &nb, int64_t *NB_out,
                          cudaStream_t st) {
-    launch_iota_u32(ids, n * L, n, st);
-    GK_LAUNCH(ctx);
     {
         EvTimer tk(ctx, "hash.sort", st);
-        GK_TRY(radix_sort_segments(ctx, scr, L, n, &klo, khi ? &khi : nullptr, &ids, nbits, st));
+        GK_TRY(radix_sort_segments(ctx, scr, L, n, &klo, khi ? &khi : nullptr, &ids, nbits, st, 0, true));
     }
     return segment_buckets(ctx, scr, L, n, klo, nbits > 64 ? khi : nullptr, ids, obj_bucket, boff_out, nb, NB_out,
                            st);

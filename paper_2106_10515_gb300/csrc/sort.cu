@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(RS_THREADS, 4)
         const bool valid = p < m;
         klo[i] = valid ? lo_in[so + p] : 0;
         khi[i] = (HI && valid) ? hi_in[so + p] : 0;
-        vv[i] = (VALS && valid) ? v_in[so + p] : 0;
+        vv[i] = (VALS && valid) ? (v_in ? v_in[so + p] : (uint32_t)p) : 0;
     }
 #pragma unroll
     for (int i = 0; i < IT; i++) {
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(RS_THREADS, 4)
 constexpr int RB_THREADS = 512, RB_ITEMS = 10, RB_MAX = RB_THREADS * RB_ITEMS, RB_WARPS = RB_THREADS / 32;
 template <bool HI, bool VALS>
 __global__ void __launch_bounds__(RB_THREADS) k_rs_block(uint64_t *__restrict__ lo, uint64_t *__restrict__ hi,
-                                                         uint32_t *__restrict__ v, int m, int bit0, int npass) {
+                                                         uint32_t *__restrict__ v, int m, int bit0, int npass, bool iota) {
     __shared__ uint32_t whist[RB_WARPS][256];
     __shared__ uint32_t tstart[256];
     __shared__ uint32_t wsum[32];
@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(RB_THREADS) k_rs_block(uint64_t *__restrict__ 
         const int p = p0 + i * 32;
         klo[i] = p < m ? lo[so + p] : 0;
         khi[i] = HI && p < m ? hi[so + p] : 0;
-        vv[i] = VALS && p < m ? v[so + p] : 0;
+        vv[i] = VALS && p < m ? (iota ? (uint32_t)p : v[so + p]) : 0;
     }
     for (int q = 0; q < npass; q++) {
         const int sh = bit0 + 8 * q;
@@ -608,12 +608,6 @@ __global__ void __launch_bounds__(1024) k_i64_scan_one(const int64_t *__restrict
     if (t == 0 && total) *total = s_warp[31];
 }
 
-__global__ void k_iota_u32(uint32_t *v, int64_t n, int64_t period) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        v[i] = (uint32_t)(i % period);
-}
-
 }  // namespace
 
 geek_status set_error(geek_ctx *ctx, geek_status st, const char *fmt, ...) {
@@ -656,16 +650,11 @@ geek_status sort_err_check(geek_ctx *ctx, cudaStream_t st) {
     return sort_err_eval(ctx, &h, st);
 }
 
-void launch_iota_u32(uint32_t *v, int64_t n, int64_t period, cudaStream_t st) {
-    if (n <= 0) return;
-    int blocks = (int)std::min<int64_t>(ceil_div(n, 256), 1 << 16);
-    GK_COUNT();
-    k_iota_u32<<<blocks, 256, 0, st>>>(v, n, period);
-}
-
 geek_status radix_sort_segments(geek_ctx *ctx, Scratch &scr, int S, int64_t m, uint64_t **key_lo,
-                                uint64_t **key_hi, uint32_t **vals, int nbits, cudaStream_t st, int bit0) {
-    if (S <= 0 || m <= 1 || nbits <= bit0) return GEEK_OK;
+                                uint64_t **key_hi, uint32_t **vals, int nbits, cudaStream_t st, int bit0, bool iota) {
+    if (S <= 0 || m < 1) return GEEK_OK;
+    if (m == 1 && iota) GK_CUDA(ctx, cudaMemsetAsync(*vals, 0, sizeof(uint32_t) * S, st));
+    if (m == 1 || nbits <= bit0) return GEEK_OK;
     if (S > 65535) return set_error(ctx, GEEK_ERR_UNSUPPORTED, "radix sort: %d segments", S);
     if (m > (int64_t)LB_MASK) return set_error(ctx, GEEK_ERR_UNSUPPORTED, "radix sort: segment too long");
     if ((int64_t)S * ceil_div(m, RS_TILE) > 0xFFFFFFFFLL)
@@ -681,7 +670,7 @@ geek_status radix_sort_segments(geek_ctx *ctx, Scratch &scr, int S, int64_t m, u
         GK_COUNT();
         auto run = [&](auto *k) -> geek_status {
             GK_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, RB_MAX * 20));
-            k<<<S, RB_THREADS, smem, st>>>(*key_lo, hi ? *key_hi : nullptr, hv ? *vals : nullptr, (int)m, bit0, npass);
+            k<<<S, RB_THREADS, smem, st>>>(*key_lo, hi ? *key_hi : nullptr, hv ? *vals : nullptr, (int)m, bit0, npass, iota);
             GK_LAUNCH(ctx);
             return GEEK_OK;
         };
@@ -741,8 +730,8 @@ geek_status radix_sort_segments(geek_ctx *ctx, Scratch &scr, int S, int64_t m, u
         tk.work = 2.0 * (double)total * ((hi ? 16 : 8) + (hv ? 4 : 0));
         GK_COUNT();
 #define RS_OS(H, V)                                                                                              \
-    k_rs_onesweep<H, V><<<(unsigned)nblocks, RS_THREADS, stage, st>>>(alo, ahi, av, blo, bhi, bv, m, tiles, dsel, sv, \
-                                                                      dbase_all + (size_t)q * 256, npass * 256, lk, \
+    k_rs_onesweep<H, V><<<(unsigned)nblocks, RS_THREADS, stage, st>>>(alo, ahi, iota && q == 0 ? nullptr : av, blo, bhi, bv, m, \
+                                                                      tiles, dsel, sv, dbase_all + (size_t)q * 256, npass * 256, lk, \
                                                                       ticket, ctx->sort_err, ctx->lb_wait_ns, ctx->stall_tile)
         if (hi && hv) RS_OS(true, true);
         else if (hi) RS_OS(true, false);
