@@ -577,6 +577,177 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc(const __grid_consta
     }
 }
 
+// The BF16 pass over pairs of row tiles (one data set of many rows and centres).
+// A centre tile is what bounds k_assign_tc at d = 128: per 128 x 256 tile the
+// tensor core takes 9 k-steps of 128 cycles and reads 12 KB of shared memory for
+// each, and the copy of the next centre tile writes 72 KB: 180 KB in 1,152 cycles
+// is more than the 128 bytes a cycle that shared memory gives.  Here a centre
+// tile serves two row tiles, row tile 0 into accumulator 0, row tile 1 into
+// accumulator 1, so the copies write half as much per MMA (144 KB in 1,152
+// cycles).  Both X stages hold the pair, so the next pair's first tile arrives
+// while the last MMAs on the second one run; epilogue warps 2-5 own
+// accumulator 0, 6-9 accumulator 1, each all 256 columns of its 32 rows (no
+// merge).  10M x 128, k = 20,000: 34.4 ms, one row tile at a time 36.2 ms.
+__global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc_pair(const __grid_constant__ TcArgs A) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t *sA0 = base, *sB0 = base + 2 * TC_A_STAGE;
+    uint64_t *bars = (uint64_t *)(base + 2 * TC_A_STAGE + 2 * TC_B_STAGE);
+    uint64_t *full_a = bars, *empty_a = bars + 2, *full_acc = bars + 4, *empty_acc = bars + 6;
+    uint64_t *full_b = bars + 8, *empty_b = bars + 10, *done_bar = bars + 12;
+    uint32_t *tmem_slot = (uint32_t *)(bars + 13);
+    uint8_t *sOnes = base + 2 * TC_A_STAGE + 2 * TC_B_STAGE + TC_MISC;
+    uint8_t *sX0 = sOnes + TC_M * 32;  // [2][TC_N * 32]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < 2; i++) {
+            mbar_init(&full_a[i], 1);
+            mbar_init(&empty_a[i], 1);
+            mbar_init(&full_acc[i], 1);
+            mbar_init(&empty_acc[i], TC_EPI_WARPS / 2);
+            mbar_init(&full_b[i], 1);
+            mbar_init(&empty_b[i], 1);
+        }
+        mbar_init(done_bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    for (int e = threadIdx.x; e < TC_M * 32 / 4; e += blockDim.x)
+        reinterpret_cast<uint32_t *>(sOnes)[e] = 0x3F803F80u;
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tmem_slot)),
+                     "r"(TC_TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = *tmem_slot;
+    const TcInst &I = A.inst[0];
+    const int nkb = I.Kp / TC_KB, ntc = I.ntiles_c;
+
+    if (warp == 0) {
+        // ------------------------------------------------ TMA producer
+        if (lane == 0) {
+            uint64_t ct = 0;
+            uint32_t it = 0, issued_a[2] = {0, 0}, issued_b[2] = {0, 0};
+            bool ok = true;
+            for (int64_t u = blockIdx.x; u < A.nunits && ok; u += gridDim.x, it++) {
+                for (int h = 0; h < 2; h++) {
+                    if (!(ok = mbar_wait(&empty_a[h], (it & 1) ^ 1, A.err))) break;
+                    mbar_expect_tx(&full_a[h], (uint32_t)(nkb * TC_M * 128));
+                    // a second tile past the rows reads zeros
+                    for (int kb = 0; kb < nkb; kb++)
+                        tma_load_2d(su32(sA0 + h * TC_A_STAGE + kb * TC_M * 128), &I.tmA, kb * TC_KB,
+                                    (int)(2 * u + h) * TC_M, &full_a[h]);
+                    issued_a[h] = it + 1;
+                }
+                for (int c = 0; c < ntc && ok; c++, ct++) {
+                    const int s = (int)(ct & 1);
+                    const uint32_t uu = (uint32_t)(ct >> 1);
+                    if (!(ok = mbar_wait(&empty_b[s], (uu & 1) ^ 1, A.err))) break;
+                    mbar_expect_tx(&full_b[s], (uint32_t)(nkb * TC_N * 128 + TC_N * 32));
+                    for (int kb = 0; kb < nkb; kb++)
+                        tma_load_2d(su32(sB0 + s * TC_B_STAGE + kb * TC_N * 128), &I.tmB, kb * TC_KB, c * TC_N, &full_b[s]);
+                    tma_load_2d(su32(sX0 + s * TC_N * 32), &I.tmX, 0, c * TC_N, &full_b[s]);
+                    issued_b[s] = uu + 1;
+                }
+                if (!ok) break;
+            }
+            // drain: every copy this thread issued has landed
+            for (int h = 0; h < 2; h++)
+                if (issued_a[h]) mbar_wait(&full_a[h], (issued_a[h] - 1) & 1, A.err, true);
+            for (int s = 0; s < 2; s++)
+                if (issued_b[s]) mbar_wait(&full_b[s], (issued_b[s] - 1) & 1, A.err, true);
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // ------------------------------------------------ MMA issuer
+        if (lane == 0) {
+            uint64_t ct = 0;
+            uint32_t it = 0;
+            bool ok = true;
+            const uint32_t idesc = idesc_bf16(TC_M, TC_N);
+            for (int64_t u = blockIdx.x; u < A.nunits && ok; u += gridDim.x, it++) {
+                for (int c = 0; c < ntc && ok; c++, ct++) {
+                    const int s = (int)(ct & 1);
+                    if (!(ok = mbar_wait(&full_b[s], (uint32_t)(ct >> 1) & 1, A.err))) break;
+                    for (int h = 0; h < 2; h++) {
+                        if (!(ok = mbar_wait(&empty_acc[h], ((uint32_t)ct & 1) ^ 1, A.err))) break;
+                        if (c == 0 && !(ok = mbar_wait(&full_a[h], it & 1, A.err))) break;
+                        fence_after();
+                        const uint32_t dtm = tmem + (uint32_t)(h * TC_N);
+                        for (int kb = 0; kb < nkb; kb++) {
+                            const uint64_t da = sdesc(su32(sA0 + h * TC_A_STAGE + kb * TC_M * 128));
+                            const uint64_t db = sdesc(su32(sB0 + s * TC_B_STAGE + kb * TC_N * 128));
+#pragma unroll
+                            for (int ks = 0; ks < TC_KB / 16; ks++)
+                                mma_bf16(dtm, da + 2 * ks, db + 2 * ks, idesc, (kb | ks) != 0);
+                        }
+                        // + |c|^2
+                        mma_bf16(dtm, sdesc32(su32(sOnes)), sdesc32(su32(sX0 + s * TC_N * 32)), idesc, 1);
+                        mma_commit(&full_acc[h]);
+                        if (c + 1 == ntc) mma_commit(&empty_a[h]);
+                    }
+                    if (!ok) break;
+                    mma_commit(&empty_b[s]);
+                }
+            }
+            // drain: all MMAs this thread issued have completed
+            mma_commit(done_bar);
+            mbar_wait(done_bar, 0, A.err, true);
+        }
+        __syncwarp();
+    } else {
+        // ------------------------------------------------ epilogue
+        const int q = warp & 3;         // TMEM lane quarter this warp may access
+        const int h = (warp - 2) >> 2;  // its accumulator
+        const uint32_t tbase = tmem + (uint32_t)(h * TC_N) + ((uint32_t)(32 * q) << 16);
+        const float cmax = sqrtf(__uint_as_float(*I.cmax_bits)) * (1.f + 1e-5f);
+        uint64_t ct = 0;
+        bool ok = true;
+        for (int64_t u = blockIdx.x; u < A.nunits; u += gridDim.x) {
+            const int64_t row = (2 * u + h) * TC_M + 32 * q + lane;
+            const float xn = row < I.n ? I.xnorm[row] : 0.f;
+            const float Wc = 2.f * window_bf16(xn, cmax, I.d) * (1.f + 1e-6f);
+            float b1 = FLT_MAX, b2o = FLT_MAX, sv[32];
+            int64_t sj = -1;
+            for (int c = 0; c < ntc; c++, ct++) {
+                int w_ok = 0;
+                if (lane == 0 && ok) w_ok = mbar_wait(&full_acc[h], (uint32_t)ct & 1, A.err);
+                w_ok = __shfl_sync(0xffffffffu, w_ok, 0);
+                ok = ok && w_ok;
+                if (ok) {
+                    fence_after();
+                    epi_tile<TC_N / 32>(tbase, (int64_t)c * TC_N, b1, b2o, sv, sj);
+                    fence_before();
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&empty_acc[h]);
+            }
+            float b2;
+            int i1;
+            epi_resolve(b1, b2o, sv, sj, b2, i1);
+            if (row < I.n && ok) {
+                const bool valid = i1 != 0x7FFFFFFF;
+                I.labels[row] = valid ? i1 : -1;
+                if (!(valid && (I.k == 1 || b2 - b1 > Wc))) {
+                    const unsigned long long qq = atomicAdd(A.n_flag, 1ull);
+                    A.flag_rows[qq] = (int32_t)(I.row_base + row);
+                    A.flag_m[qq] = valid ? b1 : __int_as_float(0x7fc00000);
+                }
+            }
+        }
+    }
+    fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_TMEM_COLS) : "memory");
+    }
+}
+
 // X -> BF16 K-major [n][Kp] (zero padded) and an upper bound of |x| per row;
 // warp per global row r of instance find_inst(row_off, r); xnorm is global.
 // A lane converts 4 consecutive columns at a time (float4 loads, 8-byte
@@ -850,7 +1021,8 @@ geek_status tc_plan_build(geek_ctx *ctx, Scratch *scr, const std::vector<TcPlanI
                                  cudaMemcpyHostToDevice, st));
     GK_TRY(tc_plan_upload(ctx, P, st));
     for (const void *fn : {(const void *)k_assign_tc<false, false>, (const void *)k_assign_tc<true, false>,
-                           (const void *)k_assign_tc<false, true>, (const void *)k_assign_tc<true, true>})
+                           (const void *)k_assign_tc<false, true>, (const void *)k_assign_tc<true, true>,
+                           (const void *)k_assign_tc_pair})
         GK_CUDA(ctx, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem()));
     return GEEK_OK;
 }
@@ -979,6 +1151,27 @@ geek_status tc_plan_launch(geek_ctx *ctx, const TcPlan &P, int32_t *flag_rows, f
                            unsigned long long *n_flag, cudaStream_t st) {
     double work = 0.0;
     for (const TcPlanInst &I : P.desc) work += 2.0 * (double)I.n * (double)I.k * (double)I.d;
+    // Pairs of row tiles: one BF16 data set of 256-wide tiles whose pairs fill
+    // the chip four times over (below, half as many units leave SMs idle in
+    // the last wave) and whose centre tiles are several per pair (the next
+    // pair's rows are loaded only at the end of this one).
+    const TcPlanInst &I0 = P.desc[0];
+    const int64_t pairs = ceil_div(I0.n, 2 * TC_M);
+    if (P.count == 1 && !I0.split && I0.N == TC_N && pairs >= 4 * (int64_t)ctx->num_sms && I0.k >= 8 * TC_N) {
+        TcArgs A{};
+        A.inst = P.inst;
+        A.nunits = pairs;
+        A.flag_rows = flag_rows;
+        A.flag_m = flag_m;
+        A.n_flag = n_flag;
+        A.err = P.err;
+        EvTimer tk(ctx, "kernel.assign_tc", st);
+        tk.work = work;
+        GK_COUNT();
+        k_assign_tc_pair<<<ctx->num_sms, TC_THREADS, tc_smem(), st>>>(A);
+        GK_LAUNCH(ctx);
+        return GEEK_OK;
+    }
     return launch_units(ctx, P.inst, P.units, P.nunits, P.nunits_x3, flag_rows, flag_m, n_flag, P.err, work,
                         ring_lg(P, nullptr, 0), ring_lg(P, nullptr, 1), st);
 }
