@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc(const __grid_consta
                 const int2 un = unit(u);
                 const TcInst &I = A.inst[un.x];
                 if (EMIT && (I.split != 0) != SPLIT) continue;
-                const int nkb = I.Kp / TC_KB, N = I.N;  // logical k-blocks
+                const int nkb = I.Kp / TC_KB, N = I.N, d = I.d;  // logical k-blocks
                 const int all = KW * nkb, bps = blocks_of(I);
                 const uint32_t idesc = idesc_bf16(TC_M, N);
                 for (int c = 0; c < I.ntiles_c && ok; c++, ct++) {
@@ -410,6 +410,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc(const __grid_consta
                                 sdesc(su32(sA0 + (int)(at & (uint64_t)(NA - 1)) * A_ST) + (SPLIT ? 0 : kb * TC_M * 128));
 #pragma unroll
                             for (int ks = 0; ks < TC_KB / 16; ks++) {
+                                if (kb * TC_KB + ks * 16 >= d) break;  // zeros from here on
                                 mma_bf16(dtm, da + 2 * ks, db + 2 * ks, idesc, (kb | ks) != 0);
                                 if (SPLIT) {  // x_l . c_h and x_h . c_l
                                     mma_bf16(dtm, da + (TC_M * 128 >> 4) + 2 * ks, db + 2 * ks, idesc, 1);
@@ -438,6 +439,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc(const __grid_consta
                             const uint64_t da = sdesc(su32(sA0 + ab * A_ST)), db = sdesc(su32(sB0 + sb * BSTR));
 #pragma unroll
                             for (int ks = 0; ks < TC_KB / 16; ks++) {
+                                if (kb * TC_KB + ks * 16 >= d) break;
                                 mma_bf16(dtm, da + 2 * ks, db + 2 * ks, idesc, (q | ks) != 0);
                                 // a hi block meets x_l too: x_h.c_h + x_l.c_h, then x_h.c_l
                                 if ((q & 1) == 0) mma_bf16(dtm, da + (TC_M * 128 >> 4) + 2 * ks, db + 2 * ks, idesc, 1);
@@ -625,7 +627,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc_pair(const __grid_c
     fence_after();
     const uint32_t tmem = *tmem_slot;
     const TcInst &I = A.inst[0];
-    const int nkb = I.Kp / TC_KB, ntc = I.ntiles_c;
+    const int nkb = I.Kp / TC_KB, ntc = I.ntiles_c, d = I.d;
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
@@ -682,8 +684,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc_pair(const __grid_c
                             const uint64_t da = sdesc(su32(sA0 + h * TC_A_STAGE + kb * TC_M * 128));
                             const uint64_t db = sdesc(su32(sB0 + s * TC_B_STAGE + kb * TC_N * 128));
 #pragma unroll
-                            for (int ks = 0; ks < TC_KB / 16; ks++)
+                            for (int ks = 0; ks < TC_KB / 16; ks++) {
+                                if (kb * TC_KB + ks * 16 >= d) break;  // zeros from here on
                                 mma_bf16(dtm, da + 2 * ks, db + 2 * ks, idesc, (kb | ks) != 0);
+                            }
                         }
                         // + |c|^2
                         mma_bf16(dtm, sdesc32(su32(sOnes)), sdesc32(su32(sX0 + s * TC_N * 32)), idesc, 1);
