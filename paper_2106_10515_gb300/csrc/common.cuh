@@ -224,10 +224,16 @@ geek_status sort_err_check(geek_ctx *ctx, cudaStream_t st);
 geek_status sort_err_fetch(geek_ctx *ctx, int *h, cudaStream_t st);
 geek_status sort_err_eval(geek_ctx *ctx, const int *h, cudaStream_t st);
 
+// the buffers a sort has finished with (from its scratch, or the caller's own)
+struct SortSpare {
+    uint64_t *lo, *hi;
+    uint32_t *vals;
+};
+
 // Stable LSD radix sort of S segments of m elements each (m < 2^30).  Keys are up to
 // 128 bits: key_lo holds bits 0..63, key_hi (may be null when nbits <= 64)
 // bits 64..127.  vals (may be null) moves with the keys.  Only bits
-// [bit0, nbits) are examined (bit0 a multiple of 8): a 32-bit key above a
+// [bit0, nbits) are examined (bit0 a multiple of 8 where nbits > 64): a 32-bit key above a
 // 32-bit value in one word moves 8 bytes per element and pass where a key and
 // vals move 12.  On return the sorted data is in the buffers
 // pointed to by *key_lo / *key_hi / *vals (which may have been swapped with
@@ -236,7 +242,12 @@ geek_status sort_err_eval(geek_ctx *ctx, const int *h, cudaStream_t st);
 // them and *vals needs no contents.
 geek_status radix_sort_segments(geek_ctx *ctx, Scratch &scr, int S, int64_t m, uint64_t **key_lo,
                                 uint64_t **key_hi, uint32_t **vals, int nbits, cudaStream_t st, int bit0 = 0,
-                                bool iota = false);
+                                bool iota = false, SortSpare *spare = nullptr);
+
+// Sorts S segments of m keys of nbits bits (ids as iota above): the same order
+// as radix_sort_segments, by the upper bits alone where few of them repeat.
+geek_status sort_ids(geek_ctx *ctx, Scratch &scr, int S, int64_t m, uint64_t **key_lo, uint64_t **key_hi,
+                     uint32_t **ids, int nbits, cudaStream_t st);
 
 // Buckets of S key-sorted segments of m elements (ids: object id at each
 // sorted position): obj_bucket[seg][id] = rank of the id's key among the

@@ -1008,7 +1008,7 @@ geek_status group_tables(geek_ctx *ctx, Scratch &scr, int64_t n, int L, uint64_t
                          cudaStream_t st) {
     {
         EvTimer tk(ctx, "hash.sort", st);
-        GK_TRY(radix_sort_segments(ctx, scr, L, n, &klo, khi ? &khi : nullptr, &ids, nbits, st, 0, true));
+        GK_TRY(sort_ids(ctx, scr, L, n, &klo, khi ? &khi : nullptr, &ids, nbits, st));
     }
     return segment_buckets(ctx, scr, L, n, klo, nbits > 64 ? khi : nullptr, ids, obj_bucket, boff_out, nb, NB_out,
                            st);

@@ -368,6 +368,215 @@ __global__ void __launch_bounds__(RB_THREADS) k_rs_block(uint64_t *__restrict__ 
     }
 }
 
+// ---- keys sorted by their upper bits, then settled ---------------------------
+// m objects rarely need all the bits of a wide key to be told apart.  So the
+// passes cover the upper bits only, and the runs of equal prefixes are put in the
+// order of the whole key afterwards: short ones by one thread each, longer ones by
+// a block each.  Both keep equal keys in the order they have, so the result is
+// the full sort's.  How many passes leave few prefixes that repeat is estimated
+// from a sample first (k_rs_twins).
+constexpr int FX_RUN = 32;                        // longest run of one thread
+constexpr int TW_SAMPLES = 8192, TW_SLOTS = 2 * TW_SAMPLES, TW_WIDTHS = 8;
+
+__device__ __forceinline__ bool same_prefix(uint64_t l0, uint64_t h0, uint64_t l1, uint64_t h1, int bit0) {
+    if (bit0 >= 64) return ((h0 ^ h1) >> (bit0 - 64)) == 0;
+    return h0 == h1 && ((l0 ^ l1) >> bit0) == 0;
+}
+
+// twins[w] += the samples of every segment whose prefix above bit0 - 8 w another
+// sample has (block per segment and w; pseudo-random positions, so that any order
+// of the objects is sampled alike)
+__global__ void __launch_bounds__(1024) k_rs_twins(const uint64_t *__restrict__ lo, const uint64_t *__restrict__ hi,
+                                                   int64_t m, int bit0, unsigned long long *__restrict__ twins) {
+    extern __shared__ unsigned long long slot[];
+    const int64_t so = (int64_t)blockIdx.x * m;
+    bit0 -= 8 * blockIdx.y;
+    for (int e = threadIdx.x; e < TW_SLOTS; e += 1024) slot[e] = ~0ull;
+    __syncthreads();
+    unsigned found = 0;
+    for (int e = threadIdx.x; e < TW_SAMPLES; e += 1024) {
+        // one position in each of TW_SAMPLES equal stretches
+        uint32_t z = (uint32_t)e * 2654435761u + blockIdx.x * 0x9E3779B9u;
+        z = (z ^ (z >> 15)) * 0x85EBCA6Bu;
+        z = (z ^ (z >> 13)) * 0xC2B2AE35u;
+        z ^= z >> 16;
+        const int64_t a = e * m / TW_SAMPLES, b = (e + 1) * m / TW_SAMPLES;
+        const int64_t p = so + a + (int64_t)(z % (uint32_t)(b - a));
+        const uint64_t l = lo[p], h = hi[p];
+        unsigned long long q = bit0 >= 64 ? h >> (bit0 - 64) : (l >> bit0) ^ (h * 0xD6E8FEB86659FD93ull);
+        if (q == ~0ull) q--;
+        uint32_t s = (uint32_t)((q * 0x9E3779B97F4A7C15ull) >> 50);  // 14 bits
+        for (;;) {
+            const unsigned long long old = atomicCAS(&slot[s], ~0ull, q);
+            if (old == ~0ull) break;
+            if (old == q) {
+                found++;
+                break;
+            }
+            s = (s + 1) & (TW_SLOTS - 1);
+        }
+    }
+    const unsigned w = __reduce_add_sync(0xffffffffu, found);
+    if ((threadIdx.x & 31) == 0 && w) atomicAdd(&twins[blockIdx.y], (unsigned long long)w);
+}
+
+// Runs of equal prefixes of 2 to FX_RUN elements into the order of the whole
+// key; the starts of longer ones go to the list.  A run belongs to the tile it
+// starts in, which may move its elements beyond the tile's end while the next
+// tile reads them: only their prefixes count there, and those are equal.  What
+// bounds it is the read of the keys and, with many short runs, the moved ids (16M
+// elements of the hetero rows' 8 tables: 0.26 ms; the passes it replaces took 1.1).
+__global__ void __launch_bounds__(RS_THREADS) k_rs_settle(uint64_t *__restrict__ lo, uint64_t *__restrict__ hi,
+                                                          uint32_t *__restrict__ v, int64_t m, int bit0,
+                                                          int64_t *__restrict__ list,
+                                                          unsigned long long *__restrict__ nlist) {
+    extern __shared__ uint64_t fx_sm[];  // elements t0 - 1 .. t0 + RS_TILE + FX_RUN - 1
+    constexpr int SPAN = RS_TILE + 1 + FX_RUN;
+    uint64_t *sl = fx_sm, *sh = fx_sm + SPAN;
+    const int64_t so = (int64_t)blockIdx.y * m, t0 = (int64_t)blockIdx.x * RS_TILE;
+    const int64_t left = m - t0;  // elements from t0 on
+    for (int e = threadIdx.x; e < SPAN; e += RS_THREADS) {
+        const int64_t p = t0 - 1 + e;
+        if (p >= 0 && p < m) {
+            sl[e] = lo[so + p];
+            sh[e] = hi[so + p];
+        }
+    }
+    __syncthreads();
+    const int cnt = (int)min((int64_t)RS_TILE, left), lim = (int)min((int64_t)(RS_TILE + FX_RUN), left);
+    for (int e = threadIdx.x; e < cnt; e += RS_THREADS) {
+        // element e of the tile at position e + 1
+        const uint64_t l = sl[e + 1], h = sh[e + 1];
+        if ((t0 + e > 0 && same_prefix(sl[e], sh[e], l, h, bit0)) || e + 1 >= lim ||
+            !same_prefix(sl[e + 2], sh[e + 2], l, h, bit0))
+            continue;
+        int len = 2;
+        while (len <= FX_RUN && e + len < lim && same_prefix(sl[e + 1 + len], sh[e + 1 + len], l, h, bit0))
+            len++;
+        if (len > FX_RUN) {
+            list[atomicAdd(nlist, 1ull)] = so + t0 + e;
+            continue;
+        }
+        // insertion; only this thread touches the run's keys and ids
+        uint32_t *ids = v + so + t0 + e;
+        bool moved = false;
+        for (int i = 1; i < len; i++) {
+            const uint64_t kl = sl[e + 1 + i], kh = sh[e + 1 + i];
+            auto above = [&](int j) { return sh[e + 1 + j] != kh ? sh[e + 1 + j] > kh : sl[e + 1 + j] > kl; };
+            if (!above(i - 1)) continue;
+            const uint32_t id = ids[i];
+            int j = i;
+            for (; j > 0 && above(j - 1); j--) {
+                sl[e + 1 + j] = sl[e + j];
+                sh[e + 1 + j] = sh[e + j];
+                ids[j] = ids[j - 1];
+            }
+            sl[e + 1 + j] = kl;
+            sh[e + 1 + j] = kh;
+            ids[j] = id;
+            moved = true;
+        }
+        if (moved)
+            for (int i = 0; i < len; i++) {
+                lo[so + t0 + e + i] = sl[e + 1 + i];
+                hi[so + t0 + e + i] = sh[e + 1 + i];
+            }
+    }
+}
+
+// The listed runs, a block each: least significant digit first over the bits
+// below the prefix, between the sorted buffers and the spare ones.
+constexpr int FL_ITEMS = 4;
+__global__ void __launch_bounds__(RB_THREADS) k_rs_settle_long(uint64_t *lo, uint64_t *hi,
+                                                               uint32_t *v, uint64_t *lo2,
+                                                               uint64_t *hi2, uint32_t *v2,
+                                                               int64_t m, int bit0, const int64_t *__restrict__ list,
+                                                               const unsigned long long *__restrict__ nlist) {
+    __shared__ uint32_t whist[RB_WARPS][256];
+    __shared__ uint32_t at[256];
+    __shared__ uint32_t wsum[32];
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const uint32_t lt = (1u << lane) - 1;
+    const int64_t nl = (int64_t)*nlist;
+    for (int64_t r = blockIdx.x; r < nl; r += gridDim.x) {
+        const int64_t p0 = list[r], room = (p0 / m + 1) * m - p0;
+        const uint64_t l0 = lo[p0], h0 = hi[p0];
+        int64_t len = 0;
+        for (;;) {
+            const int64_t p = len + t;
+            const int c = __syncthreads_count(p < room &&
+                                              same_prefix(lo[p0 + p], hi[p0 + p], l0, h0, bit0));
+            len += c;
+            if (c < RB_THREADS) break;
+        }
+        int pass = 0;
+        for (int sh = 0; sh < bit0; sh += 8, pass++) {
+            const uint64_t *sl = ((pass & 1) ? lo2 : lo) + p0, *shh = ((pass & 1) ? hi2 : hi) + p0;
+            const uint32_t *sv = ((pass & 1) ? v2 : v) + p0;
+            uint64_t *dl = ((pass & 1) ? lo : lo2) + p0, *dh = ((pass & 1) ? hi : hi2) + p0;
+            uint32_t *dv = ((pass & 1) ? v : v2) + p0;
+            auto digit = [&](uint64_t l, uint64_t h) { return (uint32_t)(((sh >= 64 ? h : l) >> (sh & 63)) & 0xFFu); };
+            if (t < 256) at[t] = 0;
+            __syncthreads();
+            for (int64_t p = t; p < len; p += RB_THREADS) atomicAdd(&at[digit(sl[p], shh[p])], 1u);
+            __syncthreads();
+            uint32_t tot;
+            const uint32_t ex = block_excl_scan<RB_THREADS>(t < 256 ? at[t] : 0u, &tot, wsum);
+            if (t < 256) at[t] = ex;
+            for (int64_t q0 = 0; q0 < len; q0 += RB_THREADS * FL_ITEMS) {
+                for (int e = t; e < RB_WARPS * 256; e += RB_THREADS) whist[e >> 8][e & 255] = 0;
+                __syncthreads();
+                uint32_t dr[FL_ITEMS];
+#pragma unroll
+                for (int i = 0; i < FL_ITEMS; i++) {
+                    const int64_t p = q0 + warp * (FL_ITEMS * 32) + i * 32 + lane;
+                    const uint32_t d = p < len ? digit(sl[p], shh[p]) : 256u;
+                    const uint32_t peers = __match_any_sync(0xffffffffu, d);
+                    const int leader = __ffs(peers) - 1;
+                    uint32_t old = 0;
+                    if (lane == leader && d < 256) {
+                        old = whist[warp][d];
+                        whist[warp][d] = old + __popc(peers);
+                    }
+                    old = __shfl_sync(0xffffffffu, old, leader);
+                    dr[i] = d | ((old + __popc(peers & lt)) << 9);
+                }
+                __syncthreads();
+                if (t < 256) {
+                    uint32_t run = at[t];
+#pragma unroll
+                    for (int w = 0; w < RB_WARPS; w++) {
+                        const uint32_t c = whist[w][t];
+                        whist[w][t] = run;
+                        run += c;
+                    }
+                    at[t] = run;
+                }
+                __syncthreads();
+#pragma unroll
+                for (int i = 0; i < FL_ITEMS; i++) {
+                    const int64_t p = q0 + warp * (FL_ITEMS * 32) + i * 32 + lane;
+                    const uint32_t d = dr[i] & 511u;
+                    if (d < 256) {
+                        const uint32_t o = whist[warp][d] + (dr[i] >> 9);
+                        dl[o] = sl[p];
+                        dh[o] = shh[p];
+                        dv[o] = sv[p];
+                    }
+                }
+                __syncthreads();
+            }
+        }
+        if (pass & 1)
+            for (int64_t p = t; p < len; p += RB_THREADS) {
+                lo[p0 + p] = lo2[p0 + p];
+                hi[p0 + p] = hi2[p0 + p];
+                v[p0 + p] = v2[p0 + p];
+            }
+        __syncthreads();
+    }
+}
+
 // ---- run detection ---------------------------------------------------------
 // a run starts where the key (lo, hi) or the optional tag changes
 __device__ __forceinline__ bool run_start_at(const uint64_t *lo, const uint64_t *hi, const uint32_t *tag, int64_t p) {
@@ -651,7 +860,7 @@ geek_status sort_err_check(geek_ctx *ctx, cudaStream_t st) {
 }
 
 geek_status radix_sort_segments(geek_ctx *ctx, Scratch &scr, int S, int64_t m, uint64_t **key_lo,
-                                uint64_t **key_hi, uint32_t **vals, int nbits, cudaStream_t st, int bit0, bool iota) {
+                                uint64_t **key_hi, uint32_t **vals, int nbits, cudaStream_t st, int bit0, bool iota, SortSpare *spare) {
     if (S <= 0 || m < 1) return GEEK_OK;
     if (m == 1 && iota) GK_CUDA(ctx, cudaMemsetAsync(*vals, 0, sizeof(uint32_t) * S, st));
     if (m == 1 || nbits <= bit0) return GEEK_OK;
@@ -686,9 +895,12 @@ geek_status radix_sort_segments(geek_ctx *ctx, Scratch &scr, int S, int64_t m, u
     GK_TRY(scr.alloc(&lo2, total));
     if (hi) GK_TRY(scr.alloc(&hi2, total));
     if (hv) GK_TRY(scr.alloc(&v2, total));
+    // iota: the first pass reads no values, so its output can be the buffer
+    // that makes *vals the last pass's
+    const bool odd = npass & 1;
     uint64_t *alo = *key_lo, *ahi = hi ? *key_hi : nullptr, *blo = lo2, *bhi = hi2;
     uint32_t *av = hv ? *vals : nullptr, *bv = v2;
-    int passes = 0;
+    if (iota && odd) std::swap(av, bv);
     const size_t stage = (size_t)RS_TILE * ((hi ? 16 : 8) + (hv ? 4 : 0));
     static bool attr_done = false;
     if (!attr_done) {
@@ -724,7 +936,7 @@ geek_status radix_sort_segments(geek_ctx *ctx, Scratch &scr, int S, int64_t m, u
         GK_LAUNCH(ctx);
     }
     const int64_t nblocks = (int64_t)S * tiles;
-    for (int q = 0; q < npass; q++, passes++) {
+    for (int q = 0; q < npass; q++) {
         const int sh = bit0 + q * 8, dsel = sh >= 64, sv = sh & 63;
         if (!one_fill) GK_CUDA(ctx, cudaMemsetAsync(look, 0, sizeof(uint32_t) * nl, st));
         uint32_t *const lk = look + (one_fill ? q * nl : 0), *const ticket = lk + (nl - 32);
@@ -745,11 +957,60 @@ geek_status radix_sort_segments(geek_ctx *ctx, Scratch &scr, int S, int64_t m, u
         std::swap(ahi, bhi);
         std::swap(av, bv);
     }
-    if (passes & 1) {  // result lives in the scratch buffers: copy back
+    if (odd && iota) {  // the values are in *vals, the keys change buffers
+        *key_lo = alo;
+        if (hi) *key_hi = ahi;
+    } else if (odd) {  // result lives in the scratch buffers: copy back
         GK_CUDA(ctx, cudaMemcpyAsync(*key_lo, alo, total * sizeof(uint64_t), cudaMemcpyDeviceToDevice, st));
         if (hi) GK_CUDA(ctx, cudaMemcpyAsync(*key_hi, ahi, total * sizeof(uint64_t), cudaMemcpyDeviceToDevice, st));
         if (hv) GK_CUDA(ctx, cudaMemcpyAsync(*vals, av, total * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st));
     }
+    if (spare) *spare = SortSpare{blo, bhi, bv};
+    return GEEK_OK;
+}
+
+geek_status sort_ids(geek_ctx *ctx, Scratch &scr, int S, int64_t m, uint64_t **key_lo, uint64_t **key_hi,
+                     uint32_t **ids, int nbits, cudaStream_t st) {
+    // The upper bits alone for keys of two words, where that saves three passes or
+    // more and the sample's cost (a launch and a wait, some 50 us) is small beside
+    // them; log2 m + 2 bits are the fewest that can do.  For one-word keys it gives
+    // nothing: 16 tables of 2M 60-bit keys saved two of eight passes (0.41 ms) and
+    // paid 0.36 ms for sampling and settling.
+    const int full = (nbits + 7) / 8, np0 = (bit_length_u64((uint64_t)m) + 2 + 7) / 8;
+    const int widths = std::min(TW_WIDTHS, full - 3 - np0 + 1);
+    if (nbits <= 64 || widths < 1 || S * m < (int64_t)8 << 20 || m < 4 * TW_SAMPLES)
+        return radix_sort_segments(ctx, scr, S, m, key_lo, key_hi, ids, nbits, st, 0, true);
+    int bit0 = (nbits - 8 * np0) & ~7;  // no digit across the words
+    unsigned long long *cnt, twins[TW_WIDTHS];  // twins, then the listed runs
+    GK_TRY(scr.alloc(&cnt, TW_WIDTHS + 1));
+    GK_CUDA(ctx, cudaMemsetAsync(cnt, 0, (TW_WIDTHS + 1) * sizeof *cnt, st));
+    const size_t tw_smem = TW_SLOTS * sizeof(unsigned long long);
+    GK_CUDA(ctx, cudaFuncSetAttribute(k_rs_twins, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tw_smem));
+    GK_COUNT();
+    k_rs_twins<<<dim3(S, widths), 1024, tw_smem, st>>>(*key_lo, *key_hi, m, bit0, cnt);
+    GK_LAUNCH(ctx);
+    GK_CUDA(ctx, cudaMemcpyAsync(twins, cnt, sizeof *cnt * widths, cudaMemcpyDeviceToHost, st));
+    GK_CUDA(ctx, cudaStreamSynchronize(st));
+    // An object with c others of its prefix has a twin among the samples with
+    // probability c TW_SAMPLES / m.  With a quarter of another on average the
+    // settling costs less than the passes it saves, even all in runs of 33 (a
+    // block each); tables of large buckets take all the passes.
+    int w = 0;
+    while (w < widths && (double)twins[w] * (double)m > 0.25 * (double)S * TW_SAMPLES * TW_SAMPLES) w++;
+    if (w == widths) return radix_sort_segments(ctx, scr, S, m, key_lo, key_hi, ids, nbits, st, 0, true);
+    bit0 -= 8 * w;
+    SortSpare sp;
+    GK_TRY(radix_sort_segments(ctx, scr, S, m, key_lo, key_hi, ids, nbits, st, bit0, true, &sp));
+    int64_t *list;
+    GK_TRY(scr.alloc(&list, (size_t)(S * m / (FX_RUN + 1) + 1)));
+    const dim3 grid((unsigned)ceil_div(m, RS_TILE), S);
+    const size_t smem = 2 * (size_t)(RS_TILE + 1 + FX_RUN) * sizeof(uint64_t);
+    GK_COUNT();
+    k_rs_settle<<<grid, RS_THREADS, smem, st>>>(*key_lo, *key_hi, *ids, m, bit0, list, cnt + TW_WIDTHS);
+    GK_COUNT();
+    k_rs_settle_long<<<2 * ctx->num_sms, RB_THREADS, 0, st>>>(*key_lo, *key_hi, *ids, sp.lo, sp.hi, sp.vals, m, bit0,
+                                                              list, cnt + TW_WIDTHS);
+    GK_LAUNCH(ctx);
     return GEEK_OK;
 }
 
