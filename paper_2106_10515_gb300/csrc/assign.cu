@@ -1628,11 +1628,60 @@ __global__ void __launch_bounds__(32) k_ul_chain(UlArgs A) {
     }
 }
 
+// A second stream for work beside the caller's, for one call (some 30 us to make
+// and give back, which a million rows outweigh; without one the work stays on the
+// caller's).  fork: its work follows what st holds now; join: st's next work
+// follows its own.  A Joined in the scope of the buffers joins before they are
+// given back, also when the call ends early.
+constexpr int64_t SIDE_MIN = 1 << 20;
+struct SideStream {
+    cudaStream_t st, s = nullptr;
+    cudaEvent_t ev = nullptr;
+    bool on = false, forked = false;
+    explicit SideStream(cudaStream_t main) : st(main) {}
+    void open() {
+        on = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess &&
+             cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) == cudaSuccess;
+        if (!on) cudaGetLastError();
+    }
+    cudaError_t fork() {
+        const cudaError_t e = cudaEventRecord(ev, st);
+        if (e != cudaSuccess) return e;
+        forked = true;
+        return cudaStreamWaitEvent(s, ev, 0);
+    }
+    cudaError_t join() {
+        if (!forked) return cudaSuccess;
+        forked = false;
+        const cudaError_t e = cudaEventRecord(ev, s);
+        return e == cudaSuccess ? cudaStreamWaitEvent(st, ev, 0) : e;
+    }
+    ~SideStream() {
+        if (ev) cudaEventDestroy(ev);
+        if (s) cudaStreamDestroy(s);
+    }
+    SideStream(const SideStream &) = delete;
+    SideStream &operator=(const SideStream &) = delete;
+};
+struct Joined {
+    SideStream &side;
+    ~Joined() { side.join(); }
+};
+
 geek_status refine_dense(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx, int64_t n, int d, double *centres,
                          int64_t k, int passes, int precision, int32_t *labels, geek_assign_stats *stats,
                          cudaStream_t st) {
+    // The rows' conversion serves every pass.  With many rows it runs beside the
+    // first centre update, on a second stream.
+    TcX xc;
+    const bool tc = (precision == GEEK_PREC_BF16 || precision == GEEK_PREC_BF16X3) && d <= 128;
+    Scratch xs(ctx, st);
+    SideStream side(st);
+    if (passes > 0 && k > 0 && n >= SIDE_MIN) side.open();
+    if (passes > 0 && k > 0 && n > 0 && tc) GK_TRY(tc_x_alloc(ctx, xs, n, d, precision == GEEK_PREC_BF16X3, &xc));
     for (int pass = 0; pass < passes && n > 0 && k > 0; pass++) {
         Scratch ps(ctx, st);
+        Joined joined{side};
         uint64_t *key;
         uint32_t *ids;
         unsigned long long *cnt;
@@ -1694,15 +1743,19 @@ geek_status refine_dense(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ld
             k_ul_starts<<<(unsigned)std::min<int64_t>(most, (int64_t)ctx->num_sms * 8), 256, 0, st>>>(U);
             GK_COUNT();
             k_ul_deltas<<<gs, 256, 0, st>>>(U);
+            if (side.on) GK_CUDA(ctx, side.fork());
             GK_COUNT();
             k_ul_chain<<<(unsigned)std::min<int64_t>(most, (int64_t)ctx->num_sms * 16), 32, 0, st>>>(U);
             GK_LAUNCH(ctx);
         }
+        const cudaStream_t us = side.on ? side.s : st;
         GK_COUNT();
         k_update_centres<<<(unsigned)std::min<int64_t>((k * ((d + 31) / 32) + UC_P - 1) / UC_P, (int64_t)ctx->num_sms),
-                           UC_T, UC_SMEM, st>>>(x, ldx, d, k, off, cnt, (const int32_t *)ids, order, n_large, next,
+                           UC_T, UC_SMEM, us>>>(x, ldx, d, k, off, cnt, (const int32_t *)ids, order, n_large, next,
                                                 centres, uc_err);
         GK_LAUNCH(ctx);
+        if (tc && pass == 0) GK_TRY(tc_x_convert(ctx, x, ldx, n, d, precision == GEEK_PREC_BF16X3, xc, us));
+        GK_CUDA(ctx, side.join());
         tu.stop();
         int h_bad = 0, h_uc = 0;
         GK_CUDA(ctx, cudaMemcpyAsync(&h_bad, bad, sizeof h_bad, cudaMemcpyDeviceToHost, st));
@@ -1713,14 +1766,14 @@ geek_status refine_dense(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ld
         EvTimer ta(ctx, "refine.assign", st);
         // the statistics describe the last pass only
         GK_TRY(assign_dense_centres(ctx, ps, x, ldx, n, d, centres, k, precision, labels,
-                                    pass + 1 == passes ? stats : nullptr, st));
+                                    pass + 1 == passes ? stats : nullptr, st, tc ? &xc : nullptr));
     }
     return GEEK_OK;
 }
 
 geek_status assign_dense_centres(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx, int64_t n, int d,
                                  const double *centres, int64_t k, int precision, int32_t *labels,
-                                 geek_assign_stats *stats, cudaStream_t st) {
+                                 geek_assign_stats *stats, cudaStream_t st, const TcX *xc) {
     if (stats) *stats = geek_assign_stats{0.0, 0.0, k, 0};
     if (n == 0) return GEEK_OK;
     if (k == 0) {
@@ -1764,6 +1817,7 @@ geek_status assign_dense_centres(geek_ctx *ctx, Scratch &scr, const float *x, in
         ~Free() { tc_plan_free(p); }
     } plan_free{&plan};
     if (precision == GEEK_PREC_BF16 || precision == GEEK_PREC_BF16X3) {
+        plan.x_done = xc;
         GK_TRY(assign_tc_bf16(ctx, scr, x, ldx, n, d, centres, k, precision == GEEK_PREC_BF16X3, labels, flag_rows,
                               flag_m, n_flag, &plan, st));
     } else {

@@ -197,6 +197,14 @@ struct TcPlanInst {
 struct TcInst;
 struct TcXPrep;
 struct TcCPrep;
+// One data set's rows in BF16 (or split-BF16 pairs) and their norms, converted
+// once for several assignments of the same rows.
+struct TcX {
+    __nv_bfloat16 *xb = nullptr;
+    float *xnorm = nullptr;
+    TcXPrep *prep = nullptr;  // the conversion's tables
+    int64_t *row_off = nullptr;
+};
 // Buffers, descriptors and the unit list (instance, row tile) of one
 // persistent tcgen05 launch over a set of instances.
 struct TcPlan {
@@ -224,6 +232,7 @@ struct TcPlan {
     CUtensorMap *tmG = nullptr;
     int kg = 0, kw = 0;
     int64_t emit_units = 0;
+    const TcX *x_done = nullptr;  // rows already converted (one instance)
     std::vector<void *> owned;
 };
 // Flagged rows grouped by instance in units of up to 128: unit u holds the
@@ -261,6 +270,9 @@ int tc_tile_candidates(const int **tiles);
 geek_status assign_tc_bf16(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx, int64_t n, int d,
                            const double *centres, int64_t k, int split, int32_t *labels, int32_t *flag_rows,
                            float *flag_m, unsigned long long *n_flag, TcPlan *P, cudaStream_t st);
+geek_status tc_x_alloc(geek_ctx *ctx, Scratch &scr, int64_t n, int d, int split, TcX *X);
+geek_status tc_x_convert(geek_ctx *ctx, const float *x, int64_t ldx, int64_t n, int d, int split, const TcX &X,
+                         cudaStream_t st);
 
 // assign.cu
 // Centre preparation of one instance (device copies): FP32 copy and |c|^2
@@ -343,7 +355,7 @@ geek_status decide_flags(geek_ctx *ctx, const TcPlan &P, const RInst *R, const i
                          const DecideBufs &B, cudaStream_t st, const FlagOrder *order = nullptr);
 geek_status assign_dense_centres(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx,
                                  int64_t n, int d, const double *centres, int64_t k, int precision,
-                                 int32_t *labels, geek_assign_stats *stats, cudaStream_t st);
+                                 int32_t *labels, geek_assign_stats *stats, cudaStream_t st, const TcX *xc = nullptr);
 geek_status cluster_radius(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx, int64_t n, int d,
                            const double *centres, int64_t k, const int32_t *labels, double *radius, cudaStream_t st);
 // Sect. 5's extra passes: per pass, centre j <- FP64 mean of the objects

@@ -990,10 +990,12 @@ geek_status tc_plan_build(geek_ctx *ctx, Scratch *scr, const std::vector<TcPlanI
     __nv_bfloat16 *xb, *cb, *cbx;
     float *cn;
     unsigned *cmax_bits;
-    GK_TRY(plan_alloc(ctx, scr, own, &xb, (size_t)std::max<int64_t>(xb_total, 1)));
+    if (P->x_done) xb = P->x_done->xb;
+    else GK_TRY(plan_alloc(ctx, scr, own, &xb, (size_t)std::max<int64_t>(xb_total, 1)));
     GK_TRY(plan_alloc(ctx, scr, own, &cb, (size_t)std::max<int64_t>(cb_total, 1)));
     GK_TRY(plan_alloc(ctx, scr, own, &cbx, (size_t)std::max<int64_t>(im.kpad_off[count] * 16, 1)));
-    GK_TRY(plan_alloc(ctx, scr, own, &P->xnorm, (size_t)std::max<int64_t>(P->N_total, 1)));
+    if (P->x_done) P->xnorm = P->x_done->xnorm;
+    else GK_TRY(plan_alloc(ctx, scr, own, &P->xnorm, (size_t)std::max<int64_t>(P->N_total, 1)));
     GK_TRY(plan_alloc(ctx, scr, own, &cn, (size_t)std::max<int64_t>(P->kpad_total, 1)));
     GK_TRY(plan_alloc(ctx, scr, own, &cmax_bits, (size_t)count));
     GK_TRY(plan_alloc(ctx, scr, own, &P->row_off, (size_t)count + 1));
@@ -1064,7 +1066,7 @@ geek_status tc_plan_convert(geek_ctx *ctx, const TcPlan &P, cudaStream_t st) {
     const int count = P.count;
     GK_CUDA(ctx, cudaMemsetAsync(P.err, 0, sizeof(int), st));
     GK_CUDA(ctx, cudaMemsetAsync(P.cmax_bits, 0, sizeof(unsigned) * count, st));
-    if (P.N_total > 0) {
+    if (P.N_total > 0 && !P.x_done) {
         GK_COUNT();
         k_x_to_bf16<<<grid_for(P.N_total * 32, 256, ctx->num_sms), 256, 0, st>>>(P.xprep, P.row_off, count,
                                                                                  P.N_total, P.xnorm);
@@ -1246,6 +1248,27 @@ void tc_plan_free(TcPlan *P) {
     P->tune_cap = 0;
     delete P->impl;
     P->impl = nullptr;
+}
+
+geek_status tc_x_alloc(geek_ctx *ctx, Scratch &scr, int64_t n, int d, int split, TcX *X) {
+    const int Kp = d <= 64 ? 64 : 128;
+    GK_TRY(scr.alloc(&X->xb, (size_t)n * Kp * (split ? 2 : 1)));
+    GK_TRY(scr.alloc(&X->xnorm, (size_t)n));
+    GK_TRY(scr.alloc(&X->prep, 1));
+    return scr.alloc(&X->row_off, 2);
+}
+
+geek_status tc_x_convert(geek_ctx *ctx, const float *x, int64_t ldx, int64_t n, int d, int split, const TcX &X,
+                         cudaStream_t st) {
+    const TcXPrep p{x, ldx, d, d <= 64 ? 64 : 128, split, X.xb};
+    const int64_t off[2] = {0, n};
+    // pageable: read on return
+    GK_CUDA(ctx, cudaMemcpyAsync(X.prep, &p, sizeof p, cudaMemcpyHostToDevice, st));
+    GK_CUDA(ctx, cudaMemcpyAsync(X.row_off, off, sizeof off, cudaMemcpyHostToDevice, st));
+    GK_COUNT();
+    k_x_to_bf16<<<grid_for(n * 32, 256, ctx->num_sms), 256, 0, st>>>(X.prep, X.row_off, 1, n, X.xnorm);
+    GK_LAUNCH(ctx);
+    return GEEK_OK;
 }
 
 // BF16 (split = 0) or split-BF16 (split = 1) tcgen05 pass of one data set:
