@@ -67,6 +67,7 @@ __global__ void __launch_bounds__(PJ_MAXT, 2) k_project_fp32(ProjArgs A, const P
     const int SR = TR + A.FPAD;  // rows per stage
     float *st0 = sm, *st1 = sm + (size_t)SR * PJ_KC;
     __shared__ int smin[512], smax[512];  // F <= 512 checked on the host
+    __shared__ float xsq[512];            // |x|^2 of the tile's rows, at most 512
     const int t = threadIdx.x;
     const int nthr = A.FG * A.RG;
     const int fg = t % A.FG, rg = t / A.FG;
@@ -77,10 +78,8 @@ __global__ void __launch_bounds__(PJ_MAXT, 2) k_project_fp32(ProjArgs A, const P
         smax[f] = INT32_MIN;
     }
     float acc[PJ_RPT][PJ_FPT];
-    float xsq[PJ_RPT];
 #pragma unroll
     for (int r = 0; r < PJ_RPT; r++) {
-        xsq[r] = 0.f;
 #pragma unroll
         for (int c = 0; c < PJ_FPT; c++) acc[r][c] = 0.f;
     }
@@ -131,6 +130,18 @@ __global__ void __launch_bounds__(PJ_MAXT, 2) k_project_fp32(ProjArgs A, const P
             asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
         __syncthreads();
+        // The norms, each row's by one thread (the FG threads that share a row
+        // would each spend an eighth more FMAs on it); lanes start at different
+        // pieces, so that eight consecutive rows fall in different banks.
+        for (int r = t; r < TR; r += blockDim.x) {
+            float s = ci ? xsq[r] : 0.f;
+#pragma unroll
+            for (int j = 0; j < 8; j++) {
+                const float4 v = *reinterpret_cast<const float4 *>(cur + r * PJ_KC + 4 * ((j + r) & 7));
+                s = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, s))));
+            }
+            xsq[r] = s;
+        }
         if (active) {
             const float *xb = cur, *ab = cur + (size_t)TR * PJ_KC;
             const int kmax = min(PJ_KC, A.d - ci * PJ_KC);
@@ -140,7 +151,6 @@ __global__ void __launch_bounds__(PJ_MAXT, 2) k_project_fp32(ProjArgs A, const P
                 for (int q = 0; q < PJ_RPT; q++) {
                     const int r = rg * PJ_RPT + q;
                     xv[q] = *reinterpret_cast<const float4 *>(xb + r * PJ_KC + 4 * (jb ^ ((r >> 3) & 7)));
-                    xsq[q] = fmaf(xv[q].x, xv[q].x, fmaf(xv[q].y, xv[q].y, fmaf(xv[q].z, xv[q].z, fmaf(xv[q].w, xv[q].w, xsq[q]))));
                 }
 #pragma unroll
                 for (int c = 0; c < PJ_FPT; c++) {
@@ -173,7 +183,7 @@ __global__ void __launch_bounds__(PJ_MAXT, 2) k_project_fp32(ProjArgs A, const P
         for (int r = 0; r < PJ_RPT; r++) {
             const int64_t row = row0 + rg * PJ_RPT + r;
             if (row >= A.n) continue;
-            const float xn = sqrtf(xsq[r]) * 1.0001f;
+            const float xn = sqrtf(xsq[rg * PJ_RPT + r]) * 1.0001f;
             int32_t out[PJ_FPT];
 #pragma unroll
             for (int c = 0; c < PJ_FPT; c++) {
