@@ -168,67 +168,74 @@ __global__ void __launch_bounds__(PJ_MAXT, 2) k_project_fp32(ProjArgs A, const P
         }
         __syncthreads();  // the next stage() overwrites this buffer
     }
+    for (int r = t; r < TR; r += blockDim.x) xsq[r] = sqrtf(xsq[r]) * 1.0001f;  // its own sums
     __syncthreads();
     unsigned nfl = 0;
     uint64_t flagmask = 0;  // bit r*8 + c: element (row r, function c) is uncertain
     if (active) {
         const float gam = (float)A.d * 6.0e-8f;  // >= gamma_d(fp32) + d 2^-53, norms' own error
-        int lmin[PJ_FPT], lmax[PJ_FPT];
+        // four functions at a time: their constants are read once for eight rows
 #pragma unroll
-        for (int c = 0; c < PJ_FPT; c++) {
-            lmin[c] = INT32_MAX;
-            lmax[c] = INT32_MIN;
-        }
+        for (int c0 = 0; c0 < PJ_FPT; c0 += 4) {
+            const int f0 = fg * PJ_FPT + c0;
+            float ga[4], bb[4];
+            int lmin[4], lmax[4];
 #pragma unroll
-        for (int r = 0; r < PJ_RPT; r++) {
-            const int64_t row = row0 + rg * PJ_RPT + r;
-            if (row >= A.n) continue;
-            const float xn = sqrtf(xsq[rg * PJ_RPT + r]) * 1.0001f;
-            int32_t out[PJ_FPT];
+            for (int c = 0; c < 4; c++) {
+                const bool in = f0 + c < A.F;
+                ga[c] = in ? gam * A.anorm[f0 + c] : 0.f;
+                bb[c] = in && !A.srp ? A.b[f0 + c] : 0.f;
+                lmin[c] = INT32_MAX;
+                lmax[c] = INT32_MIN;
+            }
 #pragma unroll
-            for (int c = 0; c < PJ_FPT; c++) {
-                const int f = fg * PJ_FPT + c;
-                out[c] = 0;
-                if (f >= A.F) continue;
-                const float p = acc[r][c];
-                const float E = gam * A.anorm[f] * xn + 1e-30f;
-                int code;
-                bool sure;
-                if (A.srp) {
-                    // s64 in [p - E, p + E]; FP32 subtraction slack 2^-23 |p|
-                    const float Es = E + fabsf(p) * 1.2e-7f;
-                    code = p >= 0.f ? 1 : 0;
-                    sure = (p - Es > 0.f) || (p + Es < 0.f);
-                } else {
-                    const float bb = A.b[f];
-                    const float tt = (p + bb) * A.inv_w;
-                    // window in t-space: model error E/w plus rounding of
-                    // p + b, of * (1/w) and of the comparisons (4 ulps)
-                    const float Et = (E + (fabsf(p) + fabsf(bb) + E) * 2.5e-7f) * A.inv_w + fabsf(tt) * 2.5e-7f;
-                    const float c0 = floorf(tt);
-                    code = fabsf(tt) < 2.0e9f ? (int)c0 : 0;
-                    sure = (tt - Et >= c0) && (tt + Et < c0 + 1.f) && fabsf(tt) < 2.0e9f;
+            for (int r = 0; r < PJ_RPT; r++) {
+                const int64_t row = row0 + rg * PJ_RPT + r;
+                if (row >= A.n) continue;
+                const float xn = xsq[rg * PJ_RPT + r];
+                int32_t out[4];
+#pragma unroll
+                for (int c = 0; c < 4; c++) {
+                    out[c] = 0;
+                    if (f0 + c >= A.F) continue;
+                    const float p = acc[r][c0 + c];
+                    const float E = ga[c] * xn + 1e-30f;
+                    int code;
+                    bool sure;
+                    if (A.srp) {
+                        // s64 in [p - E, p + E]; FP32 subtraction slack 2^-23 |p|
+                        const float Es = E + fabsf(p) * 1.2e-7f;
+                        code = p >= 0.f ? 1 : 0;
+                        sure = (p - Es > 0.f) || (p + Es < 0.f);
+                    } else {
+                        const float tt = (p + bb[c]) * A.inv_w;
+                        // window in t-space: model error E/w plus rounding of
+                        // p + b, of * (1/w) and of the comparisons (4 ulps)
+                        const float Et =
+                            (E + (fabsf(p) + fabsf(bb[c]) + E) * 2.5e-7f) * A.inv_w + fabsf(tt) * 2.5e-7f;
+                        const float c0f = floorf(tt);
+                        code = fabsf(tt) < 2.0e9f ? (int)c0f : 0;
+                        sure = (tt - Et >= c0f) && (tt + Et < c0f + 1.f) && fabsf(tt) < 2.0e9f;
+                    }
+                    out[c] = code;
+                    if (!sure) flagmask |= 1ull << (r * PJ_FPT + c0 + c);
+                    lmin[c] = min(lmin[c], code);
+                    lmax[c] = max(lmax[c], code);
                 }
-                out[c] = code;
-                if (!sure) flagmask |= 1ull << (r * PJ_FPT + c);
-                lmin[c] = min(lmin[c], code);
-                lmax[c] = max(lmax[c], code);
+                int32_t *dst = A.codes + row * A.F + f0;
+                if (f0 + 4 <= A.F && (A.F % 4) == 0) {
+                    *reinterpret_cast<int4 *>(dst) = make_int4(out[0], out[1], out[2], out[3]);
+                } else {
+                    for (int c = 0; c < 4; c++)
+                        if (f0 + c < A.F) dst[c] = out[c];
+                }
             }
-            int32_t *dst = A.codes + row * A.F + fg * PJ_FPT;
-            if (fg * PJ_FPT + PJ_FPT <= A.F && (A.F % 4) == 0) {
-                reinterpret_cast<int4 *>(dst)[0] = make_int4(out[0], out[1], out[2], out[3]);
-                reinterpret_cast<int4 *>(dst)[1] = make_int4(out[4], out[5], out[6], out[7]);
-            } else {
-                for (int c = 0; c < PJ_FPT; c++)
-                    if (fg * PJ_FPT + c < A.F) dst[c] = out[c];
-            }
-        }
 #pragma unroll
-        for (int c = 0; c < PJ_FPT; c++) {
-            const int f = fg * PJ_FPT + c;
-            if (f < A.F && lmin[c] <= lmax[c]) {
-                atomicMin(&smin[f], lmin[c]);
-                atomicMax(&smax[f], lmax[c]);
+            for (int c = 0; c < 4; c++) {
+                if (f0 + c < A.F && lmin[c] <= lmax[c]) {
+                    atomicMin(&smin[f0 + c], lmin[c]);
+                    atomicMax(&smax[f0 + c], lmax[c]);
+                }
             }
         }
         nfl = __popcll(flagmask);
