@@ -202,8 +202,7 @@ struct TcCPrep;
 struct TcX {
     __nv_bfloat16 *xb = nullptr;
     float *xnorm = nullptr;
-    TcXPrep *prep = nullptr;  // the conversion's tables
-    int64_t *row_off = nullptr;
+    TcXPrep *prep = nullptr;  // the conversion's arguments
 };
 // Buffers, descriptors and the unit list (instance, row tile) of one
 // persistent tcgen05 launch over a set of instances.
