@@ -262,7 +262,7 @@ __global__ void k_heavy_masks(int64_t k, const int64_t *__restrict__ coff, const
 // counter array (cleared after use).  Every centre is then scored exactly:
 // J_j = inter / (|A| + |C_j| - inter), compared by cross-multiplication.
 // (The dense path: every centre is scanned per set.  It serves the sets
-// with more items than k_jac_tiled takes;
+// with more items than the tiled kernels take;
 // rows lists them, na_fix >= 0 replaces |A| by a fixed size.)
 __global__ void __launch_bounds__(256) k_assign_jaccard(
     int64_t n, const int64_t *__restrict__ off, const uint32_t *__restrict__ items, int64_t k,
