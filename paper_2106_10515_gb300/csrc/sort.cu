@@ -130,7 +130,10 @@ __global__ void __launch_bounds__(256) k_rs_base_all(uint32_t *__restrict__ coun
 // digit with match-any, the block turns per-warp counts into tile offsets,
 // stages the tile in shared memory in (digit, input order) and writes it out
 // contiguously per digit: coalesced, stable.  Small tiles and 4 blocks per
-// SM: the pass is latency bound, and occupancy pays more than long tiles.
+// SM: the pass is latency bound, and occupancy pays more than long tiles (16
+// tables of 2M elements, 215 us a pass, half of HBM; tiles of 5,120 elements by
+// 512 threads 237, by 1,024 threads 365; the next tile's loads in flight during the
+// writes 222).
 template <bool HI, bool VALS>
 __global__ void __launch_bounds__(RS_THREADS, 4)
     k_rs_onesweep(const uint64_t *__restrict__ lo_in, const uint64_t *__restrict__ hi_in,
@@ -280,7 +283,10 @@ __global__ void __launch_bounds__(RS_THREADS, 4)
 // Segments of at most RB_MAX elements: one block sorts a segment in shared
 // memory, all passes in one launch (each pass of the tiled form is a launch of
 // its own plus the digit totals: 19 launches for 64 bits).  Ranking as in
-// k_rs_onesweep, the tile read back after each pass.
+// k_rs_onesweep, the tile read back after each pass.  RB_MAX is what a thread's
+// registers hold, 10 elements; a pass over it takes some 2 us, where a launch of
+// the tiled form takes 3 to 7 for so few (the 20,000 x 32 pipeline, whose SILK
+// tables are below the line: 1.85 -> 1.78 ms).
 constexpr int RB_THREADS = 512, RB_ITEMS = 10, RB_MAX = RB_THREADS * RB_ITEMS, RB_WARPS = RB_THREADS / 32;
 template <bool HI, bool VALS>
 __global__ void __launch_bounds__(RB_THREADS) k_rs_block(uint64_t *__restrict__ lo, uint64_t *__restrict__ hi,
@@ -777,8 +783,9 @@ __global__ void __launch_bounds__(RS_THREADS) k_i64_tile_apply(const int64_t *__
     for (int e = threadIdx.x; e < cnt; e += RS_THREADS) out[t0 + e] = tv[e];
 }
 
-// the same for up to SCAN_ONE values by one block (one launch instead of three):
-// thread t the values 16 t .. 16 t + 15
+// the same for up to SCAN_ONE values, what a block holds in registers, by one
+// block (one launch instead of three; with the fills of small sorts, the
+// 20,000 x 32 pipeline 1.98 -> 1.85 ms): thread t the values 16 t .. 16 t + 15
 constexpr int SCAN_ONE = 16384;
 __global__ void __launch_bounds__(1024) k_i64_scan_one(const int64_t *__restrict__ in, int64_t *__restrict__ out, int n,
                                                        int64_t *__restrict__ total) {
