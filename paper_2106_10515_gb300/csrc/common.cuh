@@ -139,7 +139,7 @@ struct Scratch {
     std::vector<void *> ptrs;
     // Requests of up to SMALL bytes are cut from slabs: a call makes dozens of
     // them, and an allocation with its release costs 1.6 us of the host's time
-    // (the 20,000 x 64 pipeline made 167 of each).
+    // (the 20,000 x 32 pipeline made 167 of each).
     static constexpr size_t SLAB = 256 << 10, SMALL = 32 << 10;
     char *slab = nullptr;
     size_t left = 0;
