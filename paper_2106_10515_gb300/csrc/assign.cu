@@ -1771,6 +1771,16 @@ geek_status refine_dense(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ld
     return GEEK_OK;
 }
 
+// After decide_flags: the candidates' pass ran to its end, and so did the sort of
+// the flagged rows (its word is read, and cleared, in the same wait).
+static geek_status decide_check(geek_ctx *ctx, const TcPlan &P, cudaStream_t st) {
+    int h_sort = 0;
+    GK_TRY(sort_err_fetch(ctx, &h_sort, st));
+    const geek_status pass = tc_plan_check(ctx, P, st);  // synchronises
+    const geek_status sort = sort_err_eval(ctx, &h_sort, st);
+    return pass != GEEK_OK ? pass : sort;
+}
+
 geek_status assign_dense_centres(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx, int64_t n, int d,
                                  const double *centres, int64_t k, int precision, int32_t *labels,
                                  geek_assign_stats *stats, cudaStream_t st, const TcX *xc) {
@@ -1852,7 +1862,7 @@ geek_status assign_dense_centres(geek_ctx *ctx, Scratch &scr, const float *x, in
             const FlagOrder order{&scr, k, labels};
             GK_TRY(decide_flags(ctx, plan, ri, roff, 1, d, flag_rows, flag_m, n_flag, (int64_t)h_flag, db, st,
                                 h_flag >= 100000 ? &order : nullptr));
-            if (!stats) GK_TRY(tc_plan_check(ctx, plan, st));  // the candidates' pass, too, ran to its end
+            if (!stats) GK_TRY(decide_check(ctx, plan, st));
         }
     }
     if (stats) {
@@ -1875,7 +1885,7 @@ geek_status assign_dense_centres(geek_ctx *ctx, Scratch &scr, const float *x, in
         GK_CUDA(ctx, cudaMemcpyAsync(&h, w, offsetof(Words, cmax_bits), cudaMemcpyDeviceToHost, st));
         if (h_flag) {
             GK_CUDA(ctx, cudaMemcpyAsync(&h_fp64, db.n_flag2, sizeof h_fp64, cudaMemcpyDeviceToHost, st));
-            GK_TRY(tc_plan_check(ctx, plan, st));  // synchronises; the candidates' pass, too, ran to its end
+            GK_TRY(decide_check(ctx, plan, st));  // synchronises
         } else {
             GK_CUDA(ctx, cudaStreamSynchronize(st));
         }

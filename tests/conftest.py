@@ -18,3 +18,12 @@ def orc():
     import oracle
     oracle.build()
     return oracle
+
+
+@pytest.fixture(scope="session")
+def geek():
+    """The binding, its library built (GPU tests)."""
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2106_10515_gb300 import geek as module
+    return module
