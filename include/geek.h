@@ -175,7 +175,8 @@ geek_status geek_ctx_destroy(geek_ctx *ctx);
  *    the call returns GEEK_ERR_TIMEOUT; -1 (default) turns it off.
  *  GEEK_OPT_TEST_FAIL_ALLOC: FOR TESTS.  Value v >= 0 makes the device
  *    allocation after the next v ones fail as if the device were out of memory
- *    (the call returns GEEK_ERR_NOMEM, the countdown then turns itself off);
+ *    (the call returns GEEK_ERR_NOMEM, or goes on with a smaller buffer where
+ *    it can; the countdown then turns itself off);
  *    -1 (default) turns it off.
  * Errors: INVALID (NULL ctx, unknown option, value out of range). */
 enum { GEEK_OPT_WAIT_LIMIT_NS = 1, GEEK_OPT_TEST_STALL_TILE = 2, GEEK_OPT_TEST_FAIL_ALLOC = 3 };
@@ -282,6 +283,10 @@ geek_status silk_seeds_free(silk_seeds *s);
  *    i.e. the label maximises the number of matching attributes.
  *  SETS: central vector = items present in more than half of the members;
  *    label maximises |A n C| / |A u C| (exact rational comparison).
+ * Device memory, DENSE in BF16 or BF16X3: besides the BF16 copies of x and the
+ * centres (2 or 4 bytes per element, d padded to 64 or 128), the decision of
+ * the flagged rows takes a buffer of up to 1 GB (256 to 512 bytes and k / 8
+ * per flagged row), smaller where the device has less room.
  * labels: n int32.  centers (nullable, DENSE only): k x d float64 out.
  * stats (nullable, HOST): filled after the stream has finished the call. */
 geek_status geek_assign(geek_ctx *ctx, const geek_data *data, const geek_buckets *b,
@@ -407,7 +412,8 @@ geek_status geek_assign_centers_noalloc(const float *x, int64_t n, int32_t d, in
  * first time a (d, seed count) class is seen on a context.
  * Results are, instance by instance, exactly those of geek_hash + silk_seed +
  * geek_assign on that instance alone (every precision gives the same,
- * exact labels). */
+ * exact labels).  The plan holds geek_assign's buffer for the flagged rows (up
+ * to 1 GB, sized for every row, smaller where the device has less room). */
 typedef struct geek_batch geek_batch;
 
 /* One dense instance: x (n x d float32, row stride ldx, n >= 0, 1 <= d <= 128),

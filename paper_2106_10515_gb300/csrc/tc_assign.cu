@@ -261,6 +261,7 @@ template <bool SPLIT, bool EMIT>
 __global__ void __launch_bounds__(TC_THREADS, 1) k_assign_tc(const __grid_constant__ TcArgs A) {
     constexpr int A_ST = TC_A_STAGE;
     constexpr int KW = SPLIT ? 2 : 1;  // stored column blocks per k-block
+    if (EMIT && (int64_t)*A.e.n_units <= A.e.u0) return;  // a wave past the flagged rows
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int NA = 1 << A.lg_na;
@@ -919,6 +920,8 @@ namespace {
 template <class T>
 geek_status plan_alloc(geek_ctx *ctx, Scratch *scr, std::vector<void *> &owned, T **p, size_t count) {
     if (scr) return scr->alloc(p, count);
+    if (alloc_injected_failure(ctx))
+        return set_error(ctx, GEEK_ERR_NOMEM, "device allocation of %zu bytes failed (injected)", count * sizeof(T));
     void *q = nullptr;
     cudaError_t e = cudaMalloc(&q, std::max<size_t>(count * sizeof(T), 16));
     if (e != cudaSuccess) {
@@ -1639,10 +1642,12 @@ geek_status tc_decide_candidates(geek_ctx *ctx, const TcPlan &P, const RInst *R,
 }
 
 // Buffers of tc_decide_candidates for at most max_rows flagged rows: a wave
-// holds as many units as fit EMIT_BYTES (gathered rows and masks), at least one
-// per SM.
+// holds as many units as fit EMIT_BYTES (gathered rows and masks), at least one,
+// and as many as the device has room for: with half the units there are twice
+// the waves and the same labels, so a request that fails is halved (down to
+// EMIT_WAVES waves for a batch, whose graph holds a few launches per wave).
 geek_status tc_emit_alloc(geek_ctx *ctx, Scratch *scr, TcPlan *P, int64_t max_rows, cudaStream_t st) {
-    constexpr int64_t EMIT_BYTES = 1ll << 30;
+    constexpr int64_t EMIT_BYTES = 1ll << 30, EMIT_WAVES = 4096;
     int kg = 64;
     int64_t kw = 8;
     for (const TcPlanInst &I : P->desc) {
@@ -1650,16 +1655,29 @@ geek_status tc_emit_alloc(geek_ctx *ctx, Scratch *scr, TcPlan *P, int64_t max_ro
         kg = std::max(kg, (I.split || P->allow_split) ? 2 * Kp : Kp);
         kw = std::max(kw, ceil_div(I.k, TC_N) * (TC_N / 32));
     }
-    const int64_t unit_bytes = TC_M * (2 * (int64_t)kg + 4 * kw + 4);
+    // one block: the tensor map, then per unit rows, masks and limits (all
+    // multiples of 256 bytes)
+    const int64_t row_bytes = TC_M * 2 * (int64_t)kg, mask_bytes = TC_M * 4 * kw, lim_bytes = TC_M * 4;
     const int64_t all = ceil_div(std::min(max_rows, P->N_total), TC_M) + P->count;
-    const int64_t units = std::min(all, std::max<int64_t>(EMIT_BYTES / unit_bytes, ctx->num_sms));
+    int64_t units = std::min(all, std::max<int64_t>(EMIT_BYTES / (row_bytes + mask_bytes + lim_bytes), 1));
+    const int64_t least = scr ? 1 : std::min(units, ceil_div(all, EMIT_WAVES));
+    char *block = nullptr;
+    const std::string msg = ctx->last_error;
+    for (;;) {
+        const geek_status rc = plan_alloc(ctx, scr, P->owned, &block,
+                                          (size_t)(256 + units * (row_bytes + mask_bytes + lim_bytes)));
+        if (rc == GEEK_OK) break;
+        if (rc != GEEK_ERR_NOMEM || units <= least) return rc;
+        units = std::max(least, units / 2);
+        ctx->last_error = msg;  // nothing has failed yet
+    }
     P->kg = kg;
     P->kw = (int)kw;
     P->emit_units = units;
-    GK_TRY(plan_alloc(ctx, scr, P->owned, &P->xg, (size_t)(units * TC_M * kg)));
-    GK_TRY(plan_alloc(ctx, scr, P->owned, &P->emit_lim, (size_t)(units * TC_M)));
-    GK_TRY(plan_alloc(ctx, scr, P->owned, &P->emit_masks, (size_t)(units * TC_M * kw)));
-    GK_TRY(plan_alloc(ctx, scr, P->owned, &P->tmG, 1));
+    P->tmG = (CUtensorMap *)block;
+    P->xg = (__nv_bfloat16 *)(block + 256);
+    P->emit_masks = (uint32_t *)(block + 256 + units * row_bytes);
+    P->emit_lim = (float *)(block + 256 + units * (row_bytes + mask_bytes));
     CUtensorMap tm;
     GK_TRY(encode_bf16_2d(ctx, &tm, P->xg, kg, (uint64_t)(units * TC_M), TC_KB, TC_M));
     GK_CUDA(ctx, cudaMemcpyAsync(P->tmG, &tm, sizeof tm, cudaMemcpyHostToDevice, st));
