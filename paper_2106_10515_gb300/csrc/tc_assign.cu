@@ -1405,6 +1405,16 @@ __device__ __forceinline__ int cand_list(uint32_t m, uint16_t *list) {
     return __shfl_sync(0xffffffffu, inc, 31);
 }
 
+// A row (in label order: 8 rows together) with more candidates than k / part goes
+// to the FP32 scan of every centre.  Data far from the origin (|x| a hundred
+// times the spread in BF16) make every centre a candidate, and a pair then costs
+// 73 ps here (48 per centre of the union of 8 rows) against 9 ps in the scan, or
+// 32 where that leaves the row to the FP64 reference: part = 6 and 4 lie between.
+// Scan tiles are 64 centres wide, so up to 64 candidates stay.
+// 90,000 x 128 in BF16, k = 2,000, all of them candidates: 1.9 ms, 13.1 by direct
+// distances; 600,000 rows in label order 10.9 ms, 57.4 by direct distances.
+__device__ __forceinline__ int cand_most(int64_t k, int part) { return (int)max((int64_t)64, k / part); }
+
 // Rows in the order of their labels (decide_flags with an order): a warp takes 8
 // neighbouring slots, whose candidates are nearly the same, and computes the
 // distances of all 8 to the union (a real distance of a centre that is no
@@ -1445,6 +1455,22 @@ __global__ void __launch_bounds__(256) k_decide_ordered(const RInst *__restrict_
             }
         }
         const int nwords = (int)((I.k + 31) >> 5);
+        int n_union = 0;
+        for (int w = lane; w < nwords; w += 32) {
+            uint32_t m = 0;
+#pragma unroll
+            for (int r = 0; r < 8; r++) m |= r0 + r < cnt ? masks[(s + r) * kw + w] : 0u;
+            n_union += __popc(m);
+        }
+        n_union = __reduce_add_sync(0xffffffffu, n_union);
+        if (n_union > cand_most(I.k, 4)) {
+            const int rows = min(8, cnt - r0);
+            unsigned long long at = 0;
+            if (lane == 0) at = atomicAdd(n_left, (unsigned long long)rows);
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (lane < rows) left[at + lane] = F.grows[F.unit_start[u] + r0 + lane];
+            continue;
+        }
         float b1[2] = {FLT_MAX, FLT_MAX}, b2[2] = {FLT_MAX, FLT_MAX};
         int bj[2] = {0x7FFFFFFF, 0x7FFFFFFF}, total = 0;
         uint32_t own = 0;  // bit r: slot s + r has a candidate
@@ -1533,6 +1559,13 @@ __global__ void __launch_bounds__(256) k_decide_candidates(const RInst *__restri
         for (int q = 0; q < 4; q++) xv[q] = cand_load4(I.x + row * I.ldx, 32 * q + 4 * sub, d, vec);
         const uint32_t *mk = masks + s * kw;
         const int nwords = (int)((I.k + 31) >> 5);
+        int n_cand = 0;
+        for (int w = lane; w < nwords; w += 32) n_cand += __popc(mk[w]);
+        n_cand = __reduce_add_sync(0xffffffffu, n_cand);
+        if (n_cand > cand_most(I.k, 6)) {
+            if (lane == 0) left[atomicAdd(n_left, 1ull)] = (int32_t)g;
+            continue;
+        }
         float b1 = FLT_MAX, b2 = FLT_MAX;  // this group's smallest and second D'
         int bj = 0x7FFFFFFF, total = 0;
         bool bad = false;
