@@ -461,11 +461,25 @@ __global__ void k_scatter_m(const int32_t *__restrict__ rows, const float *__res
 }
 
 // ---- grouping a flag list by instance (device-side, graph friendly) --------
+// A warp adds once per instance among its 32 rows (neighbours in the list nearly
+// always share theirs): 3.2M rows of 16 instances take 1.6 ms per kernel with an
+// atomic per row, all of them on 16 words, and 65 us with one per warp.
+__device__ __forceinline__ int flag_inst(const int32_t *__restrict__ flags, int64_t q, int64_t nf,
+                                         const int64_t *__restrict__ row_off, int count, int32_t &r) {
+    r = q < nf ? flags[q] : 0;
+    return q < nf ? find_inst(row_off, count, r) : -1;
+}
 __global__ void k_flag_count(const int32_t *__restrict__ flags, const unsigned long long *__restrict__ n_flag,
                              const int64_t *__restrict__ row_off, int count, int *__restrict__ cnt) {
     const int64_t nf = (int64_t)*n_flag;
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nf; q += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&cnt[find_inst(row_off, count, flags[q])], 1);
+    const int lane = threadIdx.x & 31;
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q - lane < nf;
+         q += (int64_t)gridDim.x * blockDim.x) {
+        int32_t r;
+        const int i = flag_inst(flags, q, nf, row_off, count, r);
+        const uint32_t peers = __match_any_sync(0xffffffffu, i);
+        if (i >= 0 && lane == __ffs(peers) - 1) atomicAdd(&cnt[i], __popc(peers));
+    }
 }
 
 // one block: the rows (seg_off) and 128-row units (unit_off) before each
@@ -528,9 +542,17 @@ __global__ void k_flag_scatter(const int32_t *__restrict__ flags, const unsigned
                                const int64_t *__restrict__ row_off, int count, int64_t *__restrict__ cursor,
                                int32_t *__restrict__ grows) {
     const int64_t nf = (int64_t)*n_flag;
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nf; q += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t r = flags[q];
-        grows[atomicAdd((unsigned long long *)&cursor[find_inst(row_off, count, r)], 1ull)] = r;
+    const int lane = threadIdx.x & 31;
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q - lane < nf;
+         q += (int64_t)gridDim.x * blockDim.x) {
+        int32_t r;
+        const int i = flag_inst(flags, q, nf, row_off, count, r);
+        const uint32_t peers = __match_any_sync(0xffffffffu, i);
+        const int first = __ffs(peers) - 1;
+        unsigned long long at = 0;
+        if (i >= 0 && lane == first) at = atomicAdd((unsigned long long *)&cursor[i], (unsigned long long)__popc(peers));
+        at = __shfl_sync(0xffffffffu, at, first);
+        if (i >= 0) grows[at + __popc(peers & ((1u << lane) - 1u))] = r;
     }
 }
 
