@@ -58,7 +58,7 @@ __device__ __forceinline__ Best best_merge(Best a, Best b) {
 // FMAs.  Rows are stored coordinate-contiguous with their 16-byte pieces
 // XOR-swizzled by the row, so the 2 rows and the 16 centres a warp reads at
 // once fall into different banks; the centre chunks (64 x 32) arrive by
-// cp.async two chunks ahead in a ring of three.
+// cp.async two chunks ahead in a ring of three (fp32_narrow: in chunks of 16, one ahead).
 // n = 1,000,003, d = 96, k = 2,000: the call takes 11.9 ms, against 14.6 ms with
 // scalar FMAs on transposed tiles, whose fills were 32-way bank conflicts.
 // GATHER = false: blocks walk the row tiles of the one data set A.
@@ -89,16 +89,25 @@ __device__ __forceinline__ void ffma2(unsigned long long &c, unsigned long long 
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
 }
 
-constexpr int AS_ST = 3;                    // stages of the centre ring
-constexpr int AS_CST = AS_TC * AS_KC;       // floats per stage
+// The centre ring: KC coordinates of the 64 centres per stage, ST stages.  Three
+// of 32 where two blocks fit an SM (d <= 160), or where no form lets them (d >
+// 208); between, with more than one block per SM, two of 16, with which two fit:
+// one alone has nothing to do while its rows arrive (1M x 200, k = 50: 1.40 ms,
+// 1.71 with one block; k = 1,000, 300,000 rows: 4.0 ms, 4.7).  With one block per
+// SM anyway the longer ring is the faster one (2,000 x 200, k = 3,000: 0.91, 1.00).
+static bool fp32_narrow(const geek_ctx *ctx, int64_t n, int d) {
+    return d > 160 && d <= 208 && n > (int64_t)ctx->num_sms * AS_TR;
+}
 // shared memory of k_assign_fp32: the row tile, coordinates padded to whole
 // chunks, and the centre ring
-static size_t fp32_smem(int d) {
-    return ((size_t)AS_TR * ((d + AS_KC - 1) / AS_KC * AS_KC) + AS_ST * AS_CST) * sizeof(float);
+static size_t fp32_smem(int d, bool narrow) {
+    const int kc = narrow ? 16 : 32, st = narrow ? 2 : 3;
+    return ((size_t)AS_TR * ((d + kc - 1) / kc * kc) + st * AS_TC * kc) * sizeof(float);
 }
 
-template <bool GATHER>
+template <bool GATHER, int KC, int ST>
 __global__ void __launch_bounds__(256, 2) k_assign_fp32(FArgs A, GatherUnits U) {
+    constexpr int CST = AS_TC * KC, PC = KC / 4;  // floats per stage, 16-byte pieces per chunk and centre
     extern __shared__ __align__(16) float sm[];
     __shared__ int64_t s_rows[AS_TR];
     const int t = threadIdx.x, cg = t & 15, rg = t >> 4;
@@ -125,15 +134,20 @@ __global__ void __launch_bounds__(256, 2) k_assign_fp32(FArgs A, GatherUnits U) 
         }
         const int d = A.d;
         const int64_t k = A.k;
-        const int nch = (d + AS_KC - 1) / AS_KC;   // 32-coordinate chunks
-        const int dp = nch * AS_KC, dp16 = 16 * dp;
+        const int nch = (d + KC - 1) / KC;         // chunks of KC coordinates
+        const int dp = nch * KC, dp16 = 16 * dp;
         float *xs = sm;                            // [AS_TR][dp], pieces swizzled
-        float *cs = sm + (size_t)AS_TR * dp;       // [AS_ST][AS_TC][AS_KC], pieces swizzled
+        float *cs = sm + (size_t)AS_TR * dp;       // [ST][AS_TC][KC], pieces swizzled
+        // rows of an odd number of 64-byte halves fall into different banks by themselves
+        const int xm = (dp & 16) ? 0 : 7;
         const bool xvec = ((A.ldx & 3) == 0) && ((d & 3) == 0) && (((uintptr_t)A.x & 15) == 0);
         const bool cvec = ((d & 3) == 0) && (((uintptr_t)A.c32 & 15) == 0);
         const int ntile = (int)((k + AS_TC - 1) / AS_TC);
         // 16-byte piece p of row r at position p ^ (r & 7) within each group of
-        // eight pieces; zeros outside the data
+        // eight pieces (of four in a 16-coordinate centre chunk, where two centres
+        // span the banks: p ^ (c / 2 & 3)); zeros outside the data.  Rows without
+        // 16-byte alignment arrive as asynchronously, by 4-byte copies (1M x 150, k
+        // = 50: 1.14 ms, 1.29 with loads and stores).
         auto put = [&](float *dst, const float *src, int nv, bool vec) {
             if (vec) {
                 asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(
@@ -142,25 +156,30 @@ __global__ void __launch_bounds__(256, 2) k_assign_fp32(FArgs A, GatherUnits U) 
                              : "memory");
             } else {
 #pragma unroll
-                for (int q = 0; q < 4; q++) dst[q] = q < nv ? src[q] : 0.f;
+                for (int q = 0; q < 4; q++)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                                     (uint32_t)__cvta_generic_to_shared(dst + q)),
+                                 "l"(q < nv ? src + q : A.c32), "r"(q < nv ? 4 : 0)
+                                 : "memory");
             }
         };
+        auto centre_piece = [](int c, int p) { return KC == 32 ? p ^ (c & 7) : p ^ ((c >> 1) & 3); };
         // the next chunk (tile f_t, chunk f_c) into ring slot f_s; counters instead
         // of divisions of a chunk number, which cost as much as the products
         int f_t = 0, f_c = 0, f_s = 0;
         auto stage = [&]() {
             if (f_t < ntile) {
-                const int k0 = f_c * AS_KC;
-                float *buf = cs + f_s * AS_CST;
+                const int k0 = f_c * KC;
+                float *buf = cs + f_s * CST;
 #pragma unroll
-                for (int u = 0; u < AS_CST / 4 / 256; u++) {
-                    const int e = t + 256 * u, c = e >> 3, p = e & 7;
+                for (int u = 0; u < CST / 4 / 256; u++) {
+                    const int e = t + 256 * u, c = e / PC, p = e % PC;
                     const int64_t j = (int64_t)f_t * AS_TC + c;
-                    put(buf + c * AS_KC + 4 * (p ^ (c & 7)), A.c32 + j * d + k0 + 4 * p,
+                    put(buf + c * KC + 4 * centre_piece(c, p), A.c32 + j * d + k0 + 4 * p,
                         j < k ? min(4, d - k0 - 4 * p) : 0, cvec);
                 }
                 if (++f_c == nch) f_c = 0, f_t++;
-                if (++f_s == AS_ST) f_s = 0;
+                if (++f_s == ST) f_s = 0;
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
@@ -168,17 +187,17 @@ __global__ void __launch_bounds__(256, 2) k_assign_fp32(FArgs A, GatherUnits U) 
         for (int e = t; e < AS_TR * (dp >> 2); e += 256) {
             const int r = e / (dp >> 2), p = e % (dp >> 2);
             const int64_t row = r < nrows ? (GATHER ? s_rows[r] : row0 + r) : 0;
-            put(xs + r * dp + 4 * (p ^ (r & 7)), A.x + row * A.ldx + 4 * p, r < nrows ? min(4, d - 4 * p) : 0, xvec);
+            put(xs + r * dp + 4 * (p ^ (r & xm)), A.x + row * A.ldx + 4 * p, r < nrows ? min(4, d - 4 * p) : 0, xvec);
         }
-        stage();
-        stage();
+#pragma unroll
+        for (int u = 0; u < ST - 1; u++) stage();
         Best B[AS_RPT];
 #pragma unroll
         for (int r = 0; r < AS_RPT; r++) B[r] = Best{FLT_MAX, FLT_MAX, 0x7FFFFFFF};
         unsigned long long acc[AS_RPT][AS_CPT];
         int ch = 0, slot = 0;
         for (int tile = 0; tile < ntile;) {
-            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            asm volatile("cp.async.wait_group %0;" ::"n"(ST - 2) : "memory");
             __syncthreads();  // this chunk has landed; everyone is done with the last one's slot
             stage();
             if (ch == 0) {
@@ -187,18 +206,18 @@ __global__ void __launch_bounds__(256, 2) k_assign_fp32(FArgs A, GatherUnits U) 
 #pragma unroll
                     for (int c = 0; c < AS_CPT; c++) acc[r][c] = 0ull;
             }
-            const float *buf = cs + slot * AS_CST + cg * AS_KC, *xb = xs + rg * dp + ch * AS_KC;
-            if (++slot == AS_ST) slot = 0;
-            const int np = min(AS_KC, d - ch * AS_KC + 3) >> 2;  // pieces holding data
+            const float *buf = cs + slot * CST + cg * KC, *xb = xs + rg * dp;
+            if (++slot == ST) slot = 0;
+            const int np = min(KC, d - ch * KC + 3) >> 2;  // pieces holding data
 #pragma unroll 1
             for (int p = 0; p < np; p++) {
                 ulonglong2 cv[AS_CPT];
 #pragma unroll
-                for (int c = 0; c < AS_CPT; c++)  // (cg + 16 c) & 7 == cg & 7
-                    cv[c] = *reinterpret_cast<const ulonglong2 *>(buf + 16 * c * AS_KC + 4 * (p ^ (cg & 7)));
+                for (int c = 0; c < AS_CPT; c++)  // centre_piece(cg + 16 c, p) is centre_piece(cg, p)
+                    cv[c] = *reinterpret_cast<const ulonglong2 *>(buf + 16 * c * KC + 4 * centre_piece(cg, p));
 #pragma unroll
                 for (int r = 0; r < AS_RPT; r++) {
-                    const ulonglong2 xv = *reinterpret_cast<const ulonglong2 *>(xb + r * dp16 + 4 * (p ^ (rg & 7)));
+                    const ulonglong2 xv = *reinterpret_cast<const ulonglong2 *>(xb + r * dp16 + 4 * ((ch * PC + p) ^ (rg & xm)));
 #pragma unroll
                     for (int c = 0; c < AS_CPT; c++) {
                         ffma2(acc[r][c], xv.x, cv[c].x);
@@ -242,7 +261,7 @@ __global__ void __launch_bounds__(256, 2) k_assign_fp32(FArgs A, GatherUnits U) 
         for (int r = 0; r < AS_RPT; r++) {
             xs2[r] = 0.f;
             for (int p = cg; p < (dp >> 2); p += 16) {
-                const float4 v = *reinterpret_cast<const float4 *>(xs + (rg + 16 * r) * dp + 4 * (p ^ (rg & 7)));
+                const float4 v = *reinterpret_cast<const float4 *>(xs + (rg + 16 * r) * dp + 4 * (p ^ (rg & xm)));
                 xs2[r] = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, xs2[r]))));
             }
 #pragma unroll
@@ -1853,14 +1872,16 @@ geek_status assign_dense_centres(geek_ctx *ctx, Scratch &scr, const float *x, in
         GK_TRY(assign_tc_bf16(ctx, scr, x, ldx, n, d, centres, k, precision == GEEK_PREC_BF16X3, labels, flag_rows,
                               flag_m, n_flag, &plan, st));
     } else {
-        const size_t smem = fp32_smem(d);
-        GK_CUDA(ctx, cudaFuncSetAttribute(k_assign_fp32<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)fp32_smem(AS_MAXD)));
+        const bool narrow = fp32_narrow(ctx, n, d);
+        const size_t smem = fp32_smem(d, narrow);
+        auto *const kernel = narrow ? k_assign_fp32<false, 16, 2> : k_assign_fp32<false, 32, 3>;
+        GK_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)fp32_smem(AS_MAXD, false)));
         EvTimer tk(ctx, "kernel.assign_fp32", st);
         tk.work = 2.0 * (double)n * (double)k * (double)d;
         FArgs A{x, ldx, n, d, c32, cn, k, &w->cmax_bits, labels, flag_rows, flag_m, n_flag, ceil_div(n, AS_TR)};
         GK_COUNT();
-        k_assign_fp32<false><<<(unsigned)A.ntiles, 256, smem, st>>>(A, GatherUnits{});
+        kernel<<<(unsigned)A.ntiles, 256, smem, st>>>(A, GatherUnits{});
         GK_LAUNCH(ctx);
     }
     unsigned long long h_flag = 0, h_fp64 = 0;
@@ -2100,8 +2121,8 @@ geek_status decide_flags(geek_ctx *ctx, const TcPlan &P, const RInst *R, const i
     GK_TRY(tc_decide_candidates(ctx, P, R, F, B.mrow, max_rows, order != nullptr, B.left, B.n_left, st));
     GK_TRY(group_flags(ctx, row_off, count, B.left, B.n_left, B, st));
     const size_t smem = (size_t)dmax * AS_TR * sizeof(float) + (size_t)AS_KC * AS_TC * sizeof(float);
-    GK_CUDA(ctx, cudaFuncSetAttribute(k_assign_fp32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)fp32_smem(AS_MAXD)));
+    auto *const scan = k_assign_fp32<true, 32, 3>;  // d <= 128
+    GK_CUDA(ctx, cudaFuncSetAttribute(scan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fp32_smem(AS_MAXD, false)));
     FArgs A{};
     A.flag_rows = B.flags2;
     A.flag_m = B.flags2_m;
@@ -2109,7 +2130,7 @@ geek_status decide_flags(geek_ctx *ctx, const TcPlan &P, const RInst *R, const i
     const GatherUnits U{R, F};
     EvTimer t32(ctx, "kernel.assign_refine32", st);
     GK_COUNT();
-    k_assign_fp32<true><<<ctx->num_sms * 2, 256, fp32_smem(dmax), st>>>(A, U);
+    scan<<<ctx->num_sms * 2, 256, fp32_smem(dmax, false), st>>>(A, U);
     GK_LAUNCH(ctx);
     t32.stop();
     // the rows still uncertain, grouped by instance again, go to the tiled
