@@ -390,16 +390,23 @@ __device__ __forceinline__ bool same_prefix(uint64_t l0, uint64_t h0, uint64_t l
 }
 
 // twins[w] += the samples of every segment whose prefix above bit0 - 8 w another
-// sample has (block per segment and w; pseudo-random positions, so that any order
-// of the objects is sampled alike)
+// sample has, most[w] = the most samples of one prefix (block per segment and w;
+// pseudo-random positions, so that any order of the objects is sampled alike; the
+// multipliers are those of Knuth's multiplicative hash, the MurmurHash3 finalizer,
+// degski's 64-bit mixer and SplitMix64's increment)
 __global__ void __launch_bounds__(1024) k_rs_twins(const uint64_t *__restrict__ lo, const uint64_t *__restrict__ hi,
-                                                   int64_t m, int bit0, unsigned long long *__restrict__ twins) {
+                                                   int64_t m, int bit0, unsigned long long *__restrict__ twins,
+                                                   unsigned long long *__restrict__ most) {
     extern __shared__ unsigned long long slot[];
+    uint32_t *const more = reinterpret_cast<uint32_t *>(slot + TW_SLOTS);  // samples after a slot's first
     const int64_t so = (int64_t)blockIdx.x * m;
     bit0 -= 8 * blockIdx.y;
-    for (int e = threadIdx.x; e < TW_SLOTS; e += 1024) slot[e] = ~0ull;
+    for (int e = threadIdx.x; e < TW_SLOTS; e += 1024) {
+        slot[e] = ~0ull;
+        more[e] = 0;
+    }
     __syncthreads();
-    unsigned found = 0;
+    unsigned found = 0, same = 0;
     for (int e = threadIdx.x; e < TW_SAMPLES; e += 1024) {
         // one position in each of TW_SAMPLES equal stretches
         uint32_t z = (uint32_t)e * 2654435761u + blockIdx.x * 0x9E3779B9u;
@@ -417,13 +424,18 @@ __global__ void __launch_bounds__(1024) k_rs_twins(const uint64_t *__restrict__ 
             if (old == ~0ull) break;
             if (old == q) {
                 found++;
+                same = max(same, atomicAdd(&more[s], 1u) + 2u);
                 break;
             }
             s = (s + 1) & (TW_SLOTS - 1);
         }
     }
-    const unsigned w = __reduce_add_sync(0xffffffffu, found);
-    if ((threadIdx.x & 31) == 0 && w) atomicAdd(&twins[blockIdx.y], (unsigned long long)w);
+    found = __reduce_add_sync(0xffffffffu, found);
+    same = __reduce_max_sync(0xffffffffu, same);
+    if ((threadIdx.x & 31) == 0 && found) {
+        atomicAdd(&twins[blockIdx.y], (unsigned long long)found);
+        atomicMax(&most[blockIdx.y], (unsigned long long)same);
+    }
 }
 
 // Runs of equal prefixes of 2 to FX_RUN elements into the order of the whole
@@ -988,22 +1000,31 @@ geek_status sort_ids(geek_ctx *ctx, Scratch &scr, int S, int64_t m, uint64_t **k
     if (nbits <= 64 || widths < 1 || S * m < (int64_t)8 << 20 || m < 4 * TW_SAMPLES)
         return radix_sort_segments(ctx, scr, S, m, key_lo, key_hi, ids, nbits, st, 0, true);
     int bit0 = (nbits - 8 * np0) & ~7;  // no digit across the words
-    unsigned long long *cnt, twins[TW_WIDTHS];  // twins, then the listed runs
-    GK_TRY(scr.alloc(&cnt, TW_WIDTHS + 1));
-    GK_CUDA(ctx, cudaMemsetAsync(cnt, 0, (TW_WIDTHS + 1) * sizeof *cnt, st));
-    const size_t tw_smem = TW_SLOTS * sizeof(unsigned long long);
+    unsigned long long *cnt, h[2 * TW_WIDTHS];  // twins and most, then the listed runs
+    GK_TRY(scr.alloc(&cnt, 2 * TW_WIDTHS + 1));
+    GK_CUDA(ctx, cudaMemsetAsync(cnt, 0, (2 * TW_WIDTHS + 1) * sizeof *cnt, st));
+    unsigned long long *const n_list = cnt + 2 * TW_WIDTHS;
+    const size_t tw_smem = TW_SLOTS * (sizeof(unsigned long long) + sizeof(uint32_t));
     GK_CUDA(ctx, cudaFuncSetAttribute(k_rs_twins, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tw_smem));
     GK_COUNT();
-    k_rs_twins<<<dim3(S, widths), 1024, tw_smem, st>>>(*key_lo, *key_hi, m, bit0, cnt);
+    k_rs_twins<<<dim3(S, widths), 1024, tw_smem, st>>>(*key_lo, *key_hi, m, bit0, cnt, cnt + TW_WIDTHS);
     GK_LAUNCH(ctx);
-    GK_CUDA(ctx, cudaMemcpyAsync(twins, cnt, sizeof *cnt * widths, cudaMemcpyDeviceToHost, st));
+    GK_CUDA(ctx, cudaMemcpyAsync(h, cnt, sizeof h, cudaMemcpyDeviceToHost, st));
     GK_CUDA(ctx, cudaStreamSynchronize(st));
     // An object with c others of its prefix has a twin among the samples with
     // probability c TW_SAMPLES / m.  With a quarter of another on average the
     // settling costs less than the passes it saves, even all in runs of 33 (a
-    // block each); tables of large buckets take all the passes.
+    // block each); tables of large buckets take all the passes.  So do those with
+    // one run of more than S m / 1,024 objects: a block settles an object in 18 ns,
+    // the passes saved take 33 ps of it or more (64 tables of 131,072 objects, one
+    // table a single run: 3.07 ms, 4.22 by settling; 8 tables of 2M with a run of
+    // 2,000 each: 2.75 ms by settling, 4.75).
+    auto settles = [&](int w) {
+        return (double)h[w] * (double)m <= 0.25 * (double)S * TW_SAMPLES * TW_SAMPLES &&
+               (double)h[TW_WIDTHS + w] * 1024 <= (double)S * TW_SAMPLES;
+    };
     int w = 0;
-    while (w < widths && (double)twins[w] * (double)m > 0.25 * (double)S * TW_SAMPLES * TW_SAMPLES) w++;
+    while (w < widths && !settles(w)) w++;
     if (w == widths) return radix_sort_segments(ctx, scr, S, m, key_lo, key_hi, ids, nbits, st, 0, true);
     bit0 -= 8 * w;
     SortSpare sp;
@@ -1013,10 +1034,10 @@ geek_status sort_ids(geek_ctx *ctx, Scratch &scr, int S, int64_t m, uint64_t **k
     const dim3 grid((unsigned)ceil_div(m, RS_TILE), S);
     const size_t smem = 2 * (size_t)(RS_TILE + 1 + FX_RUN) * sizeof(uint64_t);
     GK_COUNT();
-    k_rs_settle<<<grid, RS_THREADS, smem, st>>>(*key_lo, *key_hi, *ids, m, bit0, list, cnt + TW_WIDTHS);
+    k_rs_settle<<<grid, RS_THREADS, smem, st>>>(*key_lo, *key_hi, *ids, m, bit0, list, n_list);
     GK_COUNT();
     k_rs_settle_long<<<2 * ctx->num_sms, RB_THREADS, 0, st>>>(*key_lo, *key_hi, *ids, sp.lo, sp.hi, sp.vals, m, bit0,
-                                                              list, cnt + TW_WIDTHS);
+                                                              list, n_list);
     GK_LAUNCH(ctx);
     return GEEK_OK;
 }
