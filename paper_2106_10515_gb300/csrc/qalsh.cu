@@ -5,13 +5,18 @@
 // The projections are computed with compensated FP32 arithmetic (Dot2, see
 // k_qalsh_dot2): w = hi + lo lies within E of s, the pinned FP64 dot product,
 // for every object.  Only the cuts have to be exact, not the order between
-// them, so each table is sorted by r = w rounded to FP32, as one 64-bit word
+// them, so each table is sorted by r = w - p rounded to FP32, as one 64-bit word
 // (order-preserving bits of r, object id): four 8-byte passes, where sorting
-// the doubles with their ids took eight 12-byte ones.  Rounding is monotone,
-// so the sorted r are the rounded sorted w, and the w at cut position p is
-// within half an ulp of r_(p); the exact value at p is within E of that (order
+// the doubles with their ids took eight 12-byte ones.  p, one FP32 number per
+// table, is the middle of a few objects' values: on data far from the origin w
+// itself has too few bits left for the differences, and the windows below reach
+// across the tables (4M x 64 of unit spread, m = 20, t = 2,000: 8.2 ms at any
+// distance up to 10,000 from the origin, 9.3 at 100,000; rounding w itself 8.4, at
+// 3,000 16.7, at 100,000 53.8).  Rounding is monotone,
+// so the sorted r are the rounded sorted w - p, and the one at a cut position is
+// within half an ulp of its r; the exact value there is within E of that (order
 // statistics move by at most the largest perturbation).  So every object whose
-// r is more than 2E and an ulp below (above) r_(p) is exactly before (after) the
+// r is more than 2E and an ulp below (above) the cut's is exactly before (after) the
 // cut, and only the objects in that window of the sorted order can change
 // sides: their FP64 values are computed and each window (windows that overlap
 // are merged) is re-sorted by (s, id).  Outside the windows the sorted position
@@ -78,10 +83,34 @@ struct QDArgs {
     int64_t ldx, n;
     int d, F, FPAD, FG, RG;
     const float *a;
+    const float *pivot;  // F
     float *hi;           // n x F
     uint64_t *words;     // F x n: (key of the rounded value, object id)
     unsigned *xmax_bits; // max row-norm bound (float bits)
 };
+
+// pivot[f] = the median of a_f . x_i (FP32) over 31 objects spread over the ids (block
+// per table, warp per object); 0 where that is not finite, or so large that a
+// difference of two values could leave FP32's range
+__global__ void __launch_bounds__(31 * 32) k_qalsh_pivot(const float *__restrict__ x, int64_t ldx, int64_t n, int d,
+                                                         const float *__restrict__ a, float *__restrict__ pivot) {
+    __shared__ float v[31];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const float *xr = x + (w * (n - 1) / 30) * ldx, *af = a + (int64_t)blockIdx.x * d;
+    float s = 0.f;
+    for (int j = lane; j < d; j += 32) s = fmaf(af[j], xr[j], s);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) v[w] = s;
+    if (threadIdx.x == 0) pivot[blockIdx.x] = 0.f;
+    __syncthreads();
+    if (threadIdx.x < 31) {
+        const float mine = v[threadIdx.x];
+        int below = 0;
+        for (int q = 0; q < 31; q++) below += v[q] < mine || (v[q] == mine && q < (int)threadIdx.x);
+        if (below == 15 && fabsf(mine) < 1e30f) pivot[blockIdx.x] = mine;
+    }
+}
 
 __device__ __forceinline__ void qd_term(float av, float xv, float &sh, float &sc) {
     const float p = __fmul_rn(av, xv);
@@ -189,9 +218,12 @@ __global__ void __launch_bounds__(QD_T, 2) k_qalsh_dot2(QDArgs A) {
                 const int f = fg * QD_FPT + c;
                 if (f < A.F) {
                     A.hi[row * A.F + f] = sh[r][c];
-                    // + 0: -0 and 0 are equal values, tied by id
-                    const float w = __fadd_rn(__double2float_rn((double)sh[r][c] + (double)sc[r][c]), 0.f);
-                    A.words[(int64_t)f * A.n + row] = ((uint64_t)f32_key(w) << 32) | (uint64_t)row;
+                    // hi - p = s + e exactly (TwoSum); + 0: -0 and 0 are equal
+                    // values, tied by id
+                    const float p = A.pivot[f], s = __fsub_rn(sh[r][c], p), z = __fsub_rn(s, sh[r][c]);
+                    const float e = __fadd_rn(__fsub_rn(sh[r][c], __fsub_rn(s, z)), -__fadd_rn(p, z));
+                    const float v = fabsf(s) < INFINITY ? __fadd_rn(s, __fadd_rn(e, sc[r][c])) : s;
+                    A.words[(int64_t)f * A.n + row] = ((uint64_t)f32_key(__fadd_rn(v, 0.f)) << 32) | (uint64_t)row;
                 }
             }
         }
@@ -203,7 +235,7 @@ __global__ void __launch_bounds__(QD_T, 2) k_qalsh_dot2(QDArgs A) {
 
 // window of cut j (1 .. t-1) of table f: positions whose value r is within 2E
 // and an ulp of the value at floor(j n / t) (2.01 E and 2^-22 |r| cover the
-// roundings of this test, 1e-44 the subnormal ones)
+// roundings of this test and of the subtraction, 1e-44 the subnormal ones)
 __global__ void k_qalsh_windows(int64_t n, int m, int t, const uint64_t *__restrict__ words,
                                 const float *__restrict__ anorm, const unsigned *__restrict__ xmax_bits, double cf,
                                 int64_t *__restrict__ q0, int64_t *__restrict__ q1) {
@@ -296,9 +328,10 @@ geek_status hash_qalsh(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx,
     if (m < 1 || m > 512) return set_error(ctx, GEEK_ERR_UNSUPPORTED, "QALSH: 1 <= m <= 512 tables");
     if (n > 0 && (t < 1 || t > n)) return set_error(ctx, GEEK_ERR_INVALID, "QALSH: need 1 <= t <= n");
     if (n > 0x7FFFFFFFLL) return set_error(ctx, GEEK_ERR_UNSUPPORTED, "QALSH: more than 2^31 objects");
-    float *anorm;
+    float *anorm, *pivot;
     unsigned *xmax;
     GK_TRY(scr.alloc(&anorm, m));
+    GK_TRY(scr.alloc(&pivot, m));
     GK_TRY(scr.alloc(&xmax, 1));
     GK_CUDA(ctx, cudaMemsetAsync(xmax, 0, sizeof(unsigned), st));
     GK_COUNT();
@@ -315,6 +348,9 @@ geek_status hash_qalsh(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx,
     const int64_t tot = n * m;
     uint64_t *words;
     GK_TRY(scr.alloc(&words, tot));
+    GK_COUNT();
+    k_qalsh_pivot<<<m, 31 * 32, 0, st>>>(x, ldx, n, d, a, pivot);
+    GK_LAUNCH(ctx);
     {
         QDArgs Q{};
         Q.x = x; Q.ldx = ldx; Q.n = n; Q.d = d; Q.F = m; Q.a = a;
@@ -323,6 +359,7 @@ geek_status hash_qalsh(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx,
         Q.RG = std::max(1, std::min(64, QD_T / Q.FG));
         Q.hi = (float *)b->codes;  // the handle's codes: FP32 bit patterns of hi
         Q.words = words;
+        Q.pivot = pivot;
         Q.xmax_bits = xmax;
         const int TR = Q.RG * QD_RPT;
         const int threads = (int)ceil_div(Q.FG * Q.RG, 32) * 32;
@@ -344,9 +381,11 @@ geek_status hash_qalsh(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ldx,
         int64_t *q0, *q1;
         GK_TRY(scr.alloc(&q0, nc));
         GK_TRY(scr.alloc(&q1, nc));
-        // Dot2 against the exact value: gamma_d^2 <= 2.2 (2d)(d+1) 2^-48; the
-        // double sum hi + lo and the FP64 reference: (d + 2) 2^-52
-        const double cf = 2.2 * (2.0 * d) * (d + 1.0) * 3.552713678800501e-15 + (d + 2.0) * 2.220446049250313e-16;
+        // Dot2 against the exact value: gamma_d^2 <= 2.2 (2d)(d+1) 2^-48; the sum
+        // of lo and of hi - p's error, both roundings of sums of |a_j x_j|: (2d + 2)
+        // 2^-48; the FP64 reference: (d + 2) 2^-52
+        const double cf = (2.2 * (2.0 * d) * (d + 1.0) + 2.0 * d + 2.0) * 3.552713678800501e-15 +
+                          (d + 2.0) * 2.220446049250313e-16;
         GK_COUNT();
         k_qalsh_windows<<<grid_for(nc, 256, ctx->num_sms), 256, 0, st>>>(n, m, t, words, anorm, xmax, cf, q0, q1);
         GK_LAUNCH(ctx);
