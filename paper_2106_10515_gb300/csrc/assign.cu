@@ -681,34 +681,57 @@ __global__ void __launch_bounds__(256) k_assign_recheck(const RInst *__restrict_
     }
 }
 
-// centre preparation: FP32 copy, |c|^2 (FP64 then rounded), max |c|; a warp per
-// centre, lanes over coordinates (a thread per centre took 26 us for 2,000
-// centres of 96 coordinates: a serial chain of FP64 adds and scattered loads)
-__device__ __forceinline__ void centre_prep(const CInst &I, int64_t j) {
-    const int lane = threadIdx.x & 31, d = I.d;
-    double s = 0.0;
-    for (int t = lane; t < d; t += 32) {
-        const double v = I.c64[j * d + t];
-        I.c32[j * d + t] = (float)v;
-        s += v * v;
+// centre preparation: FP32 copy, |c|^2 (FP64 then rounded), max |c|.  A warp takes
+// C.steps times a few centres, C.lanes lanes over each's coordinates; lane i then
+// ends centre i.  What bounds many centres is FP64, two lanes per cycle and SM: a
+// sum over 32 lanes and a square root for one centre cost as much as 300 and 600
+// of its products (1M x 32: 185 us, with a warp per centre 1,014; 200,000 x 128: 137
+// us, 277).  (A thread per centre took 26 us for 2,000 of 96 coordinates, now 4.5:
+// scattered loads.)
+template <class Inst>  // inst(e, j): the instance and local index of centre e
+__device__ __forceinline__ void centre_prep(int64_t e0, int64_t ktot, CentreWarp C, Inst inst) {
+    const int lane = threadIdx.x & 31, per = C.per_step();
+    double mine = 0.0;
+    for (int st = 0; st < C.steps; st++) {
+        const int64_t e = e0 + per * st + lane / C.lanes;
+        double s = 0.0;
+        if (e < ktot) {
+            int64_t j;
+            const CInst &I = inst(e, j);
+            const int d = I.d;
+#pragma unroll 4
+            for (int t = lane & (C.lanes - 1); t < d; t += C.lanes) {
+                const double v = I.c64[j * d + t];
+                I.c32[j * d + t] = (float)v;
+                s += v * v;
+            }
+        }
+        for (int o = 1; o < C.lanes; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        s = __shfl_sync(0xffffffffu, s, C.lanes * (lane & (per - 1)));
+        if (lane / per == st) mine = s;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) {
-        I.cn[j] = (float)s;
-        const float nrm = (float)sqrt(s) * (1.f + 1e-6f);
-        atomicMax(I.cmax_bits, __float_as_uint(nrm));  // non-negative floats order as uints
+    unsigned bits = 0;
+    unsigned *most = nullptr;
+    if (lane < C.centres() && e0 + lane < ktot) {
+        int64_t j;
+        const CInst &I = inst(e0 + lane, j);
+        I.cn[j] = (float)mine;
+        bits = __float_as_uint((float)sqrt(mine) * (1.f + 1e-6f));  // non-negative floats order as uints
+        most = I.cmax_bits;
     }
+    max_by_warp(most, bits);
 }
 
 // global centre e of instance find_inst(k_off, e)
 __global__ void k_centre_prep(const CInst *__restrict__ C, const int64_t *__restrict__ k_off, int count,
-                              int64_t ktot) {
+                              int64_t ktot, CentreWarp W) {
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < ktot; e += nw) {
-        const CInst &I = C[find_inst(k_off, count, e)];
-        centre_prep(I, e - I.k_base);
-    }
+    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w * W.centres() < ktot; w += nw)
+        centre_prep(w * W.centres(), ktot, W, [&](int64_t e, int64_t &j) -> const CInst & {
+            const CInst &I = C[find_inst(k_off, count, e)];
+            j = e - I.k_base;
+            return I;
+        });
 }
 
 // one data set: its centres, and the one-instance tables of the kernels that
@@ -717,10 +740,15 @@ struct OneTables {
     RInst r;
     int64_t row_off[2];
 };
-__global__ void k_centre_prep_one(CInst I, int64_t k, OneTables T, OneTables *__restrict__ out) {
+__global__ void k_centre_prep_one(const __grid_constant__ CInst I, int64_t k, CentreWarp W, OneTables T,
+                                  OneTables *__restrict__ out) {
     if (blockIdx.x == 0 && threadIdx.x == 0) *out = T;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; j < k; j += nw) centre_prep(I, j);
+    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w * W.centres() < k; w += nw)
+        centre_prep(w * W.centres(), k, W, [&](int64_t e, int64_t &j) -> const CInst & {
+            j = e;
+            return I;
+        });
 }
 
 // double-float split of the FP64 centres: c = hi + lo with hi = (float)c
@@ -1855,7 +1883,9 @@ geek_status assign_dense_centres(geek_ctx *ctx, Scratch &scr, const float *x, in
         const CInst hc{centres, c32, cn, &w->cmax_bits, d, 0};
         const OneTables one{RInst{x, ldx, d, c32, cn, centres, k, &w->cmax_bits, labels, 0}, {0, n}};
         GK_COUNT();
-        k_centre_prep_one<<<grid_for(k * 32, 128, ctx->num_sms), 128, 0, st>>>(hc, k, one, &w->one);
+        const CentreWarp cw = centre_warp(ctx, k);
+        k_centre_prep_one<<<grid_for(ceil_div(k, cw.centres()) * 32, 128, ctx->num_sms), 128, 0, st>>>(hc, k, cw, one,
+                                                                                                      &w->one);
         GK_LAUNCH(ctx);
     }
     int32_t *flag_rows;
@@ -1956,7 +1986,8 @@ geek_status centre_prep_batch(geek_ctx *ctx, const CInst *C, const int64_t *k_of
                               cudaStream_t st) {
     if (ktot == 0) return GEEK_OK;
     GK_COUNT();
-    k_centre_prep<<<grid_for(ktot * 32, 128, ctx->num_sms), 128, 0, st>>>(C, k_off, count, ktot);
+    const CentreWarp cw = centre_warp(ctx, ktot);
+    k_centre_prep<<<grid_for(ceil_div(ktot, cw.centres()) * 32, 128, ctx->num_sms), 128, 0, st>>>(C, k_off, count, ktot, cw);
     GK_LAUNCH(ctx);
     return GEEK_OK;
 }

@@ -222,6 +222,21 @@ static __device__ __forceinline__ int find_inst(const int64_t *__restrict__ off,
     return lo;
 }
 
+// *p = max(*p, bits) of every lane with a p, one atomic where all have the same
+// (a whole warp calls it)
+static __device__ __forceinline__ void max_by_warp(unsigned *p, unsigned bits) {
+    const unsigned long long a = (unsigned long long)p;
+    const unsigned have = __ballot_sync(0xffffffffu, p != nullptr);
+    if (!have) return;
+    const unsigned long long first = __shfl_sync(0xffffffffu, a, __ffs((int)have) - 1);
+    if (__all_sync(0xffffffffu, !p || a == first)) {
+        bits = __reduce_max_sync(0xffffffffu, p ? bits : 0u);
+        if ((threadIdx.x & 31) == __ffs((int)have) - 1) atomicMax(p, bits);
+    } else if (p) {
+        atomicMax(p, bits);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Internal building blocks (implemented in the .cu files)
 // ---------------------------------------------------------------------------

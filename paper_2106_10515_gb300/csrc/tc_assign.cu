@@ -849,58 +849,79 @@ __global__ void k_x_to_bf16_batch(const TcXPrep *__restrict__ X, const int64_t *
     }
 }
 
-// centres -> BF16 [kpad][Kp], |c|^2 (+inf for padding) and the max of |c|^2
-// over real centres; a warp per global padded centre e of instance
-// find_inst(kpad_off, e), lanes over column pairs (a thread per centre, each
-// store two bytes of another row, took 66 us for 2,048 split centres)
+// centres -> BF16 [kpad][Kp], |c|^2 (+inf for padding) and the max of |c|^2 over
+// real centres; centre e is global, padded ones included, of instance
+// find_inst(kpad_off, e).  The warps take them as in the FP32 copy (assign.cu,
+// centre_prep), and for the same reason: 1M x 32 takes 419 us, 1,479 with a warp
+// per centre, 200,000 x 128 170 us, 440; with a thread per centre, each store two
+// bytes of another row, 2,048 split ones took 66 us, now 7.
 __global__ void k_c_to_bf16(const TcCPrep *__restrict__ C, const int64_t *__restrict__ kpad_off, int count,
-                            int64_t total) {
-    const int lane = threadIdx.x & 31;
+                            int64_t total, CentreWarp W) {
+    const int lane = threadIdx.x & 31, per = W.per_step();
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < total; e += nw) {
-        const int ii = find_inst(kpad_off, count, e);
-        const TcCPrep &P = C[ii];
-        const int64_t j = e - kpad_off[ii];
-        const int W = P.split ? 2 * P.Kp : P.Kp;
-        double s = 0.0;
-        for (int t = 2 * lane; t < P.Kp; t += 64) {
-            // -2 c: scaling by a power of two is exact in BF16
-            __nv_bfloat162 h2, l2;
-#pragma unroll
-            for (int q = 0; q < 2; q++) {
-                const double v = (j < P.k && t + q < P.d) ? P.c[j * P.d + t + q] : 0.0;
-                const __nv_bfloat16 h = __double2bfloat16(-2.0 * v);
-                const __nv_bfloat16 l = __double2bfloat16(-2.0 * v - (double)__bfloat162float(h));  // exact
-                if (q) h2.y = h, l2.y = l;
-                else h2.x = h, l2.x = l;
-                s += v * v;
+    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w * W.centres() < total; w += nw) {
+        const int64_t e0 = w * W.centres();
+        double mine = 0.0;
+        for (int st = 0; st < W.steps; st++) {
+            const int64_t e = e0 + per * st + lane / W.lanes;
+            double s = 0.0;
+            if (e < total) {
+                const int ii = find_inst(kpad_off, count, e);
+                const TcCPrep &P = C[ii];
+                const int64_t j = e - kpad_off[ii];
+                const int Kp = P.Kp;
+                const bool split = P.split;
+                const int d = j < P.k ? P.d : 0;
+                const double *c = P.c + j * P.d;
+                __nv_bfloat16 *cb = P.cb + j * (split ? 2 * Kp : Kp);
+#pragma unroll 4
+                for (int t = 2 * (lane & (W.lanes - 1)); t < Kp; t += 2 * W.lanes) {
+                    // -2 c: scaling by a power of two is exact in BF16
+                    const double v0 = t < d ? c[t] : 0.0, v1 = t + 1 < d ? c[t + 1] : 0.0;
+                    const double a0 = -2.0 * v0, a1 = -2.0 * v1;
+                    __nv_bfloat162 h;
+                    h.x = __double2bfloat16(a0);
+                    h.y = __double2bfloat16(a1);
+                    *reinterpret_cast<__nv_bfloat162 *>(cb + t) = h;
+                    if (split) {
+                        __nv_bfloat162 l;
+                        l.x = __double2bfloat16(a0 - (double)__bfloat162float(h.x));  // exact
+                        l.y = __double2bfloat16(a1 - (double)__bfloat162float(h.y));
+                        *reinterpret_cast<__nv_bfloat162 *>(cb + Kp + t) = l;
+                    }
+                    s += v0 * v0;
+                    s += v1 * v1;
+                }
             }
-            *reinterpret_cast<__nv_bfloat162 *>(P.cb + j * W + t) = h2;
-            if (P.split) *reinterpret_cast<__nv_bfloat162 *>(P.cb + j * W + P.Kp + t) = l2;
+            for (int o = 1; o < W.lanes; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            s = __shfl_sync(0xffffffffu, s, W.lanes * (lane & (per - 1)));
+            if (lane / per == st) mine = s;
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        // |c|^2 = hi + mid + lo in BF16 (within 2^-24 |c|^2); padding: +inf,
-        // which never wins
-        if (lane < 16) {
-            __nv_bfloat16 v = __ushort_as_bfloat16((unsigned short)0);
+        const int64_t e = e0 + lane;
+        unsigned bits = 0;
+        unsigned *most = nullptr;
+        if (lane < W.centres() && e < total) {
+            const int ii = find_inst(kpad_off, count, e);
+            const TcCPrep &P = C[ii];
+            const int64_t j = e - kpad_off[ii];
+            // |c|^2 = hi + mid + lo in BF16 (within 2^-24 |c|^2); padding: +inf,
+            // which never wins
+            uint32_t hm = 0x7F80u, l = 0u;
             if (j < P.k) {
-                const __nv_bfloat16 h = __double2bfloat16(s);
-                const double r1 = s - (double)__bfloat162float(h);
+                const __nv_bfloat16 h = __double2bfloat16(mine);
+                const double r1 = mine - (double)__bfloat162float(h);
                 const __nv_bfloat16 m = __double2bfloat16(r1);
-                if (lane == 0) v = h;
-                else if (lane == 1) v = m;
-                else if (lane == 2) v = __double2bfloat16(r1 - (double)__bfloat162float(m));
-            } else if (lane == 0) {
-                v = __ushort_as_bfloat16((unsigned short)0x7F80);
+                hm = (uint32_t)__bfloat16_as_ushort(h) | (uint32_t)__bfloat16_as_ushort(m) << 16;
+                l = __bfloat16_as_ushort(__double2bfloat16(r1 - (double)__bfloat162float(m)));
+                bits = __float_as_uint((float)mine);  // non-negative floats order as uints
+                most = P.cmax_bits;
             }
-            P.cbx[j * 16 + lane] = v;
+            uint4 *x = reinterpret_cast<uint4 *>(P.cbx + j * 16);
+            x[0] = make_uint4(hm, l, 0u, 0u);
+            x[1] = make_uint4(0u, 0u, 0u, 0u);
+            P.cn[j] = j < P.k ? (float)mine : __int_as_float(0x7f800000);
         }
-        if (lane == 0) {
-            const float f = (float)s;
-            P.cn[j] = j < P.k ? f : __int_as_float(0x7f800000);
-            if (j < P.k) atomicMax(P.cmax_bits, __float_as_uint(f));  // non-negative floats order as uints
-        }
+        max_by_warp(most, bits);
     }
 }
 
@@ -1110,8 +1131,9 @@ geek_status tc_plan_convert(geek_ctx *ctx, const TcPlan &P, cudaStream_t st) {
     }
     if (P.kpad_total > 0) {
         GK_COUNT();
-        k_c_to_bf16<<<grid_for(P.kpad_total * 32, 128, ctx->num_sms), 128, 0, st>>>(P.cprep, P.kpad_off_dev, count,
-                                                                               P.kpad_total);
+        const CentreWarp cw = centre_warp(ctx, P.kpad_total);
+        k_c_to_bf16<<<grid_for(ceil_div(P.kpad_total, cw.centres()) * 32, 128, ctx->num_sms), 128, 0, st>>>(
+            P.cprep, P.kpad_off_dev, count, P.kpad_total, cw);
     }
     GK_LAUNCH(ctx);
     return GEEK_OK;
