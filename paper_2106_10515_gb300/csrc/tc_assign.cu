@@ -1174,6 +1174,24 @@ Rings ring_lg(const TcPlan &P, const std::vector<int> *which, int split) {
     return Rings{lg, lg, lg_na};
 }
 
+// Pairs of row tiles: one BF16 data set of 256-wide tiles, several centre tiles per
+// pair (the next pair's rows are loaded only at the end of this one), four pairs
+// or more per SM.  Pairs come out even on the SMs less often than single tiles:
+// what the longer last round costs, 2 ceil(pairs / SMs) against ceil(tiles / SMs),
+// must stay below what a pair saves, 1 % and a part that shrinks with the centres
+// (the ends of a row tile, twice as large a share with d <= 64).  Times against one
+// tile at a time, k = 2,048 / 4,000 / 20,000 / 100,000: with even rounds (n =
+// 311,296) d = 64: 0.89 / 0.92 / 0.97 / 0.99, d = 128: 0.94 / 1.00 / 0.97 / 0.89; with
+// 22 for 21 (n = 400,000) d = 64: 0.92 / 0.95 / 1.02 / 1.04, d = 128: 0.99 / 1.04 / 1.02;
+// with 10 for 9 (n = 156,000) d = 64: 0.97 / 1.02 / 1.07 / 1.10, d = 128: 1.05 / 1.10 /
+// 1.09 / 1.03.
+bool pairs_pay(const TcPlanInst &I, int num_sms) {
+    const int64_t pairs = ceil_div(I.n, 2 * TC_M), tiles_c = ceil_div(I.k, TC_N);
+    if (I.split || I.N != TC_N || pairs < 4 * (int64_t)num_sms || tiles_c < 8) return false;
+    const double rounds = (double)ceil_div(I.n, (int64_t)TC_M * num_sms);
+    return 2.0 * (double)ceil_div(pairs, num_sms) <= rounds * (1.01 + (I.d <= 64 ? 1.0 : 0.4) / (double)tiles_c);
+}
+
 geek_status launch_units(geek_ctx *ctx, const TcInst *inst, const int2 *units, int64_t n0, int64_t n1,
                          int32_t *flag_rows, float *flag_m, unsigned long long *n_flag, int *err, double work,
                          Rings r0, Rings r1, cudaStream_t st) {
@@ -1216,16 +1234,10 @@ geek_status tc_plan_launch(geek_ctx *ctx, const TcPlan &P, int32_t *flag_rows, f
                            unsigned long long *n_flag, cudaStream_t st) {
     double work = 0.0;
     for (const TcPlanInst &I : P.desc) work += 2.0 * (double)I.n * (double)I.k * (double)I.d;
-    // Pairs of row tiles: one BF16 data set of 256-wide tiles whose pairs fill
-    // the chip four times over (below, half as many units leave SMs idle in
-    // the last wave) and whose centre tiles are several per pair (the next
-    // pair's rows are loaded only at the end of this one).
-    const TcPlanInst &I0 = P.desc[0];
-    const int64_t pairs = ceil_div(I0.n, 2 * TC_M);
-    if (P.count == 1 && !I0.split && I0.N == TC_N && pairs >= 4 * (int64_t)ctx->num_sms && I0.k >= 8 * TC_N) {
+    if (P.count == 1 && pairs_pay(P.desc[0], ctx->num_sms)) {
         TcArgs A{};
         A.inst = P.inst;
-        A.nunits = pairs;
+        A.nunits = ceil_div(P.desc[0].n, 2 * TC_M);
         A.flag_rows = flag_rows;
         A.flag_m = flag_m;
         A.n_flag = n_flag;
