@@ -174,7 +174,7 @@ __global__ void k_group_emit(const int64_t *__restrict__ nruns, const int64_t *_
 
 // heavy items: up to 64 * JX_HW of the items with the longest posting lists
 // are counted by bitmasks instead of posting lists
-constexpr int JX_HW = 1;
+constexpr int JX_HW = 3;
 
 // item -> centres inverted index helpers
 __global__ void k_centre_pairs(int64_t k, const int64_t *__restrict__ coff, const uint32_t *__restrict__ citems,
@@ -365,8 +365,8 @@ __global__ void __launch_bounds__(256) k_assign_jaccard(
 //    gives the first bound; a tile met while the threshold is not positive is
 //    taken again at the end, and if it still is not (a set unlike every
 //    centre), the set goes to the second pass.
-//  k_jac_count (those sets): only the 64 most frequent items stay out, and
-//    every centre is scored, lane per centre.
+//  k_jac_count (those sets): only the most frequent items stay out, 64 to 64
+//    JX_HW of them (jx_heavy_words), and every centre is scored, lane per centre.
 // Sets with more than MAXI items are listed for the dense path.
 // 2,000,000 sets of 59 items against 47,686 centres (mean 58 items): the
 // counters get 3,200 increments per set instead of 28,600, and the two passes
@@ -451,11 +451,31 @@ __global__ void k_freq_lut(int nfreq, const uint32_t *__restrict__ fq_item, cons
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nfreq; q += gridDim.x * blockDim.x)
         lut[fq_item[q]] = -2 - (int32_t)fq_bit[q];
 }
-// posting list of each frequent item by rank (ranks below 64 JX_HW have none)
-__global__ void k_freq_list(int nfreq, const int64_t *__restrict__ fq_run, const int16_t *__restrict__ fq_bit,
+// posting list of each frequent item by rank (ranks below nheavy have none)
+__global__ void k_freq_list(int nfreq, int nheavy, const int64_t *__restrict__ fq_run, const int16_t *__restrict__ fq_bit,
                             const int64_t *__restrict__ lrun_pos, int32_t *__restrict__ fq_list) {
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nfreq; q += gridDim.x * blockDim.x)
-        fq_list[fq_bit[q]] = fq_bit[q] < 64 * JX_HW ? -1 : (int32_t)lrun_pos[fq_run[q]];
+        fq_list[fq_bit[q]] = fq_bit[q] < nheavy ? -1 : (int32_t)lrun_pos[fq_run[q]];
+}
+
+// Mask words of the heaviest items (ord: by posting list) that pay in the second
+// pass.  64 more items in the mask cost a load and a popcount per centre, and save
+// a set the counter increments of those it holds, about k sum (len / k)^2 when sets
+// resemble centres: they pay from a quarter of an increment per centre on.  2M
+// sets, k = 47,686 (0.28 for a second word, 0.11 for a third): 81 ms with one word,
+// 78 with two; 200,000 sets of 60 of 1,500 items, k = 2,605 (0.17) 2.49 and 2.57; of 100
+// of 600 items, k = 744 (2.2 and 2.0) 4.6 with one, 4.1 with three.
+int jx_heavy_words(const std::vector<int64_t> &rs, const std::vector<int32_t> &ord, int nfreq, int64_t k) {
+    int words = 1;
+    for (; words < JX_HW && 64 * words < nfreq; words++) {
+        double sum = 0.0;
+        for (int q = 64 * words; q < std::min(nfreq, 64 * words + 64); q++) {
+            const double len = (double)(rs[ord[q] + 1] - rs[ord[q]]) / (double)k;
+            sum += len * len;
+        }
+        if (sum < 0.25) break;
+    }
+    return words;
 }
 
 // how the kernels find an item: the table when the items are small numbers
@@ -681,7 +701,7 @@ __global__ void __launch_bounds__(JX_THREADS, 3) k_jac_prune(JxArgs A, const uin
     }
 }
 
-template <bool NARROW>
+template <bool NARROW, int MW>  // MW: mask words per centre, at least HW
 __global__ void __launch_bounds__(JX_THREADS, 3) k_jac_count(JxArgs A, const uint64_t *__restrict__ cmask, int HW,
                                                              const int32_t *__restrict__ fq_list,
                                                              const int4 *__restrict__ rows,
@@ -701,21 +721,25 @@ __global__ void __launch_bounds__(JX_THREADS, 3) k_jac_count(JxArgs A, const uin
         const int64_t s0 = A.off[i];
         const int ni = (int)(A.off[i + 1] - s0);  // <= MAXI: the first pass listed it
         const uint32_t na = (uint32_t)(A.na_fix >= 0 ? A.na_fix : ni);
-        uint64_t am = 0;
+        uint64_t am[MW] = {};
         __syncwarp();
 #pragma unroll 2
         for (int p = lane; p < ni; p += 32) {
             int32_t r = A.X.find(A.items[s0 + p]);
             if (r < -1) {
                 const int hb = -2 - r;
-                if (hb < 64 * JX_HW) am |= 1ull << hb;
+#pragma unroll
+                for (int h = 0; h < MW; h++)
+                    if (h < HW && hb >> 6 == h) am[h] |= 1ull << (hb & 63);
                 r = fq_list[hb];
             }
             ridx[p] = r;
         }
         __syncwarp();
-        am = ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(am >> 32)) << 32) |
-             __reduce_or_sync(0xffffffffu, (uint32_t)am);
+#pragma unroll
+        for (int h = 0; h < MW; h++)
+            am[h] = ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(am[h] >> 32)) << 32) |
+                    __reduce_or_sync(0xffffffffu, (uint32_t)am[h]);
         JxBest best;
         best.n = (uint32_t)row.y;
         best.d = (uint32_t)row.z;
@@ -729,7 +753,9 @@ __global__ void __launch_bounds__(JX_THREADS, 3) k_jac_count(JxArgs A, const uin
 #pragma unroll 4
             for (int cc = lane; cc < nc; cc += 32) {
                 uint32_t in = (cw[cc >> C::LG] >> ((cc & ((1 << C::LG) - 1)) * C::CBITS)) & C::CMASK;
-                if (HW) in += __popcll(am & cmask[c0 + cc]);
+#pragma unroll
+                for (int h = 0; h < MW; h++)
+                    if (h < HW) in += __popcll(am[h] & cmask[(c0 + cc) * (MW == 1 ? 1 : HW) + h]);
                 if (in >= need) best.push(in, na + (uint32_t)A.clen[c0 + cc] - in, (int)(c0 + cc));
             }
             best.warp_merge();
@@ -740,7 +766,6 @@ __global__ void __launch_bounds__(JX_THREADS, 3) k_jac_count(JxArgs A, const uin
         if (lane == 0) A.labels[i] = best.n > 0 ? best.j : 0;
     }
 }
-static_assert(JX_HW == 1, "k_jac_count holds one mask word per centre");
 
 }  // namespace
 
@@ -951,14 +976,14 @@ geek_status jaccard_core(geek_ctx *ctx, Scratch &scr, const int64_t *off, const 
     std::vector<int32_t> ord(ni);
     GK_CUDA(ctx, cudaStreamSynchronize(st));
     for (int64_t r = 0; r < ni; r++) ord[r] = (int32_t)r;
-    const int64_t fmax = std::min<int64_t>(64 * JX_MW, ni), hmax = std::min<int64_t>(64 * JX_HW, ni);
+    const int64_t fmax = std::min<int64_t>(64 * JX_MW, ni);
     std::partial_sort(ord.begin(), ord.begin() + fmax, ord.end(), [&](int32_t a, int32_t b) {
         const int64_t la = hrs[a + 1] - hrs[a], lb = hrs[b + 1] - hrs[b];
         return la != lb ? la > lb : a < b;
     });
-    int nfreq = 0;  // frequent items, by rank: the first 64 JX_HW of them are the heavy ones
+    int nfreq = 0;  // frequent items, by rank: the first nheavy of them are the heavy ones
     while (nfreq < fmax && hrs[ord[nfreq] + 1] - hrs[ord[nfreq]] >= 2) nfreq++;
-    const int nheavy = (int)std::min<int64_t>(nfreq, hmax);
+    const int nheavy = std::min(nfreq, 64 * jx_heavy_words(hrs, ord, nfreq, k));
     const int HW = (nheavy + 63) / 64, FW = (nfreq + 63) / 64;
     std::vector<int32_t> fq_runs(ord.begin(), ord.begin() + nfreq);
     std::sort(fq_runs.begin(), fq_runs.end());
@@ -1032,7 +1057,7 @@ geek_status jaccard_core(geek_ctx *ctx, Scratch &scr, const int64_t *off, const 
     GK_LAUNCH(ctx);
     if (nfreq) {
         GK_COUNT();
-        k_freq_list<<<G(ctx, nfreq), 256, 0, st>>>(nfreq, fq_run_dev, fq_bit, lrun_pos, fq_list);
+        k_freq_list<<<G(ctx, nfreq), 256, 0, st>>>(nfreq, nheavy, fq_run_dev, fq_bit, lrun_pos, fq_list);
         GK_LAUNCH(ctx);
     }
     uint64_t *cmask, *fmask;
@@ -1140,8 +1165,8 @@ geek_status jaccard_core(geek_ctx *ctx, Scratch &scr, const int64_t *off, const 
             GK_LAUNCH(ctx);
             return GEEK_OK;
         };
-        if (narrow) GK_TRY(run(k_jac_prune<true>, k_jac_count<true>));
-        else GK_TRY(run(k_jac_prune<false>, k_jac_count<false>));
+        if (narrow) GK_TRY(run(k_jac_prune<true>, HW > 1 ? k_jac_count<true, JX_HW> : k_jac_count<true, 1>));
+        else GK_TRY(run(k_jac_prune<false>, HW > 1 ? k_jac_count<false, JX_HW> : k_jac_count<false, 1>));
         GK_LAUNCH(ctx);
         }
     }
