@@ -1110,19 +1110,56 @@ __global__ void k_label_keys(int64_t n, const int32_t *__restrict__ labels, int6
     }
 }
 
-// sort key of centre j: descending member count, then ascending index; nseg[j] =
-// segments of a large centre (else 0), *n_large += 1 for each
-constexpr int UL_M = 128;        // members per segment
-constexpr int UL_MIN = 16384;    // a centre of more members is cut into segments
-__global__ void k_size_order(int64_t k, const unsigned long long *__restrict__ cnt, uint64_t *__restrict__ key,
-                             int64_t *__restrict__ nseg, unsigned long long *__restrict__ n_large) {
+// sort key of centre j: descending member count, then ascending index
+__global__ void k_size_order(int64_t k, const unsigned long long *__restrict__ cnt, uint64_t *__restrict__ key) {
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < k; j += (int64_t)gridDim.x * blockDim.x) {
         const uint64_t cj = cnt[j] > 0xFFFFFFFFull ? 0xFFFFFFFFull : cnt[j];
         key[j] = ((0xFFFFFFFFull - cj) << 32) | (uint64_t)j;
-        const bool large = cj > UL_MIN;
-        nseg[j] = large ? (int64_t)((cj + UL_M - 1) / UL_M) : 0;
-        if (large) atomicAdd(n_large, 1ull);
     }
+}
+
+// The centres whose chains are cut into segments (the large ones): nseg[j] = their
+// segments (zeros before), *n_large = how many.  A chain takes 41 ns per member on its
+// warp pair, segments two more passes over the rows and a walk that is the slower the
+// more chains there are.  With r the longest chain over the members per pair (of
+// the clusters above UL_MIN; of all where the others' chains run beside the walk on
+// a second stream), both ways take about the same time at UL_MIN (0.85 + 9.5 / r + 110
+// / r^2) members, at least UL_MIN; measured, clusters of one size around 10 in each coordinate,
+// spread 1:
+//   r = 152 (1 x 128 coordinates) 18,000; 30 (20 x 32) 30,000; 19 (8 x 128) 30,000;
+//   12 (8 x 200) 48,000; 10 (60 x 32) 50,000; 7.6 (20 x 128) 62,000; 4.9 (20 x 200) 125,000.
+// 60 clusters of 20,000 x 128: 0.83 ms by chains, 2.6 by segments; 8 of 80,000 3.1 and
+// 2.1; one of 250,000 9.7 and 2.4; 10M x 128 of 20,000 Zipf clusters (r = 14): 14.1 ms,
+// 15.8 with all above UL_MIN cut.
+constexpr int UL_M = 128;        // members per segment
+constexpr int UL_MIN = 16384;    // no smaller centre is large
+__global__ void __launch_bounds__(256) k_large(int64_t most_large, const unsigned long long *__restrict__ cnt,
+                                               const uint64_t *__restrict__ order, double pairs_per_row,
+                                               int64_t all_rows, int64_t *__restrict__ nseg, unsigned long long *__restrict__ n_large) {
+    __shared__ unsigned long long s_sum, s_count;
+    if (threadIdx.x == 0) s_sum = s_count = 0;
+    __syncthreads();
+    unsigned long long sum = 0;
+    for (int64_t q = threadIdx.x; q < most_large; q += blockDim.x) {
+        const unsigned long long cj = cnt[order[q] & 0xFFFFFFFFull];
+        if (cj <= UL_MIN) break;  // descending
+        sum += cj;
+    }
+    atomicAdd(&s_sum, sum);
+    __syncthreads();
+    const double r = (double)cnt[order[0] & 0xFFFFFFFFull] / ((double)(all_rows ? all_rows : s_sum) * pairs_per_row);
+    const double line = UL_MIN * (1.0 + fmax(9.5 / r - 0.15, 0.0) + 110.0 / (r * r));
+    unsigned count = 0;
+    for (int64_t q = threadIdx.x; q < most_large; q += blockDim.x) {
+        const int64_t j = (int64_t)(order[q] & 0xFFFFFFFFull);
+        const unsigned long long cj = cnt[j];
+        if (cj <= UL_MIN || (double)cj <= line) break;
+        nseg[j] = (int64_t)((cj + UL_M - 1) / UL_M);
+        count++;
+    }
+    atomicAdd(&s_count, (unsigned long long)count);
+    __syncthreads();
+    if (threadIdx.x == 0) *n_large = s_count;
 }
 
 // centre j <- mean of its members (ascending id, the seeds' centroid sum);
@@ -1454,9 +1491,7 @@ __global__ void __launch_bounds__(UC_T) k_update_centres(const float *__restrict
 //               otherwise (the first segments, a segment that crosses a power
 //               of two, a member comparable to s or not finite) the segment
 //               runs through chain_chunk.
-// Both sides of the line: a centre of UL_MIN members takes 0.7 ms on one warp
-// pair, about what the whole pass over the segments takes at 10M x 128, and
-// its first segments run through chain_chunk either way.
+// Which centres are cut: k_large.
 struct UlArgs {
     const float *x;
     int64_t ldx;
@@ -1779,10 +1814,17 @@ geek_status refine_dense(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ld
         GK_TRY(ps.alloc(&n_large, 1));
         GK_CUDA(ctx, cudaMemsetAsync(n_large, 0, sizeof(unsigned long long), st));
         GK_COUNT();
-        k_size_order<<<grid_for(k, 256, ctx->num_sms), 256, 0, st>>>(k, cnt, order, nseg, n_large);
+        k_size_order<<<grid_for(k, 256, ctx->num_sms), 256, 0, st>>>(k, cnt, order);
         GK_LAUNCH(ctx);
         GK_TRY(radix_sort_segments(ctx, ps, 1, k, &order, nullptr, nullptr, 64, st));
-        GK_TRY(exclusive_scan_i64(ctx, ps, nseg, seg_off, k, seg_tot, st));
+        if (n > UL_MIN) {  // else no centre is large
+            GK_CUDA(ctx, cudaMemsetAsync(nseg, 0, sizeof(int64_t) * k, st));
+            GK_COUNT();
+            k_large<<<1, 256, 0, st>>>(std::min(k, n / UL_MIN), cnt, order, d / (32.0 * UC_P * ctx->num_sms),
+                                       side.on ? n : 0, nseg, n_large);
+            GK_LAUNCH(ctx);
+            GK_TRY(exclusive_scan_i64(ctx, ps, nseg, seg_off, k, seg_tot, st));
+        }
         tg.stop();
         unsigned long long *next;
         int *uc_err;
@@ -1796,7 +1838,7 @@ geek_status refine_dense(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ld
             uc_attr = true;
         }
         EvTimer tu(ctx, "kernel.update_centres", st);
-        if (n > UL_MIN) {  // else no centre is large
+        if (n > UL_MIN) {
             const size_t segs = (size_t)(n / UL_M + n / UL_MIN + 1);  // at most
             UlArgs U{x, ldx, d, k, off, cnt, (const int32_t *)ids, seg_off, seg_tot, order, n_large};
             GK_TRY(ps.alloc(&U.start, segs * d));
