@@ -1110,56 +1110,84 @@ __global__ void k_label_keys(int64_t n, const int32_t *__restrict__ labels, int6
     }
 }
 
-// sort key of centre j: descending member count, then ascending index
-__global__ void k_size_order(int64_t k, const unsigned long long *__restrict__ cnt, uint64_t *__restrict__ key) {
+// sort key of centre j: descending member count, then ascending index; nseg[j] = 0
+__global__ void k_size_order(int64_t k, const unsigned long long *__restrict__ cnt, uint64_t *__restrict__ key,
+                             int64_t *__restrict__ nseg) {
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < k; j += (int64_t)gridDim.x * blockDim.x) {
         const uint64_t cj = cnt[j] > 0xFFFFFFFFull ? 0xFFFFFFFFull : cnt[j];
         key[j] = ((0xFFFFFFFFull - cj) << 32) | (uint64_t)j;
+        nseg[j] = 0;
     }
 }
 
-// The centres whose chains are cut into segments (the large ones): nseg[j] = their
-// segments (zeros before), *n_large = how many.  A chain takes 41 ns per member on its
-// warp pair, segments two more passes over the rows and a walk that is the slower the
-// more chains there are.  With r the longest chain over the members per pair (of
-// the clusters above UL_MIN; of all where the others' chains run beside the walk on
-// a second stream), both ways take about the same time at UL_MIN (0.85 + 9.5 / r + 110
-// / r^2) members, at least UL_MIN; measured, clusters of one size around 10 in each coordinate,
-// spread 1:
-//   r = 152 (1 x 128 coordinates) 18,000; 30 (20 x 32) 30,000; 19 (8 x 128) 30,000;
-//   12 (8 x 200) 48,000; 10 (60 x 32) 50,000; 7.6 (20 x 128) 62,000; 4.9 (20 x 200) 125,000.
-// 60 clusters of 20,000 x 128: 0.83 ms by chains, 2.6 by segments; 8 of 80,000 3.1 and
-// 2.1; one of 250,000 9.7 and 2.4; 10M x 128 of 20,000 Zipf clusters (r = 14): 14.1 ms,
-// 15.8 with all above UL_MIN cut.
+// How many of the centres, the largest first, are cut into segments (the large
+// ones): *n_large, and their segments in nseg.  Estimated, in ms, for every count
+// (block of one):
+//  the others' chains, 41 ns per member: the longest of them, or their balanced load
+//  on the warp pairs;
+//  the large ones' segments: two passes over their rows, 0.1 + 5.2 ps per value, and a
+//  walk that grows as the root of the longest chain (most of its steps are near the
+//  start), 0.1 + a sqrt(members / 1000), a = 0.11 with 32 coordinates per warp, 0.04
+//  with 8.  It depends on the data (spread 1 around 10: up to 1.5 times that, around
+//  100: down to 0.7) and is taken for 1.25 times that where the others' chains follow
+//  it, for 0.55 where they run beside the walk: a chain left beside a short walk
+//  costs more than a segment too many.
+// Measured, chains and segments: 60 clusters of 20,000 x 128 0.82 and 2.6 ms, 20 of
+// 50,000 1.9 and 2.4, 8 of 80,000 3.1 and 2.1, one of 20,000 0.77 and 0.73, one of
+// 250,000 9.7 and 2.4; 111,000 x 128 of 105 Zipf clusters, one above UL_MIN, two
+// passes 2.3 and 3.1 in all; 10M x 128 of 20,000 Zipf clusters 14 ms as chosen, 16
+// with all above UL_MIN cut.
 constexpr int UL_M = 128;        // members per segment
 constexpr int UL_MIN = 16384;    // no smaller centre is large
-__global__ void __launch_bounds__(256) k_large(int64_t most_large, const unsigned long long *__restrict__ cnt,
-                                               const uint64_t *__restrict__ order, double pairs_per_row,
-                                               int64_t all_rows, int64_t *__restrict__ nseg, unsigned long long *__restrict__ n_large) {
-    __shared__ unsigned long long s_sum, s_count;
-    if (threadIdx.x == 0) s_sum = s_count = 0;
+__global__ void __launch_bounds__(256) k_large(int64_t k, int64_t most_large, int64_t n, int d, int pairs, bool beside,
+                                               const unsigned long long *__restrict__ cnt,
+                                               const uint64_t *__restrict__ order, int64_t *__restrict__ nseg,
+                                               unsigned long long *__restrict__ n_large) {
+    __shared__ unsigned long long s_best;
+    __shared__ double s_warp[8];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    auto size = [&](int64_t q) { return q < k ? (double)cnt[order[q] & 0xFFFFFFFFull] : 0.0; };
+    auto chains = [&](double longest, double rows) {
+        return 41e-6 * fmax(longest, rows * d / (32.0 * pairs));
+    };
+    const double first = size(0);
+    const double walk = (beside ? 0.55 : 1.25) * (0.1 + (0.02 + 0.09 * min(d, 32) / 32) * sqrt(first * 1e-3));
+    // (estimate, count) of the best: positive floats order as their bits
+    if (t == 0) s_best = (unsigned long long)__float_as_uint((float)chains(first, (double)n)) << 32;
     __syncthreads();
-    unsigned long long sum = 0;
-    for (int64_t q = threadIdx.x; q < most_large; q += blockDim.x) {
-        const unsigned long long cj = cnt[order[q] & 0xFFFFFFFFull];
-        if (cj <= UL_MIN) break;  // descending
-        sum += cj;
+    double before = 0.0;
+    for (int64_t q0 = 0; q0 < most_large; q0 += 256) {
+        const int64_t q = q0 + t;
+        const double c = q < most_large ? size(q) : 0.0, next = size(q + 1);
+        double x = c > UL_MIN ? c : 0.0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) s_warp[w] = x;
+        __syncthreads();
+        double all = 0.0;
+        for (int v = 0; v < 8; v++) {
+            if (v < w) x += s_warp[v];
+            all += s_warp[v];
+        }
+        if (c > UL_MIN) {  // the first q + 1
+            const double rows = before + x;
+            const double passes = 1.25 * (0.1 + 5.2e-9 * rows * d), rest = chains(next, (double)n - rows);
+            const float est = (float)(passes + (beside ? fmax(walk, rest) : walk + rest));
+            atomicMin(&s_best, ((unsigned long long)__float_as_uint(est) << 32) | (unsigned long long)(q + 1));
+        }
+        before += all;
+        if (__syncthreads_or(c <= UL_MIN)) break;  // descending
     }
-    atomicAdd(&s_sum, sum);
     __syncthreads();
-    const double r = (double)cnt[order[0] & 0xFFFFFFFFull] / ((double)(all_rows ? all_rows : s_sum) * pairs_per_row);
-    const double line = UL_MIN * (1.0 + fmax(9.5 / r - 0.15, 0.0) + 110.0 / (r * r));
-    unsigned count = 0;
-    for (int64_t q = threadIdx.x; q < most_large; q += blockDim.x) {
+    const int64_t nl = (int64_t)(s_best & 0xFFFFFFFFull);
+    for (int64_t q = t; q < nl; q += 256) {
         const int64_t j = (int64_t)(order[q] & 0xFFFFFFFFull);
-        const unsigned long long cj = cnt[j];
-        if (cj <= UL_MIN || (double)cj <= line) break;
-        nseg[j] = (int64_t)((cj + UL_M - 1) / UL_M);
-        count++;
+        nseg[j] = (int64_t)((cnt[j] + UL_M - 1) / UL_M);
     }
-    atomicAdd(&s_count, (unsigned long long)count);
-    __syncthreads();
-    if (threadIdx.x == 0) *n_large = s_count;
+    if (t == 0) *n_large = (unsigned long long)nl;
 }
 
 // centre j <- mean of its members (ascending id, the seeds' centroid sum);
@@ -1812,16 +1840,15 @@ geek_status refine_dense(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ld
         GK_TRY(ps.alloc(&seg_off, k));
         GK_TRY(ps.alloc(&seg_tot, 1));
         GK_TRY(ps.alloc(&n_large, 1));
-        GK_CUDA(ctx, cudaMemsetAsync(n_large, 0, sizeof(unsigned long long), st));
+        if (n <= UL_MIN) GK_CUDA(ctx, cudaMemsetAsync(n_large, 0, sizeof(unsigned long long), st));
         GK_COUNT();
-        k_size_order<<<grid_for(k, 256, ctx->num_sms), 256, 0, st>>>(k, cnt, order);
+        k_size_order<<<grid_for(k, 256, ctx->num_sms), 256, 0, st>>>(k, cnt, order, nseg);
         GK_LAUNCH(ctx);
         GK_TRY(radix_sort_segments(ctx, ps, 1, k, &order, nullptr, nullptr, 64, st));
         if (n > UL_MIN) {  // else no centre is large
-            GK_CUDA(ctx, cudaMemsetAsync(nseg, 0, sizeof(int64_t) * k, st));
             GK_COUNT();
-            k_large<<<1, 256, 0, st>>>(std::min(k, n / UL_MIN), cnt, order, d / (32.0 * UC_P * ctx->num_sms),
-                                       side.on ? n : 0, nseg, n_large);
+            k_large<<<1, 256, 0, st>>>(k, std::min(k, n / UL_MIN), n, d, UC_P * ctx->num_sms, side.on, cnt, order, nseg,
+                                       n_large);
             GK_LAUNCH(ctx);
             GK_TRY(exclusive_scan_i64(ctx, ps, nseg, seg_off, k, seg_tot, st));
         }

@@ -9,8 +9,9 @@ import torch
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("d,sizes", [(1, [16_384]), (1, [16_398]), (1, [16_420]), (3, [16_400] * 40), (24, [17_000] * 40), (5, [500_000] + [30_000] * 12),
-                                     (2, [900_000] + [20_000] * 10 + [17_000] * 3), (40, [70_000, 18_500, 18_000, 16_385, 5])])
+@pytest.mark.parametrize("d,sizes", [(1, [16_384]), (1, [16_385]), (1, [16_420]), (3, [16_400] * 40), (24, [17_000] * 40), (5, [500_000] + [30_000] * 12),
+                                     (2, [900_000] + [20_000] * 10 + [17_000] * 3), (40, [70_000, 18_500, 18_000, 16_385, 5]),
+                                     (1, [16_400] * 300 + [16_384] * 3 + [100] * 40), (35, [100_000] * 3 + [50_000] * 4 + [24_000] * 8)])
 def test_sums_are_sequential(geek, d, sizes):
     rng = np.random.default_rng(d + len(sizes))
     lab = rng.permutation(np.repeat(np.arange(len(sizes)), sizes)).astype(np.int32)
