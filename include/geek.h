@@ -167,12 +167,13 @@ geek_status geek_ctx_destroy(geek_ctx *ctx);
  * error paths can be tested without faulting a GPU.
  *  GEEK_OPT_WAIT_LIMIT_NS: limit of one bounded wait of a radix-sort pass on a
  *    predecessor tile's published count, in ns (default 2e9, range
- *    [1e3, 6e10]).  A wait that runs out gives up with a partial prefix (the
- *    pass's writes stay inside its segment; its result is wrong), and the
+ *    [1e3, 6e10]).  A tile whose wait runs out counts its predecessors' keys
+ *    itself (the pass stays right and its writes inside its segment), and the
  *    call that sorted returns GEEK_ERR_TIMEOUT.
- *  GEEK_OPT_TEST_STALL_TILE: FOR TESTS.  Tile t >= 0 of every radix pass never
- *    publishes its count, so the tiles after it wait until the wait limit and
- *    the call returns GEEK_ERR_TIMEOUT; -1 (default) turns it off.
+ *  GEEK_OPT_TEST_STALL_TILE: FOR TESTS.  Tile t >= 0 of every tiled radix pass
+ *    never publishes its count, so the tiles after it wait until the wait limit
+ *    and the call returns GEEK_ERR_TIMEOUT; -1 (default) turns it off.  (Sorts
+ *    of up to 5,120 elements per segment take one block each, without waits.)
  *  GEEK_OPT_TEST_FAIL_ALLOC: FOR TESTS.  Value v >= 0 makes the device
  *    allocation after the next v ones fail as if the device were out of memory
  *    (the call returns GEEK_ERR_NOMEM, or goes on with a smaller buffer where

@@ -306,6 +306,3 @@ geek_status segment_runs_tagged(geek_ctx *ctx, Scratch &scr, int S, int64_t m, c
 // Exclusive prefix sum of n int64 values (in place allowed); total -> *total_dev.
 geek_status exclusive_scan_i64(geek_ctx *ctx, Scratch &scr, const int64_t *in, int64_t *out,
                                int64_t n, int64_t *total_dev, cudaStream_t st);
-
-// iota fill
-void launch_iota_u32(uint32_t *v, int64_t n, int64_t period, cudaStream_t st);

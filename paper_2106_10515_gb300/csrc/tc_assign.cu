@@ -6,9 +6,9 @@
 // approximate values are closer than the rigorous error window.
 //
 // Persistent kernel, one CTA per SM, 10 warps:
-//   warp 0     TMA producer: X row tiles (double buffered) and centre tiles
-//              (2-stage ring), 128-byte swizzled, K-major, plus |c|^2 of
-//              each centre tile by bulk copy
+//   warp 0     TMA producer: X row tiles (a ring of 2 or 4 stages) and centre
+//              tiles (2 to 8 stages, whole tiles or 64-column parts), 128-byte
+//              swizzled, K-major, plus |c|^2 of each centre tile
 //   warp 1     MMA issuer: tcgen05.mma.cta_group::1.kind::f16, M=128, N=256,
 //              into one of two TMEM accumulators (2 x 256 columns)
 //   warps 2-9  epilogue: tcgen05.ld of the accumulator, d' = |c|^2 - 2 s,
@@ -1004,7 +1004,6 @@ void make_units(const TcPlan &P, const std::vector<int> &which, int split, std::
 
 size_t tc_smem() {
     static_assert(32 * 8 + (TC_EPI_GROUPS - 1) * TC_M * 3 * 4 <= TC_MISC, "misc region too small");
-    // tile stages + barriers / TMEM slot / merge buffer + |c|^2 ring + alignment
     // tile stages + barriers / TMEM slot / merge buffer + ones block + two
     // |c|^2 stages + alignment
     return 1024 + 2 * (size_t)TC_A_STAGE + 2 * (size_t)TC_B_STAGE + TC_MISC + TC_M * 32 + 2 * TC_N * 32;
@@ -1670,8 +1669,9 @@ __global__ void __launch_bounds__(256) k_decide_candidates(const RInst *__restri
 // decide_flags: F, every row's smallest value in mrow), gather the rows, find
 // their candidates with a second tcgen05 pass over them, and decide among the
 // candidates; what stays undecided is appended to left / n_left.  max_rows
-// bounds the flagged rows, ordered: they are in the order of their labels; no allocation and no host synchronisation (the
-// buffers are the plan's, tc_emit_alloc).
+// bounds the flagged rows; ordered: they are in the order of their labels.  No
+// allocation and no host synchronisation (the buffers are the plan's,
+// tc_emit_alloc).
 geek_status tc_decide_candidates(geek_ctx *ctx, const TcPlan &P, const RInst *R, const FlagUnits &F, const float *mrow,
                                  int64_t max_rows, bool ordered, int32_t *left, unsigned long long *n_left,
                                  cudaStream_t st) {
