@@ -1840,12 +1840,21 @@ geek_status refine_dense(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ld
         GK_TRY(ps.alloc(&seg_off, k));
         GK_TRY(ps.alloc(&seg_tot, 1));
         GK_TRY(ps.alloc(&n_large, 1));
-        if (n <= UL_MIN) GK_CUDA(ctx, cudaMemsetAsync(n_large, 0, sizeof(unsigned long long), st));
+        // the segments' arrays (at most so many), n d / 4 bytes; without room for them
+        // every centre is one chain
+        UlArgs U{x, ldx, d, k, off, cnt, (const int32_t *)ids, seg_off, seg_tot, nullptr, n_large};
+        U.segs = n / UL_M + n / UL_MIN + 1;
+        U.c = centres;
+        bool cut = n > UL_MIN;  // else no centre is large
+        if (cut) GK_TRY(ps.try_alloc(&U.start, (size_t)U.segs * d, &cut));
+        if (cut) GK_TRY(ps.try_alloc(&U.rec, 3 * (size_t)U.segs * d, &cut));
+        if (!cut) GK_CUDA(ctx, cudaMemsetAsync(n_large, 0, sizeof(unsigned long long), st));
         GK_COUNT();
         k_size_order<<<grid_for(k, 256, ctx->num_sms), 256, 0, st>>>(k, cnt, order, nseg);
         GK_LAUNCH(ctx);
         GK_TRY(radix_sort_segments(ctx, ps, 1, k, &order, nullptr, nullptr, 64, st));
-        if (n > UL_MIN) {  // else no centre is large
+        U.order = order;
+        if (cut) {
             GK_COUNT();
             k_large<<<1, 256, 0, st>>>(k, std::min(k, n / UL_MIN), n, d, UC_P * ctx->num_sms, side.on, cnt, order, nseg,
                                        n_large);
@@ -1865,15 +1874,9 @@ geek_status refine_dense(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ld
             uc_attr = true;
         }
         EvTimer tu(ctx, "kernel.update_centres", st);
-        if (n > UL_MIN) {
-            const size_t segs = (size_t)(n / UL_M + n / UL_MIN + 1);  // at most
-            UlArgs U{x, ldx, d, k, off, cnt, (const int32_t *)ids, seg_off, seg_tot, order, n_large};
-            GK_TRY(ps.alloc(&U.start, segs * d));
-            GK_TRY(ps.alloc(&U.rec, 3 * segs * d));
-            U.segs = (int64_t)segs;
-            U.c = centres;
+        if (cut) {
             const int nsl = (d + 31) / 32;
-            const int gs = grid_for((int64_t)segs * nsl * 32, 256, ctx->num_sms);
+            const int gs = grid_for(U.segs * nsl * 32, 256, ctx->num_sms);
             const int64_t most = (n / UL_MIN) * nsl;  // (large centre, slice) items, at most
             GK_COUNT();
             k_ul_sums<<<gs, 256, 0, st>>>(U);
@@ -1881,12 +1884,12 @@ geek_status refine_dense(geek_ctx *ctx, Scratch &scr, const float *x, int64_t ld
             k_ul_starts<<<(unsigned)std::min<int64_t>(most, (int64_t)ctx->num_sms * 8), 256, 0, st>>>(U);
             GK_COUNT();
             k_ul_deltas<<<gs, 256, 0, st>>>(U);
-            if (side.on) GK_CUDA(ctx, side.fork());
+            if (side.on) GK_CUDA(ctx, side.fork());  // with the chains that are not cut
             GK_COUNT();
             k_ul_chain<<<(unsigned)std::min<int64_t>(most, (int64_t)ctx->num_sms * 16), 32, 0, st>>>(U);
             GK_LAUNCH(ctx);
         }
-        const cudaStream_t us = side.on ? side.s : st;
+        const cudaStream_t us = cut && side.on ? side.s : st;
         GK_COUNT();
         k_update_centres<<<(unsigned)std::min<int64_t>((k * ((d + 31) / 32) + UC_P - 1) / UC_P, (int64_t)ctx->num_sms),
                            UC_T, UC_SMEM, us>>>(x, ldx, d, k, off, cnt, (const int32_t *)ids, order, n_large, next,

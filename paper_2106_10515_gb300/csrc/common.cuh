@@ -176,6 +176,16 @@ struct Scratch {
         *out = (T *)p;
         return GEEK_OK;
     }
+    // A buffer the call can do without: *got is false when there is no room.
+    template <class T>
+    geek_status try_alloc(T **out, size_t count, bool *got) {
+        const std::string msg = ctx->last_error;
+        const geek_status rc = alloc(out, count);
+        *got = rc == GEEK_OK;
+        if (rc != GEEK_ERR_NOMEM) return rc;
+        ctx->last_error = msg;  // nothing has failed
+        return GEEK_OK;
+    }
 };
 
 // Device buffer owned by a result handle.
