@@ -881,9 +881,10 @@ geek_status assign_hetero(geek_ctx *ctx, Scratch &scr, const geek_buckets *b, co
     unsigned long long *hist;  // rows by their number of matching attributes
     GK_TRY(scr.alloc(&hist, A + 1));
     GK_CUDA(ctx, cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * (A + 1), st));
-    if (match_bits_eligible(k, A)) {
-        GK_TRY(match_bits_assign(ctx, scr, n, A, attrs, k, modes, labels, stats ? hist : nullptr, st));
-    } else {
+    bool done = false;
+    if (match_bits_eligible(k, A))
+        GK_TRY(match_bits_assign(ctx, scr, n, A, attrs, k, modes, labels, stats ? hist : nullptr, &done, st));
+    if (!done) {
         GK_COUNT();
         k_assign_cat<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(n, A, k, attrs, modes, labels, stats ? hist : nullptr);
         GK_LAUNCH(ctx);
@@ -1230,8 +1231,8 @@ __global__ void k_run_flags(int64_t m, const uint64_t *__restrict__ sorted, int6
 // seed's members (Sect. 3.3: the mode of sparse data after DOPH; ties to the
 // smallest token); distance 1 - Jaccard of the token sets, i.e. the label
 // maximises the number of dimensions equal to the centre's mode
-// (match_bits.cu).  Where the mask table would be too large, tokens map to
-// 32-bit ids of the distinct mode tokens and the Jaccard engine decides, with
+// (match_bits.cu).  Where the mask table would be too large, or has no room,
+// tokens map to 32-bit ids of the distinct mode tokens and the Jaccard engine decides, with
 // |A| = |C| = D'.
 geek_status assign_doph(geek_ctx *ctx, Scratch &scr, const geek_buckets *b, const silk_seeds *s, int32_t *labels,
                         geek_assign_stats *stats, geek_centres *keep, cudaStream_t st) {
@@ -1257,7 +1258,10 @@ geek_status assign_doph(geek_ctx *ctx, Scratch &scr, const geek_buckets *b, cons
     k_modes<<<G(ctx, km), 256, 0, st>>>(k, D, s->off, s->ids, b->doph_tok, modes, nullptr);
     GK_LAUNCH(ctx);
     if (keep) GK_CUDA(ctx, cudaMemcpyAsync(keep->modes, modes, 8 * km, cudaMemcpyDeviceToDevice, st));
-    if (match_bits_eligible(k, D)) return match_bits_assign(ctx, scr, n, D, b->doph_tok, k, modes, labels, nullptr, st);
+    bool done = false;
+    if (match_bits_eligible(k, D))
+        GK_TRY(match_bits_assign(ctx, scr, n, D, b->doph_tok, k, modes, labels, nullptr, &done, st));
+    if (done) return GEEK_OK;
     // distinct mode tokens, ascending
     GK_CUDA(ctx, cudaMemcpyAsync(srt, modes, 8 * km, cudaMemcpyDeviceToDevice, st));
     GK_TRY(radix_sort_segments(ctx, scr, 1, km, &srt, nullptr, nullptr, 64, st));

@@ -396,7 +396,8 @@ struct geek_centres {
 // match_bits.cu: label = centre with the most attributes equal to the row's.
 bool match_bits_eligible(int64_t k, int A);
 geek_status match_bits_assign(geek_ctx *ctx, Scratch &scr, int64_t n, int A, const uint64_t *attrs, int64_t k,
-                              const uint64_t *modes, int32_t *labels, unsigned long long *hist, cudaStream_t st);
+                              const uint64_t *modes, int32_t *labels, unsigned long long *hist, bool *done,
+                              cudaStream_t st);
 // Stream-ordered allocation of a result handle's buffer (NOMEM on failure).
 geek_status own_alloc(geek_ctx *ctx, void **p, size_t bytes, cudaStream_t st);
 // keep (nullable): receives the central vectors the assignment used.

@@ -219,20 +219,24 @@ bool match_bits_eligible(int64_t k, int A) {
 
 // labels[i] = argmax_j #{a : attrs[i][a] == modes[j][a]}, ties to the smallest j
 // (attrs n x A, modes k x A, attribute by attribute); hist (nullable, A + 1
-// counters, zeroed by the caller): rows by their largest match count.
+// counters, zeroed by the caller): rows by their largest match count.  *done is
+// false, and nothing has run, where there is no room for the tables.
 geek_status match_bits_assign(geek_ctx *ctx, Scratch &scr, int64_t n, int A, const uint64_t *attrs, int64_t k,
-                              const uint64_t *modes, int32_t *labels, unsigned long long *hist, cudaStream_t st) {
+                              const uint64_t *modes, int32_t *labels, unsigned long long *hist, bool *done,
+                              cudaStream_t st) {
     const int64_t m = k * A;
     const int W = (int)ceil_div(k, 32);
     const uint64_t ns = mb_slots(k, A);
     uint32_t *owner, *slot_of, *masks;
     unsigned *next;
     MbSlot *slots;
-    GK_TRY(scr.alloc(&owner, ns));
-    GK_TRY(scr.alloc(&slot_of, m));
-    GK_TRY(scr.alloc(&slots, ns));
-    GK_TRY(scr.alloc(&masks, (size_t)m * W));
+    *done = true;
     GK_TRY(scr.alloc(&next, 1));
+    GK_TRY(scr.try_alloc(&masks, (size_t)m * W, done));
+    if (*done) GK_TRY(scr.try_alloc(&owner, ns, done));
+    if (*done) GK_TRY(scr.try_alloc(&slots, ns, done));
+    if (*done) GK_TRY(scr.try_alloc(&slot_of, m, done));
+    if (!*done) return GEEK_OK;
     GK_CUDA(ctx, cudaMemsetAsync(owner, 0, sizeof(uint32_t) * ns, st));
     GK_CUDA(ctx, cudaMemsetAsync(masks, 0, sizeof(uint32_t) * (size_t)m * W, st));
     GK_CUDA(ctx, cudaMemsetAsync(next, 0, sizeof(unsigned), st));
