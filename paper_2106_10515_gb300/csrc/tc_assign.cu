@@ -1346,9 +1346,13 @@ geek_status assign_tc_bf16(geek_ctx *ctx, Scratch &scr, const float *x, int64_t 
                            float *flag_m, unsigned long long *n_flag, TcPlan *P, cudaStream_t st) {
     if (d > 128) return set_error(ctx, GEEK_ERR_UNSUPPORTED, "BF16 tensor-core assignment supports d <= 128");
     std::vector<TcPlanInst> one(1);
-    // the widest tiles: 128-wide ones read the X tile from shared memory twice
-    // as often per flop and measured ~60% slower (BF16, d = 128)
-    one[0] = TcPlanInst{x, ldx, n, d, centres, k, labels, 0, TC_N, split};
+    // the widest tiles (128-wide ones read the X tile from shared memory twice as
+    // often per flop and measured ~60% slower, BF16, d = 128), but none wider than
+    // the centres need: 2M x 128, split, k = 30: 64-wide 217 us, 128-wide 308, 256-wide
+    // 369; k = 100: 314 (128-wide), 370; BF16, d = 64, k = 8: 152, 168, 222; k = 100: 186
+    // (128-wide), 191
+    const int N = k <= 64 ? 64 : k <= 128 ? 128 : TC_N;
+    one[0] = TcPlanInst{x, ldx, n, d, centres, k, labels, 0, N, split};
     GK_TRY(tc_plan_build(ctx, &scr, one, P, st));
     return tc_plan_enqueue(ctx, *P, flag_rows, flag_m, n_flag, st);
 }
