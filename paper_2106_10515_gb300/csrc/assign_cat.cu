@@ -264,10 +264,11 @@ __global__ void k_heavy_masks(int64_t k, const int64_t *__restrict__ coff, const
 // (The dense path: every centre is scanned per set.  It serves the sets
 // with more items than the tiled kernels take;
 // rows lists them, na_fix >= 0 replaces |A| by a fixed size.)
+template <int MW>  // mask words per centre
 __global__ void __launch_bounds__(256) k_assign_jaccard(
     int64_t n, const int64_t *__restrict__ off, const uint32_t *__restrict__ items, int64_t k,
     const int32_t *__restrict__ clen, const uint64_t *__restrict__ cmask, const uint32_t *__restrict__ hv_item,
-    const int16_t *__restrict__ hv_bit, int nheavy, int HW, const uint32_t *__restrict__ post_item,
+    const int16_t *__restrict__ hv_bit, int nheavy, const uint32_t *__restrict__ post_item,
     const int64_t *__restrict__ post_off, int64_t n_post_items, const uint32_t *__restrict__ post_centre,
     int32_t *__restrict__ counts, int32_t *__restrict__ labels, const int32_t *__restrict__ rows,
     const unsigned long long *__restrict__ n_rows, int na_fix) {
@@ -280,13 +281,15 @@ __global__ void __launch_bounds__(256) k_assign_jaccard(
         const int64_t i = rows ? (int64_t)rows[ii] : ii;
         const int64_t s = off[i], e = off[i + 1];
         const int64_t na = na_fix >= 0 ? na_fix : e - s;
-        uint64_t am[JX_HW] = {};
+        uint64_t am[MW] = {};
         // light items: binary search in the sorted item list of the index
         for (int64_t p = s + lane; p < e; p += 32) {
             const uint32_t it = items[p];
             const int hb = heavy_bit(it, hv_item, hv_bit, nheavy);
             if (hb >= 0) {
-                am[hb >> 6] |= 1ull << (hb & 63);
+#pragma unroll
+                for (int w = 0; w < MW; w++)
+                    if (hb >> 6 == w) am[w] |= 1ull << (hb & 63);
                 continue;
             }
             int64_t lo = 0, hi = n_post_items;
@@ -299,7 +302,7 @@ __global__ void __launch_bounds__(256) k_assign_jaccard(
                 for (int64_t q = post_off[lo]; q < post_off[lo + 1]; q++) atomicAdd(&cnt[post_centre[q]], 1);
         }
 #pragma unroll
-        for (int w = 0; w < JX_HW; w++)
+        for (int w = 0; w < MW; w++)
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) am[w] |= __shfl_xor_sync(0xffffffffu, am[w], o);
         __syncwarp();
@@ -308,7 +311,8 @@ __global__ void __launch_bounds__(256) k_assign_jaccard(
         int bj = 0x7FFFFFFF;
         for (int64_t j = lane; j < k; j += 32) {
             int64_t in = cnt[j];
-            for (int w = 0; w < HW; w++) in += __popcll(am[w] & cmask[j * HW + w]);
+#pragma unroll
+            for (int w = 0; w < MW; w++) in += __popcll(am[w] & cmask[j * MW + w]);
             cnt[j] = 0;
             const int64_t un = na + clen[j] - in;
             const int64_t num = un ? in : 0, den = un ? un : 1;
@@ -368,9 +372,9 @@ __global__ void __launch_bounds__(256) k_assign_jaccard(
 //  k_jac_count (those sets): only the most frequent items stay out, 64 to 64
 //    JX_HW of them (jx_heavy_words), and every centre is scored, lane per centre.
 // Sets with more than MAXI items are listed for the dense path.
-// 2,000,000 sets of 59 items against 47,686 centres (mean 58 items): the
+// 2,000,000 sets of 59 items against 46,553 centres (mean 58 items): the
 // counters get 3,200 increments per set instead of 28,600, and the two passes
-// take 44 + 37 ms; scoring every pair took 173 ms.  500,000 DOPH rows of 400
+// take 41 + 23 ms; scoring every pair took 173 ms.  500,000 DOPH rows of 400
 // tokens against 425 centres: 4.5 + 5.0 ms, before 31 ms.
 constexpr int JX_WARPS = 8;
 constexpr int JX_THREADS = 32 * JX_WARPS;
@@ -461,11 +465,16 @@ __global__ void k_freq_list(int nfreq, int nheavy, const int64_t *__restrict__ f
 // Mask words of the heaviest items (ord: by posting list) that pay in the second
 // pass.  64 more items in the mask cost a load and a popcount per centre, and save
 // a set the counter increments of those it holds, about k sum (len / k)^2 when sets
-// resemble centres: they pay from a quarter of an increment per centre on.  2M
-// sets, k = 47,686 (0.28 for a second word, 0.11 for a third): 81 ms with one word,
-// 78 with two; 200,000 sets of 60 of 1,500 items, k = 2,605 (0.17) 2.49 and 2.57; of 100
-// of 600 items, k = 744 (2.2 and 2.0) 4.6 with one, 4.1 with three.
-int jx_heavy_words(const std::vector<int64_t> &rs, const std::vector<int32_t> &ord, int nfreq, int64_t k) {
+// resemble centres.  Second pass with one, two and three words, the sum for the
+// second word in brackets: 200,000 sets of 60 of 300 items, k = 674 (2.9) 1.00, 0.91
+// and 0.75 ms; of 100 of 600, k = 605 (2.5) 1.24, 1.22, 1.07; of 60 of 500, k = 3,057 (1.06)
+// 3.08, 3.45, 3.28.  With more than a tile of centres they pay earlier: 300,000 of 60 of
+// 500, k = 12,796 (1.07) 21.2, 20.4, 18.8; 200,000 of 40 of 400, k = 10,420 (0.72) 8.6, 8.2, 7.8;
+// of 60 of 700, k = 12,299 (0.58) 9.97, 10.15, 9.86; 2M sets, k = 46,553 (0.28) 22.9, 24.3, 27.4.
+// Wide sets, whose loop over the items costs more: 100,000 of 300 of 2,000, k = 177 (2.5)
+// 1.14, 1.45, 1.46; of 300 of 1,200, k = 1,864 (4.9) 1.79, 1.94, 1.83.
+int jx_heavy_words(const std::vector<int64_t> &rs, const std::vector<int32_t> &ord, int nfreq, int64_t k, bool narrow) {
+    if (!narrow) return 1;
     int words = 1;
     for (; words < JX_HW && 64 * words < nfreq; words++) {
         double sum = 0.0;
@@ -473,7 +482,7 @@ int jx_heavy_words(const std::vector<int64_t> &rs, const std::vector<int32_t> &o
             const double len = (double)(rs[ord[q] + 1] - rs[ord[q]]) / (double)k;
             sum += len * len;
         }
-        if (sum < 0.25) break;
+        if (sum < (k > Jx<true>::KT ? 0.65 : 1.5)) break;
     }
     return words;
 }
@@ -516,10 +525,16 @@ struct JxArgs {
 };
 
 // Counts one tile: every item of the warp's set adds one to the counter of
-// each centre of its posting list there.  The lanes take 32 items at a time; a
-// prefix sum of their range lengths turns the ranges into one run of entries,
-// walked 32 at a time with every lane busy (a range is 16 entries on
-// average).  Returns the lane's largest (count << 16 | counter) it produced.
+// each centre of its posting list there.  The lanes take 32 items at a time.
+// Ranges of JX_LONG entries and more are walked one after the other, lane per
+// entry.  A prefix sum turns the shorter ones into one run of entries, walked 32
+// at a time with every lane busy (a range is 16 entries on average), at six
+// shuffles a step to find each lane's range.  With those steps for long ranges too
+// the passes over 200,000 sets of 40 of 400 items, k = 10,420, took 22.1 ms, 8.9
+// this way; over 2M sets of 59 of 64,000, k = 46,553: 81.5 and 63.6.  Lines of 32 and
+// 64 measured the same, but for 100 of 600 items, k = 339: 1.5 and 1.8 ms.
+// Returns the lane's largest (count << 16 | counter) it produced.
+constexpr int JX_LONG = 32;
 template <class C>
 __device__ __forceinline__ uint32_t jx_count(uint32_t *cw, const int32_t *ridx, int ni, int t, const JxArgs &A) {
     const int lane = threadIdx.x & 31, ld = A.ntiles + 1;
@@ -531,6 +546,18 @@ __device__ __forceinline__ uint32_t jx_count(uint32_t *cw, const int32_t *ridx, 
             ps = A.tile_off[(int64_t)r * ld + t];
             len = A.tile_off[(int64_t)r * ld + t + 1] - ps;
         }
+        auto add = [&](uint32_t cc) {
+            const int sh = (cc & ((1 << C::LG) - 1)) * C::CBITS;
+            const uint32_t old = atomicAdd(&cw[cc >> C::LG], 1u << sh);
+            lm = max(lm, (((old >> sh) & C::CMASK) << 16) + 65536u + cc);
+        };
+        for (uint32_t m = __ballot_sync(0xffffffffu, len >= JX_LONG); m; m &= m - 1) {
+            const int src = __ffs((int)m) - 1;
+            const int at = __shfl_sync(0xffffffffu, ps, src), ln = __shfl_sync(0xffffffffu, len, src);
+#pragma unroll 4
+            for (int e = lane; e < ln; e += 32) add(A.post_local[at + e]);
+        }
+        if (len >= JX_LONG) len = 0;
         int inc = len;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -547,12 +574,7 @@ __device__ __forceinline__ uint32_t jx_count(uint32_t *cw, const int32_t *ridx, 
             for (int o = 16; o > 0; o >>= 1)
                 if (__shfl_sync(0xffffffffu, ex, src + o) <= e) src += o;
             const int at = __shfl_sync(0xffffffffu, base, src) + e;
-            if (e < tot) {
-                const uint32_t cc = A.post_local[at];
-                const int sh = (cc & ((1 << C::LG) - 1)) * C::CBITS;
-                const uint32_t old = atomicAdd(&cw[cc >> C::LG], 1u << sh);
-                lm = max(lm, (((old >> sh) & C::CMASK) << 16) + 65536u + cc);
-            }
+            if (e < tot) add(A.post_local[at]);
         }
     }
     return lm;
@@ -701,8 +723,8 @@ __global__ void __launch_bounds__(JX_THREADS, 3) k_jac_prune(JxArgs A, const uin
     }
 }
 
-template <bool NARROW, int MW>  // MW: mask words per centre, at least HW
-__global__ void __launch_bounds__(JX_THREADS, 3) k_jac_count(JxArgs A, const uint64_t *__restrict__ cmask, int HW,
+template <bool NARROW, int MW>  // MW: mask words per centre
+__global__ void __launch_bounds__(JX_THREADS, 3) k_jac_count(JxArgs A, const uint64_t *__restrict__ cmask,
                                                              const int32_t *__restrict__ fq_list,
                                                              const int4 *__restrict__ rows,
                                                              const unsigned long long *__restrict__ n_rows) {
@@ -730,7 +752,7 @@ __global__ void __launch_bounds__(JX_THREADS, 3) k_jac_count(JxArgs A, const uin
                 const int hb = -2 - r;
 #pragma unroll
                 for (int h = 0; h < MW; h++)
-                    if (h < HW && hb >> 6 == h) am[h] |= 1ull << (hb & 63);
+                    if (hb >> 6 == h) am[h] |= 1ull << (hb & 63);
                 r = fq_list[hb];
             }
             ridx[p] = r;
@@ -754,8 +776,7 @@ __global__ void __launch_bounds__(JX_THREADS, 3) k_jac_count(JxArgs A, const uin
             for (int cc = lane; cc < nc; cc += 32) {
                 uint32_t in = (cw[cc >> C::LG] >> ((cc & ((1 << C::LG) - 1)) * C::CBITS)) & C::CMASK;
 #pragma unroll
-                for (int h = 0; h < MW; h++)
-                    if (h < HW) in += __popcll(am[h] & cmask[(c0 + cc) * (MW == 1 ? 1 : HW) + h]);
+                for (int h = 0; h < MW; h++) in += __popcll(am[h] & cmask[(c0 + cc) * MW + h]);
                 if (in >= need) best.push(in, na + (uint32_t)A.clen[c0 + cc] - in, (int)(c0 + cc));
             }
             best.warp_merge();
@@ -970,12 +991,23 @@ geek_status jaccard_core(geek_ctx *ctx, Scratch &scr, const int64_t *off, const 
     int64_t ni = 0;
     GK_CUDA(ctx, cudaMemcpyAsync(&ni, nr_dev, 8, cudaMemcpyDeviceToHost, st));
     GK_CUDA(ctx, cudaStreamSynchronize(st));
+    unsigned long long h_amax = 0, *d_amax;  // items of the largest set
+    GK_TRY(scr.alloc(&d_amax, 1));
+    GK_CUDA(ctx, cudaMemsetAsync(d_amax, 0, sizeof(unsigned long long), st));
+    if (na_fix < 0 && n > 0) {
+        GK_COUNT();
+        k_max_len<<<G(ctx, n), 256, 0, st>>>(n, off, d_amax);
+        GK_LAUNCH(ctx);
+    }
     // heavy items: the (up to 64 JX_HW) longest posting lists of length >= 2,
     // chosen on the host from the run lengths; the others keep posting lists
     std::vector<int64_t> hrs(ni + 1);
     GK_CUDA(ctx, cudaMemcpyAsync(hrs.data(), rs, 8 * (ni + 1), cudaMemcpyDeviceToHost, st));
     std::vector<int32_t> ord(ni);
+    GK_CUDA(ctx, cudaMemcpyAsync(&h_amax, d_amax, sizeof h_amax, cudaMemcpyDeviceToHost, st));
     GK_CUDA(ctx, cudaStreamSynchronize(st));
+    // the narrow kernels when no set has more than their MAXI items
+    const bool narrow = (na_fix >= 0 ? (int64_t)na_fix : (int64_t)h_amax) <= Jx<true>::MAXI;
     for (int64_t r = 0; r < ni; r++) ord[r] = (int32_t)r;
     const int64_t fmax = std::min<int64_t>(64 * JX_MW, ni);
     std::partial_sort(ord.begin(), ord.begin() + fmax, ord.end(), [&](int32_t a, int32_t b) {
@@ -984,7 +1016,7 @@ geek_status jaccard_core(geek_ctx *ctx, Scratch &scr, const int64_t *off, const 
     });
     int nfreq = 0;  // frequent items, by rank: the first nheavy of them are the heavy ones
     while (nfreq < fmax && hrs[ord[nfreq] + 1] - hrs[ord[nfreq]] >= 2) nfreq++;
-    const int nheavy = std::min(nfreq, 64 * jx_heavy_words(hrs, ord, nfreq, k));
+    const int nheavy = std::min(nfreq, 64 * jx_heavy_words(hrs, ord, nfreq, k, narrow));
     const int HW = (nheavy + 63) / 64, FW = (nfreq + 63) / 64;
     std::vector<int32_t> fq_runs(ord.begin(), ord.begin() + nfreq);
     std::sort(fq_runs.begin(), fq_runs.end());
@@ -1073,29 +1105,18 @@ geek_status jaccard_core(geek_ctx *ctx, Scratch &scr, const int64_t *off, const 
     GK_LAUNCH(ctx);
     if (nci > 0x7FFFFFFFLL) return set_error(ctx, GEEK_ERR_UNSUPPORTED, "more than 2^31 centre items");
     // the tiled kernel compares fractions in 32 bits: |A| <= MAXI (else the
-    // dense path) and every |C| below 2^15; the narrow variant when no set has
-    // more than its MAXI items
+    // dense path) and every |C| below 2^15
     bool tiled_ok = na_fix < 32768;
-    unsigned long long h_amax = 0, *d_amax;
     uint64_t h_last = 0;  // the largest item of any centre
-    GK_TRY(scr.alloc(&d_amax, 1));
-    GK_CUDA(ctx, cudaMemsetAsync(d_amax, 0, sizeof(unsigned long long), st));
-    if (na_fix < 0 && n > 0) {
-        GK_COUNT();
-        k_max_len<<<G(ctx, n), 256, 0, st>>>(n, off, d_amax);
-        GK_LAUNCH(ctx);
-    }
     {
         std::vector<int64_t> hco(k + 1);
         GK_CUDA(ctx, cudaMemcpyAsync(hco.data(), coff, 8 * (k + 1), cudaMemcpyDeviceToHost, st));
-        GK_CUDA(ctx, cudaMemcpyAsync(&h_amax, d_amax, sizeof h_amax, cudaMemcpyDeviceToHost, st));
         // the items ascend with the runs: the last entry holds the largest
         if (nci > 0)
             GK_CUDA(ctx, cudaMemcpyAsync(&h_last, ikey + nci - 1, sizeof h_last, cudaMemcpyDeviceToHost, st));
         GK_CUDA(ctx, cudaStreamSynchronize(st));
         for (int64_t j = 0; j < k && tiled_ok; j++) tiled_ok = hco[j + 1] - hco[j] < 32768;
     }
-    const bool narrow = (na_fix >= 0 ? (int64_t)na_fix : (int64_t)h_amax) <= Jx<true>::MAXI;
     int32_t *ovf;
     unsigned long long *n_ovf;
     GK_TRY(scr.alloc(&ovf, n));
@@ -1162,12 +1183,12 @@ geek_status jaccard_core(geek_ctx *ctx, Scratch &scr, const int64_t *off, const 
             GK_COUNT();
             prune<<<grid(0), JX_THREADS, smem, st>>>(A, fmask, FW, ovf, n_ovf, hard, n_hard);
             GK_COUNT();
-            count<<<grid(1), JX_THREADS, smem, st>>>(A, cmask, HW, fq_list, hard, n_hard);
+            count<<<grid(1), JX_THREADS, smem, st>>>(A, cmask, fq_list, hard, n_hard);
             GK_LAUNCH(ctx);
             return GEEK_OK;
         };
-        if (narrow) GK_TRY(run(k_jac_prune<true>, HW > 1 ? k_jac_count<true, JX_HW> : k_jac_count<true, 1>));
-        else GK_TRY(run(k_jac_prune<false>, HW > 1 ? k_jac_count<false, JX_HW> : k_jac_count<false, 1>));
+        if (narrow) GK_TRY(run(k_jac_prune<true>, HW > 2 ? k_jac_count<true, 3> : HW > 1 ? k_jac_count<true, 2> : k_jac_count<true, 1>));
+        else GK_TRY(run(k_jac_prune<false>, HW > 2 ? k_jac_count<false, 3> : HW > 1 ? k_jac_count<false, 2> : k_jac_count<false, 1>));
         GK_LAUNCH(ctx);
         }
     }
@@ -1181,8 +1202,9 @@ geek_status jaccard_core(geek_ctx *ctx, Scratch &scr, const int64_t *off, const 
         GK_TRY(scr.alloc(&counts, (size_t)nwarps * k));
         GK_CUDA(ctx, cudaMemsetAsync(counts, 0, sizeof(int32_t) * nwarps * k, st));
         GK_COUNT();
-        k_assign_jaccard<<<blocks, 256, 0, st>>>(n, off, items, k, clen, cmask, hv_item, hv_bit, nheavy, HW, d_litem,
-                                                 d_loff, h_nlight, d_lcentre, counts, labels, ovf, n_ovf, na_fix);
+        auto *dense = HW > 2 ? k_assign_jaccard<3> : HW > 1 ? k_assign_jaccard<2> : k_assign_jaccard<1>;
+        dense<<<blocks, 256, 0, st>>>(n, off, items, k, clen, cmask, hv_item, hv_bit, nheavy, d_litem, d_loff, h_nlight,
+                                      d_lcentre, counts, labels, ovf, n_ovf, na_fix);
         GK_LAUNCH(ctx);
     }
     if (stats) stats->n_recheck_rows = (int64_t)h_ovf;  // sets decided by the dense path
