@@ -366,9 +366,12 @@ __global__ void __launch_bounds__(256) k_assign_jaccard(
 //    threshold with one add and mask per word and scores the few that pass
 //    exactly (64-bit cross products, larger fraction then smaller index; with
 //    no positive J the label is 0).  The centre of a tile's largest counter
-//    gives the first bound; a tile met while the threshold is not positive is
-//    taken again at the end, and if it still is not (a set unlike every
-//    centre), the set goes to the second pass.
+//    gives the first bound; a tile met while the threshold is not positive, or
+//    so near the mean counter that most centres would be scored, is taken
+//    again at the end, and if it still is (a set unlike every centre), the set
+//    goes to the second pass.  200,000 sets of 60 of 700 items, k = 12,299: this pass
+//    8.7 ms with the sign alone, 3.9 with the mean, the second pass 10.0 either way;
+//    2M sets of 59 of 64,000 items: 40.7 and 41.2, 23.
 //  k_jac_count (those sets): only the most frequent items stay out, 64 to 64
 //    JX_HW of them (jx_heavy_words), and every centre is scored, lane per centre.
 // Sets with more than MAXI items are listed for the dense path.
@@ -533,10 +536,12 @@ struct JxArgs {
 // the passes over 200,000 sets of 40 of 400 items, k = 10,420, took 22.1 ms, 8.9
 // this way; over 2M sets of 59 of 64,000, k = 46,553: 81.5 and 63.6.  Lines of 32 and
 // 64 measured the same, but for 100 of 600 items, k = 339: 1.5 and 1.8 ms.
-// Returns the lane's largest (count << 16 | counter) it produced.
+// Returns the lane's largest (count << 16 | counter) it produced, and adds the
+// entries of the lane's items to sum.
 constexpr int JX_LONG = 32;
 template <class C>
-__device__ __forceinline__ uint32_t jx_count(uint32_t *cw, const int32_t *ridx, int ni, int t, const JxArgs &A) {
+__device__ __forceinline__ uint32_t jx_count(uint32_t *cw, const int32_t *ridx, int ni, int t, const JxArgs &A,
+                                             int &sum) {
     const int lane = threadIdx.x & 31, ld = A.ntiles + 1;
     uint32_t lm = 0;
     for (int q0 = 0; q0 < ni; q0 += 32) {
@@ -546,6 +551,7 @@ __device__ __forceinline__ uint32_t jx_count(uint32_t *cw, const int32_t *ridx, 
             ps = A.tile_off[(int64_t)r * ld + t];
             len = A.tile_off[(int64_t)r * ld + t + 1] - ps;
         }
+        sum += len;
         auto add = [&](uint32_t cc) {
             const int sh = (cc & ((1 << C::LG) - 1)) * C::CBITS;
             const uint32_t old = atomicAdd(&cw[cc >> C::LG], 1u << sh);
@@ -656,6 +662,12 @@ __global__ void __launch_bounds__(JX_THREADS, 3) k_jac_prune(JxArgs A, const uin
         // tiles met without a positive threshold, taken again at the end
         uint64_t again = 0;
         bool hard = false;
+        // a threshold at most two deviations above the mean counter (as of a Poisson count)
+        auto weak = [](int need, float entries, int64_t centres) {
+            const float d = (float)need * (float)centres - entries;
+            return d <= 0.0f || d * d <= 4.0f * entries * (float)centres;
+        };
+        float total = 0.0f;
         for (int tt = 0, t = 0; !hard; tt++) {
             const bool second = tt >= A.ntiles;
             if (!second) {
@@ -668,22 +680,30 @@ __global__ void __launch_bounds__(JX_THREADS, 3) k_jac_prune(JxArgs A, const uin
             const int64_t c0 = (int64_t)t * A.kt;
             const uint32_t cmin = (uint32_t)A.tile_min[t];
             int need = (int)best.need(na, cmin) - hcnt;
-            if (second && need <= 0) {
+            if (second && weak(need, total, A.k)) {
                 hard = true;
                 break;
             }
-            const uint32_t lm = __reduce_max_sync(0xffffffffu, jx_count<C>(cw, ridx, ni, t, A));
+            int sum = 0;
+            const uint32_t lm = __reduce_max_sync(0xffffffffu, jx_count<C>(cw, ridx, ni, t, A, sum));
             __syncwarp();
-            if (need <= 0) {
+            bool low = false;
+            if (!second) {
+                sum = __reduce_add_sync(0xffffffffu, sum);
+                total += (float)sum;
+                low = weak(need, (float)sum, min((int64_t)A.kt, A.k - c0));
+            }
+            if (low) {
                 // the centre of the tile's largest counter as a first bound
                 if (lm >> 16) score(c0 + (lm & 0xFFFFu), lm >> 16, best);
                 need = (int)best.need(na, cmin) - hcnt;
-                if (need <= 0) {
+                low = weak(need, (float)sum, min((int64_t)A.kt, A.k - c0));
+                if (low) {
                     if (t < 64) again |= 1ull << t;
                     else hard = true;
                 }
             }
-            if (need <= 0 || need > (int)(lm >> 16)) {  // taken again, or above every counter
+            if (low || need > (int)(lm >> 16)) {  // taken again, or above every counter
                 for (int v = 0; v < nv; v++) c4[v * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
                 __syncwarp();
                 continue;
@@ -768,7 +788,8 @@ __global__ void __launch_bounds__(JX_THREADS, 3) k_jac_count(JxArgs A, const uin
         best.j = row.w;
         for (int t = 0; t < A.ntiles; t++) {
             const int64_t c0 = (int64_t)t * A.kt;
-            jx_count<C>(cw, ridx, ni, t, A);
+            int sum = 0;
+            jx_count<C>(cw, ridx, ni, t, A, sum);
             __syncwarp();
             const uint32_t need = best.need(na, (uint32_t)A.tile_min[t]);
             const int nc = (int)min((int64_t)A.kt, A.k - c0);

@@ -1,5 +1,5 @@
 """GPU: Jaccard assignment of sets over a small universe, where a tile of centres holds
-an item hundreds of times: the labels, and that its counters fill at a lane per entry."""
+an item hundreds of times: the labels, and the rate of the passes."""
 import numpy as np
 import pytest
 import torch
@@ -29,7 +29,7 @@ def _case(geek, n, base, size, universe, keep):
 
 
 @pytest.mark.parametrize("n,base,size,universe", [(20_000, 300, 40, 400), (40_000, 1_000, 60, 500),
-                                                  (20_000, 200, 140, 900), (60_000, 2_000, 40, 400)])
+                                                  (20_000, 200, 140, 900), (30_000, 1_000, 60, 700), (60_000, 2_000, 40, 400)])
 def test_labels_are_the_exact_argmax(geek, n, base, size, universe):
     ctx, data, bk, seeds, off, items = _case(geek, n, base, size, universe, 0.9)
     labels = torch.empty(n, dtype=torch.int32, device="cuda")
@@ -42,9 +42,12 @@ def test_labels_are_the_exact_argmax(geek, n, base, size, universe):
     assert np.array_equal(labels.cpu().numpy()[f:], ref)
 
 
-def test_pairs_per_second(geek):
+# (set, centre) pairs a second: 2.6e11, or 0.95e11 with a search for every entry's list; and
+# 1.77e11, or 1.31e11 with nearly every centre of a tile scored before its set is set aside
+@pytest.mark.parametrize("size,universe,least", [(40, 400, 1.6e11), (60, 700, 1.5e11)])
+def test_pairs_per_second(geek, size, universe, least):
     n = 200_000
-    ctx, data, bk, seeds, _, _ = _case(geek, n, 1_000, 40, 400, 0.85)
+    ctx, data, bk, seeds, _, _ = _case(geek, n, 1_000, size, universe, 0.85)
     assert seeds.k > 8_192
     labels, ms = torch.empty(n, dtype=torch.int32, device="cuda"), []
     ctx.timing(True)
@@ -53,5 +56,4 @@ def test_pairs_per_second(geek):
         ctx.assign_ex(data, bk, seeds, labels)
         ms.append(ctx.timing_get("kernel.jaccard")[0])
     ctx.timing(False)
-    # 2.6e11 (set, centre) pairs a second; 0.95e11 with a search for every entry's list
-    assert n * seeds.k / (min(ms[1:]) * 1e-3) > 1.6e11
+    assert n * seeds.k / (min(ms[1:]) * 1e-3) > least
