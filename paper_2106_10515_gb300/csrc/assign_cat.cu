@@ -373,12 +373,16 @@ __global__ void __launch_bounds__(256) k_assign_jaccard(
 //    8.7 ms with the sign alone, 3.9 with the mean, the second pass 10.0 either way;
 //    2M sets of 59 of 64,000 items: 40.7 and 41.2, 23.
 //  k_jac_count (those sets): only the most frequent items stay out, 64 to 64
-//    JX_HW of them (jx_heavy_words), and every centre is scored, lane per centre.
+//    JX_HW of them (jx_heavy_words), and every centre is scored, lane per centre
+//    (k_jac_count8: thread per four centres, eight sets).
 // Sets with more than MAXI items are listed for the dense path.
 // 2,000,000 sets of 59 items against 46,553 centres (mean 58 items): the
 // counters get 3,200 increments per set instead of 28,600, and the two passes
-// take 41 + 23 ms; scoring every pair took 173 ms.  500,000 DOPH rows of 400
+// take 41 + 22 ms; scoring every pair took 173 ms.  500,000 DOPH rows of 400
 // tokens against 425 centres: 4.5 + 5.0 ms, before 31 ms.
+// centres from which the second pass scores by blocks (k_jac_count8): k = 3,020 0.99 ms by
+// warps, 1.29 by blocks; 4,279 0.090, 0.129; 5,831 4.11, 3.79; 6,393 5.21, 4.69; 7,762 1.06, 0.79
+constexpr int JX_BLOCKS = 5120;
 constexpr int JX_WARPS = 8;
 constexpr int JX_THREADS = 32 * JX_WARPS;
 constexpr int JX_MW = 8;  // mask words of the frequent items k_jac_prune leaves out
@@ -809,6 +813,119 @@ __global__ void __launch_bounds__(JX_THREADS, 3) k_jac_count(JxArgs A, const uin
     }
 }
 
+// The same for narrow sets and one mask word, eight sets of a block scored together,
+// thread per counter word: a centre's mask and size are loaded once for eight
+// sets.  A warp of k_jac_count loads them for its one set, from L2 once the masks of
+// k centres no longer fit the L1 beside the counters: 1.1M sets of 59 items, k = 6,993,
+// 7.2 ms, here 5.4; 180,242 of 21, k = 10,817, 3.3 and 2.2; 2M of 59, k = 46,553, 23.0 and 21.5;
+// where increments outweigh the scoring it is the other way, the warps of a block wait
+// for one another: 300,000 of 59, k = 19,375, 5.5 and 5.8.
+__global__ void __launch_bounds__(JX_THREADS, 3) k_jac_count8(JxArgs A, const uint64_t *__restrict__ cmask,
+                                                              const int32_t *__restrict__ fq_list,
+                                                              const int4 *__restrict__ rows,
+                                                              const unsigned long long *__restrict__ n_rows) {
+    using C = Jx<true>;
+    constexpr int V = 1 << C::LG;  // counters of a word
+    extern __shared__ uint4 jx_smem[];
+    __shared__ int4 s_row[JX_WARPS];  // the sets and their best centres so far
+    __shared__ uint64_t s_am[JX_WARPS];
+    __shared__ uint32_t s_na[JX_WARPS];
+    __shared__ uint32_t s_best[JX_WARPS][JX_WARPS][3];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int nv = A.kt / C::STEP;
+    uint4 *c4 = jx_smem + (size_t)w * nv * 32;
+    uint32_t *cw = reinterpret_cast<uint32_t *>(c4);
+    const uint32_t *all = reinterpret_cast<const uint32_t *>(jx_smem);
+    int32_t *ridx = reinterpret_cast<int32_t *>(jx_smem + (size_t)JX_WARPS * nv * 32) + w * C::MAXI;
+    for (int v = lane; v < nv * 32; v += 32) c4[v] = make_uint4(0u, 0u, 0u, 0u);
+    const int64_t nr = (int64_t)*n_rows;
+    for (int64_t q0 = (int64_t)blockIdx.x * JX_WARPS; q0 < nr; q0 += (int64_t)gridDim.x * JX_WARPS) {
+        const bool on = q0 + w < nr;
+        const int4 row = on ? rows[q0 + w] : make_int4(-1, 0, 1, 0x7FFFFFFF);
+        const int64_t s0 = on ? A.off[row.x] : 0;
+        const int ni = on ? (int)(A.off[row.x + 1] - s0) : 0;  // <= MAXI: the first pass listed it
+        uint64_t am = 0;
+        for (int p = lane; p < ni; p += 32) {
+            int32_t r = A.X.find(A.items[s0 + p]);
+            if (r < -1) {
+                const int hb = -2 - r;
+                if (hb < 64) am |= 1ull << hb;
+                r = fq_list[hb];
+            }
+            ridx[p] = r;
+        }
+        am = ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(am >> 32)) << 32) |
+             __reduce_or_sync(0xffffffffu, (uint32_t)am);
+        if (lane == 0) {
+            s_row[w] = row;
+            s_am[w] = am;
+            s_na[w] = (uint32_t)(A.na_fix >= 0 ? A.na_fix : ni);
+        }
+        __syncthreads();
+        JxBest best[JX_WARPS];
+        uint64_t ams[JX_WARPS];
+        uint32_t na[JX_WARPS];
+#pragma unroll
+        for (int u = 0; u < JX_WARPS; u++) {
+            best[u].n = (uint32_t)s_row[u].y;
+            best[u].d = (uint32_t)s_row[u].z;
+            best[u].j = s_row[u].w;
+            ams[u] = s_am[u];
+            na[u] = s_na[u];
+        }
+        for (int t = 0; t < A.ntiles; t++) {
+            const int64_t c0 = (int64_t)t * A.kt;
+            int sum = 0;
+            jx_count<C>(cw, ridx, ni, t, A, sum);
+            __syncthreads();
+            const int nc = (int)min((int64_t)A.kt, A.k - c0);
+            for (int x = threadIdx.x; x * V < nc; x += JX_THREADS) {
+                // whole words: masks and sizes have room for the last one's
+                uint64_t cm[V];
+                int cl[V];
+#pragma unroll
+                for (int v = 0; v < V; v += 2) {
+                    const ulonglong2 m2 = *reinterpret_cast<const ulonglong2 *>(cmask + c0 + x * V + v);
+                    const int2 l2 = *reinterpret_cast<const int2 *>(A.clen + c0 + x * V + v);
+                    cm[v] = m2.x;
+                    cm[v + 1] = m2.y;
+                    cl[v] = l2.x;
+                    cl[v + 1] = l2.y;
+                }
+#pragma unroll
+                for (int u = 0; u < JX_WARPS; u++) {
+                    const uint32_t word = all[(size_t)u * nv * 128 + x];
+#pragma unroll
+                    for (int v = 0; v < V; v++) {
+                        const uint32_t in = ((word >> (v * C::CBITS)) & C::CMASK) + (uint32_t)__popcll(ams[u] & cm[v]);
+                        const uint32_t un = na[u] + (uint32_t)cl[v] - in;
+                        if (in * best[u].d >= best[u].n * un && x * V + v < nc && in)
+                            best[u].push(in, un, (int)(c0 + x * V + v));
+                    }
+                }
+            }
+            __syncthreads();
+            for (int v = lane; v < nv * 32; v += 32) c4[v] = make_uint4(0u, 0u, 0u, 0u);
+            __syncwarp();
+        }
+#pragma unroll
+        for (int u = 0; u < JX_WARPS; u++) {
+            best[u].warp_merge();
+            if (lane == 0) {
+                s_best[u][w][0] = best[u].n;
+                s_best[u][w][1] = best[u].d;
+                s_best[u][w][2] = (uint32_t)best[u].j;
+            }
+        }
+        __syncthreads();
+        if (on && lane == 0) {
+            JxBest b;
+            for (int u = 0; u < JX_WARPS; u++) b.push(s_best[w][u][0], s_best[w][u][1], (int)s_best[w][u][2]);
+            A.labels[row.x] = b.n > 0 ? b.j : 0;
+        }
+    }
+}
+
 }  // namespace
 
 // Majority set of each group of sets: items present in more than half of
@@ -1116,8 +1233,8 @@ geek_status jaccard_core(geek_ctx *ctx, Scratch &scr, const int64_t *off, const 
     }
     uint64_t *cmask, *fmask;
     int32_t *clen, *counts;
-    GK_TRY(scr.alloc(&cmask, (size_t)k * std::max(HW, 1)));
-    GK_TRY(scr.alloc(&clen, k));
+    GK_TRY(scr.alloc(&cmask, (size_t)k * std::max(HW, 1) + 4));  // k_jac_count8 reads whole counter words
+    GK_TRY(scr.alloc(&clen, k + 4));
     GK_COUNT();
     k_heavy_masks<JX_HW><<<G(ctx, k), 256, 0, st>>>(k, coff, citems, hv_item, hv_bit, nheavy, HW, cmask, clen);
     GK_TRY(scr.alloc(&fmask, (size_t)k * std::max(FW, 1)));
@@ -1208,8 +1325,12 @@ geek_status jaccard_core(geek_ctx *ctx, Scratch &scr, const int64_t *off, const 
             GK_LAUNCH(ctx);
             return GEEK_OK;
         };
-        if (narrow) GK_TRY(run(k_jac_prune<true>, HW > 2 ? k_jac_count<true, 3> : HW > 1 ? k_jac_count<true, 2> : k_jac_count<true, 1>));
-        else GK_TRY(run(k_jac_prune<false>, HW > 2 ? k_jac_count<false, 3> : HW > 1 ? k_jac_count<false, 2> : k_jac_count<false, 1>));
+        if (narrow)
+            GK_TRY(run(k_jac_prune<true>, HW > 2           ? k_jac_count<true, 3>
+                                          : HW > 1         ? k_jac_count<true, 2>
+                                          : k >= JX_BLOCKS ? k_jac_count8
+                                                           : k_jac_count<true, 1>));
+        else GK_TRY(run(k_jac_prune<false>, k_jac_count<false, 1>));
         GK_LAUNCH(ctx);
         }
     }

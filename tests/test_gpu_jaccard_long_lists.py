@@ -57,3 +57,46 @@ def test_pairs_per_second(geek, size, universe, least):
         ms.append(ctx.timing_get("kernel.jaccard")[0])
     ctx.timing(False)
     assert n * seeds.k / (min(ms[1:]) * 1e-3) > least
+
+
+@pytest.mark.parametrize("k", [5_000, 5_119, 5_120, 5_121, 8_191, 8_193, 9_001])
+@pytest.mark.parametrize("universe,size", [(3_000, 9), (60, 12)])
+def test_scoring_by_blocks_of_sets(geek, k, universe, size):
+    rng = np.random.default_rng(k + universe)
+    base = {tuple(sorted(rng.choice(universe, size, replace=False))) for _ in range(k)}
+    while len(base) < k:
+        base.add(tuple(sorted(rng.choice(universe, size, replace=False))))
+    base = [np.array(b) for b in base]
+    rows = [b for b in base for _ in range(2)]  # each pair becomes a seed
+    # sets far from every centre, and subsets: 203, not a multiple of a block's eight
+    rows += [np.sort(rng.choice(universe, int(rng.integers(1, 30)), replace=False)) for _ in range(203)]
+    off = np.zeros(len(rows) + 1, np.int64)
+    off[1:] = np.cumsum([r.size for r in rows])
+    items = np.concatenate(rows).astype(np.uint32)
+    ctx = geek.Context(0)
+    u64 = lambda c: geek._dev(rng.integers(0, 1 << 63, c, dtype=np.uint64))  # noqa: E731
+    bk = ctx.hash(data := ctx.sets(geek._dev(off), geek._dev(items.astype(np.int32))), 4, 4, mh_a=u64(16), mh_b=u64(16))
+    seeds = ctx.silk(bk, 2, 4, 2, u64(8), u64(8), u64(2), u64(2))
+    labels = torch.empty(len(rows), dtype=torch.int32, device="cuda")
+    _, cen = ctx.assign_ex(data, bk, seeds, labels)
+    f = len(rows) - 300
+    ref, _, _ = oracle.assign_jaccard(off[f:] - off[f], items[off[f]:], cen["item_off"].cpu().numpy(),
+                                      cen["items"].cpu().numpy().view(np.uint32))
+    assert np.array_equal(labels.cpu().numpy()[f:], ref)
+    if k > 8_000 and universe > 1_000:
+        assert seeds.k > 5_120
+
+
+def test_rate_of_small_sets(geek):
+    n = 200_000
+    ctx, data, bk, seeds, _, _ = _case(geek, n, 1_000, 12, 300, 0.7)
+    assert seeds.k > 5_120
+    labels, ms = torch.empty(n, dtype=torch.int32, device="cuda"), []
+    ctx.timing(True)
+    for _ in range(4):
+        ctx.timing_reset()
+        ctx.assign_ex(data, bk, seeds, labels)
+        ms.append(ctx.timing_get("kernel.jaccard")[0])
+    ctx.timing(False)
+    # 5.5e11 (set, centre) pairs a second with the masks loaded once for eight sets, 3.96e11 by set
+    assert n * seeds.k / (min(ms[1:]) * 1e-3) > 4.7e11
