@@ -380,6 +380,7 @@ __global__ void __launch_bounds__(256) k_assign_jaccard(
 // counters get 3,200 increments per set instead of 28,600, and the two passes
 // take 41 + 22 ms; scoring every pair took 173 ms.  500,000 DOPH rows of 400
 // tokens against 425 centres: 4.5 + 5.0 ms, before 31 ms.
+
 // centres from which the second pass scores by blocks (k_jac_count8): k = 3,020 0.99 ms by
 // warps, 1.29 by blocks; 4,279 0.090, 0.129; 5,831 4.11, 3.79; 6,393 5.21, 4.69; 7,762 1.06, 0.79
 constexpr int JX_BLOCKS = 5120;
